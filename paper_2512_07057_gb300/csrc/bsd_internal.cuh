@@ -39,6 +39,7 @@ constexpr int kMaxColDeg = 16;   // the generic engines' largest column degree b
 constexpr int kMaxBeam = 64;
 constexpr int kSmallMaxCpl = 5;   // the single-warp engine's largest code: 5 words of columns
 constexpr int kSmallMaxRpl = 3;   // and 3 of rows
+constexpr int kSmallRowWords = 8; // words kept per row of H for its stopping rule (kSmallMaxCpl used)
 constexpr int kMaxResults = 64;
 constexpr double kFixScale = 65536.0;   // fixed-point grid 2^-16 for scores and weights
 
@@ -88,8 +89,8 @@ struct DevGraph {
     const uint32_t* scol;  // [3 N], null when the code has no such placement
     const float* sD0;      // [Epad]
     const void* slamE;     // [Epad] in the storage format
-    const uint4* slamh;    // [32 WN] with the placement: per column slot j the bits of Lambda_j and the
-                           // (at most 3) words of column j of H; zero past N
+    const uint32_t* shrow; // [32 ceil(M / 32)][kSmallRowWords] with the placement: the columns of row i of H
+                           // as a bit set (the stopping rule's parities); zero past M
 };
 
 struct DecCfg {

@@ -477,7 +477,7 @@ struct GenericEngine {
     static constexpr bool kPriorStart = true;   // runs from E(0) need no copy of E(0)
     static constexpr bool kPriorSetsSums = true;  // ... nor cleared sums: their first iteration sets them
     G grp;
-    __device__ void load_graph(const DevGraph&) {}
+    __device__ void load_graph(const DevGraph&, const WarpState&) {}
     // E(0) in this engine's message layout (the CSR edge order)
     static __device__ const void* prior_E(const DevGraph& g) { return g.lamE; }
     // the sentinel +L_MAX on every message of the newly fixed node j (at the
@@ -500,9 +500,7 @@ struct GenericEngine {
     {
         for (int j = grp.rank(); j < g.N; j += grp.size()) st.sumllr[j] = 0.f;
     }
-    // (kAtomicStop selects the small engine's form of the stopping rule; the
-    // generic engines have one form)
-    template <bool kPostOut = false, bool kAtomicStop = false>
+    template <bool kPostOut = false>
     __device__ int run(const DevGraph& g, const DecCfg& cfg, const WarpState& st, int max_iters, bool stop,
                        int* success, float* post_out, bool from_prior = false, const AbortCheck& ab = AbortCheck{})
     {
@@ -521,51 +519,113 @@ struct GenericEngine {
 
 // SmallEngine: codes with every column of degree exactly 3, every row of
 // degree exactly RD = 6, N <= 32*CPL, M <= 32*RPL and fewer than 65536 edges
-// -- the bivariate bicycle codes.  A candidate's messages E and D sit at the
-// words of the code's placement (bsd_layout.cu): the pair h of row i at
-// h kPlane + 2 i, so the detector pass moves 32 consecutive pairs per access,
-// and the error pass gathers and scatters through a per-(column, k) word
-// table chosen to put the 32 lanes in 32 distinct banks.  Each lane keeps its
-// columns' words, sum_LLR and mask bits in registers for the warp's lifetime.
-// The stopping rule forms H e^ from the columns of H of the lane's columns
-// with e^_j = 1 and three warp XOR reductions, with no shared-memory atomics
-// (kAtomicStop: XOR of the set columns' rows into shared words instead, which
-// the seed kernel uses: most of its runs stop after one or two iterations,
-// where the reductions' latency is not hidden).  The warp's e^ words stay in
-// registers and are written once, after the last iteration.
-// The detector pass writes D_{i->j} itself for every edge, so the
-// error-node pass gathers one 4-byte message per edge; the ascending-order
-// sums of three messages are formed from min / max / median directly.  Every
-// value it produces is the one GenericEngine produces (same operations, same
-// order; the placement only permutes where a row's edges and a column's
+// -- the bivariate bicycle codes.  A candidate's messages sit at the words of
+// the code's placement (bsd_layout.cu): the pair h of row i at h kPlane + 2 i,
+// so the detector pass moves 32 consecutive pairs per access, and the error
+// pass gathers and scatters through a per-(column, k) word table chosen to
+// put the 32 lanes in 32 distinct banks.  With single-precision storage D is
+// written over E (each word belongs to one row and to one (column, k), so
+// either pass reads its words before it writes them); 16-bit storage keeps D
+// in float beside E.  Each lane keeps its columns' shared-memory addresses,
+// Lambda_j, sum_LLR and its first row's columns in registers.
+//
+// What bounds the iteration: 4 shared-memory transfers per edge (54
+// wavefronts at 100% for 432 edges), and the ALU pipe, which runs min, max,
+// compare, select and logic at 64 lanes per clock (an add or multiply runs on
+// the other pipe at 128).  So the detector pass takes each edge's minimum over
+// the other five directly, with the sign product in the same instruction
+// (min.xorsign.abs: the sign of the result is the xor of the operands'), 15
+// such operations per row of six instead of 13 min/max, 6 compares, 6 selects
+// and 12 logic operations; the cap at L_MAX carries the syndrome sign.  The
+// stopping rule tests the parity of e^ on rows 0..31 from registers and goes on
+// to the others only if these agree with s' (before: XOR of the set columns of
+// H in every column pass and three warp reductions).  k_round on 10^6
+// [[144,12,12]] shots at p = 0.05: 25.9 -> 17.4 ms; with 32 results on 3001
+// shots: 21.3 -> 13.7 ms, 94 cycles per SM and candidate iteration against
+// the 54 of its shared-memory transfers.
+//
+// Every value it produces is the one GenericEngine produces (same operations,
+// same order; the placement only permutes where a row's edges and a column's
 // edges are kept, and neither pass depends on that order).
+__device__ __forceinline__ float xmin(float a, float b)
+{
+    float r;
+    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+// two single-precision operations in one instruction, each rounded to nearest
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+// shared-memory accesses by 32-bit address, kept in program order (the code
+// below loads a step ahead of its stores; the compiler cannot see that the
+// words differ)
+__device__ __forceinline__ float lds(uint32_t a)
+{
+    float r;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(r) : "r"(a) : "memory");
+    return r;
+}
+__device__ __forceinline__ float2 lds2(uint32_t a)
+{
+    float2 r;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "r"(a) : "memory");
+    return r;
+}
+__device__ __forceinline__ void sts(uint32_t a, float v)
+{
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts2(uint32_t a, float2 v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+
 template <int CPL, int RPL, int RD, int P, bool W = false>
 struct SmallEngine {
     using Grp = WarpGroup;
-    static constexpr int kMinBlocks = 2;   // at most 128 registers: two 8-warp blocks per SM
+    // three 8-warp blocks per SM (at most 80 registers): k_round of 10^6
+    // [[144,12,12]] shots at p = 0.05 took 17.4 ms against 18.0 with two
+    // blocks (128 registers) and 18.1 with four (64 registers, 4 bytes spilled)
+    static constexpr int kMinBlocks = 3;
     static constexpr int kMaxThreads = 256;
     static constexpr int kPrec = P;
     static constexpr bool kPriorStart = !W;  // unweighted runs from E(0) start from the table D0
     static constexpr bool kPriorSetsSums = false;
+    static constexpr bool kInPlace = P == 0; // D over E
     WarpGroup grp;
     using S = Store<P>;
     static_assert(RD == 6, "the placement holds rows of degree 6");
-    static_assert(RPL <= 3, "the per-column record holds at most three words of a column of H");
     static constexpr int kPlane = small_plane_stride_rpl(RPL);   // words between a row's pairs
-    uint32_t ci[CPL][3];   // (word << 16) | row of the k-th edge of column lane + 32 c
+    uint32_t ca[CPL][3];   // shared-memory address of the D message on the k-th edge of column lane + 32 c
+    uint32_t hq[CPL];      // the columns of row `lane` of H
     float sum[CPL];
     uint32_t mb;           // bit c: column lane + 32 c is masked or beyond N
 
-    __device__ void load_graph(const DevGraph& g)
+    static __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+    __device__ void load_graph(const DevGraph& g, const WarpState& st)
     {
         const int lane = threadIdx.x & 31;
+        const uint32_t base = saddr(kInPlace ? st.E : (void*)st.D);
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
             const int j = lane + 32 * c;
-            ci[c][0] = ci[c][1] = ci[c][2] = 0u;
+            ca[c][0] = ca[c][1] = ca[c][2] = base;
+            hq[c] = __ldg(g.shrow + (size_t)kSmallRowWords * lane + c);
             if (j < g.N) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) ci[c][k] = __ldg(g.scol + 3 * j + k);
+                for (int k = 0; k < 3; ++k) ca[c][k] = base + 4u * (__ldg(g.scol + 3 * j + k) >> 16);
             }
         }
     }
@@ -581,25 +641,35 @@ struct SmallEngine {
 #pragma unroll
         for (int c = 0; c < CPL; ++c) sum[c] = 0.f;
     }
-    template <bool kPostOut = false, bool kAtomicStop = false>
+    template <bool kPostOut = false>
     __device__ int run(const DevGraph& g, const DecCfg& cfg, const WarpState& st, int max_iters, bool stop,
                        int* success, float* post_out, bool from_prior = false, const AbortCheck& ab = AbortCheck{})
     {
         const int lane = threadIdx.x & 31;
-        const float alpha = cfg.alpha;
-        const float L = cfg.L;
+        const float2 alpha2 = make_float2(cfg.alpha, cfg.alpha);
         typename S::T* const E = reinterpret_cast<typename S::T*>(st.E);
+        const uint32_t dbase = saddr(kInPlace ? st.E : (void*)st.D);
+        const uint32_t drow = dbase + 8u * lane;         // D of the lane's first row
+        // Lambda_j of the lane's columns; +inf for a masked column or one past
+        // N: its messages and posterior are then +inf, which the detector
+        // pass reads as L_MAX and positive (the sentinel of a masked node) and
+        // Eq. 4 as e^_j = 0, with no test in the loop
+        float l[CPL];
         mb = 0u;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
             const int j = lane + 32 * c;
-            if (j >= g.N || ((st.mask[c] >> lane) & 1u)) mb |= 1u << c;
+            const bool out = j >= g.N || ((st.mask[c] >> lane) & 1u);
+            if (out) mb |= 1u << c;
+            l[c] = out ? INFINITY : __ldg(g.lam + j);
         }
-        // s'_i of the lane's rows in bit 31 (s' is fixed for the whole run)
-        uint32_t sb[RPL];
+        // L_MAX with the sign (-1)^{s'_i} of the lane's rows (s' is fixed for the run)
+        float sL[RPL];
 #pragma unroll
-        for (int r = 0; r < RPL; ++r) sb[r] = (lane + 32 * r < g.M) ? ((st.sp[r] >> lane) & 1u) << 31 : 0u;
-        const uint32_t spw = lane < RPL ? st.sp[lane] : 0u;
+        for (int r = 0; r < RPL; ++r) {
+            const uint32_t sb = (lane + 32 * r < g.M) ? ((st.sp[r] >> lane) & 1u) << 31 : 0u;
+            sL[r] = __uint_as_float(__float_as_uint(cfg.L) | sb);
+        }
         int iters = 0;
         int ok = 0;
         uint32_t bal[CPL];     // e^ words of the last iteration (the same in every lane)
@@ -608,165 +678,115 @@ struct SmallEngine {
         for (int t = 1; t <= max_iters; ++t) {
             unsigned long long ab_key = 0ull;
             if (ab.key != nullptr && lane == 0) ab_key = *((volatile const unsigned long long*)ab.key);
-            if (kAtomicStop && lane < RPL) st.par[lane] = spw;
             // weighted min-sum: row min(t, wT) - 1 of the weights in place of alpha
             const float* wt = W ? cfg.sweights + (size_t)((t < cfg.wT ? t : cfg.wT) - 1) * (size_t)g.Epad : nullptr;
-            // ---- detector pass (Eq. 1); a run from E(0) takes its first check
-            // messages from the table D0, flipping the sign where s_i = 1
+            // ---- detector pass (Eq. 1)
             if (!W && from_prior && t == 1) {
+                // a run from E(0) takes its first check messages from the table
+                // D0, flipping the sign where s_i = 1
 #pragma unroll
                 for (int r = 0; r < RPL; ++r) {
                     const int i = lane + 32 * r;
                     if (i < g.M) {
-                        const uint32_t sb = ((st.sp[i >> 5] >> (i & 31)) & 1u) << 31;
+                        const uint32_t sb = __float_as_uint(sL[r]) & 0x80000000u;
 #pragma unroll
-                        for (int h = 0; h < RD / 2; ++h) {
+                        for (int h = 0; h < 3; ++h) {
                             const int wd = h * kPlane + 2 * i;
                             const float2 v = __ldg(reinterpret_cast<const float2*>(g.sD0 + wd));
-                            *reinterpret_cast<float2*>(st.D + wd) =
-                                make_float2(__uint_as_float(__float_as_uint(v.x) ^ sb),
-                                            __uint_as_float(__float_as_uint(v.y) ^ sb));
+                            sts2(drow + 4u * (h * kPlane + 64 * r),
+                                 make_float2(__uint_as_float(__float_as_uint(v.x) ^ sb),
+                                             __uint_as_float(__float_as_uint(v.y) ^ sb)));
                         }
                     }
                 }
-            }
+            } else {
 #pragma unroll
-            for (int r = 0; r < ((!W && from_prior && t == 1) ? 0 : RPL); ++r) {
-                const int i = lane + 32 * r;
-                if (i < g.M) {
-                    float x[RD];
+                for (int r = 0; r < RPL; ++r) {
+                    const int i = lane + 32 * r;
+                    if (i < g.M) {
+                        float2 x[3];
 #pragma unroll
-                    for (int h = 0; h < RD / 2; ++h) {
-                        const float2 x2 = S::ld2(E, h * kPlane + 2 * i);
-                        x[2 * h] = x2.x;
-                        x[2 * h + 1] = x2.y;
-                    }
-                    // the two smallest magnitudes m1 <= m2 of min(|x|, L_MAX)
-                    // (R3; m2 = m1 when the minimum is attained twice): the
-                    // pairs (lo, hi) of edges 2h, 2h + 1; m1 and the runner-up
-                    // among the lo; m2 = min(runner-up, every hi), since a hi
-                    // is never below its own lo
-                    float lo[RD / 2], hi[RD / 2];
+                        for (int h = 0; h < 3; ++h)
+                            x[h] = kInPlace ? lds2(drow + 4u * (h * kPlane + 64 * r)) : S::ld2(E, h * kPlane + 2 * i);
+                        // D_{i->j} = alpha (-1)^{s_i} prod sign min over the other
+                        // five messages (R3, R4): p[h] the signed minimum of pair
+                        // h, q[h] that of the other two pairs capped at L_MAX with
+                        // the syndrome sign (a stored message is never -0, so its
+                        // sign bit is exactly x < 0; min(|x|, L_MAX) is exact)
+                        float p[3], q[3];
 #pragma unroll
-                    for (int h = 0; h < RD / 2; ++h) {
-                        lo[h] = fminf(fabsf(x[2 * h]), fabsf(x[2 * h + 1]));
-                        hi[h] = fmaxf(fabsf(x[2 * h]), fabsf(x[2 * h + 1]));
-                    }
-                    // (three pairs: t <= u the pair minima lo0, lo1 in order;
-                    // the runner-up among the lo is min(u, max(t, lo2)); the
-                    // caps at L_MAX folded into three-input minima)
-                    const float t = fminf(lo[0], lo[1]), u = fmaxf(lo[0], lo[1]);
-                    const float m1 = fmin3(t, lo[2], L);
-                    const float m2 = fminf(fmin3(u, fmaxf(t, lo[2]), hi[0]), fmin3(hi[1], hi[2], L));
-                    // sign parity in bit 31: a stored message is never -0 (it is
-                    // a clamped sum of terms that starts at Lambda_j or the
-                    // sentinel), so its sign bit is exactly x < 0
-                    uint32_t nb = sb[r];
+                        for (int h = 0; h < 3; ++h) p[h] = xmin(x[h].x, x[h].y);
+                        q[0] = xmin(xmin(p[1], p[2]), sL[r]);
+                        q[1] = xmin(xmin(p[0], p[2]), sL[r]);
+                        q[2] = xmin(xmin(p[0], p[1]), sL[r]);
 #pragma unroll
-                    for (int k = 0; k < RD; ++k) nb ^= __float_as_uint(x[k]);
-                    nb &= 0x80000000u;
-                    // D_{i->j} for every edge of the row: alpha * (minimum over the
-                    // others), which is m2 for an edge holding the minimum and m1
-                    // otherwise; sign = s'_i xor parity of all signs xor the
-                    // edge's own sign.  The row's part of the sign is applied to
-                    // both candidates once (negating a factor negates the
-                    // product exactly), the edge's own per edge.
-                    const float m1s = __uint_as_float(__float_as_uint(m1) | nb);
-                    const float m2s = __uint_as_float(__float_as_uint(m2) | nb);
-                    const float d1 = W ? m1s : __fmul_rn(alpha, m1s), d2 = W ? m2s : __fmul_rn(alpha, m2s);
-#pragma unroll
-                    for (int h = 0; h < RD / 2; ++h) {
-                        const int wd = h * kPlane + 2 * i;
-                        float dd[2];
-                        float2 w2 = make_float2(alpha, alpha);
-                        if (W) w2 = __ldg(reinterpret_cast<const float2*>(wt + wd));
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const int k = 2 * h + u;
-                            const float sel = (fabsf(x[k]) == m1) ? d2 : d1;
-                            const float d = W ? __fmul_rn(u ? w2.y : w2.x, sel) : sel;
-                            dd[u] = __uint_as_float(__float_as_uint(d) ^ (__float_as_uint(x[k]) & 0x80000000u));
+                        for (int h = 0; h < 3; ++h) {
+                            float2 w2 = alpha2;
+                            if (W) w2 = __ldg(reinterpret_cast<const float2*>(wt + h * kPlane + 2 * i));
+                            sts2(drow + 4u * (h * kPlane + 64 * r),
+                                 mul2(w2, make_float2(xmin(x[h].y, q[h]), xmin(x[h].x, q[h]))));
                         }
-                        *reinterpret_cast<float2*>(st.D + wd) = make_float2(dd[0], dd[1]);
                     }
                 }
             }
             __syncwarp();
-            // ---- error-node pass (Eqs. 2-4); hx: the XOR of the columns of H
-            // of the lane's columns with e^_j = 1, reduced over the warp into
-            // H e^ after the pass (the code's M bits fill RPL words)
-            uint32_t hx[RPL];
+            // ---- error-node pass (Eqs. 2-4), the next column's messages loaded
+            // before this one's are stored
+            float v[2][3];
 #pragma unroll
-            for (int q = 0; q < RPL; ++q) hx[q] = 0u;
+            for (int k = 0; k < 3; ++k) v[0][k] = lds(ca[0][k]);
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
-                // every column is computed; a masked column or one beyond N
-                // stores nothing
-                const bool inr = (lane + 32 * c) < g.N;
-                const bool act = !((mb >> c) & 1u);
-                float v[3];
-                int ed[3];
+                if (c + 1 < CPL) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    ed[k] = (int)(ci[c][k] >> 16);
-                    v[k] = st.D[ed[k]];
+                    for (int k = 0; k < 3; ++k) v[(c + 1) & 1][k] = lds(ca[c + 1][k]);
                 }
-                // Lambda_j and column j of H in one 16-byte record (zero past N)
-                const uint4 lh = __ldg(g.slamh + lane + 32 * c);
-                const float l = __uint_as_float(lh.x);
+                const float v0 = v[c & 1][0], v1 = v[c & 1][1], v2 = v[c & 1][2];
                 // Eq. 2: each message leaves its own detector out; the other two
                 // are added in ascending order.  Messages are stored unclamped:
                 // the detector pass reads min(|E|, L_MAX) and the sign, which is
-                // what a clamp at store time (R4) would leave, and |E| stays below
-                // Lambda_j + 3 alpha L_MAX.  A masked column stores nothing: its
-                // messages hold the sentinel +L_MAX from the moment it was fixed.
-                const float e0 = __fadd_rn(__fadd_rn(l, fminf(v[1], v[2])), fmaxf(v[1], v[2]));
-                const float e1 = __fadd_rn(__fadd_rn(l, fminf(v[0], v[2])), fmaxf(v[0], v[2]));
-                const float e2 = __fadd_rn(__fadd_rn(l, fminf(v[0], v[1])), fmaxf(v[0], v[1]));
-                if (act) {
-                    S::st(E, ed[0], e0);
-                    S::st(E, ed[1], e1);
-                    S::st(E, ed[2], e2);
+                // what a clamp at store time (R4) would leave.  Eq. 3 in ascending
+                // order: smallest, median (the least of the pair maxima), largest.
+                const float lo12 = fminf(v1, v2), hi12 = fmaxf(v1, v2);
+                const float lo02 = fminf(v0, v2), hi02 = fmaxf(v0, v2);
+                const float lo01 = fminf(v0, v1), hi01 = fmaxf(v0, v1);
+                const float2 ll = make_float2(l[c], l[c]);
+                const float2 e01 = add2(add2(ll, make_float2(lo12, lo02)), make_float2(hi12, hi02));
+                const float2 e2p = add2(add2(ll, make_float2(lo01, fminf(lo01, v2))),
+                                        make_float2(hi01, fmin3(hi01, hi02, hi12)));
+                const float post = __fadd_rn(e2p.y, fmaxf(hi01, v2));
+                const bool inr = c + 1 < CPL || lane + 32 * c < g.N;   // only the last word may pass N
+                if (inr) {
+                    const float e[3] = {e01.x, e01.y, e2p.x};
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        if (kInPlace) sts(ca[c][k], e[k]);
+                        else S::st(E, (ca[c][k] - dbase) >> 2, e[k]);
+                    }
                 }
-                // Eq. 3 in ascending order: smallest, median, largest
-                const float lo01 = fminf(v[0], v[1]), hi01 = fmaxf(v[0], v[1]);
-                const float a0 = fminf(lo01, v[2]);
-                const float a2 = fmaxf(hi01, v[2]);
-                const float a1 = fmaxf(lo01, fminf(hi01, v[2]));
-                const float post = __fadd_rn(__fadd_rn(__fadd_rn(l, a0), a1), a2);
                 sum[c] = __fadd_rn(sum[c], post);           // unused for masked columns
                 if (kPostOut && t == max_iters && inr) post_out[lane + 32 * c] = post;
-                const uint32_t ebit = (act && post <= 0.f) ? 1u : 0u;                // Eq. 4
-                if (kAtomicStop) {
-                    if (ebit) {
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            const int r = (int)(ci[c][k] & 0xffffu);
-                            atomicXor(&st.par[r >> 5], 1u << (r & 31));
-                        }
-                    }
-                } else {
-                    // column j of H where e^_j = 1
-                    const uint32_t em = 0u - ebit;
-                    const uint32_t hw[3] = {lh.y, lh.z, lh.w};
-#pragma unroll
-                    for (int q = 0; q < RPL; ++q) hx[q] ^= hw[q] & em;
-                }
-                bal[c] = __ballot_sync(FULLMASK, ebit);
+                bal[c] = __ballot_sync(FULLMASK, post <= 0.f);                       // Eq. 4
             }
-            // stopping rule: H e^ = s' word by word (every lane gets the same
-            // reductions, so the decision needs no vote)
-            if (kAtomicStop) {
-                __syncwarp();
-                uint32_t nz = 0;
-                if (lane < RPL) nz = st.par[lane];
-                ok = !__any_sync(FULLMASK, nz != 0u);
-            } else {
-                uint32_t nz = 0u;
+            __syncwarp();
+            // ---- stopping rule H e^ = s': the parity of e^ on the lane's row
+            // against s'_i, first on rows 0..31 (their columns stay in
+            // registers: most iterations end here), then on the others
+            uint32_t acc = 0u;
 #pragma unroll
-                for (int q = 0; q < RPL; ++q) nz |= __reduce_xor_sync(FULLMASK, hx[q]) ^ st.sp[q];
-                __syncwarp();
-                ok = (nz == 0u);
+            for (int c = 0; c < CPL; ++c) acc ^= bal[c] & hq[c];
+            ok = !__any_sync(FULLMASK, ((__popc(acc) & 1u) ^ (__float_as_uint(sL[0]) >> 31)) != 0u);
+            if (RPL > 1 && ok) {
+                uint32_t bad = 0u;
+#pragma unroll
+                for (int r = 1; r < RPL; ++r) {
+                    const uint32_t* hr = g.shrow + (size_t)kSmallRowWords * (lane + 32 * r);
+                    uint32_t a2 = 0u;
+#pragma unroll
+                    for (int c = 0; c < CPL; ++c) a2 ^= bal[c] & __ldg(hr + c);
+                    bad |= (__popc(a2) & 1u) ^ (__float_as_uint(sL[r]) >> 31);
+                }
+                ok = !__any_sync(FULLMASK, bad != 0u);
             }
             iters = t;
             if (ok && stop) break;
@@ -1207,7 +1227,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
     const WarpState st = carve(smem + (size_t)grp.index() * warp_smem_bytes(g), g);
     const RunDesc* dp = w.desc;                  // read fields when needed (keeps registers free)
     count_launch(w);
-    eng.load_graph(g);
+    eng.load_graph(g, st);
     unsigned long long seed_iters = 0;           // BP iterations (group rank 0)
     // a warp claims its shots kBatch at a time (one atomic per batch on the
     // chunk's counter, which a million one-iteration seeds would otherwise
@@ -1256,7 +1276,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
         if (!Eng::kPriorSetsSums) eng.clear_sums(g, st);
         grp.sync();
         int succ = 0;
-        const int it = eng.template run<false, true>(g, cfg, st, cfg.initial_iters, true, &succ, nullptr, true);
+        const int it = eng.run(g, cfg, st, cfg.initial_iters, true, &succ, nullptr, true);
         if (grp.rank() == 0) seed_iters += (unsigned long long)it;
         grp.sync();
         if ((succ && cfg.num_results == 1) || cfg.max_rounds == 0) {
@@ -1314,7 +1334,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(Dev
     const int nitems = (r == 1) ? 2 * cnt : *((volatile int*)(rc + 2));
     const int2* items = w.items + (size_t)(r & 1) * (size_t)w.A * (size_t)W2;
     const int cb = r & 1;
-    eng.load_graph(g);
+    eng.load_graph(g, st);
     for (;;) {
         int it = 0;
         if (grp.rank() == 0) it = atomicAdd(&rc[0], 1);
@@ -1688,7 +1708,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_bp_llr(De
     eng.grp = Eng::Grp::make(smem + warp_smem_bytes(g));
     const auto& grp = eng.grp;
     const WarpState st = carve(smem + (size_t)grp.index() * warp_smem_bytes(g), g);
-    eng.load_graph(g);
+    eng.load_graph(g, st);
     const long long nw = (long long)gridDim.x * grp.per_block();
     for (long long b = (long long)blockIdx.x * grp.per_block() + grp.index(); b < B; b += nw) {
         for (int q = grp.rank(); q < g.WM; q += grp.size()) st.sp[q] = synd[b * g.WM + q];
@@ -1813,9 +1833,10 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     } else {
         const int kind = skind >= 0 ? skind : gkind;
         eng = weighted ? kWeightedEngine + kind : 3 * kind + g.prec;
-        // the small engine keeps D per edge in float; the generic one a record per detector
-        const size_t recs = sizeof(float2) * (size_t)g.M, msgs = sizeof(float) * (size_t)g.Epad;
-        g.det_bytes = (int)align16(kind >= 3 && msgs > recs ? msgs : recs);
+        // the small engine keeps D per edge in float (over E with single-precision
+        // messages, else beside it); the generic one a record per detector
+        g.det_bytes = (int)align16(kind < 3 ? sizeof(float2) * (size_t)g.M
+                                            : (g.prec == 0 ? 0 : sizeof(float) * (size_t)g.Epad));
         const size_t per_warp = warp_smem_bytes(g);
         if (per_warp > (size_t)max_optin) return -5;
         wpb = warps_per_block > 0 ? warps_per_block : (int)((96 * 1024) / per_warp);
@@ -2259,7 +2280,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_serve(Dev
     eng.grp = Eng::Grp::make(smem + warp_smem_bytes(g));
     const auto& grp = eng.grp;
     const WarpState st = carve(smem, g);
-    eng.load_graph(g);
+    eng.load_graph(g, st);
     volatile uint32_t* const synd = reinterpret_cast<volatile uint32_t*>(box + 1);
     uint32_t* const obuf = reinterpret_cast<uint32_t*>(box + 1) + g.WM;
     const Outputs out{obuf, g.K > 0 ? obuf + g.WN : nullptr, &box->status, &box->iters};

@@ -429,7 +429,7 @@ def run_reference(args, rank: int):
     print(json.dumps(line), flush=True)
 
 
-KIND_NAMES = {0: "k_seed", 1: "k_round", 2: "k_select", 8: "k_bs_check", 9: "k_bs_var", 10: "k_bs_retire",
+KIND_NAMES = {0: "k_seed", 1: "k_round", 2: "beam set-up", 8: "k_bs_check", 9: "k_bs_var", 10: "k_bs_retire",
               11: "k_screen"}
 
 

@@ -306,8 +306,8 @@ int bsd_profile_enable(bsd_decoder *dec, int enable);
 
 /* Synchronise the decode stream, then return and reset, since the previous
  * read: the summed event-timed duration in milliseconds and the launch count
- * of each kernel kind (index 0: seed BP, 1: expand + masked BP of a round,
- * 2: per-shot selection of a round), the full BP iterations executed on the
+ * of each kernel kind (index 0: seed BP, 1: the beam -- expand, masked BP and
+ * selection of every round, 2: the beam's set-up), the full BP iterations executed on the
  * device (index 0: seed candidates, 1: round candidates, counting children
  * evaluated after a shot's first success, 2: the part of index 0 run by the
  * batched seed BP of bsd_params.batch_slots), the number of kernels of this

@@ -144,7 +144,6 @@ LaunchShape small_shape(const LaunchShape& ls, const DecCfg& cfg, int n)
     s.screen = 0;
     s.batch = 0;
     s.grid_round = cap(((long long)n * 2 * cfg.w + per_block - 1) / per_block, ls.grid_round);
-    s.grid_select = cap((n + ls.select_warps - 1) / ls.select_warps, ls.grid_select);
     return s;
 }
 
@@ -611,8 +610,9 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     rc = configure_kernels(g, cfg, device, params->group_warps, 0, &dec->ls);
     if (rc) { bsd_destroy(dec); return rc == -5 ? BSD_ERR_UNSUPPORTED : BSD_ERR_CUDA; }
 
-    // ---- workspace: a seed store of S shots and a beam window of A active
-    // entries (two banks of 2w child slots each), about 1 : 4 in bytes
+    // ---- workspace: a seed store of S shots and a beam window of A entries
+    // (two banks of 2w child slots each): four fifths for the window up to
+    // kBeamEntries, the rest for the store
     const int W2 = 2 * cfg.w;
     const int SB = WM + 3 * WN;
     const int NR = cfg.num_results;
@@ -642,11 +642,11 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
         }
     }
     long long A = (long long)(0.8 * (double)budget / win_b);
+    if (A > kBeamEntries) A = kBeamEntries;
     if (A < 1) A = 1;
     long long S = (long long)(((double)budget - (double)A * win_b) / seed_b);
     if (S > (1ll << 22)) S = 1ll << 22;
     if (S < A) S = A;
-    if (A > (1ll << 22)) A = 1ll << 22;
     // with the batched seed BP a chunk can hold far more shots than the seed
     // store: only the shots it hands on need an entry, and they are decoded
     // in windows of S
@@ -662,13 +662,13 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     }
     Work& w = dec->w;
     work_layout(g, cfg, S, A, (char*)dec->work_mem, &w, bs_slots, S1);
-    dec->ctr_bytes = work_head_bytes(cfg);
+    dec->ctr_bytes = work_head_bytes();
     if (CUDA_FAILED(cudaMemset(dec->work_mem, 0, dec->ctr_bytes)) ||
         CUDA_FAILED(cudaMallocHost(&dec->h_nactive, sizeof(int)))) {
         bsd_destroy(dec);
         return BSD_ERR_CUDA;
     }
-    // the per-chunk graph: seed kernel + WHILE over beam passes; without it
+    // the per-chunk graph: seed kernel, then the beam if needed; without it
     // decoding falls back to plain launches
     dec->small_n = params->small_batch > 0 ? params->small_batch : (params->small_batch == 0 ? 32 : 0);
     rebuild_graphs(dec);

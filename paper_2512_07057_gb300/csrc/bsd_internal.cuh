@@ -20,10 +20,10 @@
 // Workspace (one decoder):
 //   seed store, S entries: the snapshot (E, s', mask, vals, e^, record) of
 //   every shot of a chunk of S shots whose seed BP did not end the search;
-//   beam window, A entries: the active shots of the current beam pass
-//   (entries pass*A .. pass*A + A - 1 of the seed store), with two banks of
-//   2w child slots each; round r writes bank r % 2 and reads its parents from
-//   bank (r - 1) % 2 (or the seed store for r = 1) through a rank -> slot
+//   beam window, A entries: the shots whose beam is running (an entry takes
+//   the next shot of the seed store when its shot has ended), with two banks
+//   of 2w child slots each; round r writes bank r % 2 and reads its parents
+//   from bank (r - 1) % 2 (or the seed store for r = 1) through a rank -> slot
 //   table, so surviving paths are never copied.
 #pragma once
 #include <cuda_runtime.h>
@@ -155,8 +155,6 @@ struct RunDesc {
     Outputs out;
     long long chunk_base;  // index of the chunk's first shot in the caller's batch
     long long chunk_n;     // shots in the chunk
-    int pass;              // current beam pass
-    int round;             // current beam round of the pass (graph launches read it from here)
     int win_base;          // batched seed BP: first entry of the fail list in the current window
 };
 
@@ -172,15 +170,39 @@ struct Counters {
     int bs_active_next;    // active slots after the current retirement (counted by its blocks)
     int bs_done_blocks;    // blocks of the current retirement that have finished
     int n_fail;            // shots passed on to the per-candidate seed kernel
-    // followed by 3 * (max_rounds + 2) ints for the current pass:
-    // claim_round[r], claim_select[r], work_count[r] (reset by k_pass_end)
+    // the beam over the n_active entries of the seed store
+    unsigned b_head;       // tickets drawn from the ring of items
+    unsigned b_tail;       // items put on it
+    unsigned b_mask;       // slots of the ring in use, less one
+    int b_left;            // shots that have not ended
+    int b_next;            // first seed-store entry that no window entry has taken
 };
+
+// what a window entry runs (16 bytes, read in one load)
+struct __align__(16) BeamEntry {
+    int seed;              // seed-store entry of its shot
+    int round;             // current round, from 1
+    int pending;           // children of the round that have not finished
+    int stamp;             // of the round, never 0, grows over the shots of the entry
+};
+
+// an item of the ring: child c (< 2w <= 128) of window entry a, never one of
+// the two marks
+constexpr uint32_t kRingEmpty = 0u;
+constexpr uint32_t kRingLeft = 0xffffffffu;   // the group that held this slot's ticket has left
+__host__ __device__ inline uint32_t ring_item(int a, int c) { return (((uint32_t)a << 7) | (uint32_t)c) + 1u; }
+__host__ __device__ inline int ring_entry(uint32_t it) { return (int)((it - 1u) >> 7); }
+__host__ __device__ inline int ring_child(uint32_t it) { return (int)((it - 1u) & 127u); }
+// window entries in use at once: enough that the items of their shots (two in
+// the first round, up to 2w later) keep every candidate group busy
+constexpr long long kBeamEntries = 4096;
+constexpr int kErrBeam = 2;                   // Counters::err: the beam left a shot behind
 
 struct Work {
     long long S;           // shots per chunk = seed-store entries
     long long S1;          // with the batched seed BP: shots per chunk (>= S); the shots it hands on are
                            // decoded from the seed on in windows of S
-    long long A;           // active entries per beam pass
+    long long A;           // window entries: shots whose beam runs at once
     int SB;                // words per slot bit record: sp[WM] mask[WN] vals[WN] ehat[WN]
     int* queue;            // [S1] chunk-local shots the screen passed on to the seed BP
     // batched seed BP over slots (bsd_batch.cu); bs_slots = 0: not used
@@ -205,16 +227,15 @@ struct Work {
     int* set_size;         // [A]
     uint8_t* set_idx;      // [A][w] child index (in the parent bank) of the path of rank k
     unsigned long long* iters_acc;   // [A]
-    int* done;             // [A]
     uint32_t* res_bits;    // [A][num_results][WN]
     long long* res_w;      // [A][num_results]
     int* res_origin;       // [A][num_results]: 0 = seed, 1 = masked BP round
     int* res_n;            // [A]
     int* near;             // [A] a near-tie met by this shot's search so far
     unsigned long long* first_ok;  // [A] (round stamp << 32) | ~c of the lowest-index successful child so far
-    int2* items;           // [2][A * 2w] (window entry, child index) for rounds >= 2
+    BeamEntry* ent;        // [A]
+    uint32_t* ring;        // items to run, Counters::b_mask + 1 slots in use
     Counters* ctr;
-    int* round_ctr;        // 3 * (max_rounds + 2) ints after ctr
     RunDesc* desc;
     unsigned long long* stats;   // [5]: executed full BP iterations (seed, rounds), kernel launches, message
                                  // updates of first-iteration screens, seed iterations run by the batch
@@ -235,30 +256,28 @@ bool cuda_failed_at(cudaError_t e, const char* file, int line);
 
 // workspace layout for S seed entries and A window entries starting at base
 // (base may be null to size it); returns the bytes used.  The counters and the
-// run descriptor come first, in the first head_bytes(cfg) bytes.
+// run descriptor come first, in the first work_head_bytes() bytes.
 size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long A, char* base, Work* w,
                    int bs_slots = 0, long long S1 = 0);
-size_t work_head_bytes(const DecCfg& cfg);
+size_t work_head_bytes();
 
 // host-side launch helpers (bsd_kernels.cu)
 struct LaunchShape {
     int warps_per_block;
     int group_warps;       // warps per BP candidate: 1 (a warp) or the whole block
-    int select_warps;      // block size of the selection kernel, in warps (<= 8)
-    int grid_seed, grid_round, grid_select;
+    int grid_seed, grid_round;
     int screen;            // a first-iteration screen kernel runs before the seed BP
     int grid_screen;       // its blocks of 8 warps (one shot per warp)
     int dv_screen;         // its column degree bound: 0 -> 3, 1 -> 6, 2 -> 16
     size_t smem_screen;
     size_t smem_bp;        // dynamic shared memory of the seed / round kernels
-    size_t smem_select;
     int dv;                // engine id
     int batch;             // the seed BP runs batched over slots (when the workspace has them)
     int grid_bs;           // blocks of the batched passes (persistent)
 };
 
-// optional callbacks around every kernel launch; kinds 0 seed, 1 round,
-// 2 select, 3..6 the unrolled decoder's check / error / error adjoint / check
+// optional callbacks around every kernel launch; kinds 0 seed, 1 the beam,
+// 2 its set-up, 3..6 the unrolled decoder's check / error / error adjoint / check
 // adjoint passes, 7 its other kernels, 8..10 the batched seed BP's check pass,
 // error-node pass and retirement, 11 the first-iteration screen
 constexpr int kProfKinds = BSD_PROFILE_KINDS;
@@ -275,13 +294,13 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
                       LaunchShape* ls);
 
 // decode one chunk: reset counters and set the run descriptor, then the seed
-// kernel and as many beam passes as the chunk has active windows.  With a
-// graph (built by build_graph) the passes run under a conditional WHILE node;
-// without one, n_active is read back after the seed kernel.
+// kernel and, if a shot needs it, the beam.  With a graph (built by
+// build_graph) the beam runs under a conditional node; without one, n_active
+// is read back after the seed kernel.
 int launch_chunk(const DevGraph& g, const DecCfg& cfg, const Work& w, const LaunchShape& ls,
                  const uint32_t* synd, long long chunk_base, long long chunk_n, const Outputs& out,
                  void* stream, const LaunchHooks* hooks, void* graph_exec, int* host_n_active);
-// build and instantiate the per-chunk graph (seed kernel + WHILE over beam passes)
+// build and instantiate the per-chunk graph (seed kernel, then the beam if it is needed)
 int build_graph(const DevGraph& g, const DecCfg& cfg, const Work& w, const LaunchShape& ls, void** graph_exec);
 
 // batched seed BP (bsd_batch.cu): slots that fit a byte budget (0: none)

@@ -14,9 +14,11 @@
 //                 finalises the shots that converge there, queues the rest
 //   k_seed<DV>    the seed BP of every shot in a chunk, or of the queued ones
 //                 (Alg. 3, first BP run)
-//   k_round<DV>   expand + masked BP for every child of round r (Alg. 2)
-//   k_select      per shot: first success in visit order, results, top-w
-//                 pruning and the work list of round r + 1 (Alg. 3, App. B)
+//   k_round<DV>   the beam of every shot: expand + masked BP of its children
+//                 (Alg. 2) round by round; after the last child of a round
+//                 select_entry takes the first success in visit order, the
+//                 results, the top-w pruning and the next round's children
+//                 (Alg. 3, App. B)
 //   k_bp_llr<DV>  plain BP for a fixed number of iterations (LLR measurement)
 //
 // Arithmetic follows the readings stated in include/bsd.h: D = alpha * sign *
@@ -62,13 +64,15 @@ struct AbortCheck {
     }
 };
 
-// copy n16 16-byte vectors (the E snapshot) with the threads of a candidate group
-template <class G>
+// copy n16 16-byte vectors (the E snapshot) with the threads of a candidate
+// group; kL2: the source was written by other SMs during this kernel, so it is
+// read past the L1 cache, which is not coherent between them
+template <bool kL2 = false, class G>
 __device__ __forceinline__ void group_copy16(const G& grp, void* dst, const void* src, int n16)
 {
     const uint4* s = reinterpret_cast<const uint4*>(src);
     uint4* d = reinterpret_cast<uint4*>(dst);
-    for (int q = grp.rank(); q < n16; q += grp.size()) d[q] = s[q];
+    for (int q = grp.rank(); q < n16; q += grp.size()) d[q] = kL2 ? __ldcg(s + q) : s[q];
 }
 
 
@@ -149,10 +153,12 @@ __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(
 // with the engine choice
 __host__ __device__ inline size_t det_region_bytes(const DevGraph& g) { return (size_t)g.det_bytes; }
 
+constexpr size_t kSelectBytes = 2 * kMaxBeam * (sizeof(double) + 2 * sizeof(int));
 __host__ __device__ inline size_t warp_smem_bytes(const DevGraph& g)
 {
-    return align16((size_t)g.msg_bytes * (size_t)g.Epad) + det_region_bytes(g) +
-           align16(sizeof(float) * (size_t)g.Npad) + align16(sizeof(uint32_t) * (size_t)(2 * g.WM + 3 * g.WN));
+    const size_t n = align16((size_t)g.msg_bytes * (size_t)g.Epad) + det_region_bytes(g) +
+                     align16(sizeof(float) * (size_t)g.Npad) + align16(sizeof(uint32_t) * (size_t)(2 * g.WM + 3 * g.WN));
+    return n > kSelectBytes ? n : kSelectBytes;   // the selection's scratch lies over the candidate's state
 }
 
 struct WarpState {
@@ -826,20 +832,22 @@ struct SmallEngine {
 
 // write one shot's outputs: e^, A e^, status, iteration count
 // (kSparse: A e^ from the set bits of e^, for the seed kernel, where e^ is
-// long and sparse)
-template <class G = WarpGroup, bool kSparse = false>
+// long and sparse; kL2: e^ is in global memory and was written by other SMs
+// during this kernel)
+template <class G = WarpGroup, bool kSparse = false, bool kL2 = false>
 __device__ void finalize_shot(const DevGraph& g, const Outputs& out, long long gb, const uint32_t* ehat,
                               uint32_t status, unsigned long long iters, const G& grp = G{})
 {
     uint32_t* corr = out.corr + gb * g.WN;
-    for (int q = grp.rank(); q < g.WN; q += grp.size()) corr[q] = ehat[q];
+    auto word = [&](int q) -> uint32_t { return kL2 ? __ldcg(ehat + q) : ehat[q]; };
+    for (int q = grp.rank(); q < g.WN; q += grp.size()) corr[q] = word(q);
     if (out.obs != nullptr) {
         for (int wq = 0; wq < g.WK; ++wq) {
             uint32_t acc = 0;
             if constexpr (kSparse) {
                 // over the set bits of e^ only (bits past N are never set)
                 for (int q = grp.rank(); q < g.WN; q += grp.size()) {
-                    uint32_t bits = ehat[q];
+                    uint32_t bits = word(q);
                     while (bits != 0u) {
                         const int b = __ffs(bits) - 1;
                         bits &= bits - 1u;
@@ -848,7 +856,7 @@ __device__ void finalize_shot(const DevGraph& g, const Outputs& out, long long g
                 }
             } else {
                 for (int j = grp.rank(); j < g.N; j += grp.size())
-                    if ((ehat[j >> 5] >> (j & 31)) & 1u) acc ^= __ldg(g.acol + (size_t)j * g.WK + wq);
+                    if ((word(j >> 5) >> (j & 31)) & 1u) acc ^= __ldg(g.acol + (size_t)j * g.WK + wq);
             }
             acc = grp.xor_all(acc);
             if (grp.rank() == 0) out.obs[gb * g.WK + wq] = acc;
@@ -866,13 +874,11 @@ __device__ inline long long vector_weight(const DevGraph& g, const uint32_t* bit
     const int lane = threadIdx.x & 31;
     unsigned long long s = 0;
     for (int j = lane; j < g.N; j += 32)
-        if ((bits[j >> 5] >> (j & 31)) & 1u) s += (unsigned long long)__ldg(g.lamq + j);
+        if ((__ldcg(bits + (j >> 5)) >> (j & 31)) & 1u) s += (unsigned long long)__ldg(g.lamq + j);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULLMASK, s, o);
     return (long long)s;
 }
-
-__device__ inline int* round_ctr(const Work& w, int r) { return w.round_ctr + 3 * r; }
 
 // slot of child c of window entry a in bank `bank`
 __device__ inline size_t slot_index(const Work& w, int bank, int a, int c, int W2)
@@ -881,24 +887,25 @@ __device__ inline size_t slot_index(const Work& w, int bank, int a, int c, int W
 }
 
 // the parent of the rank-k path of window entry a in round r: the seed-store
-// entry for r = 1, else the slot of the previous round that won rank k
+// entry of its shot for r = 1, else the slot of the previous round that won
+// rank k
 struct SlotRef {
     const unsigned char* E;   // snapshot, Epad messages in the storage format
     const uint32_t* bits;
     const SlotMeta* meta;
 };
 
-__device__ inline SlotRef parent_ref(const DevGraph& g, const DecCfg& cfg, const Work& w, int r, long long pbase,
+__device__ inline SlotRef parent_ref(const DevGraph& g, const DecCfg& cfg, const Work& w, int r, int seed,
                                      int a, int k)
 {
     SlotRef s;
     if (r == 1) {
-        const size_t e = (size_t)(pbase + a);
+        const size_t e = (size_t)seed;
         s.E = w.seedE + e * snap_bytes(g);
         s.bits = w.seedBits + e * (size_t)w.SB;
         s.meta = w.seedMeta + e;
     } else {
-        const size_t e = slot_index(w, (r - 1) & 1, a, w.set_idx[(size_t)a * cfg.w + k], 2 * cfg.w);
+        const size_t e = slot_index(w, (r - 1) & 1, a, __ldcg(w.set_idx + (size_t)a * cfg.w + k), 2 * cfg.w);
         s.E = w.slotE + e * snap_bytes(g);
         s.bits = w.slotBits + e * (size_t)w.SB;
         s.meta = w.slotMeta + e;
@@ -906,34 +913,37 @@ __device__ inline SlotRef parent_ref(const DevGraph& g, const DecCfg& cfg, const
     return s;
 }
 
-// entries of the current pass's window: [pbase, pbase + count)
-__device__ inline int window(const Work& w, long long* pbase)
+// records written by other SMs during the beam kernel, read past L1
+__device__ inline SlotMeta load_meta(const SlotMeta* p)
 {
-    const int pass = *((volatile int*)&w.desc->pass);
-    const long long n_active = *((volatile int*)&w.ctr->n_active);
-    *pbase = (long long)pass * w.A;
-    long long cnt = n_active - *pbase;
-    if (cnt > w.A) cnt = w.A;
-    return cnt > 0 ? (int)cnt : 0;
+    static_assert(sizeof(SlotMeta) == 24, "three 8-byte loads");
+    const unsigned long long* q = reinterpret_cast<const unsigned long long*>(p);
+    const unsigned long long x = __ldcg(q), y = __ldcg(q + 1), z = __ldcg(q + 2);
+    SlotMeta m;
+    m.S = (long long)x;
+    m.iters = (int)(uint32_t)y;
+    m.next_pos = (int)(uint32_t)(y >> 32);
+    m.success = (int)(uint32_t)z;
+    m.flags = (int)(uint32_t)(z >> 32);
+    return m;
+}
+__device__ inline BeamEntry load_entry(const BeamEntry* p)
+{
+    const int4 v = __ldcg(reinterpret_cast<const int4*>(p));
+    return BeamEntry{v.x, v.y, v.z, v.w};
 }
 
 // ----------------------------------------------------------------------------
-// chunk set-up and pass advance (one warp each)
+// chunk set-up and beam set-up
 // ----------------------------------------------------------------------------
 __device__ inline void count_launch(const Work& w)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&w.stats[2], 1ull);
 }
 
-__global__ void k_begin_chunk(Work w, int n_round_ints, const uint32_t* synd, Outputs out, long long base,
-                              long long n)
+__global__ void k_begin_chunk(Work w, const uint32_t* synd, Outputs out, long long base, long long n)
 {
     count_launch(w);
-    for (int q = threadIdx.x; q < n_round_ints; q += blockDim.x) w.round_ctr[q] = 0;
-    // early-abort keys of the window entries this chunk can use (stamps grow
-    // within a chunk, so only a new chunk needs them cleared)
-    const long long na = n < w.A ? n : w.A;
-    for (long long q = threadIdx.x; q < na; q += blockDim.x) w.first_ok[q] = 0ull;
     if (threadIdx.x == 0) {
         w.ctr->claim_seed = 0;
         w.ctr->n_active = 0;
@@ -949,56 +959,55 @@ __global__ void k_begin_chunk(Work w, int n_round_ints, const uint32_t* synd, Ou
         d.out = out;
         d.chunk_base = base;
         d.chunk_n = n;
-        d.pass = 0;
-        d.round = 1;
         d.win_base = 0;
         *w.desc = d;
     }
 }
 
-// after the last round of a pass: move to the next window, reset the per-pass
-// counters and, under a graph, set the WHILE condition (another window left)
-__global__ void k_pass_end(Work w, int n_round_ints, cudaGraphConditionalHandle cond, int use_cond)
-{
-    count_launch(w);
-    for (int q = threadIdx.x; q < n_round_ints; q += blockDim.x) w.round_ctr[q] = 0;
-    if (threadIdx.x == 0) {
-        const int pass = w.desc->pass + 1;
-        w.desc->pass = pass;
-        w.desc->round = 1;
-        if (use_cond) cudaGraphSetConditional(cond, ((long long)pass * w.A < (long long)w.ctr->n_active) ? 1u : 0u);
-    }
-}
-
-// graph only, after the seed kernel: enter the loop over beam passes only if
-// some shot of the chunk needs beam rounds
-__global__ void k_pass_gate(Work w, cudaGraphConditionalHandle cond)
+// graph only, after the seed kernel: run the beam only if some shot of the
+// chunk needs it
+__global__ void k_beam_gate(Work w, cudaGraphConditionalHandle cond)
 {
     count_launch(w);
     if (threadIdx.x == 0) cudaGraphSetConditional(cond, w.ctr->n_active > 0 ? 1u : 0u);
 }
 
-// graph only, at the start of a pass: the loop over rounds begins with round 1
-__global__ void k_rounds_begin(Work w, cudaGraphConditionalHandle cond)
+// counters of a beam search over the n_active entries of the seed store: the
+// first of them take the window entries, the others follow as entries end
+__global__ void k_beam_begin(Work w, int beam_width)
 {
     count_launch(w);
     if (threadIdx.x == 0) {
-        w.desc->round = 1;
-        cudaGraphSetConditional(cond, 1u);
+        const int n = w.ctr->n_active;
+        const int cnt = (long long)n < w.A ? n : (int)w.A;
+        w.ctr->b_head = 0u;
+        w.ctr->b_tail = 2u * (unsigned)cnt;
+        w.ctr->b_left = n;
+        w.ctr->b_next = cnt;
+        // the ring for these entries: at most 2w items of each are on it at
+        // once, and it has at least twice as many slots
+        uint32_t slots = 4;
+        while ((unsigned long long)slots < 4ull * (unsigned long long)cnt * (unsigned)beam_width) slots *= 2;
+        w.ctr->b_mask = slots - 1;
     }
 }
 
-// graph only, after the selection of round r: run round r + 1 only if it has
-// children to expand (a shot with none left was finalised by the selection)
-__global__ void k_round_end(Work w, int max_rounds, cudaGraphConditionalHandle cond)
+// the first items of the ring, two children per window entry, and empty
+// slots after them
+__global__ void k_beam_ring(Work w)
 {
     count_launch(w);
-    if (threadIdx.x == 0) {
-        const int r = w.desc->round;
-        const int more = (r < max_rounds && *((volatile int*)(w.round_ctr + 3 * (r + 1) + 2)) > 0) ? 1 : 0;
-        w.desc->round = r + 1;
-        cudaGraphSetConditional(cond, (unsigned)more);
-    }
+    const uint32_t n = w.ctr->b_tail, mask = w.ctr->b_mask;
+    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q <= mask; q += gridDim.x * blockDim.x)
+        w.ring[q] = q < n ? ring_item((int)(q >> 1), (int)(q & 1u)) : kRingEmpty;
+}
+
+// every shot of the beam ended with its outputs written, or the device-side
+// error word says so (the beam kernel cannot leave one behind by design)
+__global__ void k_beam_end(Work w)
+{
+    count_launch(w);
+    if (threadIdx.x == 0 && w.ctr->b_left != 0) w.ctr->err = kErrBeam;
 }
 
 // batched seed BP: the shots it hands on are decoded from the seed on in
@@ -1013,18 +1022,14 @@ __global__ void k_win_gate(Work w, cudaGraphConditionalHandle cond)
     }
 }
 
-// start of a window: the per-window counters and early-abort keys start
-// afresh, as at the start of a chunk (base < 0: keep the window base)
-__global__ void k_win_begin(Work w, int n_round_ints, int base)
+// start of a window: the per-window counters start afresh, as at the start of
+// a chunk (base < 0: keep the window base)
+__global__ void k_win_begin(Work w, int base)
 {
     count_launch(w);
-    for (int q = threadIdx.x; q < n_round_ints; q += blockDim.x) w.round_ctr[q] = 0;
-    for (long long q = threadIdx.x; q < w.A; q += blockDim.x) w.first_ok[q] = 0ull;
     if (threadIdx.x == 0) {
         w.ctr->claim_seed = 0;
         w.ctr->n_active = 0;
-        w.desc->pass = 0;
-        w.desc->round = 1;
         if (base >= 0) w.desc->win_base = base;
     }
 }
@@ -1312,386 +1317,482 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
 }
 
 // ----------------------------------------------------------------------------
-// one beam round: expand every child and run masked BP (Alg. 2)
+// the beam: every round of every shot in one kernel
 // ----------------------------------------------------------------------------
-template <class Eng>
-__global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(DevGraph g, DecCfg cfg, Work w, int r)
+// A shot's rounds depend only on one another, so no round waits for another
+// shot: the children to run are items of a ring that the candidate groups of
+// one persistent kernel draw from; the group that finishes the last child of a
+// shot's round selects (k_round's select_entry), and pushes the children of
+// the next round or, when the shot has ended, gives its window entry to the
+// next shot of the seed store.  (Before: a launch of all children and one of
+// all selections per round and window of shots, each ending with most of the
+// GPU idle: 10^6 [[144,12,12]] shots at p = 0.05 took 280 launches of 21.3 ms
+// in all.)
+//
+// The ring: a group draws a ticket (b_head) and waits for the item that will
+// be put at it (b_tail).  An item is exchanged in and out of its slot, so a
+// slot still full when the ring has come round gives its item back to the
+// pusher, which pushes it again; a group that has waited kIdleNs leaves
+// and marks its ticket's slot, and the pusher that meets the mark pushes its
+// item again too.  No item is lost, no wait is unbounded, and the running
+// groups alone finish the work, so nothing rests on two groups being resident
+// at once.
+constexpr unsigned long long kIdleNs = 1000ull * 1000 * 1000;
+
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p)
 {
-    extern __shared__ __align__(16) char smem[];
-    count_launch(w);
-    if (r <= 0) r = *((volatile int*)&w.desc->round);   // graph launches: the round counter
-    long long pbase;
-    const int cnt = window(w, &pbase);
-    if (cnt == 0) return;
-    const int pass = *((volatile int*)&w.desc->pass);
-    Eng eng;
-    eng.grp = Eng::Grp::make(smem + warp_smem_bytes(g));
-    const auto& grp = eng.grp;
-    const WarpState st = carve(smem + (size_t)grp.index() * warp_smem_bytes(g), g);
-    const int W2 = 2 * cfg.w;
-    int* rc = round_ctr(w, r);
-    // round 1: two children of every window entry; later rounds: the work list
-    const int nitems = (r == 1) ? 2 * cnt : *((volatile int*)(rc + 2));
-    const int2* items = w.items + (size_t)(r & 1) * (size_t)w.A * (size_t)W2;
-    const int cb = r & 1;
-    eng.load_graph(g, st);
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long global_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ inline void push_item(const Work& w, uint32_t item)
+{
     for (;;) {
-        int it = 0;
-        if (grp.rank() == 0) it = atomicAdd(&rc[0], 1);
-        it = grp.bcast(it);
-        if (it >= nitems) break;
-        const int2 item = (r == 1) ? make_int2(it >> 1, it & 1) : items[it];
-        const int a = item.x, c = item.y;
-        const int k = c >> 1, v = c & 1;
-        const SlotRef par = parent_ref(g, cfg, w, r, pbase, a, k);
-        const int pos = par.meta->next_pos;
-        if (pos < 0) continue;                     // a path with no unmasked node has no children
-        const size_t cslot = slot_index(w, cb, a, c, W2);
-        // s' of the child: flip the detectors of pos when it is fixed to 1
-        for (int q = grp.rank(); q < g.WM; q += grp.size()) {
-            uint32_t x = par.bits[q];
-            if (v) x ^= __ldg(g.hcol + (size_t)pos * g.WM + q);
-            st.sp[q] = x;
+        uint32_t* slot = w.ring + (atomicAdd(&w.ctr->b_tail, 1u) & w.ctr->b_mask);
+        const uint32_t old = atomicExch(slot, item);
+        if (old == kRingEmpty) return;
+        if (old == kRingLeft) {
+            // this ticket's group has left: take the item back unless the
+            // ring's next lap has drawn it already
+            if (atomicCAS(slot, item, kRingEmpty) != item) return;
+        } else {
+            item = old;                        // an item of the lap before, not drawn yet
         }
-        for (int q = grp.rank(); q < g.WN; q += grp.size()) {
-            uint32_t m = par.bits[g.WM + q];
-            uint32_t vv = par.bits[g.WM + g.WN + q];
-            if (q == (pos >> 5)) {
-                m |= 1u << (pos & 31);
-                if (v) vv |= 1u << (pos & 31);
-            }
-            st.mask[q] = m;
-            st.vals[q] = vv;
-        }
-        // warm start from the parent's snapshot
-        group_copy16(grp, st.E, par.E, snap_vec16(g));
-        eng.clear_sums(g, st);
-        grp.sync();
-        eng.fix_node(g, st, pos, cfg.L);
-        grp.sync();
-        // with num_results = 1, only the first success in visit order matters:
-        // a child stops once a lower-index sibling of this round has succeeded
-        AbortCheck ab{};
-        if (cfg.num_results == 1) {
-            ab.key = w.first_ok + a;
-            ab.stamp = (unsigned long long)(pass * (cfg.max_rounds + 1) + r) << 32;
-            ab.c = (unsigned)c;
-        }
-        int succ = 0;
-        const int iters = eng.run(g, cfg, st, cfg.iters_per_round, true, &succ, nullptr, false, ab);
-        int superseded = 0;
-        if (grp.rank() == 0) {
-            atomicAdd(&w.stats[1], (unsigned long long)iters);
-            if (ab.key != nullptr) {
-                if (succ) atomicMax(w.first_ok + a, ab.stamp | (0xffffffffull - (unsigned)c));
-                else superseded = ab.hit(*((volatile const unsigned long long*)ab.key)) ? 1 : 0;
-            }
-        }
-        // a superseded child's slot is never read: record only that it exists
-        if (grp.bcast(superseded)) {
-            if (grp.rank() == 0) {
-                SlotMeta m;
-                m.S = 0; m.iters = iters; m.next_pos = -1; m.success = 0; m.flags = 0;
-                w.slotMeta[cslot] = m;
-            }
-            grp.sync();
-            continue;
-        }
-        grp.sync();
-        for (int q = grp.rank(); q < g.WN; q += grp.size()) st.ehat[q] = (st.ehat[q] & ~st.mask[q]) | st.vals[q];
-        grp.sync();
-        int np, tie;
-        long long S;
-        eng.argmin_score(g, st, cfg.tie_guard, &np, &S, &tie);
-        group_copy16(grp, w.slotE + cslot * snap_bytes(g), st.E, snap_vec16(g));
-        uint32_t* cbits = w.slotBits + cslot * (size_t)w.SB;
-        for (int q = grp.rank(); q < g.WM; q += grp.size()) cbits[q] = st.sp[q];
-        for (int q = grp.rank(); q < g.WN; q += grp.size()) {
-            cbits[g.WM + q] = st.mask[q];
-            cbits[g.WM + g.WN + q] = st.vals[q];
-            cbits[g.WM + 2 * g.WN + q] = st.ehat[q];
-        }
-        if (grp.rank() == 0) {
-            SlotMeta m;
-            m.S = S; m.iters = iters; m.next_pos = np; m.success = succ; m.flags = tie;
-            w.slotMeta[cslot] = m;
-        }
-        grp.sync();
     }
 }
 
-// ----------------------------------------------------------------------------
-// per-shot selection after round r
-// ----------------------------------------------------------------------------
+// the next item, or kRingEmpty when every shot has ended (or none came for kIdleNs)
+__device__ inline uint32_t draw_item(const Work& w)
+{
+    uint32_t* slot = w.ring + (atomicAdd(&w.ctr->b_head, 1u) & w.ctr->b_mask);
+    unsigned long long t0 = 0ull;
+    for (unsigned spins = 0;; ++spins) {
+        const uint32_t v = ld_relaxed(slot);
+        if (v != kRingEmpty && v != kRingLeft) {
+            const uint32_t it = atomicExch(slot, kRingEmpty);
+            if (it != kRingEmpty && it != kRingLeft) {
+                __threadfence();               // the item before what it names
+                return it;
+            }
+            continue;
+        }
+        if ((spins & 3u) == 0u && ld_relaxed(reinterpret_cast<const uint32_t*>(&w.ctr->b_left)) == 0u) return kRingEmpty;
+        if (spins >= 4u) __nanosleep(200);
+        if ((spins & 63u) == 0u) {
+            const unsigned long long t = global_ns();
+            if (t0 == 0ull) t0 = t;
+            else if (t - t0 > kIdleNs && atomicCAS(slot, kRingEmpty, kRingLeft) == kRingEmpty) return kRingEmpty;
+        }
+    }
+}
+
 struct SelScratch {
     double score[2 * kMaxBeam];
     int iters[2 * kMaxBeam];
     int flags[2 * kMaxBeam];     // bit0 exists, bit1 success, bit2 argmin near-tie
 };
+static_assert(sizeof(SelScratch) == kSelectBytes, "the scratch warp_smem_bytes makes room for");
+
+// window entry a takes the shot of seed-store entry e (one warp): the seed
+// path is its only path (Alg. 3)
+__device__ inline void init_entry(const DevGraph& g, const DecCfg& cfg, const Work& w, int a, int e, int stamp)
+{
+    const int lane = threadIdx.x & 31;
+    const SlotMeta sm = w.seedMeta[e];
+    if (sm.success) {                  // num_results > 1: the seed result opens `results`
+        const uint32_t* eb = w.seedBits + (size_t)e * (size_t)w.SB + g.WM + 2 * g.WN;
+        uint32_t* rb = w.res_bits + (size_t)a * cfg.num_results * g.WN;
+        for (int q = lane; q < g.WN; q += 32) rb[q] = eb[q];
+        const long long W = vector_weight(g, eb);
+        if (lane == 0) {
+            w.res_w[(size_t)a * cfg.num_results] = W;
+            w.res_origin[(size_t)a * cfg.num_results] = 0;
+        }
+    }
+    if (lane == 0) {
+        w.shot_of[a] = w.seed_shot[e];
+        w.set_size[a] = 1;
+        w.iters_acc[a] = (unsigned long long)sm.iters;
+        w.res_n[a] = sm.success ? 1 : 0;
+        w.near[a] = sm.flags & 1;      // the seed path branches on its argmin
+        w.ent[a] = BeamEntry{e, 1, 2, stamp};
+    }
+    __syncwarp();
+}
+
+// the entries of the first items (the ring is filled by k_beam_ring)
+__global__ void k_beam_entries(DevGraph g, DecCfg cfg, Work w)
+{
+    count_launch(w);
+    const int cnt = w.ctr->b_next;
+    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int a = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); a < cnt; a += nw) {
+        init_entry(g, cfg, w, a, a, 1);
+        if ((threadIdx.x & 31) == 0) w.first_ok[a] = 0ull;   // no stamp is 0
+    }
+}
 
 __device__ void finalize_results(const DevGraph& g, const DecCfg& cfg, const Work& w, const Outputs& out,
                                  int a, long long gb, unsigned long long total, uint32_t extra)
 {
-    const int n = w.res_n[a];
+    const int n = __ldcg(w.res_n + a);
     const long long* rw = w.res_w + (size_t)a * cfg.num_results;
     int bi = 0;
-    for (int q = 1; q < n; ++q)
-        if (rw[q] < rw[bi]) bi = q;
-    const uint32_t st = (w.res_origin[(size_t)a * cfg.num_results + bi] == 0) ? ST_SEED : ST_BEAM;
-    finalize_shot(g, out, gb, w.res_bits + ((size_t)a * cfg.num_results + bi) * g.WN, st | extra, total);
+    long long wb = __ldcg(rw);
+    for (int q = 1; q < n; ++q) {
+        const long long wq = __ldcg(rw + q);
+        if (wq < wb) { bi = q; wb = wq; }
+    }
+    const uint32_t st = (__ldcg(w.res_origin + (size_t)a * cfg.num_results + bi) == 0) ? ST_SEED : ST_BEAM;
+    finalize_shot<WarpGroup, false, true>(g, out, gb, w.res_bits + ((size_t)a * cfg.num_results + bi) * g.WN,
+                                          st | extra, total);
 }
 
-__global__ void __launch_bounds__(256) k_select(DevGraph g, DecCfg cfg, Work w, int r)
+// one warp, after the last child of the round of window entry a: first success
+// in visit order, `results`, top-w pruning (Alg. 3, App. B), then the next
+// round's items, or the shot's outputs and the entry's next shot.  Everything
+// read here was written by other SMs during this kernel (__ldcg).
+__device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, const Work& w, int a, SelScratch* sc)
+{
+    const int lane = threadIdx.x & 31;
+    const int W2 = 2 * cfg.w;
+    const RunDesc d = *w.desc;
+    const BeamEntry ent = load_entry(w.ent + a);
+    const int r = ent.round;
+    const int cb = r & 1;
+    const long long gb = d.chunk_base + __ldcg(w.shot_of + a);
+    const int npar = __ldcg(w.set_size + a);
+    const int nch = 2 * npar;
+    // gather the children of this round in canonical order c = 2 * rank + val
+    for (int c = lane; c < nch; c += 32) {
+        const int pnp = __ldcg(&parent_ref(g, cfg, w, r, ent.seed, a, c >> 1).meta->next_pos);
+        int fl = 0, it = 0;
+        double scv = 0.0;
+        if (pnp >= 0) {
+            const SlotMeta m = load_meta(w.slotMeta + slot_index(w, cb, a, c, W2));
+            fl = 1 | (m.success ? 2 : 0) | ((m.flags & 1) << 2);
+            it = m.iters;
+            scv = ((double)m.S / kFixScale) / (double)m.iters;
+        }
+        sc->flags[c] = fl;
+        sc->iters[c] = it;
+        sc->score[c] = scv;
+    }
+    __syncwarp();
+    unsigned long long acc = __ldcg(w.iters_acc + a);
+    bool done = false;
+    // near-tie record: argmin margins of the children the sequential
+    // algorithm visits, and the pruning margin of the round
+    int near = __ldcg(w.near + a);
+    auto near_upto = [&](int last) {
+        int f = 0;
+        for (int c = lane; c <= last && c < nch; c += 32) f |= (sc->flags[c] >> 2) & 1;
+        return __any_sync(FULLMASK, f != 0) ? 1 : 0;
+    };
+    if (cfg.num_results == 1) {
+        // Alg. 3: the first successful child in visit order ends the search
+        int first = 0x7fffffff;
+        for (int c = lane; c < nch; c += 32)
+            if ((sc->flags[c] & 3) == 3 && c < first) first = c;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) first = min(first, __shfl_xor_sync(FULLMASK, first, o));
+        if (first != 0x7fffffff) {
+            unsigned long long sum = 0;
+            for (int c = lane; c <= first; c += 32)
+                if (sc->flags[c] & 1) sum += (unsigned long long)sc->iters[c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULLMASK, sum, o);
+            const uint32_t* eb = w.slotBits + slot_index(w, cb, a, first, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
+            near |= near_upto(first);
+            finalize_shot<WarpGroup, false, true>(g, d.out, gb, eb, ST_BEAM | (near ? ST_NEAR : 0u), acc + sum);
+            done = true;
+        }
+    } else {
+        // results collection in visit order (dedupe by equality, App. B)
+        unsigned long long sum = 0;
+        for (int c = 0; c < nch && !done; ++c) {
+            const int fl = sc->flags[c];
+            if (!(fl & 1)) continue;
+            sum += (unsigned long long)sc->iters[c];
+            if (!(fl & 2)) continue;
+            const uint32_t* eb = w.slotBits + slot_index(w, cb, a, c, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
+            const int nres = __ldcg(w.res_n + a);
+            bool dup = false;
+            for (int q = 0; q < nres && !dup; ++q) {
+                const uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + q) * g.WN;
+                bool eq = true;
+                for (int x = lane; x < g.WN; x += 32) eq = eq && (__ldcg(rb + x) == __ldcg(eb + x));
+                dup = __all_sync(FULLMASK, eq);
+            }
+            if (!dup) {
+                uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + nres) * g.WN;
+                for (int x = lane; x < g.WN; x += 32) rb[x] = __ldcg(eb + x);
+                const long long W = vector_weight(g, eb);
+                __syncwarp();
+                if (lane == 0) {
+                    w.res_w[(size_t)a * cfg.num_results + nres] = W;
+                    w.res_origin[(size_t)a * cfg.num_results + nres] = 1;
+                    w.res_n[a] = nres + 1;
+                }
+                __syncwarp();
+                if (nres + 1 >= cfg.num_results) {
+                    near |= near_upto(c);
+                    finalize_results(g, cfg, w, d.out, a, gb, acc + sum, near ? ST_NEAR : 0u);
+                    done = true;
+                }
+            }
+        }
+    }
+    if (!done) {
+        unsigned long long sum = 0;
+        int nex = 0;
+        for (int c = lane; c < nch; c += 32) {
+            if (sc->flags[c] & 1) { sum += (unsigned long long)sc->iters[c]; ++nex; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sum += __shfl_xor_sync(FULLMASK, sum, o);
+            nex += __shfl_xor_sync(FULLMASK, nex, o);
+        }
+        acc += sum;
+        near |= near_upto(nch - 1);
+        // rank of each existing child under (score desc, canonical index asc)
+        int myrank[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = lane + 32 * q;
+            myrank[q] = -1;
+            if (c < nch && (sc->flags[c] & 1)) {
+                const double s0 = sc->score[c];
+                int rk = 0;
+                for (int c2 = 0; c2 < nch; ++c2) {
+                    if (!(sc->flags[c2] & 1)) continue;
+                    const double s2 = sc->score[c2];
+                    rk += (s2 > s0 || (s2 == s0 && c2 < c)) ? 1 : 0;
+                }
+                myrank[q] = rk;
+            }
+        }
+        // the kept paths of a round before the last, and how many of them
+        // have a node left to branch on (their children make round r + 1)
+        const bool last = (r >= cfg.max_rounds || nex == 0);
+        int keep = 0, tot = 0;
+        if (!last) {
+            __syncwarp();
+            keep = nex < cfg.w ? nex : cfg.w;
+            if (cfg.tie_guard > 0.0 && nex > keep) {
+                // pruning margin: last kept (rank keep-1) against first dropped (rank keep)
+                double s_in = -INFINITY, s_out = -INFINITY;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (myrank[q] == keep - 1) s_in = sc->score[lane + 32 * q];
+                    if (myrank[q] == keep) s_out = sc->score[lane + 32 * q];
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    s_in = fmax(s_in, __shfl_xor_sync(FULLMASK, s_in, o));
+                    s_out = fmax(s_out, __shfl_xor_sync(FULLMASK, s_out, o));
+                }
+                const double den = fabs(s_in) > 1.0 ? fabs(s_in) : 1.0;
+                const double gap = (s_in - s_out) / den;
+                if (gap > 0.0 && gap < cfg.tie_guard) near = 1;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (myrank[q] >= 0 && myrank[q] < keep)
+                    w.set_idx[(size_t)a * cfg.w + myrank[q]] = (uint8_t)(lane + 32 * q);
+            __syncwarp();
+            int cntp = 0;
+            for (int k = lane; k < keep; k += 32) {
+                const int c = w.set_idx[(size_t)a * cfg.w + k];
+                cntp += (__ldcg(&w.slotMeta[slot_index(w, cb, a, c, W2)].next_pos) >= 0) ? 1 : 0;
+            }
+            tot = cntp;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(FULLMASK, tot, o);
+        }
+        if (last || tot == 0) {
+            // the search ends here: the last round, no child, or no kept
+            // path with a node left (the next round would have no child)
+            if (cfg.num_results > 1 && __ldcg(w.res_n + a) > 0) {
+                finalize_results(g, cfg, w, d.out, a, gb, acc, near ? ST_NEAR : 0u);
+            } else {
+                // no valid solution: the best path of the final set
+                int best = 0x7fffffff;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (myrank[q] == 0) best = lane + 32 * q;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(FULLMASK, best, o));
+                const uint32_t* eb;
+                if (best != 0x7fffffff)
+                    eb = w.slotBits + slot_index(w, cb, a, best, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
+                else
+                    eb = parent_ref(g, cfg, w, r, ent.seed, a, 0).bits + g.WM + 2 * g.WN;
+                finalize_shot<WarpGroup, false, true>(g, d.out, gb, eb, ST_FAILED | (near ? ST_NEAR : 0u), acc);
+            }
+            done = true;
+        } else {
+            // the kept slots become the next round's parents: two children per
+            // kept path that has a next_pos
+            if (lane == 0) {
+                w.set_size[a] = keep;
+                w.iters_acc[a] = acc;
+                w.near[a] = near;
+                w.ent[a] = BeamEntry{ent.seed, r + 1, 2 * tot, ent.stamp + 1};
+            }
+            __syncwarp();
+            __threadfence();                   // the entry before its items
+            for (int k = lane; k < keep; k += 32) {
+                const int c = __ldcg(w.set_idx + (size_t)a * cfg.w + k);
+                if (__ldcg(&w.slotMeta[slot_index(w, cb, a, c, W2)].next_pos) >= 0) {
+                    push_item(w, ring_item(a, 2 * k));
+                    push_item(w, ring_item(a, 2 * k + 1));
+                }
+            }
+        }
+    }
+    if (done) {
+        // the entry's next shot, then this one is counted off
+        __syncwarp();
+        int e = 0;
+        if (lane == 0) e = atomicAdd(&w.ctr->b_next, 1);
+        e = __shfl_sync(FULLMASK, e, 0);
+        if (e < w.ctr->n_active) {
+            init_entry(g, cfg, w, a, e, ent.stamp + 1);
+            __threadfence();
+            if (lane < 2) push_item(w, ring_item(a, lane));
+        }
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            atomicSub(&w.ctr->b_left, 1);
+        }
+    }
+}
+
+// expand a child and run masked BP (Alg. 2), item by item
+template <class Eng>
+__global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(DevGraph g, DecCfg cfg, Work w)
 {
     extern __shared__ __align__(16) char smem[];
     count_launch(w);
-    if (r <= 0) r = *((volatile int*)&w.desc->round);   // graph launches: the round counter
-    long long pbase;
-    const int cnt = window(w, &pbase);
-    if (cnt == 0) return;
-    const int lane = threadIdx.x & 31;
-    const int wid = threadIdx.x >> 5;
-    SelScratch* sc = reinterpret_cast<SelScratch*>(smem) + wid;
+    Eng eng;
+    eng.grp = Eng::Grp::make(smem + warp_smem_bytes(g));
+    const auto& grp = eng.grp;
+    char* const own = smem + (size_t)grp.index() * warp_smem_bytes(g);
+    const WarpState st = carve(own, g);
+    // never more tickets waiting than half the ring
+    if ((uint32_t)(blockIdx.x * grp.per_block() + grp.index()) > w.ctr->b_mask / 2) return;
     const int W2 = 2 * cfg.w;
-    const RunDesc d = *w.desc;
-    int* rc = round_ctr(w, r);
-    const int cb = r & 1;
-    int acur = 0, aend = 0;                      // window entries claimed four at a time
+    unsigned long long ran = 0;                // BP iterations (group rank 0)
     for (;;) {
-        if (acur >= aend) {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(&rc[1], 4);
-            acur = __shfl_sync(FULLMASK, base, 0);
-            aend = acur + 4;
-        }
-        const int a = acur++;
-        if (a >= cnt) break;
-        if (r == 1) {
-            // a new window entry: the seed path is its only path (Alg. 3)
-            const size_t e = (size_t)(pbase + a);
-            const SlotMeta sm = w.seedMeta[e];
-            if (sm.success) {                  // num_results > 1: the seed result opens `results`
-                const uint32_t* eb = w.seedBits + e * (size_t)w.SB + g.WM + 2 * g.WN;
-                uint32_t* rb = w.res_bits + (size_t)a * cfg.num_results * g.WN;
-                for (int q = lane; q < g.WN; q += 32) rb[q] = eb[q];
-                const long long W = vector_weight(g, eb);
-                if (lane == 0) {
-                    w.res_w[(size_t)a * cfg.num_results] = W;
-                    w.res_origin[(size_t)a * cfg.num_results] = 0;
+        uint32_t item = kRingEmpty;
+        if (grp.rank() == 0) item = draw_item(w);
+        item = (uint32_t)grp.bcast((int)item);
+        if (item == kRingEmpty) break;
+        const int a = ring_entry(item), c = ring_child(item);
+        const BeamEntry ent = load_entry(w.ent + a);
+        const int r = ent.round;
+        const int k = c >> 1, v = c & 1;
+        const SlotRef par = parent_ref(g, cfg, w, r, ent.seed, a, k);
+        const int pos = __ldcg(&par.meta->next_pos);
+        if (pos >= 0) {                        // (a path with no unmasked node has no children)
+            const size_t cslot = slot_index(w, r & 1, a, c, W2);
+            // s' of the child: flip the detectors of pos when it is fixed to 1
+            for (int q = grp.rank(); q < g.WM; q += grp.size()) {
+                uint32_t x = __ldcg(par.bits + q);
+                if (v) x ^= __ldg(g.hcol + (size_t)pos * g.WM + q);
+                st.sp[q] = x;
+            }
+            for (int q = grp.rank(); q < g.WN; q += grp.size()) {
+                uint32_t m = __ldcg(par.bits + g.WM + q);
+                uint32_t vv = __ldcg(par.bits + g.WM + g.WN + q);
+                if (q == (pos >> 5)) {
+                    m |= 1u << (pos & 31);
+                    if (v) vv |= 1u << (pos & 31);
+                }
+                st.mask[q] = m;
+                st.vals[q] = vv;
+            }
+            // (the engine's tables are read again for each child: nothing of them
+            // is kept in registers across the selection's call)
+            eng.load_graph(g, st);
+            // warm start from the parent's snapshot
+            group_copy16<true>(grp, st.E, par.E, snap_vec16(g));
+            eng.clear_sums(g, st);
+            grp.sync();
+            eng.fix_node(g, st, pos, cfg.L);
+            grp.sync();
+            // with num_results = 1, only the first success in visit order matters:
+            // a child stops once a lower-index sibling of this round has succeeded
+            AbortCheck ab{};
+            if (cfg.num_results == 1) {
+                ab.key = w.first_ok + a;
+                ab.stamp = (unsigned long long)(unsigned)ent.stamp << 32;
+                ab.c = (unsigned)c;
+            }
+            int succ = 0;
+            const int iters = eng.run(g, cfg, st, cfg.iters_per_round, true, &succ, nullptr, false, ab);
+            int superseded = 0;
+            if (grp.rank() == 0) {
+                ran += (unsigned long long)iters;
+                if (ab.key != nullptr) {
+                    if (succ) atomicMax(w.first_ok + a, ab.stamp | (0xffffffffull - (unsigned)c));
+                    else superseded = ab.hit(*((volatile const unsigned long long*)ab.key)) ? 1 : 0;
                 }
             }
-            if (lane == 0) {
-                w.shot_of[a] = w.seed_shot[e];
-                w.set_size[a] = 1;
-                w.iters_acc[a] = (unsigned long long)sm.iters;
-                w.done[a] = 0;
-                w.res_n[a] = sm.success ? 1 : 0;
-                w.near[a] = sm.flags & 1;      // the seed path branches on its argmin
-            }
-            __syncwarp();
-        } else if (w.done[a]) {
-            continue;
-        }
-        const long long gb = d.chunk_base + w.shot_of[a];
-        const int npar = w.set_size[a];
-        const int nch = 2 * npar;
-        // gather the children of this round in canonical order c = 2 * rank + val
-        for (int c = lane; c < nch; c += 32) {
-            const int pnp = parent_ref(g, cfg, w, r, pbase, a, c >> 1).meta->next_pos;
-            int fl = 0, it = 0;
-            double scv = 0.0;
-            if (pnp >= 0) {
-                const SlotMeta m = w.slotMeta[slot_index(w, cb, a, c, W2)];
-                fl = 1 | (m.success ? 2 : 0) | ((m.flags & 1) << 2);
-                it = m.iters;
-                scv = ((double)m.S / kFixScale) / (double)m.iters;
-            }
-            sc->flags[c] = fl;
-            sc->iters[c] = it;
-            sc->score[c] = scv;
-        }
-        __syncwarp();
-        unsigned long long acc = w.iters_acc[a];
-        bool done = false;
-        // near-tie record: argmin margins of the children the sequential
-        // algorithm visits, and the pruning margin of the round
-        int near = w.near[a];
-        auto near_upto = [&](int last) {
-            int f = 0;
-            for (int c = lane; c <= last && c < nch; c += 32) f |= (sc->flags[c] >> 2) & 1;
-            return __any_sync(FULLMASK, f != 0) ? 1 : 0;
-        };
-        if (cfg.num_results == 1) {
-            // Alg. 3: the first successful child in visit order ends the search
-            int first = 0x7fffffff;
-            for (int c = lane; c < nch; c += 32)
-                if ((sc->flags[c] & 3) == 3 && c < first) first = c;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) first = min(first, __shfl_xor_sync(FULLMASK, first, o));
-            if (first != 0x7fffffff) {
-                unsigned long long sum = 0;
-                for (int c = lane; c <= first; c += 32)
-                    if (sc->flags[c] & 1) sum += (unsigned long long)sc->iters[c];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULLMASK, sum, o);
-                const uint32_t* eb = w.slotBits + slot_index(w, cb, a, first, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
-                near |= near_upto(first);
-                finalize_shot(g, d.out, gb, eb, ST_BEAM | (near ? ST_NEAR : 0u), acc + sum);
-                done = true;
-            }
-        } else {
-            // results collection in visit order (dedupe by equality, App. B)
-            unsigned long long sum = 0;
-            for (int c = 0; c < nch && !done; ++c) {
-                const int fl = sc->flags[c];
-                if (!(fl & 1)) continue;
-                sum += (unsigned long long)sc->iters[c];
-                if (!(fl & 2)) continue;
-                const uint32_t* eb = w.slotBits + slot_index(w, cb, a, c, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
-                const int nres = w.res_n[a];
-                bool dup = false;
-                for (int q = 0; q < nres && !dup; ++q) {
-                    const uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + q) * g.WN;
-                    bool eq = true;
-                    for (int x = lane; x < g.WN; x += 32) eq = eq && (rb[x] == eb[x]);
-                    dup = __all_sync(FULLMASK, eq);
+            // a superseded child's slot is never read: record only that it exists
+            if (grp.bcast(superseded)) {
+                if (grp.rank() == 0) {
+                    SlotMeta m;
+                    m.S = 0; m.iters = iters; m.next_pos = -1; m.success = 0; m.flags = 0;
+                    w.slotMeta[cslot] = m;
                 }
-                if (!dup) {
-                    uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + nres) * g.WN;
-                    for (int x = lane; x < g.WN; x += 32) rb[x] = eb[x];
-                    const long long W = vector_weight(g, eb);
-                    __syncwarp();
-                    if (lane == 0) {
-                        w.res_w[(size_t)a * cfg.num_results + nres] = W;
-                        w.res_origin[(size_t)a * cfg.num_results + nres] = 1;
-                        w.res_n[a] = nres + 1;
-                    }
-                    __syncwarp();
-                    if (nres + 1 >= cfg.num_results) {
-                        near |= near_upto(c);
-                        finalize_results(g, cfg, w, d.out, a, gb, acc + sum, near ? ST_NEAR : 0u);
-                        done = true;
-                    }
-                }
-            }
-        }
-        if (!done) {
-            unsigned long long sum = 0;
-            int nex = 0;
-            for (int c = lane; c < nch; c += 32) {
-                if (sc->flags[c] & 1) { sum += (unsigned long long)sc->iters[c]; ++nex; }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sum += __shfl_xor_sync(FULLMASK, sum, o);
-                nex += __shfl_xor_sync(FULLMASK, nex, o);
-            }
-            acc += sum;
-            near |= near_upto(nch - 1);
-            // rank of each existing child under (score desc, canonical index asc)
-            int myrank[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = lane + 32 * q;
-                myrank[q] = -1;
-                if (c < nch && (sc->flags[c] & 1)) {
-                    const double s0 = sc->score[c];
-                    int rk = 0;
-                    for (int c2 = 0; c2 < nch; ++c2) {
-                        if (!(sc->flags[c2] & 1)) continue;
-                        const double s2 = sc->score[c2];
-                        rk += (s2 > s0 || (s2 == s0 && c2 < c)) ? 1 : 0;
-                    }
-                    myrank[q] = rk;
-                }
-            }
-            // the kept paths of a round before the last, and how many of them
-            // have a node left to branch on (their children make round r + 1)
-            const bool last = (r >= cfg.max_rounds || nex == 0);
-            int keep = 0, tot = 0;
-            if (!last) {
-                __syncwarp();
-                keep = nex < cfg.w ? nex : cfg.w;
-                if (cfg.tie_guard > 0.0 && nex > keep) {
-                    // pruning margin: last kept (rank keep-1) against first dropped (rank keep)
-                    double s_in = -INFINITY, s_out = -INFINITY;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if (myrank[q] == keep - 1) s_in = sc->score[lane + 32 * q];
-                        if (myrank[q] == keep) s_out = sc->score[lane + 32 * q];
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        s_in = fmax(s_in, __shfl_xor_sync(FULLMASK, s_in, o));
-                        s_out = fmax(s_out, __shfl_xor_sync(FULLMASK, s_out, o));
-                    }
-                    const double den = fabs(s_in) > 1.0 ? fabs(s_in) : 1.0;
-                    const double gap = (s_in - s_out) / den;
-                    if (gap > 0.0 && gap < cfg.tie_guard) near = 1;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (myrank[q] >= 0 && myrank[q] < keep)
-                        w.set_idx[(size_t)a * cfg.w + myrank[q]] = (uint8_t)(lane + 32 * q);
-                __syncwarp();
-                int cntp = 0;
-                for (int k = lane; k < keep; k += 32) {
-                    const int c = w.set_idx[(size_t)a * cfg.w + k];
-                    cntp += (w.slotMeta[slot_index(w, cb, a, c, W2)].next_pos >= 0) ? 1 : 0;
-                }
-                tot = cntp;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(FULLMASK, tot, o);
-            }
-            if (last || tot == 0) {
-                // the search ends here: the last round, no child, or no kept
-                // path with a node left (the next round would have no child)
-                if (cfg.num_results > 1 && w.res_n[a] > 0) {
-                    finalize_results(g, cfg, w, d.out, a, gb, acc, near ? ST_NEAR : 0u);
-                } else {
-                    // no valid solution: the best path of the final set
-                    int best = 0x7fffffff;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (myrank[q] == 0) best = lane + 32 * q;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(FULLMASK, best, o));
-                    const uint32_t* eb;
-                    if (best != 0x7fffffff)
-                        eb = w.slotBits + slot_index(w, cb, a, best, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
-                    else
-                        eb = parent_ref(g, cfg, w, r, pbase, a, 0).bits + g.WM + 2 * g.WN;
-                    finalize_shot(g, d.out, gb, eb, ST_FAILED | (near ? ST_NEAR : 0u), acc);
-                }
-                done = true;
             } else {
-                // the kept slots become the next round's parents: two children per
-                // kept path that has a next_pos
-                int wbase = 0;
-                if (lane == 0) {
-                    w.set_size[a] = keep;
-                    w.iters_acc[a] = acc;
-                    w.near[a] = near;
-                    wbase = atomicAdd(&round_ctr(w, r + 1)[2], 2 * tot);
+                grp.sync();
+                for (int q = grp.rank(); q < g.WN; q += grp.size())
+                    st.ehat[q] = (st.ehat[q] & ~st.mask[q]) | st.vals[q];
+                grp.sync();
+                int np, tie;
+                long long S;
+                eng.argmin_score(g, st, cfg.tie_guard, &np, &S, &tie);
+                group_copy16(grp, w.slotE + cslot * snap_bytes(g), st.E, snap_vec16(g));
+                uint32_t* cbits = w.slotBits + cslot * (size_t)w.SB;
+                for (int q = grp.rank(); q < g.WM; q += grp.size()) cbits[q] = st.sp[q];
+                for (int q = grp.rank(); q < g.WN; q += grp.size()) {
+                    cbits[g.WM + q] = st.mask[q];
+                    cbits[g.WM + g.WN + q] = st.vals[q];
+                    cbits[g.WM + 2 * g.WN + q] = st.ehat[q];
                 }
-                wbase = __shfl_sync(FULLMASK, wbase, 0);
-                if (lane == 0) {
-                    int2* items = w.items + (size_t)((r + 1) & 1) * (size_t)w.A * (size_t)W2;
-                    int o = 0;
-                    for (int k = 0; k < keep; ++k) {
-                        const int c = w.set_idx[(size_t)a * cfg.w + k];
-                        if (w.slotMeta[slot_index(w, cb, a, c, W2)].next_pos >= 0) {
-                            items[wbase + o] = make_int2(a, 2 * k);
-                            items[wbase + o + 1] = make_int2(a, 2 * k + 1);
-                            o += 2;
-                        }
-                    }
+                if (grp.rank() == 0) {
+                    SlotMeta m;
+                    m.S = S; m.iters = iters; m.next_pos = np; m.success = succ; m.flags = tie;
+                    w.slotMeta[cslot] = m;
                 }
             }
         }
-        if (done && lane == 0) w.done[a] = 1;
-        __syncwarp();
+        // the slot before the count; the round's last child selects
+        __threadfence();
+        grp.sync();
+        int last = 0;
+        if (grp.rank() == 0) {
+            last = atomicSub(&w.ent[a].pending, 1) == 1 ? 1 : 0;
+            __threadfence();
+        }
+        if (grp.bcast(last)) {
+            if (grp.warp() == 0) select_entry(g, cfg, w, a, reinterpret_cast<SelScratch*>(own));
+            grp.sync();
+        }
     }
+    if (grp.rank() == 0 && ran != 0ull) atomicAdd(&w.stats[1], ran);
 }
 
 // ----------------------------------------------------------------------------
@@ -1849,12 +1950,9 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     ls->warps_per_block = wpb;
     ls->smem_bp = gw >= 2 ? per_cand + 16 * sizeof(ArgRec) : per_cand * (size_t)wpb;
     if (ls->smem_bp > (size_t)max_optin) return -5;
-    // the selection kernel handles one shot per warp in blocks of at most 8 warps
-    ls->select_warps = wpb < 8 ? wpb : 8;
-    ls->smem_select = sizeof(SelScratch) * (size_t)ls->select_warps;
     ls->dv = eng;
     const int threads = 32 * wpb;
-    int rc = 0, bps_bp = 0, bps_sel = 0;
+    int rc = 0, bps_bp = 0;
     // The dynamic shared-memory limit is a property of the kernel, shared by
     // every decoder that launches it; it is raised to the device maximum so
     // that no decoder created later can lower it below what an earlier one
@@ -1871,11 +1969,7 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
         default: return -5;
     }
     if (rc) return rc;
-    if (CUDA_FAILED(cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin)) ||
-        CUDA_FAILED(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_sel, k_select, 32 * ls->select_warps,
-                                                                  ls->smem_select)))
-        return -2;
-    if (bps_bp < 1 || bps_sel < 1) return -5;
+    if (bps_bp < 1) return -5;
     // the first-iteration screen: generic engines, the scale alpha, every
     // Lambda_j > 0, one result
     ls->screen = 0;
@@ -1903,7 +1997,6 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     }
     ls->grid_seed = sms * bps_bp;
     ls->grid_round = sms * bps_bp;
-    ls->grid_select = sms * bps_sel;
     // the batched seed BP: generic engines with the scale alpha and one result
     // (the shots it finishes need no snapshot; the others are decoded again by
     // the per-candidate seed kernel)
@@ -1931,8 +2024,7 @@ static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, c
                           const LaunchHooks* hk, cudaGraphExec_t gx, int* host_n_active)
 {
     const int threads = 32 * ls.warps_per_block;
-    const int nri = 3 * (cfg.max_rounds + 2);
-    k_begin_chunk<<<1, 128, 0, s>>>(w, nri, synd, out, base, n);
+    k_begin_chunk<<<1, 32, 0, s>>>(w, synd, out, base, n);
     if (CUDA_FAILED(cudaGetLastError())) return -2;
     if (gx != nullptr) return !CUDA_FAILED(cudaGraphLaunch(gx, s)) ? 0 : -2;
     if (ls.screen) {
@@ -1940,9 +2032,9 @@ static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, c
         launch_screen(g, cfg, w, ls, s);
         if (hk) hk->after(hk->ctx, 11);
     }
-    // the seed kernel on its shots, then exactly the beam passes they need
-    // (without a graph the number of active entries is read back)
-    auto seed_and_passes = [&](int seed_src) -> int {
+    // the seed kernel on its shots, then the beam if any needs it (without a
+    // graph the number of active entries is read back)
+    auto seed_and_beam = [&](int seed_src) -> int {
         if (hk) hk->before(hk->ctx, 0);
         k_seed<Eng><<<ls.grid_seed, threads, ls.smem_bp, s>>>(g, cfg, w, seed_src);
         if (hk) hk->after(hk->ctx, 0);
@@ -1951,21 +2043,18 @@ static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, c
         if (CUDA_FAILED(cudaMemcpyAsync(host_n_active, &w.ctr->n_active, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
             CUDA_FAILED(cudaStreamSynchronize(s)))
             return -2;
-        const long long passes = (*host_n_active + w.A - 1) / w.A;
-        for (long long p = 0; p < passes; ++p) {
-            for (int r = 1; r <= cfg.max_rounds; ++r) {
-                if (hk) hk->before(hk->ctx, 1);
-                k_round<Eng><<<ls.grid_round, threads, ls.smem_bp, s>>>(g, cfg, w, r);
-                if (hk) { hk->after(hk->ctx, 1); hk->before(hk->ctx, 2); }
-                k_select<<<ls.grid_select, 32 * ls.select_warps, ls.smem_select, s>>>(g, cfg, w, r);
-                if (hk) hk->after(hk->ctx, 2);
-            }
-            k_pass_end<<<1, 128, 0, s>>>(w, nri, cudaGraphConditionalHandle{}, 0);
-            if (CUDA_FAILED(cudaGetLastError())) return -2;
-        }
-        return 0;
+        if (*host_n_active == 0) return 0;
+        if (hk) hk->before(hk->ctx, 2);
+        k_beam_begin<<<1, 32, 0, s>>>(w, cfg.w);
+        k_beam_ring<<<ls.grid_seed, 256, 0, s>>>(w);
+        k_beam_entries<<<ls.grid_seed, 256, 0, s>>>(g, cfg, w);
+        if (hk) { hk->after(hk->ctx, 2); hk->before(hk->ctx, 1); }
+        k_round<Eng><<<ls.grid_round, threads, ls.smem_bp, s>>>(g, cfg, w);
+        if (hk) hk->after(hk->ctx, 1);
+        k_beam_end<<<1, 32, 0, s>>>(w);
+        return CUDA_FAILED(cudaGetLastError()) ? -2 : 0;
     };
-    if (!(ls.batch && w.bs_slots > 0)) return seed_and_passes(ls.screen);
+    if (!(ls.batch && w.bs_slots > 0)) return seed_and_beam(ls.screen);
     // batched seed BP over the chunk, then the shots it handed on in windows
     // of at most S (the seed store)
     if (launch_batch_direct(g, cfg, w, ls, ls.screen, s, hk, host_n_active)) return -2;
@@ -1974,9 +2063,9 @@ static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, c
         return -2;
     const long long n_fail = *host_n_active;
     for (long long wb = 0; wb < n_fail; wb += w.S) {
-        k_win_begin<<<1, 128, 0, s>>>(w, nri, (int)wb);
+        k_win_begin<<<1, 32, 0, s>>>(w, (int)wb);
         if (CUDA_FAILED(cudaGetLastError())) return -2;
-        const int rc = seed_and_passes(2);
+        const int rc = seed_and_beam(2);
         if (rc) return rc;
     }
     return 0;
@@ -1997,7 +2086,7 @@ int launch_chunk(const DevGraph& g, const DecCfg& cfg, const Work& w, const Laun
     }
 }
 
-// ---- the per-chunk graph: k_seed, then WHILE(another window) { rounds, k_pass_end }
+// ---- the per-chunk graph: k_seed, then IF (a shot needs the beam) { the beam }
 static int add_kernel(cudaGraph_t graph, cudaGraphNode_t* node, const cudaGraphNode_t* dep, void* func, int grid,
                       int block, size_t smem, void** args)
 {
@@ -2010,64 +2099,43 @@ static int add_kernel(cudaGraph_t graph, cudaGraphNode_t* node, const cudaGraphN
     return !CUDA_FAILED(cudaGraphAddKernelNode(node, graph, dep, dep ? 1 : 0, &p)) ? 0 : -2;
 }
 
-// WHILE (a window of active shots left) { round 1, WHILE (the next round has
-// children) { round r, selection, round end }, pass end }, after `dep` in
-// `graph`: a chunk runs exactly the passes and rounds it needs
+// IF (a shot needs the beam) { its set-up, the beam, the check that no shot is
+// left } after `dep` in `graph`
 template <class Eng>
 static int add_beam_nodes(cudaGraph_t graph, cudaGraphNode_t dep, cudaGraphNode_t* last, DevGraph& g, DecCfg& cfg,
                           Work& w, const LaunchShape& ls)
 {
-    const int threads = 32 * ls.warps_per_block;
-    int nri = 3 * (cfg.max_rounds + 2);
     int rc = 0;
-    cudaGraphConditionalHandle cpass, cround;
-    cudaGraphNode_t gate, wpass, rbegin, wround, pend;
-    cudaGraphNodeParams cp{};
-    if (CUDA_FAILED(cudaGraphConditionalHandleCreate(&cpass, graph, 0, cudaGraphCondAssignDefault))) rc = -2;
+    cudaGraphConditionalHandle cbeam;
+    cudaGraphNode_t gate, beam, begin, ring, entries, round, end;
+    if (CUDA_FAILED(cudaGraphConditionalHandleCreate(&cbeam, graph, 0, cudaGraphCondAssignDefault))) rc = -2;
     if (!rc) {
-        void* gargs[] = {&w, &cpass};
-        rc = add_kernel(graph, &gate, &dep, (void*)k_pass_gate, 1, 32, 0, gargs);
+        void* gargs[] = {&w, &cbeam};
+        rc = add_kernel(graph, &gate, &dep, (void*)k_beam_gate, 1, 32, 0, gargs);
     }
+    cudaGraphNodeParams cp{};
     if (!rc) {
         cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = cpass;
-        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.handle = cbeam;
+        cp.conditional.type = cudaGraphCondTypeIf;
         cp.conditional.size = 1;
-        if (CUDA_FAILED(cudaGraphAddNode(&wpass, graph, &gate, nullptr, 1, &cp))) rc = -2;
-    }
-    cudaGraph_t body = rc ? nullptr : cp.conditional.phGraph_out[0];
-    if (!rc && CUDA_FAILED(cudaGraphConditionalHandleCreate(&cround, body, 0, 0))) rc = -2;
-    if (!rc) {
-        void* bargs[] = {&w, &cround};
-        rc = add_kernel(body, &rbegin, nullptr, (void*)k_rounds_begin, 1, 32, 0, bargs);
-    }
-    cudaGraphNodeParams cr{};
-    if (!rc) {
-        cr.type = cudaGraphNodeTypeConditional;
-        cr.conditional.handle = cround;
-        cr.conditional.type = cudaGraphCondTypeWhile;
-        cr.conditional.size = 1;
-        if (CUDA_FAILED(cudaGraphAddNode(&wround, body, &rbegin, nullptr, 1, &cr))) rc = -2;
+        if (CUDA_FAILED(cudaGraphAddNode(&beam, graph, &gate, nullptr, 1, &cp))) rc = -2;
     }
     if (!rc) {
-        // kernel parameters are copied when a node is added; round 0 means
-        // "read the round counter"
-        cudaGraph_t rbody = cr.conditional.phGraph_out[0];
-        cudaGraphNode_t nr, ns, ne;
-        int r0 = 0, maxr = cfg.max_rounds;
-        void* rargs[] = {&g, &cfg, &w, &r0};
-        rc = add_kernel(rbody, &nr, nullptr, (void*)k_round<Eng>, ls.grid_round, threads, ls.smem_bp, rargs);
-        if (!rc) rc = add_kernel(rbody, &ns, &nr, (void*)k_select, ls.grid_select, 32 * ls.select_warps,
-                                    ls.smem_select, rargs);
-        void* eargs[] = {&w, &maxr, &cround};
-        if (!rc) rc = add_kernel(rbody, &ne, &ns, (void*)k_round_end, 1, 32, 0, eargs);
+        // kernel parameters are copied when a node is added
+        cudaGraph_t body = cp.conditional.phGraph_out[0];
+        void* wargs[] = {&w};
+        void* rargs[] = {&g, &cfg, &w};
+        void* bargs[] = {&w, &cfg.w};
+        rc = add_kernel(body, &begin, nullptr, (void*)k_beam_begin, 1, 32, 0, bargs);
+        if (!rc) rc = add_kernel(body, &ring, &begin, (void*)k_beam_ring, ls.grid_seed, 256, 0, wargs);
+        if (!rc) rc = add_kernel(body, &entries, &ring, (void*)k_beam_entries, ls.grid_seed, 256, 0, rargs);
+        if (!rc)
+            rc = add_kernel(body, &round, &entries, (void*)k_round<Eng>, ls.grid_round, 32 * ls.warps_per_block,
+                            ls.smem_bp, rargs);
+        if (!rc) rc = add_kernel(body, &end, &round, (void*)k_beam_end, 1, 32, 0, wargs);
     }
-    if (!rc) {
-        int use = 1;
-        void* pargs[] = {&w, &nri, &cpass, &use};
-        rc = add_kernel(body, &pend, &wround, (void*)k_pass_end, 1, 128, 0, pargs);
-    }
-    if (!rc) *last = wpass;
+    if (!rc) *last = beam;
     return rc;
 }
 
@@ -2079,7 +2147,6 @@ static int build_graph_t(const DevGraph& g0, const DecCfg& cfg0, const Work& w0,
     DecCfg cfg = cfg0;
     Work w = w0;
     const int threads = 32 * ls.warps_per_block;
-    int nri = 3 * (cfg.max_rounds + 2);
     cudaGraph_t graph = nullptr;
     if (CUDA_FAILED(cudaGraphCreate(&graph, 0))) return -2;
     int rc = 0;
@@ -2092,7 +2159,7 @@ static int build_graph_t(const DevGraph& g0, const DecCfg& cfg0, const Work& w0,
         rc = add_kernel(graph, &scr, nullptr, screen_func(ls), ls.grid_screen, 32 * kScreenWarps, ls.smem_screen,
                         cargs);
     if (!batched) {
-        // seed, then the beam passes
+        // seed, then the beam
         if (!rc)
             rc = add_kernel(graph, &seed, ls.screen ? &scr : nullptr, (void*)k_seed<Eng>, ls.grid_seed, threads,
                             ls.smem_bp, sargs);
@@ -2100,7 +2167,7 @@ static int build_graph_t(const DevGraph& g0, const DecCfg& cfg0, const Work& w0,
     } else {
         // the batched seed BP over the chunk, then WHILE (shots handed on
         // remain) { window start, the seed kernel on at most S of them, the
-        // beam passes, window end }
+        // beam, window end }
         cudaGraphNode_t bs, wgate, wwin;
         cudaGraphConditionalHandle cwin;
         if (!rc) rc = add_batch_nodes(graph, ls.screen ? scr : nullptr, &bs, g, cfg, w, ls, ls.screen);
@@ -2122,8 +2189,8 @@ static int build_graph_t(const DevGraph& g0, const DecCfg& cfg0, const Work& w0,
             cudaGraph_t body = cp.conditional.phGraph_out[0];
             cudaGraphNode_t wbeg, wend;
             int keep = -1;
-            void* bargs[] = {&w, &nri, &keep};
-            rc = add_kernel(body, &wbeg, nullptr, (void*)k_win_begin, 1, 128, 0, bargs);
+            void* bargs[] = {&w, &keep};
+            rc = add_kernel(body, &wbeg, nullptr, (void*)k_win_begin, 1, 32, 0, bargs);
             if (!rc)
                 rc = add_kernel(body, &seed, &wbeg, (void*)k_seed<Eng>, ls.grid_seed, threads, ls.smem_bp, sargs);
             cudaGraphNode_t tail = seed;
@@ -2166,10 +2233,9 @@ void destroy_graph(void* graph_exec)
 // ---- workspace layout
 static inline size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
-size_t work_head_bytes(const DecCfg& cfg)
+size_t work_head_bytes()
 {
-    return a256(sizeof(Counters) + sizeof(int) * 3 * (size_t)(cfg.max_rounds + 2)) + a256(sizeof(RunDesc)) +
-           a256(kStats * sizeof(unsigned long long));
+    return a256(sizeof(Counters)) + a256(sizeof(RunDesc)) + a256(kStats * sizeof(unsigned long long));
 }
 
 size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long A, char* base, Work* w,
@@ -2185,7 +2251,7 @@ size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long 
         off += a256(bytes > 0 ? bytes : 1);
         return p;
     };
-    char* ctr = take(sizeof(Counters) + sizeof(int) * 3 * (size_t)(cfg.max_rounds + 2));
+    char* ctr = take(sizeof(Counters));
     char* desc = take(sizeof(RunDesc));
     char* stats = take(kStats * sizeof(unsigned long long));
     Work v{};
@@ -2194,7 +2260,6 @@ size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long 
     v.A = A;
     v.SB = (int)SB;
     v.ctr = reinterpret_cast<Counters*>(ctr);
-    v.round_ctr = ctr ? reinterpret_cast<int*>(ctr + sizeof(Counters)) : nullptr;
     v.desc = reinterpret_cast<RunDesc*>(desc);
     v.stats = reinterpret_cast<unsigned long long*>(stats);
     v.seedE = (unsigned char*)take((size_t)S * snap_bytes(g));
@@ -2207,7 +2272,7 @@ size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long 
     v.slotMeta = (SlotMeta*)take(sizeof(SlotMeta) * 2 * (size_t)A * W2);
     v.shot_of = (int*)take(sizeof(int) * (size_t)A);
     v.set_size = (int*)take(sizeof(int) * (size_t)A);
-    v.done = (int*)take(sizeof(int) * (size_t)A);
+    v.ent = (BeamEntry*)take(sizeof(BeamEntry) * (size_t)A);
     v.set_idx = (uint8_t*)take((size_t)A * (size_t)cfg.w);
     v.iters_acc = (unsigned long long*)take(sizeof(unsigned long long) * (size_t)A);
     v.res_bits = (uint32_t*)take(sizeof(uint32_t) * (size_t)A * NR * (size_t)g.WN);
@@ -2216,7 +2281,10 @@ size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long 
     v.res_n = (int*)take(sizeof(int) * (size_t)A);
     v.first_ok = (unsigned long long*)take(sizeof(unsigned long long) * (size_t)A);
     v.near = (int*)take(sizeof(int) * (size_t)A);
-    v.items = (int2*)take(sizeof(int2) * 2 * (size_t)A * W2);
+    // a power of two of at least 2 * A * 2w slots (k_beam_begin)
+    size_t slots = 4;
+    while (slots < 2 * (size_t)A * W2) slots *= 2;
+    v.ring = (uint32_t*)take(sizeof(uint32_t) * slots);
     // the batched seed BP's slots and the shots it passes on
     v.bs_slots = bs_slots;
     if (bs_slots > 0) {
@@ -2256,13 +2324,6 @@ __device__ __forceinline__ uint32_t ld_acquire_sys(const uint32_t* p)
 __device__ __forceinline__ void st_release_sys(uint32_t* p, uint32_t v)
 {
     asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
 }
 
 // The loop answers a request (ServeBox::req != the last answered number) by

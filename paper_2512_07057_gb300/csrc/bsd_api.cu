@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <chrono>
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -94,6 +95,9 @@ inline int words_of(long long bits) { return (int)((bits + 31) / 32); }
 // this many slots
 constexpr long long kBatchMinEdges = 16384;
 constexpr int kBatchDefaultSlots = 2048;
+// the second-iteration screen is built while the columns next to flipped
+// detectors are expected to be at most this share of all
+constexpr double kScreen2MaxShare = 0.125;
 
 const char* kPresetNames[] = {"beam8_230iters", "beam32_340iters", "beam64_640iters", "beam64_32res_640iters"};
 // Table I: max_rounds, beam_width, initial_iters, iters_per_round, num_results
@@ -142,6 +146,7 @@ LaunchShape small_shape(const LaunchShape& ls, const DecCfg& cfg, int n)
     // no first-iteration screen and no batched seed BP: for a few shots their
     // extra launches cost more latency than they save
     s.screen = 0;
+    s.grid_screen2 = 0;
     s.batch = 0;
     s.grid_round = cap(((long long)n * 2 * cfg.w + per_block - 1) / per_block, ls.grid_round);
     return s;
@@ -458,6 +463,50 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
             std::memcpy(&colRD[((size_t)j * rdk + k) * 2 + 1], &r, 4);
         }
     }
+    // the second-iteration screen's tables: E0(1), the messages after one
+    // iteration with s = 0 (D0 of the column's other edges added to Lambda_j in
+    // ascending order, clamped and rounded to the storage format), and each
+    // row's four smallest.  Built where the columns next to flipped detectors
+    // are few: the screen's work grows with them (sum over rows of the chance of
+    // a flip times the degree, against N), the seed BP's does not.  Measured at
+    // 3% (synthetic 936 x 8800 DEM) and 2 to 6% (phenomenological DEM at
+    // p = 1e-3 to 3e-3) of the columns it pays; at 78% (depolarizing noise on
+    // [[144,12,12]], p = 0.05) 3% of the shots converge at t = 2.
+    std::vector<float> E1, row4;
+    if (all_pos && rdk > 0 && N < 65536 && params->num_results == 1) {
+        double next = 0.0;
+        for (int i = 0; i < M; ++i) {
+            double q = 1.0;
+            for (int e = H_row_ptr[i]; e < H_row_ptr[i + 1]; ++e) q *= 1.0 - 2.0 * priors[H_col_idx[e]];
+            next += 0.5 * (1.0 - q) * (H_row_ptr[i + 1] - H_row_ptr[i]);
+        }
+        if (next <= kScreen2MaxShare * N) {
+            E1.assign((size_t)E, 0.f);
+            std::vector<int> ord;
+            for (int j = 0; j < N; ++j) {
+                ord.assign(col_edge.begin() + col_ptr[j], col_edge.begin() + col_ptr[j + 1]);
+                std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return D0[a] < D0[b]; });
+                for (int e : ord) {
+                    float acc = lam[j];
+                    for (int e2 : ord)
+                        if (e2 != e) acc = acc + D0[e2];
+                    const float v = store_round(std::fmin(std::fmax(acc, -L), L));
+                    E1[e] = v == 0.f ? 0.f : v;
+                }
+            }
+            row4.assign((size_t)M * 8, 0.f);
+            for (int i = 0; i < M; ++i) {
+                ord.resize(H_row_ptr[i + 1] - H_row_ptr[i]);
+                for (size_t k = 0; k < ord.size(); ++k) ord[k] = H_row_ptr[i] + (int)k;
+                std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return E1[a] < E1[b]; });
+                for (size_t k = 0; k < 4; ++k) {
+                    const int c = k < ord.size() ? H_col_idx[ord[k]] : -1;
+                    row4[(size_t)i * 8 + 2 * k] = k < ord.size() ? E1[ord[k]] : L;
+                    std::memcpy(&row4[(size_t)i * 8 + 2 * k + 1], &c, 4);
+                }
+            }
+        }
+    }
     // the columns ordered by degree, each column's (edge, row) pairs contiguous
     // in the order of the column lists (the batched seed BP walks runs of
     // columns of one degree)
@@ -504,6 +553,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     gb += align256(sizeof(int) * colperm.size());
     gb += align256(sizeof(int2) * colseq.size());
     gb += align256(sizeof(float) * colRD.size());
+    gb += align256(sizeof(float) * E1.size()) + align256(sizeof(float) * row4.size());
     // the single-warp engine's rows of H as column sets (the stopping rule's parities)
     std::vector<uint32_t> shrow;
     if (has_sl) {
@@ -537,6 +587,8 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     unsigned char* d_lamEc = carve<unsigned char>(p, lamEc_st.size());
     int* d_colperm = colperm.empty() ? nullptr : carve<int>(p, colperm.size());
     int2* d_colseq = colseq.empty() ? nullptr : carve<int2>(p, colseq.size());
+    float* d_E1 = E1.empty() ? nullptr : carve<float>(p, E1.size());
+    float* d_row4 = row4.empty() ? nullptr : carve<float>(p, row4.size());
     float* d_colRD = colRD.empty() ? nullptr : carve<float>(p, colRD.size());
     uint32_t* d_scol = has_sl ? carve<uint32_t>(p, sl.col.size()) : nullptr;
     float* d_sD0 = has_sl ? carve<float>(p, sD0.size()) : nullptr;
@@ -561,6 +613,9 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
                !CUDA_FAILED(cudaMemcpy(d_colperm, colperm.data(), sizeof(int) * colperm.size(), cudaMemcpyHostToDevice))) &&
               (colseq.empty() ||
                !CUDA_FAILED(cudaMemcpy(d_colseq, colseq.data(), sizeof(int2) * colseq.size(), cudaMemcpyHostToDevice))) &&
+              (E1.empty() ||
+               (!CUDA_FAILED(cudaMemcpy(d_E1, E1.data(), sizeof(float) * E1.size(), cudaMemcpyHostToDevice)) &&
+                !CUDA_FAILED(cudaMemcpy(d_row4, row4.data(), sizeof(float) * row4.size(), cudaMemcpyHostToDevice)))) &&
               (colRD.empty() ||
                !CUDA_FAILED(cudaMemcpy(d_colRD, colRD.data(), sizeof(float) * colRD.size(), cudaMemcpyHostToDevice))) &&
               (!has_sl ||
@@ -583,6 +638,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     g.colperm = d_colperm; g.colseq = d_colseq;
     g.colRD = reinterpret_cast<const float4*>(d_colRD); g.colRDk = rdk;
     for (int d = 0; d < kMaxColDeg + 2; ++d) { g.dstart[d] = dstart[d]; g.dbase[d] = dbase[d]; }
+    g.E1 = d_E1; g.row4 = reinterpret_cast<const float4*>(d_row4);
     g.scol = d_scol; g.sD0 = d_sD0; g.slamE = d_slamE; g.shrow = d_shrow;
     if (has_gl) dec->generic_pos = gl.pos;
     if (has_sl) {

@@ -78,6 +78,11 @@ struct DevGraph {
     // the degree bounds 3, 6 and 16 (two pairs per float4)
     const float4* colRD;   // [Npad][colRDk / 2]
     int colRDk;
+    // second-iteration screen (null where it does not pay): per row the four
+    // smallest E0(1) -- E(1) for s = 0, every Lambda_j > 0 -- with their
+    // columns, ascending, padded with (L_MAX, -1); and E0(1) of every CSR edge
+    const float4* row4;    // [M][2], two (value, column) pairs each
+    const float* E1;       // [E]
     int dstart[kMaxColDeg + 2];
     int dbase[kMaxColDeg + 2];
     // the single-warp engine's shared-memory placement of a candidate's
@@ -163,7 +168,8 @@ struct Counters {
     int claim_seed;
     int n_active;          // seed-store entries written by k_seed
     int err;
-    int n_queue;           // shots the first-iteration screen passed on to the seed BP
+    int n_queue;           // shots the screens passed on to the seed BP
+    int n_queue1;          // shots the first screen passed on to the second
     // batched seed BP (bsd_batch.cu)
     int bs_claim;          // queue entries handed to slots so far
     int bs_run;            // the batch has active slots: another iteration runs
@@ -204,7 +210,8 @@ struct Work {
                            // decoded from the seed on in windows of S
     long long A;           // window entries: shots whose beam runs at once
     int SB;                // words per slot bit record: sp[WM] mask[WN] vals[WN] ehat[WN]
-    int* queue;            // [S1] chunk-local shots the screen passed on to the seed BP
+    int* queue;            // [S1] chunk-local shots the screens passed on to the seed BP
+    int* queue1;           // [S1] those the first screen passed on to the second (shares another array's memory)
     // batched seed BP over slots (bsd_batch.cu); bs_slots = 0: not used
     int bs_slots;          // Bs, a multiple of kBsChunk
     unsigned char* bsE;    // [Epad][Bs] messages in the storage format, shots contiguous
@@ -270,6 +277,8 @@ struct LaunchShape {
     int grid_screen;       // its blocks of 8 warps (one shot per warp)
     int dv_screen;         // its column degree bound: 0 -> 3, 1 -> 6, 2 -> 16
     size_t smem_screen;
+    int grid_screen2;      // blocks of the second-iteration screen, 0: it does not run
+    size_t smem_screen2;
     size_t smem_bp;        // dynamic shared memory of the seed / round kernels
     int dv;                // engine id
     int batch;             // the seed BP runs batched over slots (when the workspace has them)

@@ -12,6 +12,8 @@
 //   k_screen<DV>  (generic engines, every Lambda_j > 0, one result) a warp per
 //                 shot forms e^(1) from the columns next to flipped detectors;
 //                 finalises the shots that converge there, queues the rest
+//   k_screen2<DV> the same for e^(2) of the shots k_screen passes on, from the
+//                 columns that may flip (sparse syndromes)
 //   k_seed<DV>    the seed BP of every shot in a chunk, or of the queued ones
 //                 (Alg. 3, first BP run)
 //   k_round<DV>   the beam of every shot: expand + masked BP of its children
@@ -948,6 +950,7 @@ __global__ void k_begin_chunk(Work w, const uint32_t* synd, Outputs out, long lo
         w.ctr->claim_seed = 0;
         w.ctr->n_active = 0;
         w.ctr->n_queue = 0;
+        w.ctr->n_queue1 = 0;
         w.ctr->err = 0;
         w.ctr->bs_claim = 0;
         w.ctr->bs_run = 0;
@@ -1069,8 +1072,9 @@ __host__ __device__ inline size_t screen_warp_words(const DevGraph& g)
     return 2 * (size_t)g.WN + 2 * (size_t)g.WM + 2 * (size_t)kMaxFlip;
 }
 
+// (more: the shots that do not converge go to the second-iteration screen)
 template <int DV>
-__global__ void k_screen(DevGraph g, DecCfg cfg, Work w)
+__global__ void k_screen(DevGraph g, DecCfg cfg, Work w, int more)
 {
     extern __shared__ __align__(16) uint32_t ssm[];
     const int lane = threadIdx.x & 31;
@@ -1208,14 +1212,340 @@ __global__ void k_screen(DevGraph g, DecCfg cfg, Work w)
         if (conv) {
             finalize_shot<WarpGroup, true>(g, dp->out, gb, eh, ST_SEED, 1ull);
         } else if (lane == 0) {
-            const int k = atomicAdd(&w.ctr->n_queue, 1);
-            w.queue[k] = (int)b;
+            const int k = atomicAdd(more ? &w.ctr->n_queue1 : &w.ctr->n_queue, 1);
+            (more ? w.queue1 : w.queue)[k] = (int)b;
         }
         __syncwarp();
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) upd += __shfl_xor_sync(FULLMASK, upd, o);
     if (lane == 0 && upd != 0ull) atomicAdd(&w.stats[3], upd);
+}
+
+// ----------------------------------------------------------------------------
+// second-iteration screen (generic engines, sparse syndromes)
+// ----------------------------------------------------------------------------
+// E(1) differs from its value for s = 0 (the create-time E0(1) > 0) only on the
+// columns next to flipped detectors.  So the row records of E(1) -- the two
+// smallest magnitudes and the parity P_i of s_i and the negative messages --
+// follow from the row's few smallest E0(1) on other columns (DevGraph::row4)
+// and those columns' messages, and at t = 2 a column meets a negative check
+// message, without which Lambda_j(2) > 0, only in a row with P_i odd or through
+// a negative E(1) of its own.  One warp per shot forms Lambda_j(2) for these
+// columns, by the operations and in the order of the seed BP's second
+// iteration, and tests H e^(2) = s.  A shot that converges is finalised here
+// with two iterations; the others (and any whose lists overflow) go to the seed
+// BP.
+//
+// It pays where the flipped detectors' columns are few (configure_kernels): of
+// the synthetic 936 x 8800 DEM's shots 14% pass the first screen and 97% of
+// those end here, after about 300 columns each way instead of two passes over
+// 35110 edges.
+constexpr int kScreen2Cols = 1024;       // columns next to flipped detectors, and
+constexpr int kScreen2Cand = 512;        // columns that may flip at t = 2, of one shot
+
+__host__ __device__ inline size_t screen2_warp_words(const DevGraph& g)
+{
+    return (size_t)g.WN + 3 * (size_t)g.WM + 2 * (size_t)kMaxFlip + (kScreen2Cols + kScreen2Cand) / 2 +
+           2 * (size_t)g.M;
+}
+
+// the set rows of a bit set: each one's first edge (first) and its edges'
+// offset (off) in the list of all their edges; returns the rows, *tot = the
+// edges (nothing is listed when there are more than kMaxFlip)
+__device__ inline int list_rows(const DevGraph& g, const uint32_t* bits, int* first, int* off, int* tot)
+{
+    const int lane = threadIdx.x & 31;
+    int n = 0;
+    for (int q0 = 0; q0 < g.WM; q0 += 32) {
+        const int q = q0 + lane;
+        const uint32_t word = q < g.WM ? bits[q] : 0u;
+        const int c = __popc(word);
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULLMASK, incl, o);
+            if (lane >= o) incl += y;
+        }
+        int k = n + incl - c;
+        if (k + c <= kMaxFlip) {
+            for (uint32_t w2 = word; w2 != 0u; w2 &= w2 - 1u) first[k++] = 32 * q + __ffs(w2) - 1;
+        }
+        n += __shfl_sync(FULLMASK, incl, 31);
+    }
+    *tot = 0;
+    if (n > kMaxFlip) return n;
+    __syncwarp();
+    for (int k0 = 0; k0 < n; k0 += 32) {
+        const int k = k0 + lane;
+        int rb = 0, d = 0;
+        if (k < n) {
+            const int i = first[k];
+            rb = __ldg(g.row_ptr + i);
+            d = __ldg(g.row_ptr + i + 1) - rb;
+        }
+        int incl = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULLMASK, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (k < n) {
+            first[k] = rb;
+            off[k] = *tot + incl - d;
+        }
+        *tot += __shfl_sync(FULLMASK, incl, 31);
+    }
+    __syncwarp();
+    return n;
+}
+
+// the columns on the listed rows' edges that `seen` does not hold yet, appended
+// to list[cap]; returns the list's length, above cap when it overflows
+__device__ inline int list_columns(const DevGraph& g, const int* first, const int* off, int n, int tot,
+                                   uint32_t* seen, uint16_t* list, int len, int cap)
+{
+    const int lane = threadIdx.x & 31;
+    for (int t0 = 0; t0 < tot && len <= cap; t0 += 32) {
+        const int t = t0 + lane;
+        bool add = false;
+        int j = 0;
+        if (t < tot) {
+            int lo = 0, hi = n - 1;                        // last row with off <= t
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (off[mid] <= t) lo = mid; else hi = mid - 1;
+            }
+            j = __ldg(g.row_col + first[lo] + (t - off[lo]));
+            const uint32_t bit = 1u << (j & 31);
+            add = !(atomicOr(&seen[j >> 5], bit) & bit);
+        }
+        const uint32_t bal = __ballot_sync(FULLMASK, add);
+        const int at = len + __popc(bal & ((1u << lane) - 1u));
+        if (add && at < cap) list[at] = (uint16_t)j;
+        len += __popc(bal);
+    }
+    __syncwarp();
+    return len;
+}
+
+// E_{j->i}(1) of column j in the storage format's values: v[k] on row rr[k],
+// k < the column's degree (returned)
+template <int KD, int P>
+__device__ __forceinline__ int column_E1(const DevGraph& g, const uint32_t* sp, int j, float L, float (&v)[KD],
+                                         int (&rr)[KD])
+{
+    using S = Store<P>;
+    const float4* cr = g.colRD + (size_t)j * (KD / 2);
+    float d[KD];
+    int deg = 0;
+#pragma unroll
+    for (int h = 0; h < KD / 2; ++h) {
+        const float4 q = __ldg(cr + h);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int r = __float_as_int(u ? q.w : q.y);
+            const uint32_t si = (r >= 0) ? (sp[(r >= 0 ? r : 0) >> 5] >> (r & 31)) & 1u : 0u;
+            d[2 * h + u] = __uint_as_float(__float_as_uint(u ? q.z : q.x) ^ (si << 31));
+            rr[2 * h + u] = r;
+            deg += (r >= 0) ? 1 : 0;
+        }
+    }
+    // ascending order of value, the padding (+inf) last
+#pragma unroll
+    for (int a = 0; a < KD; ++a) {
+#pragma unroll
+        for (int k = 0; k + 1 < KD - a; ++k) {
+            if (d[k] > d[k + 1]) {
+                const float tv = d[k]; d[k] = d[k + 1]; d[k + 1] = tv;
+                const int tr = rr[k]; rr[k] = rr[k + 1]; rr[k + 1] = tr;
+            }
+        }
+    }
+    const float lj = __ldg(g.lam + j);
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {                            // Eq. 2: leave d_i out
+        float acc = lj;
+#pragma unroll
+        for (int k2 = 0; k2 < KD; ++k2)
+            if (k2 != k && k2 < deg) acc = __fadd_rn(acc, d[k2]);
+        typename S::T x;
+        S::st(&x, 0, fminf(fmaxf(acc, -L), L));
+        v[k] = S::ld(&x, 0);
+    }
+    return deg;
+}
+
+template <int DV, int P>
+__global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCfg cfg, Work w)
+{
+    extern __shared__ __align__(16) uint32_t ssm[];
+    constexpr int KD = DV == 3 ? 4 : DV;
+    const int lane = threadIdx.x & 31;
+    const size_t stride = screen2_warp_words(g);
+    uint32_t* rec = ssm + (size_t)(threadIdx.x >> 5) * stride;      // [M] (min1, min2)
+    uint32_t* bits = rec + 2 * (size_t)g.M;                          // [WN] columns listed, then e^(2)
+    uint32_t* sp = bits + g.WN;
+    uint32_t* pr = sp + g.WM;                                        // P_i
+    uint32_t* par = pr + g.WM;                                       // s xor H e^(2)
+    int* first = reinterpret_cast<int*>(par + g.WM);
+    int* off = first + kMaxFlip;
+    uint16_t* cols = reinterpret_cast<uint16_t*>(off + kMaxFlip);
+    uint16_t* cand = cols + kScreen2Cols;
+    count_launch(w);
+    const RunDesc* dp = w.desc;
+    const int nq = *((volatile int*)&w.ctr->n_queue1);
+    const int nw = gridDim.x * kScreenWarps;
+    const float L = cfg.L;
+    unsigned long long upd = 0;                                      // message updates formed (lane)
+    unsigned long long ended = 0;
+    for (int k0 = blockIdx.x * kScreenWarps + (threadIdx.x >> 5); k0 < nq; k0 += nw) {
+        const int b = w.queue1[k0];
+        const long long gb = dp->chunk_base + b;
+        const uint32_t* s = dp->synd + gb * g.WM;
+        for (int q = lane; q < g.WM; q += 32) sp[q] = pr[q] = par[q] = s[q];
+        for (int q = lane; q < g.WN; q += 32) bits[q] = 0u;
+        __syncwarp();
+        bool conv = false;
+        int tot;
+        const int nflip = list_rows(g, sp, first, off, &tot);
+        const int nc = nflip <= kMaxFlip ? list_columns(g, first, off, nflip, tot, bits, cols, 0, kScreen2Cols)
+                                         : kScreen2Cols + 1;
+        if (nc <= kScreen2Cols) {
+            // the records of E0(1) over the other columns: the first two of the
+            // row's four smallest; a row that has fewer (more than two of the
+            // four are next to flipped detectors) is read whole
+            for (int i = lane; i < g.M; i += 32) {
+                const float4 a0 = __ldg(g.row4 + 2 * i), a1 = __ldg(g.row4 + 2 * i + 1);
+                const float x[4] = {a0.x, a0.z, a1.x, a1.z};
+                const int c[4] = {__float_as_int(a0.y), __float_as_int(a0.w), __float_as_int(a1.y),
+                                  __float_as_int(a1.w)};
+                float m1 = L, m2 = L;
+                int n = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool other = c[u] < 0 || !((bits[c[u] >> 5] >> (c[u] & 31)) & 1u);
+                    if (other) {
+                        if (n == 0) m1 = x[u];
+                        else if (n == 1) m2 = x[u];
+                        ++n;
+                    }
+                }
+                if (n < 2) {
+                    m1 = m2 = L;
+                    for (int e = __ldg(g.row_ptr + i); e < __ldg(g.row_ptr + i + 1); ++e) {
+                        const int j = __ldg(g.row_col + e);
+                        if ((bits[j >> 5] >> (j & 31)) & 1u) continue;
+                        const float a = __ldg(g.E1 + e);
+                        m2 = fminf(m2, fmaxf(m1, a));
+                        m1 = fminf(m1, a);
+                    }
+                }
+                rec[2 * i] = __float_as_uint(m1);
+                rec[2 * i + 1] = __float_as_uint(m2);
+            }
+            __syncwarp();
+            for (int q = lane; q < g.WN; q += 32) bits[q] = 0u;
+            __syncwarp();
+            // the messages of the columns next to flipped detectors; the larger
+            // of a message and the minimum it meets goes on to the second one,
+            // which in the end is the least of all but the minimum
+            int ncand = 0;
+            for (int t0 = 0; t0 < nc; t0 += 32) {
+                bool neg = false;
+                int j = 0;
+                if (t0 + lane < nc) {
+                    j = cols[t0 + lane];
+                    float v[KD];
+                    int rr[KD];
+                    const int deg = column_E1<KD, P>(g, sp, j, L, v, rr);
+#pragma unroll
+                    for (int k = 0; k < KD; ++k) {
+                        if (k < deg) {
+                            const uint32_t a = __float_as_uint(fabsf(v[k]));
+                            const uint32_t old = atomicMin(&rec[2 * rr[k]], a);
+                            atomicMin(&rec[2 * rr[k] + 1], old > a ? old : a);
+                            if (v[k] < 0.f) {
+                                neg = true;
+                                atomicXor(&pr[rr[k] >> 5], 1u << (rr[k] & 31));
+                            }
+                        }
+                    }
+                    upd += (unsigned long long)deg;
+                }
+                const uint32_t bal = __ballot_sync(FULLMASK, neg);
+                const int at = ncand + __popc(bal & ((1u << lane) - 1u));
+                if (neg) {
+                    atomicOr(&bits[j >> 5], 1u << (j & 31));
+                    if (at < kScreen2Cand) cand[at] = (uint16_t)j;
+                }
+                ncand += __popc(bal);
+            }
+            __syncwarp();
+            if (ncand <= kScreen2Cand) {
+                const int nodd = list_rows(g, pr, first, off, &tot);
+                ncand = nodd <= kMaxFlip ? list_columns(g, first, off, nodd, tot, bits, cand, ncand, kScreen2Cand)
+                                         : kScreen2Cand + 1;
+            }
+            if (ncand <= kScreen2Cand) {
+                for (int q = lane; q < g.WN; q += 32) bits[q] = 0u;
+                __syncwarp();
+                for (int t = lane; t < ncand; t += 32) {
+                    const int j = cand[t];
+                    float v[KD];
+                    int rr[KD];
+                    const int deg = column_E1<KD, P>(g, sp, j, L, v, rr);
+#pragma unroll
+                    for (int k = 0; k < KD; ++k) {            // Eq. 1
+                        if (k < deg) {
+                            const float m1 = __uint_as_float(rec[2 * rr[k]]), m2 = __uint_as_float(rec[2 * rr[k] + 1]);
+                            const float d = __fmul_rn(cfg.alpha, fabsf(v[k]) == m1 ? m2 : m1);
+                            const uint32_t sg = ((pr[rr[k] >> 5] >> (rr[k] & 31)) << 31) ^
+                                                (__float_as_uint(v[k]) & 0x80000000u);
+                            v[k] = __uint_as_float(__float_as_uint(d) ^ sg);
+                        } else {
+                            v[k] = INFINITY;
+                        }
+                    }
+#pragma unroll
+                    for (int a = 0; a < KD; ++a) {
+#pragma unroll
+                        for (int k = 0; k + 1 < KD - a; ++k) {
+                            if (v[k] > v[k + 1]) { const float tv = v[k]; v[k] = v[k + 1]; v[k + 1] = tv; }
+                        }
+                    }
+                    float post = __ldg(g.lam + j);            // Eq. 3 in ascending order
+#pragma unroll
+                    for (int k = 0; k < KD; ++k)
+                        if (k < deg) post = __fadd_rn(post, v[k]);
+                    upd += (unsigned long long)deg;
+                    if (post <= 0.f) {                        // Eq. 4
+                        atomicOr(&bits[j >> 5], 1u << (j & 31));
+#pragma unroll
+                        for (int k = 0; k < KD; ++k)
+                            if (k < deg) atomicXor(&par[rr[k] >> 5], 1u << (rr[k] & 31));
+                    }
+                }
+                __syncwarp();
+                uint32_t nz = 0;
+                for (int q = lane; q < g.WM; q += 32) nz |= par[q];
+                conv = !__any_sync(FULLMASK, nz != 0u);
+            }
+        }
+        if (conv) {
+            finalize_shot<WarpGroup, true>(g, dp->out, gb, bits, ST_SEED, 2ull);
+            ended += 2ull;
+        } else if (lane == 0) {
+            w.queue[atomicAdd(&w.ctr->n_queue, 1)] = b;
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) upd += __shfl_xor_sync(FULLMASK, upd, o);
+    if (lane == 0 && upd != 0ull) {
+        atomicAdd(&w.stats[3], upd);
+        if (ended != 0ull) atomicAdd(&w.stats[0], ended);
+    }
 }
 
 // ----------------------------------------------------------------------------
@@ -1890,6 +2220,15 @@ static int occupancy(int threads, size_t smem_bp, int* bps)
     return 0;
 }
 
+static void* screen2_func(int dv, int prec)
+{
+    if (dv == 0)
+        return prec == 0 ? (void*)k_screen2<3, 0> : prec == 1 ? (void*)k_screen2<3, 1> : (void*)k_screen2<3, 2>;
+    if (dv == 1)
+        return prec == 0 ? (void*)k_screen2<6, 0> : prec == 1 ? (void*)k_screen2<6, 1> : (void*)k_screen2<6, 2>;
+    return prec == 0 ? (void*)k_screen2<16, 0> : prec == 1 ? (void*)k_screen2<16, 1> : (void*)k_screen2<16, 2>;
+}
+
 // can the small engine run this code? (column degree 3, row degree 6, with
 // the placement of its messages built)
 static bool small_fits(const DevGraph& g, int cpl, int rpl)
@@ -1974,6 +2313,7 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     // Lambda_j > 0, one result
     ls->screen = 0;
     ls->grid_screen = 0;
+    ls->grid_screen2 = 0;
     ls->smem_screen = sizeof(uint32_t) * screen_warp_words(g) * kScreenWarps;
     if (eng < 9 || eng >= kBlockEngine) {                   // not a small engine
         if (!weighted && g.all_lam_pos && cfg.num_results == 1 && ls->smem_screen <= (size_t)max_optin) {
@@ -1993,6 +2333,18 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
                 ls->grid_screen = sms * bps_scr;
                 ls->dv_screen = gkind;
             }
+            // the second-iteration screen where its tables were built (sparse
+            // syndromes) and the seed BP has a second iteration
+            ls->smem_screen2 = sizeof(uint32_t) * (screen2_warp_words(g)) * kScreenWarps;
+            if (ls->screen && g.row4 != nullptr && cfg.initial_iters >= 2 &&
+                ls->smem_screen2 <= (size_t)max_optin) {
+                kf = screen2_func(gkind, g.prec);
+                if (CUDA_FAILED(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin)) ||
+                    CUDA_FAILED(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_scr, kf, 32 * kScreenWarps,
+                                                                              ls->smem_screen2)))
+                    return -2;
+                if (bps_scr >= 1) ls->grid_screen2 = sms * bps_scr;
+            }
         }
     }
     ls->grid_seed = sms * bps_bp;
@@ -2010,14 +2362,6 @@ static void* screen_func(const LaunchShape& ls)
     return ls.dv_screen == 0 ? (void*)k_screen<3> : ls.dv_screen == 1 ? (void*)k_screen<6> : (void*)k_screen<16>;
 }
 
-static void launch_screen(const DevGraph& g, const DecCfg& cfg, const Work& w, const LaunchShape& ls, cudaStream_t s)
-{
-    const dim3 grid((unsigned)ls.grid_screen), block(32 * kScreenWarps);
-    if (ls.dv_screen == 0) k_screen<3><<<grid, block, ls.smem_screen, s>>>(g, cfg, w);
-    else if (ls.dv_screen == 1) k_screen<6><<<grid, block, ls.smem_screen, s>>>(g, cfg, w);
-    else k_screen<16><<<grid, block, ls.smem_screen, s>>>(g, cfg, w);
-}
-
 template <class Eng>
 static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, const LaunchShape& ls,
                           const uint32_t* synd, long long base, long long n, const Outputs& out, cudaStream_t s,
@@ -2029,7 +2373,16 @@ static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, c
     if (gx != nullptr) return !CUDA_FAILED(cudaGraphLaunch(gx, s)) ? 0 : -2;
     if (ls.screen) {
         if (hk) hk->before(hk->ctx, 11);
-        launch_screen(g, cfg, w, ls, s);
+        DevGraph gg = g;
+        DecCfg cc = cfg;
+        Work ww = w;
+        int more = ls.grid_screen2 > 0;
+        void* cargs[] = {&gg, &cc, &ww, &more};
+        if (CUDA_FAILED(cudaLaunchKernel(screen_func(ls), dim3((unsigned)ls.grid_screen), dim3(32 * kScreenWarps),
+                                         cargs, ls.smem_screen, s)) ||
+            (more && CUDA_FAILED(cudaLaunchKernel(screen2_func(ls.dv_screen, g.prec), dim3((unsigned)ls.grid_screen2),
+                                                  dim3(32 * kScreenWarps), cargs, ls.smem_screen2, s))))
+            return -2;
         if (hk) hk->after(hk->ctx, 11);
     }
     // the seed kernel on its shots, then the beam if any needs it (without a
@@ -2154,10 +2507,16 @@ static int build_graph_t(const DevGraph& g0, const DecCfg& cfg0, const Work& w0,
     const bool batched = ls.batch && w.bs_slots > 0;
     int screened = batched ? 2 : ls.screen;
     void* sargs[] = {&g, &cfg, &w, &screened};
-    void* cargs[] = {&g, &cfg, &w};
+    int more = ls.grid_screen2 > 0;
+    void* cargs[] = {&g, &cfg, &w, &more};
     if (ls.screen)
         rc = add_kernel(graph, &scr, nullptr, screen_func(ls), ls.grid_screen, 32 * kScreenWarps, ls.smem_screen,
                         cargs);
+    if (ls.screen && more && !rc) {
+        cudaGraphNode_t scr1 = scr;
+        rc = add_kernel(graph, &scr, &scr1, screen2_func(ls.dv_screen, g.prec), ls.grid_screen2, 32 * kScreenWarps,
+                        ls.smem_screen2, cargs);
+    }
     if (!batched) {
         // seed, then the beam
         if (!rc)
@@ -2297,6 +2656,9 @@ size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long 
         v.bs_list = (int*)take(sizeof(int) * Bs * (size_t)kBsList);
         v.fail = (int*)take(sizeof(int) * (size_t)S1);
     }
+    // the first screen's queue for the second lies where the chunk's later
+    // steps write (the hand-on list of the batch, or the seed store's shots)
+    v.queue1 = bs_slots > 0 ? v.fail : v.seed_shot;
     if (w) *w = v;
     return off;
 }

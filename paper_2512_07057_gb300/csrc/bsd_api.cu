@@ -413,26 +413,52 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     // the generic engines' column table: (edge, row) of the k-th edge of column
     // j at [k][j], (-1, -1) past the column's degree, for degree bounds 3 and 6
     const int colK = max_col <= 3 ? 3 : max_col <= 6 ? 6 : 0;
-    std::vector<int2> colER((size_t)colK * Npad, make_int2(-1, -1));
-    // the generic engines keep a candidate's messages at the words of their
-    // own placement (bsd_layout.cu: each row's edges permuted inside the row's
-    // window, each column's edges in the k slots of a colouring), so that the
-    // 32 lanes of an error-pass access meet distinct banks where possible
-    GenericLayout gl;
-    const bool has_gl = colK > 0 && generic_layout(M, N, H_row_ptr, H_col_idx, colK, &gl);
-    if (has_gl) {
-        std::vector<int> erow(E);
-        for (int i = 0; i < M; ++i)
-            for (int e = H_row_ptr[i]; e < H_row_ptr[i + 1]; ++e) erow[e] = i;
-        for (int k = 0; k < colK; ++k)
-            for (int j = 0; j < N; ++j) {
-                const int e = gl.kedge[(size_t)k * N + j];
-                if (e >= 0) colER[(size_t)k * Npad + j] = make_int2(gl.pos[e], erow[e]);
+    // the jagged engine's tables: rows by falling degree, the planes of their
+    // k-th edges, the words of every column's edges
+    std::vector<int2> rowQ;
+    std::vector<int> jplanes, colW, jpos;
+    std::vector<uint8_t> colG;
+    std::vector<float> jD0;
+    if (colK > 0) {
+        std::vector<int> ord(M), start((size_t)E);
+        for (int i = 0; i < M; ++i) ord[i] = i;
+        auto rdeg = [&](int i) { return H_row_ptr[i + 1] - H_row_ptr[i]; };
+        std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return rdeg(x) > rdeg(y); });
+        jplanes.assign(max_row > 0 ? max_row : 1, 0);
+        for (int k = 0, at = 0; k < max_row; ++k) {
+            jplanes[k] = at;
+            for (int q = 0; q < M && rdeg(ord[q]) > k; ++q) start[(size_t)H_row_ptr[ord[q]] + k] = at++;
+        }
+        for (int q = 0; q < M; ++q) rowQ.push_back(make_int2(ord[q], rdeg(ord[q])));
+        GenericLayout gl;
+        const bool has_gl = generic_layout(M, N, H_row_ptr, H_col_idx, colK, &gl, start.data());
+        jpos = has_gl ? gl.pos : start;
+        // a group of 32 columns of one degree keeps its edges in the first slots
+        colW.assign((size_t)colK * Npad, -1);
+        colG.assign((size_t)WN, 0);
+        for (int q = 0; q < WN; ++q) {
+            int lo = colK, hi = 0;
+            for (int j = 32 * q; j < std::min(N, 32 * q + 32); ++j) {
+                lo = std::min(lo, col_ptr[j + 1] - col_ptr[j]);
+                hi = std::max(hi, col_ptr[j + 1] - col_ptr[j]);
             }
-    } else {
-        for (int j = 0; j < N && colK > 0; ++j)
-            for (int k = 0; k < col_ptr[j + 1] - col_ptr[j]; ++k)
-                colER[(size_t)k * Npad + j] = make_int2(col_edge[col_ptr[j] + k], col_row[col_ptr[j] + k]);
+            colG[q] = (uint8_t)(lo == hi ? hi : hi + 8);
+            for (int j = 32 * q; j < std::min(N, 32 * q + 32); ++j) {
+                std::vector<int> slot(colK, -1), rest;
+                for (int k = 0; k < colK; ++k) {
+                    const int e = has_gl ? gl.kedge[(size_t)k * N + j]
+                                         : (k < col_ptr[j + 1] - col_ptr[j] ? col_edge[col_ptr[j] + k] : -1);
+                    if (e < 0) continue;
+                    if (k < hi) slot[k] = e; else rest.push_back(e);
+                }
+                for (int k = 0; k < hi && !rest.empty(); ++k)
+                    if (slot[k] < 0) { slot[k] = rest.back(); rest.pop_back(); }
+                for (int k = 0; k < hi; ++k)
+                    if (slot[k] >= 0) colW[(size_t)k * Npad + j] = jpos[slot[k]];
+            }
+        }
+        jD0.assign((size_t)(E > 0 ? E : 1), 0.f);
+        for (long long e = 0; e < E; ++e) jD0[jpos[e]] = D0[e];
     }
     // E(0) of column j in the storage format (every edge of the column holds it)
     std::vector<unsigned char> lamEc_st((size_t)Npad * msg_bytes, 0);
@@ -548,7 +574,8 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     gb += align256(sizeof(long long) * N);
     gb += align256(sizeof(float4) * M);
     gb += align256(sizeof(float) * Epad);
-    gb += align256(sizeof(int2) * colER.size());
+    gb += align256(sizeof(int) * colW.size()) + align256(colG.size()) + align256(sizeof(int2) * rowQ.size()) +
+          align256(sizeof(int) * jplanes.size()) + align256(sizeof(float) * jD0.size());
     gb += align256(lamEc_st.size());
     gb += align256(sizeof(int) * colperm.size());
     gb += align256(sizeof(int2) * colseq.size());
@@ -583,7 +610,11 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     long long* d_lamq = carve<long long>(p, N);
     float4* d_rs0 = carve<float4>(p, M);
     float* d_D0 = carve<float>(p, Epad);
-    int2* d_colER = colER.empty() ? nullptr : carve<int2>(p, colER.size());
+    int* d_colW = colW.empty() ? nullptr : carve<int>(p, colW.size());
+    uint8_t* d_colG = colG.empty() ? nullptr : carve<uint8_t>(p, colG.size());
+    int2* d_rowQ = rowQ.empty() ? nullptr : carve<int2>(p, rowQ.size());
+    int* d_jplanes = jplanes.empty() ? nullptr : carve<int>(p, jplanes.size());
+    float* d_jD0 = jD0.empty() ? nullptr : carve<float>(p, jD0.size());
     unsigned char* d_lamEc = carve<unsigned char>(p, lamEc_st.size());
     int* d_colperm = colperm.empty() ? nullptr : carve<int>(p, colperm.size());
     int2* d_colseq = colseq.empty() ? nullptr : carve<int2>(p, colseq.size());
@@ -606,8 +637,12 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
               !CUDA_FAILED(cudaMemcpy(d_lamq, lamq.data(), sizeof(long long) * N, cudaMemcpyHostToDevice)) &&
               !CUDA_FAILED(cudaMemcpy(d_rs0, rs0.data(), sizeof(float4) * M, cudaMemcpyHostToDevice)) &&
               !CUDA_FAILED(cudaMemcpy(d_D0, D0.data(), sizeof(float) * Epad, cudaMemcpyHostToDevice)) &&
-              (colER.empty() ||
-               !CUDA_FAILED(cudaMemcpy(d_colER, colER.data(), sizeof(int2) * colER.size(), cudaMemcpyHostToDevice))) &&
+              (colW.empty() ||
+               (!CUDA_FAILED(cudaMemcpy(d_colW, colW.data(), sizeof(int) * colW.size(), cudaMemcpyHostToDevice)) &&
+                !CUDA_FAILED(cudaMemcpy(d_colG, colG.data(), colG.size(), cudaMemcpyHostToDevice)) &&
+                !CUDA_FAILED(cudaMemcpy(d_rowQ, rowQ.data(), sizeof(int2) * rowQ.size(), cudaMemcpyHostToDevice)) &&
+                !CUDA_FAILED(cudaMemcpy(d_jplanes, jplanes.data(), sizeof(int) * jplanes.size(), cudaMemcpyHostToDevice)) &&
+                !CUDA_FAILED(cudaMemcpy(d_jD0, jD0.data(), sizeof(float) * jD0.size(), cudaMemcpyHostToDevice)))) &&
               !CUDA_FAILED(cudaMemcpy(d_lamEc, lamEc_st.data(), lamEc_st.size(), cudaMemcpyHostToDevice)) &&
               (colperm.empty() ||
                !CUDA_FAILED(cudaMemcpy(d_colperm, colperm.data(), sizeof(int) * colperm.size(), cudaMemcpyHostToDevice))) &&
@@ -634,13 +669,15 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     g.all_lam_pos = all_pos;
     g.row_ptr = d_row_ptr; g.row_col = d_row_col; g.col_ptr = d_col_ptr; g.col_edge = d_col_edge; g.col_row = d_col_row;
     g.lam = d_lam; g.lamE = d_lamE; g.hcol = d_hcol; g.acol = d_acol; g.lamq = d_lamq; g.rs0 = d_rs0; g.D0 = d_D0;
-    g.colER = d_colER; g.colK = colK; g.lamEc = d_lamEc;
+    g.colW = d_colW; g.colK = colK; g.colG = d_colG; g.rowQ = d_rowQ; g.jplanes = d_jplanes; g.jD0 = d_jD0;
+    for (int k = 0; k < kJaggedPlanes; ++k) g.jplane[k] = k < (int)jplanes.size() ? jplanes[k] : 0;
+    g.lamEc = d_lamEc;
     g.colperm = d_colperm; g.colseq = d_colseq;
     g.colRD = reinterpret_cast<const float4*>(d_colRD); g.colRDk = rdk;
     for (int d = 0; d < kMaxColDeg + 2; ++d) { g.dstart[d] = dstart[d]; g.dbase[d] = dbase[d]; }
     g.E1 = d_E1; g.row4 = reinterpret_cast<const float4*>(d_row4);
     g.scol = d_scol; g.sD0 = d_sD0; g.slamE = d_slamE; g.shrow = d_shrow;
-    if (has_gl) dec->generic_pos = gl.pos;
+    dec->generic_pos = jpos;
     if (has_sl) {
         dec->small_excess = sl.excess;
         dec->small_extent = sl.extent;

@@ -13,8 +13,8 @@
 //   lamq[N]               Lambda_j on the 2^-16 fixed-point grid (weights)
 //   rs0[M]                the detector records of E(0) (a seed run's first check pass, up to the syndrome)
 //   D0[Epad]              the check messages of E(0) with the scale alpha, before the syndrome sign
-//   colER[colK][Npad]     (word, row) of the edge in slot k of column j at the
-//                         generic engines' placement, (-1, -1) for an empty slot
+//   colW[colK][Npad]      word of the edge in slot k of column j at the jagged
+//                         engine's placement, -1 for an empty slot
 //   lamEc[Npad]           clamp(Lambda_j) in the storage format (E(0) of every edge of column j)
 //
 // Workspace (one decoder):
@@ -52,6 +52,7 @@ struct DevGraph {
     int max_col_deg, max_row_deg;
     int all_lam_pos;       // every Lambda_j > 0 (all p_j < 1/2)
     int det_bytes;         // per-warp detector-side shared memory (set with the engine)
+    int e_bytes;           // bytes of a message in shared memory (set with the engine)
     const int* row_ptr;
     const int* row_col;    // [E] column of CSR edge e
     const int* col_ptr;
@@ -64,8 +65,17 @@ struct DevGraph {
     const long long* lamq;
     const float4* rs0;     // [M] detector records of E(0): (min1, min2, argmin edge, parity of negatives)
     const float* D0;       // [Epad] check messages of E(0) with scale alpha, before the syndrome sign
-    const int2* colER;     // [colK][Npad] (word, row) of the edge in slot k of column j, (-1, -1): empty
-    int colK;              // 3 or 6 (the generic engines' degree bound), 0 when colER is absent
+    // the jagged engine's placement of a candidate's messages (column degrees
+    // up to 6; bsd_layout.cu): the rows in order of falling degree, the k-th
+    // edges of all rows that have one adjacent: the k-th edge of the row of rank
+    // q at word jplane[k] + q (jplane[] holds the first kJaggedPlanes, jplanes all)
+    const int* colW;       // [colK][Npad] word of the edge in slot k of column j, -1: empty
+    int colK;              // 3 or 6 (the engine's degree bound), 0 when colW is absent
+    const uint8_t* colG;   // [ceil(N / 32)] degree of the group's columns, + 8 when they differ
+    const int2* rowQ;      // [M] (row, degree) of rank q
+    const int* jplanes;    // [max_row_deg]
+    int jplane[16];
+    const float* jD0;      // [E] D0 at those words
     const void* lamEc;     // [Npad] E(0) of column j (clamp(Lambda_j)) in the storage format
     // the columns ordered by degree (batched seed BP): colperm[q] is the
     // column at position q, the columns of degree d hold positions
@@ -120,9 +130,9 @@ struct SmallLayout {
     int excess;
 };
 bool small_layout(int M, int N, const int* row_ptr, const int* col_idx, SmallLayout* out);
-// the generic engines' placement of a candidate's messages for column degree
-// bounds up to 6 (bsd_layout.cu): pos[e] = the word of CSR edge e inside its
-// row's storage window [row_ptr[i], row_ptr[i + 1]); kedge[k * N + j] = the
+// a placement of a candidate's messages for column degree bounds up to 6
+// (bsd_layout.cu): pos[e] = the word of CSR edge e among its row's words (the
+// storage window [row_ptr[i], row_ptr[i + 1]), or the jagged engine's); kedge[k * N + j] = the
 // CSR edge in slot k of column j (-1: a hole); excess = bank loads above each
 // column group's largest degree left by the search; false for codes beyond
 // kGenericLayoutMaxEdges edges or with a column above colK
@@ -132,7 +142,10 @@ struct GenericLayout {
     int excess;
 };
 constexpr int kGenericLayoutMaxEdges = 1 << 20;
-bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, GenericLayout* out);
+// (start: the words to permute within each row, null for the storage windows)
+bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, GenericLayout* out,
+                    const int* start = nullptr);
+constexpr int kJaggedPlanes = 16;        // planes whose offsets travel with the kernel parameters
 // the placement's plane stride for codes of M rows (the engine holds
 // ceil(M / 32) rows per lane); every plane spans 2 M <= 64 ceil(M / 32) words
 __host__ __device__ constexpr int small_plane_stride_rpl(int rpl) { return 64 * rpl + 12; }

@@ -158,7 +158,7 @@ __host__ __device__ inline size_t det_region_bytes(const DevGraph& g) { return (
 constexpr size_t kSelectBytes = 2 * kMaxBeam * (sizeof(double) + 2 * sizeof(int));
 __host__ __device__ inline size_t warp_smem_bytes(const DevGraph& g)
 {
-    const size_t n = align16((size_t)g.msg_bytes * (size_t)g.Epad) + det_region_bytes(g) +
+    const size_t n = align16((size_t)g.e_bytes * (size_t)g.Epad) + det_region_bytes(g) +
                      align16(sizeof(float) * (size_t)g.Npad) + align16(sizeof(uint32_t) * (size_t)(2 * g.WM + 3 * g.WN));
     return n > kSelectBytes ? n : kSelectBytes;   // the selection's scratch lies over the candidate's state
 }
@@ -179,7 +179,7 @@ __device__ inline WarpState carve(char* base, const DevGraph& g)
 {
     WarpState s;
     char* p = base;
-    s.E = p;                                 p += align16((size_t)g.msg_bytes * (size_t)g.Epad);
+    s.E = p;                                 p += align16((size_t)g.e_bytes * (size_t)g.Epad);
     s.rs = reinterpret_cast<float2*>(p);
     s.D = reinterpret_cast<float*>(p);       p += det_region_bytes(g);
     s.sumllr = reinterpret_cast<float*>(p);  p += align16(sizeof(float) * (size_t)g.Npad);
@@ -273,29 +273,14 @@ __device__ int bp_iterate(const G& grp, const DevGraph& g, const DecCfg& cfg, co
         // D_{i->j} of column j's edges in ascending order (padding +inf last),
         // with their CSR edge ids; returns the column's degree
         auto gather = [&](int j, float (&v)[DV], int (&ed)[DV]) -> int {
-            // the column's edges: from the padded (edge, row) table for degree
-            // bounds up to 6 (one coalesced load per slot), else from the
-            // column lists
-            int kb = 0, deg = 0;
-            if constexpr (DV > 6) {
-                kb = __ldg(g.col_ptr + j);
-                deg = __ldg(g.col_ptr + j + 1) - kb;
-            }
+            const int kb = __ldg(g.col_ptr + j), deg = __ldg(g.col_ptr + j + 1) - kb;
             // E(0) is the same on every edge of a column: one load
             const float x0 = prior ? S::ld(reinterpret_cast<const T*>(g.lamEc), j) : 0.f;
 #pragma unroll
             for (int k = 0; k < DV; ++k) {
-                int e = -1, r = 0;
-                if constexpr (DV <= 6) {
-                    const int2 er = __ldg(g.colER + (size_t)k * g.Npad + j);
-                    e = er.x;
-                    r = er.y;
-                    deg += (e >= 0) ? 1 : 0;
-                } else if (k < deg) {
-                    e = __ldg(g.col_edge + kb + k);
-                    r = __ldg(g.col_row + kb + k);
-                }
-                if (e >= 0) {
+                if (k < deg) {
+                    const int e = __ldg(g.col_edge + kb + k);
+                    const int r = __ldg(g.col_row + kb + k);
                     const float2 r2 = st.rs[r];
                     const float x = prior ? x0 : S::ld(E, e);
                     // the minimum over the row's other edges: min2 on an edge
@@ -325,18 +310,9 @@ __device__ int bp_iterate(const G& grp, const DevGraph& g, const DecCfg& cfg, co
             return deg;
         };
         auto flip_rows = [&](int j, int deg) {                 // s' xor H e^: the rows of column j
-            if constexpr (DV <= 6) {
-                // the column's slots of the padded table (a slot may be a hole)
-#pragma unroll
-                for (int k = 0; k < DV; ++k) {
-                    const int r = __ldg(g.colER + (size_t)k * g.Npad + j).y;
-                    if (r >= 0) atomicXor(&st.par[r >> 5], 1u << (r & 31));
-                }
-            } else {
-                for (int k = 0; k < deg; ++k) {
-                    const int r = __ldg(g.col_row + __ldg(g.col_ptr + j) + k);
-                    atomicXor(&st.par[r >> 5], 1u << (r & 31));
-                }
+            for (int k = 0; k < deg; ++k) {
+                const int r = __ldg(g.col_row + __ldg(g.col_ptr + j) + k);
+                atomicXor(&st.par[r >> 5], 1u << (r & 31));
             }
         };
 
@@ -471,38 +447,35 @@ __device__ inline void argmin_and_score(const G& grp, const DevGraph& g, const W
 // ----------------------------------------------------------------------------
 // BP engines: how one warp runs the iterations of one candidate
 // ----------------------------------------------------------------------------
-// GenericEngine: any code whose column degree is at most DV; graph tables
-// are read from global memory (L1-resident) and sum_LLR lives in shared memory.
+// GenericEngine: any code whose column degree is at most DV (used for degrees
+// above 6); graph tables are read from global memory (L1-resident) and sum_LLR
+// lives in shared memory.
 template <int DV, int P, bool W = false, class G = WarpGroup>
 struct GenericEngine {
     using Grp = G;
-    // blocks of up to 16 warps: for column degrees up to 6 the kernels fit in
-    // 64 registers, so two such blocks stay resident on an SM; one warp per
-    // candidate: 80 registers, three 8-warp blocks
-    static constexpr int kMinBlocks = (DV <= 6) ? (G::kBlock ? 2 : 3) : 1;
+    static constexpr int kMinBlocks = 1;
     static constexpr int kMaxThreads = G::kBlock ? 512 : 256;
     static constexpr int kPrec = P;
     static constexpr bool kPriorStart = true;   // runs from E(0) need no copy of E(0)
     static constexpr bool kPriorSetsSums = true;  // ... nor cleared sums: their first iteration sets them
     G grp;
     __device__ void load_graph(const DevGraph&, const WarpState&) {}
-    // E(0) in this engine's message layout (the CSR edge order)
-    static __device__ const void* prior_E(const DevGraph& g) { return g.lamE; }
-    // the sentinel +L_MAX on every message of the newly fixed node j (at the
-    // words of the padded column table for degree bounds up to 6, which may
-    // have holes; at the CSR edges for the column lists)
+    __device__ void start_prior(const DevGraph&, const WarpState&) const {}
+    // snapshots: the messages as they are kept
+    __device__ void load_E(const DevGraph& g, const WarpState& st, const void* src) const
+    {
+        group_copy16<true>(grp, st.E, src, snap_vec16(g));
+    }
+    __device__ void save_E(const DevGraph& g, const WarpState& st, void* dst) const
+    {
+        group_copy16(grp, dst, st.E, snap_vec16(g));
+    }
+    // the sentinel +L_MAX on every message of the newly fixed node j
     __device__ void fix_node(const DevGraph& g, const WarpState& st, int j, float L) const
     {
         typename Store<P>::T* const E = reinterpret_cast<typename Store<P>::T*>(st.E);
-        if constexpr (DV <= 6) {
-            for (int k = grp.rank(); k < DV; k += grp.size()) {
-                const int e = __ldg(g.colER + (size_t)k * g.Npad + j).x;
-                if (e >= 0) Store<P>::st(E, e, L);
-            }
-        } else {
-            for (int q = __ldg(g.col_ptr + j) + grp.rank(); q < __ldg(g.col_ptr + j + 1); q += grp.size())
-                Store<P>::st(E, __ldg(g.col_edge + q), L);
-        }
+        for (int q = __ldg(g.col_ptr + j) + grp.rank(); q < __ldg(g.col_ptr + j + 1); q += grp.size())
+            Store<P>::st(E, __ldg(g.col_edge + q), L);
     }
     __device__ void clear_sums(const DevGraph& g, const WarpState& st)
     {
@@ -637,7 +610,19 @@ struct SmallEngine {
             }
         }
     }
-    static __device__ const void* prior_E(const DevGraph& g) { return g.slamE; }
+    __device__ void start_prior(const DevGraph& g, const WarpState& st) const
+    {
+        group_copy16(grp, st.E, g.slamE, snap_vec16(g));
+    }
+    // snapshots: the messages as they are kept
+    __device__ void load_E(const DevGraph& g, const WarpState& st, const void* src) const
+    {
+        group_copy16<true>(grp, st.E, src, snap_vec16(g));
+    }
+    __device__ void save_E(const DevGraph& g, const WarpState& st, void* dst) const
+    {
+        group_copy16(grp, dst, st.E, snap_vec16(g));
+    }
     __device__ void fix_node(const DevGraph& g, const WarpState& st, int j, float L) const
     {
         const int lane = threadIdx.x & 31;
@@ -829,6 +814,323 @@ struct SmallEngine {
 #pragma unroll
         for (int c = 0; c < CPL; ++c)
             if (lane + 32 * c < g.N) dst[lane + 32 * c] = sum[c];
+    }
+};
+
+// exchange networks of 2 to 6 inputs (the last three with the fewest
+// comparators known): comparator c orders inputs x(c) < y(c), the c-th digits of
+// two hexadecimal numbers
+template <int N> struct SortNet;
+template <> struct SortNet<1> { static constexpr int n = 0; static constexpr unsigned long long x = 0x0ull, y = 0x0ull; };
+template <> struct SortNet<2> { static constexpr int n = 1; static constexpr unsigned long long x = 0x0ull, y = 0x1ull; };
+template <> struct SortNet<3> { static constexpr int n = 3; static constexpr unsigned long long x = 0x100ull, y = 0x212ull; };
+template <> struct SortNet<4> { static constexpr int n = 5; static constexpr unsigned long long x = 0x12010ull, y = 0x23132ull; };
+template <> struct SortNet<5> { static constexpr int n = 9; static constexpr unsigned long long x = 0x231201010ull, y = 0x342413243ull; };
+template <> struct SortNet<6> { static constexpr int n = 12; static constexpr unsigned long long x = 0x314202031210ull, y = 0x425315342435ull; };
+
+// JaggedEngine: any code whose column degree is at most DV <= 6 (the detector
+// error models, stacked X and Z checks).  The rows stand in order of falling
+// degree and the k-th edges of all rows lie side by side (jagged diagonals,
+// DevGraph::jplane), so the detector pass -- lane = row -- moves 32 consecutive
+// words per access whatever the degrees; a row's edges are permuted among its
+// words and a column's among its slots so that the error pass meets few bank
+// conflicts (bsd_layout.cu).  D is written over E: a row's and a column's words
+// are its own in either pass.  Messages are floats holding values of the
+// storage format; snapshots are converted.
+//
+// The detector pass takes each edge's minimum over the others with its sign
+// from running signed minima from both ends (three min.xorsign.abs per edge, the
+// cap at L_MAX with the syndrome sign in the first; rows above degree 16 read
+// their messages twice instead).  The error pass runs the exact network of the
+// columns' degree where the 32 columns of a group have the same one (degree 3
+// without a sort, as the single-warp engine), and one padded to the largest
+// degree where they differ.  Masked columns and the clamp are handled as in the
+// single-warp engine.
+//
+// Before (records of the two smallest magnitudes per row, one thread per CSR
+// row, networks of DV inputs for every column) the detector pass of rows of
+// equal degree met 4- to 8-way bank conflicts and an iteration took 2.9 warp
+// instructions per edge.
+template <int DV, int P, bool W = false, class G = WarpGroup>
+struct JaggedEngine {
+    using Grp = G;
+    // blocks of up to 16 warps in 64 registers: two of them resident on an SM;
+    // one warp per candidate: 80 registers, three 8-warp blocks
+    static constexpr int kMinBlocks = G::kBlock ? 2 : 3;
+    static constexpr int kMaxThreads = G::kBlock ? 512 : 256;
+    static constexpr int kPrec = P;
+    static constexpr bool kPriorStart = !W;       // unweighted runs from E(0) start from the table D0
+    static constexpr bool kPriorSetsSums = true;  // a run from E(0) needs no cleared sums
+    using S = Store<P>;
+    G grp;
+
+    // the storage format's value of a message
+    static __device__ __forceinline__ float rnd(float x)
+    {
+        if constexpr (P == 0) return x;
+        typename S::T t;
+        S::st(&t, 0, x);
+        return S::ld(&t, 0);
+    }
+    static __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+    __device__ void load_graph(const DevGraph&, const WarpState&) {}
+    __device__ void start_prior(const DevGraph& g, const WarpState& st) const
+    {
+        float* const E = reinterpret_cast<float*>(st.E);
+        for (int j = grp.rank(); j < g.N; j += grp.size()) {
+            const float v = S::ld(reinterpret_cast<const typename S::T*>(g.lamEc), j);
+#pragma unroll
+            for (int k = 0; k < DV; ++k) {
+                const int e = __ldg(g.colW + (size_t)k * g.Npad + j);
+                if (e >= 0) E[e] = v;
+            }
+        }
+    }
+    __device__ void load_E(const DevGraph& g, const WarpState& st, const void* src) const
+    {
+        if constexpr (P == 0) {
+            group_copy16<true>(grp, st.E, src, snap_vec16(g));
+        } else {
+            const uint4* s = reinterpret_cast<const uint4*>(src);
+            float4* d = reinterpret_cast<float4*>(st.E);
+            for (int q = grp.rank(); q < snap_vec16(g); q += grp.size()) {
+                const uint4 v = __ldcg(s + q);
+                const typename S::T* h = reinterpret_cast<const typename S::T*>(&v);
+                d[2 * q] = make_float4(S::ld(h, 0), S::ld(h, 1), S::ld(h, 2), S::ld(h, 3));
+                d[2 * q + 1] = make_float4(S::ld(h, 4), S::ld(h, 5), S::ld(h, 6), S::ld(h, 7));
+            }
+        }
+    }
+    __device__ void save_E(const DevGraph& g, const WarpState& st, void* dst) const
+    {
+        if constexpr (P == 0) {
+            group_copy16(grp, dst, st.E, snap_vec16(g));
+        } else {
+            uint4* d = reinterpret_cast<uint4*>(dst);
+            const float* s = reinterpret_cast<const float*>(st.E);
+            for (int q = grp.rank(); q < snap_vec16(g); q += grp.size()) {
+                uint4 v;
+                typename S::T* h = reinterpret_cast<typename S::T*>(&v);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) S::st(h, u, s[8 * q + u]);
+                d[q] = v;
+            }
+        }
+    }
+    // the sentinel +L_MAX on every message of the newly fixed node j
+    __device__ void fix_node(const DevGraph& g, const WarpState& st, int j, float L) const
+    {
+        for (int k = grp.rank(); k < DV; k += grp.size()) {
+            const int e = __ldg(g.colW + (size_t)k * g.Npad + j);
+            if (e >= 0) reinterpret_cast<float*>(st.E)[e] = L;
+        }
+    }
+    __device__ void clear_sums(const DevGraph& g, const WarpState& st)
+    {
+        for (int j = grp.rank(); j < g.N; j += grp.size()) st.sumllr[j] = 0.f;
+    }
+
+    // D over E on the row of rank q, of degree deg <= RD, whose words start at eb
+    template <int RD>
+    static __device__ __forceinline__ void row_pass(const DevGraph& g, uint32_t eb, int q, int deg, float sL, float alpha,
+                                                    const float* wt)
+    {
+        float x[RD], after[RD];
+#pragma unroll
+        for (int k = 0; k < RD; ++k) x[k] = k < deg ? lds(eb + 4u * (uint32_t)(g.jplane[k] + q)) : INFINITY;
+        after[RD - 1] = INFINITY;                  // the messages after k
+#pragma unroll
+        for (int k = RD - 1; k > 0; --k) after[k - 1] = k == RD - 1 ? x[k] : xmin(x[k], after[k]);
+        float before = sL;                         // those before k, capped, with the syndrome sign
+#pragma unroll
+        for (int k = 0; k < RD; ++k) {
+            if (k < deg) {
+                const float m = k == RD - 1 ? before : xmin(before, after[k]);
+                sts(eb + 4u * (uint32_t)(g.jplane[k] + q), __fmul_rn(W ? __ldg(wt + g.jplane[k] + q) : alpha, m));
+            }
+            if (k + 1 < RD) before = xmin(before, x[k]);
+        }
+    }
+
+    // Eqs. 2-3 for a column of degree DD (kSame), or at most DD with holes in its
+    // slots: the messages over the column's words, the posterior returned
+    template <int DD, bool kSame>
+    static __device__ __forceinline__ float column(const DevGraph& g, uint32_t eb, int j, float l)
+    {
+        if constexpr (DD == 0) {
+            return l;
+        } else {
+            float v[DD];
+            uint32_t a[DD];
+            const int* cw = g.colW + j;
+#pragma unroll
+            for (int k = 0; k < DD; ++k) {
+                const int e = __ldg(cw + (size_t)k * g.Npad);
+                a[k] = (kSame || e >= 0) ? eb + 4u * (uint32_t)e : 0xffffffffu;
+            }
+#pragma unroll
+            for (int k = 0; k < DD; ++k) v[k] = (kSame || a[k] != 0xffffffffu) ? lds(a[k]) : INFINITY;
+            if constexpr (DD == 3 && kSame) {
+                const float lo12 = fminf(v[1], v[2]), hi12 = fmaxf(v[1], v[2]);
+                const float lo02 = fminf(v[0], v[2]), hi02 = fmaxf(v[0], v[2]);
+                const float lo01 = fminf(v[0], v[1]), hi01 = fmaxf(v[0], v[1]);
+                const float2 ll = make_float2(l, l);
+                const float2 e01 = add2(add2(ll, make_float2(lo12, lo02)), make_float2(hi12, hi02));
+                const float2 e2p = add2(add2(ll, make_float2(lo01, fminf(lo01, v[2]))),
+                                        make_float2(hi01, fmin3(hi01, hi02, hi12)));
+                sts(a[0], rnd(e01.x));
+                sts(a[1], rnd(e01.y));
+                sts(a[2], rnd(e2p.x));
+                return __fadd_rn(e2p.y, fmaxf(hi01, v[2]));
+            } else {
+                // ascending order of value, the addresses along
+#pragma unroll
+                for (int c = 0; c < SortNet<DD>::n; ++c) {
+                    const int x = (int)((SortNet<DD>::x >> (4 * c)) & 15u), y = (int)((SortNet<DD>::y >> (4 * c)) & 15u);
+                    const bool sw = v[x] > v[y];
+                    const float lo = fminf(v[x], v[y]), hi = fmaxf(v[x], v[y]);
+                    const uint32_t al = sw ? a[y] : a[x], ah = sw ? a[x] : a[y];
+                    v[x] = lo; v[y] = hi;
+                    a[x] = al; a[y] = ah;
+                }
+                // (a hole adds +0, which changes no sum)
+                if (!kSame) {
+#pragma unroll
+                    for (int k = 0; k < DD; ++k) v[k] = a[k] == 0xffffffffu ? 0.f : v[k];
+                }
+                float pre = l;
+#pragma unroll
+                for (int k = 0; k < DD; ++k) {                    // Eq. 2: leave d_i out
+                    float acc = pre;
+#pragma unroll
+                    for (int k2 = k + 1; k2 < DD; ++k2) acc = __fadd_rn(acc, v[k2]);
+                    if (kSame || a[k] != 0xffffffffu) sts(a[k], rnd(acc));
+                    pre = __fadd_rn(pre, v[k]);
+                }
+                return pre;                                       // Eq. 3
+            }
+        }
+    }
+
+    template <bool kPostOut = false>
+    __device__ int run(const DevGraph& g, const DecCfg& cfg, const WarpState& st, int max_iters, bool stop,
+                       int* success, float* post_out, bool from_prior = false, const AbortCheck& ab = AbortCheck{})
+    {
+        const int lane = threadIdx.x & 31;
+        const uint32_t eb = saddr(st.E);
+        int iters = 0;
+        int ok = 0;
+        for (int t = 1; t <= max_iters; ++t) {
+            unsigned long long ab_key = 0ull;
+            if (ab.key != nullptr && grp.rank() == 0) ab_key = *((volatile const unsigned long long*)ab.key);
+            for (int q = grp.rank(); q < g.WM; q += grp.size()) st.par[q] = st.sp[q];
+            // weighted min-sum: row min(t, wT) - 1 of the weights in place of alpha
+            const float* wt = W ? cfg.weights + (size_t)((t < cfg.wT ? t : cfg.wT) - 1) * (size_t)g.Epad : nullptr;
+            // ---- detector pass (Eq. 1); a run from E(0) takes its first check
+            // messages from the table D0, flipping the sign where s_i = 1
+            const bool prior = from_prior && t == 1;
+            for (int q = grp.rank(); q < g.M; q += grp.size()) {
+                const int2 rd = __ldg(g.rowQ + q);
+                const uint32_t sb = ((st.sp[rd.x >> 5] >> (rd.x & 31)) & 1u) << 31;
+                if (!W && prior) {
+                    for (int k = 0; k < rd.y; ++k) {
+                        const int e = __ldg(g.jplanes + k) + q;
+                        sts(eb + 4u * (uint32_t)e, __uint_as_float(__float_as_uint(__ldg(g.jD0 + e)) ^ sb));
+                    }
+                    continue;
+                }
+                const float sL = __uint_as_float(__float_as_uint(cfg.L) | sb);
+                const int dmax = __ldg(&g.rowQ[q & ~31].y);       // the warp's largest degree
+                if (dmax <= 8) {
+                    row_pass<8>(g, eb, q, rd.y, sL, cfg.alpha, wt);
+                } else if (dmax <= 12) {
+                    row_pass<12>(g, eb, q, rd.y, sL, cfg.alpha, wt);
+                } else if (dmax <= 16) {
+                    row_pass<16>(g, eb, q, rd.y, sL, cfg.alpha, wt);
+                } else {
+                    // the two smallest magnitudes and the sign parity, then D:
+                    // the minimum over the others is m2 on an edge holding the
+                    // minimum (a tie makes m2 = m1), m1 elsewhere
+                    float m1 = cfg.L, m2 = cfg.L;
+                    uint32_t sg = sb;
+#pragma unroll 4
+                    for (int k = 0; k < rd.y; ++k) {
+                        const float x = lds(eb + 4u * (uint32_t)(__ldg(g.jplanes + k) + q)), m = fabsf(x);
+                        m2 = fminf(m2, fmaxf(m1, m));
+                        m1 = fminf(m1, m);
+                        sg ^= __float_as_uint(x) & 0x80000000u;
+                    }
+#pragma unroll 4
+                    for (int k = 0; k < rd.y; ++k) {
+                        const int e = __ldg(g.jplanes + k) + q;
+                        const float x = lds(eb + 4u * (uint32_t)e);
+                        const float d = __fmul_rn(W ? __ldg(wt + e) : cfg.alpha, fabsf(x) == m1 ? m2 : m1);
+                        sts(eb + 4u * (uint32_t)e,
+                            __uint_as_float(__float_as_uint(d) ^ sg ^ (__float_as_uint(x) & 0x80000000u)));
+                    }
+                }
+            }
+            grp.sync();
+            // ---- error-node pass (Eqs. 2-4) and syndrome parity; each warp owns
+            // whole 32-column words of e^ (one column per lane)
+            for (int jb = 32 * grp.warp(); jb < g.N; jb += 32 * grp.nwarps()) {
+                const int j = jb + lane;
+                bool ebit = false;
+                const int gd = __ldg(g.colG + (jb >> 5));
+                if (j < g.N) {
+                    const float l = ((st.mask[jb >> 5] >> lane) & 1u) ? INFINITY : __ldg(g.lam + j);
+                    float post;
+                    switch (gd) {
+                        case 0: post = column<0, true>(g, eb, j, l); break;
+                        case 1: post = column<1, true>(g, eb, j, l); break;
+                        case 2: post = column<2, true>(g, eb, j, l); break;
+                        case 3: post = column<3, true>(g, eb, j, l); break;
+                        case 9: case 10: case 11: post = column<3, false>(g, eb, j, l); break;
+                        default:
+                            if constexpr (DV == 6) {
+                                if (gd == 4) post = column<4, true>(g, eb, j, l);
+                                else if (gd == 5) post = column<5, true>(g, eb, j, l);
+                                else if (gd == 6) post = column<6, true>(g, eb, j, l);
+                                else post = column<6, false>(g, eb, j, l);
+                            } else {
+                                post = l;
+                            }
+                    }
+                    // a run from E(0) starts its sums here (0 + post, as a sum from zero)
+                    st.sumllr[j] = __fadd_rn(prior ? 0.f : st.sumllr[j], post);
+                    if (kPostOut && t == max_iters) post_out[j] = post;
+                    ebit = post <= 0.f;                               // Eq. 4
+                    if (ebit) {
+                        for (int k = __ldg(g.col_ptr + j); k < __ldg(g.col_ptr + j + 1); ++k) {
+                            const int r = __ldg(g.col_row + k);
+                            atomicXor(&st.par[r >> 5], 1u << (r & 31));
+                        }
+                    }
+                }
+                const uint32_t bal = __ballot_sync(FULLMASK, ebit);
+                if (lane == 0) st.ehat[jb >> 5] = bal;
+            }
+            grp.sync();
+            // ---- stopping rule: H e^(t) = s'
+            uint32_t nz = 0;
+            for (int q = grp.rank(); q < g.WM; q += grp.size()) nz |= st.par[q];
+            ok = !grp.any(nz != 0u);
+            iters = t;
+            grp.sync();
+            if (ok && stop) break;
+            if (ab.key != nullptr && grp.any(grp.rank() == 0 && ab.hit(ab_key))) { ok = 0; break; }
+        }
+        *success = ok;
+        return iters;
+    }
+    __device__ void argmin_score(const DevGraph& g, const WarpState& st, double guard, int* np, long long* S,
+                                 int* tie)
+    {
+        argmin_and_score(grp, g, st, guard, np, S, tie);
+    }
+    __device__ void write_sums(const DevGraph& g, const WarpState& st, float* dst)
+    {
+        for (int j = grp.rank(); j < g.N; j += grp.size()) dst[j] = st.sumllr[j];
     }
 };
 
@@ -1607,7 +1909,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
             grp.sync();
             continue;
         }
-        if (!Eng::kPriorStart) group_copy16(grp, st.E, Eng::prior_E(g), snap_vec16(g));
+        if (!Eng::kPriorStart) eng.start_prior(g, st);
         if (!Eng::kPriorSetsSums) eng.clear_sums(g, st);
         grp.sync();
         int succ = 0;
@@ -1627,7 +1929,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
         if (grp.rank() == 0) a = atomicAdd(&w.ctr->n_active, 1);
         a = grp.bcast(a);
         // the seed path (Alg. 3): snapshot, s' = s, no fixed node, e^, next_pos
-        group_copy16(grp, w.seedE + (size_t)a * snap_bytes(g), st.E, snap_vec16(g));
+        eng.save_E(g, st, w.seedE + (size_t)a * snap_bytes(g));
         uint32_t* bits = w.seedBits + (size_t)a * (size_t)w.SB;
         for (int q = grp.rank(); q < g.WM; q += grp.size()) bits[q] = st.sp[q];
         for (int q = grp.rank(); q < g.WN; q += grp.size()) {
@@ -2056,7 +2358,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(Dev
             // is kept in registers across the selection's call)
             eng.load_graph(g, st);
             // warm start from the parent's snapshot
-            group_copy16<true>(grp, st.E, par.E, snap_vec16(g));
+            eng.load_E(g, st, par.E);
             eng.clear_sums(g, st);
             grp.sync();
             eng.fix_node(g, st, pos, cfg.L);
@@ -2094,7 +2396,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(Dev
                 int np, tie;
                 long long S;
                 eng.argmin_score(g, st, cfg.tie_guard, &np, &S, &tie);
-                group_copy16(grp, w.slotE + cslot * snap_bytes(g), st.E, snap_vec16(g));
+                eng.save_E(g, st, w.slotE + cslot * snap_bytes(g));
                 uint32_t* cbits = w.slotBits + cslot * (size_t)w.SB;
                 for (int q = grp.rank(); q < g.WM; q += grp.size()) cbits[q] = st.sp[q];
                 for (int q = grp.rank(); q < g.WN; q += grp.size()) {
@@ -2144,7 +2446,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_bp_llr(De
     for (long long b = (long long)blockIdx.x * grp.per_block() + grp.index(); b < B; b += nw) {
         for (int q = grp.rank(); q < g.WM; q += grp.size()) st.sp[q] = synd[b * g.WM + q];
         for (int q = grp.rank(); q < g.WN; q += grp.size()) { st.mask[q] = 0u; st.vals[q] = 0u; }
-        if (!Eng::kPriorStart) group_copy16(grp, st.E, Eng::prior_E(g), snap_vec16(g));
+        if (!Eng::kPriorStart) eng.start_prior(g, st);
         if (!Eng::kPriorSetsSums) eng.clear_sums(g, st);
         grp.sync();
         int succ;
@@ -2159,12 +2461,12 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_bp_llr(De
 // host-side launch helpers
 // ----------------------------------------------------------------------------
 // engine id = 3 * kind + storage precision, or 15 + kind for weighted min-sum;
-// kinds: 0..2 generic with column degree bound 3 / 6 / 16, 3: small (CPL 3,
+// kinds: 0, 1 jagged with column degree bound 3 / 6, 2 generic (16), 3: small (CPL 3,
 // RPL 2, row degree 6), 4: small (CPL 5, RPL 3, row degree 6); precision 0
 // float, 1 binary16, 2 bfloat16
 #define BSD_KIND_ALIASES(P, SFX)                          \
-    using Generic3##SFX = GenericEngine<3, P>;            \
-    using Generic6##SFX = GenericEngine<6, P>;            \
+    using Generic3##SFX = JaggedEngine<3, P>;             \
+    using Generic6##SFX = JaggedEngine<6, P>;             \
     using Generic16##SFX = GenericEngine<16, P>;          \
     using Small326##SFX = SmallEngine<3, 2, 6, P>;        \
     using Small536##SFX = SmallEngine<5, 3, 6, P>;
@@ -2172,22 +2474,22 @@ BSD_KIND_ALIASES(0, _f32)
 BSD_KIND_ALIASES(1, _f16)
 BSD_KIND_ALIASES(2, _bf16)
 // weighted min-sum (per-edge, per-iteration weights), single-precision messages: id 15 + kind
-using Generic3_w = GenericEngine<3, 0, true>;
-using Generic6_w = GenericEngine<6, 0, true>;
+using Generic3_w = JaggedEngine<3, 0, true>;
+using Generic6_w = JaggedEngine<6, 0, true>;
 using Generic16_w = GenericEngine<16, 0, true>;
 using Small326_w = SmallEngine<3, 2, 6, 0, true>;
 using Small536_w = SmallEngine<5, 3, 6, 0, true>;
 constexpr int kWeightedEngine = 15;
 // a block of warps per candidate (generic engines only): id 20 + 4 * kind + (0 float, 1 binary16,
 // 2 bfloat16, 3 weighted float)
-#define BSD_BLOCK_ALIASES(DV)                                                   \
-    using Block##DV##_f32 = GenericEngine<DV, 0, false, BlockGroup>;            \
-    using Block##DV##_f16 = GenericEngine<DV, 1, false, BlockGroup>;            \
-    using Block##DV##_bf16 = GenericEngine<DV, 2, false, BlockGroup>;           \
-    using Block##DV##_w = GenericEngine<DV, 0, true, BlockGroup>;
-BSD_BLOCK_ALIASES(3)
-BSD_BLOCK_ALIASES(6)
-BSD_BLOCK_ALIASES(16)
+#define BSD_BLOCK_ALIASES(DV, ENGINE)                                    \
+    using Block##DV##_f32 = ENGINE<DV, 0, false, BlockGroup>;            \
+    using Block##DV##_f16 = ENGINE<DV, 1, false, BlockGroup>;            \
+    using Block##DV##_bf16 = ENGINE<DV, 2, false, BlockGroup>;           \
+    using Block##DV##_w = ENGINE<DV, 0, true, BlockGroup>;
+BSD_BLOCK_ALIASES(3, JaggedEngine)
+BSD_BLOCK_ALIASES(6, JaggedEngine)
+BSD_BLOCK_ALIASES(16, GenericEngine)
 constexpr int kBlockEngine = 20;
 #define BSD_ENGINES(X)                                                                          \
     X(0, Generic3_f32) X(1, Generic3_f16) X(2, Generic3_bf16)                                   \
@@ -2257,8 +2559,10 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     if (CUDA_FAILED(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device)) ||
         CUDA_FAILED(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)))
         return -2;
-    // per-candidate state with the generic engine's detector records
-    g.det_bytes = (int)align16(sizeof(float2) * (size_t)g.M);
+    // per-candidate state: the jagged engine keeps float messages, D over E;
+    // the generic one the stored format and a record per detector
+    g.e_bytes = gkind < 2 ? (int)sizeof(float) : g.msg_bytes;
+    g.det_bytes = gkind < 2 ? 0 : (int)align16(sizeof(float2) * (size_t)g.M);
     const size_t generic_bytes = warp_smem_bytes(g);
     // automatic choice: the small engine where it fits; otherwise a warp per
     // candidate while eight or more candidates fit on an SM, a block of 8
@@ -2274,9 +2578,11 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
         const int kind = skind >= 0 ? skind : gkind;
         eng = weighted ? kWeightedEngine + kind : 3 * kind + g.prec;
         // the small engine keeps D per edge in float (over E with single-precision
-        // messages, else beside it); the generic one a record per detector
-        g.det_bytes = (int)align16(kind < 3 ? sizeof(float2) * (size_t)g.M
-                                            : (g.prec == 0 ? 0 : sizeof(float) * (size_t)g.Epad));
+        // messages, else beside it)
+        if (kind >= 3) {
+            g.e_bytes = g.msg_bytes;
+            g.det_bytes = g.prec == 0 ? 0 : (int)align16(sizeof(float) * (size_t)g.Epad);
+        }
         const size_t per_warp = warp_smem_bytes(g);
         if (per_warp > (size_t)max_optin) return -5;
         wpb = warps_per_block > 0 ? warps_per_block : (int)((96 * 1024) / per_warp);
@@ -2737,7 +3043,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_serve(Dev
             // s = 0 with every Lambda_j > 0: the seed converges at t = 1 with e^ = 0
             finalize_shot<typename Eng::Grp, true>(g, out, 0, st.ehat, ST_SEED, 1ull, grp);
         } else {
-            if (!Eng::kPriorStart) group_copy16(grp, st.E, Eng::prior_E(g), snap_vec16(g));
+            if (!Eng::kPriorStart) eng.start_prior(g, st);
             if (!Eng::kPriorSetsSums) eng.clear_sums(g, st);
             grp.sync();
             int succ = 0;

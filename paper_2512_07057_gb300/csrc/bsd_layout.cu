@@ -296,7 +296,8 @@ void colour_group_n(const std::vector<int>& eu, const std::vector<int>& ev, int 
 
 }  // namespace
 
-bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, GenericLayout* out)
+bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, GenericLayout* out,
+                    const int* start)
 {
     if (M < 1 || N < 1 || colK < 1 || colK > kMaxColour) return false;
     const int E = row_ptr[M];
@@ -308,11 +309,11 @@ bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int co
     const int NG = (N + 31) / 32;
     std::vector<int> cap(NG, 0);                  // the largest column degree of each group
     for (int j = 0; j < N; ++j) cap[j >> 5] = std::max(cap[j >> 5], cdeg[j]);
-    // position of every CSR edge inside its row's storage window: start from
-    // the CSR order and swap within rows while the bank loads above each
-    // group's cap fall
+    // position of every CSR edge among its row's words: start from the given
+    // order (the CSR order) and swap within rows while the bank loads above
+    // each group's cap fall
     std::vector<int> pos(E);
-    for (int e = 0; e < E; ++e) pos[e] = e;
+    for (int e = 0; e < E; ++e) pos[e] = start ? start[e] : e;
     std::vector<int> cnt((size_t)NG * 32, 0);
     for (int e = 0; e < E; ++e) cnt[(size_t)(col_idx[e] >> 5) * 32 + (pos[e] & 31)]++;
     auto over = [&](int g, int b) { return std::max(0, cnt[(size_t)g * 32 + b] - cap[g]); };

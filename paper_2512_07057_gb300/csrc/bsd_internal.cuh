@@ -76,6 +76,8 @@ struct DevGraph {
     const int* jplanes;    // [max_row_deg]
     int jplane[16];
     const float* jD0;      // [E] D0 at those words
+    const int4* tile_word; // [N][1 or 2] kTileShots * tile_slot of the column's edges, -1 past its degree
+                           // (one int4 for column degrees up to 4, two up to 8; null above)
     const void* lamEc;     // [Npad] E(0) of column j (clamp(Lambda_j)) in the storage format
     // the columns ordered by degree (batched seed BP): colperm[q] is the
     // column at position q, the columns of degree d hold positions
@@ -107,6 +109,11 @@ struct DevGraph {
     const uint32_t* shrow; // [32 ceil(M / 32)][kSmallRowWords] with the placement: the columns of row i of H
                            // as a bit set (the stopping rule's parities); zero past M
 };
+
+// shots of a tile of the unrolled decoder's on-chip path (bsd_unrolled.cu), and
+// the place of an edge's kTileShots values in units of them
+constexpr int kTileShots = 8;
+__host__ __device__ inline int tile_slot(int e) { return e ^ ((e >> 3) & 3); }
 
 struct DecCfg {
     int max_rounds, w, initial_iters, iters_per_round, num_results;

@@ -35,6 +35,7 @@
 // result is deterministic.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -446,6 +447,443 @@ __global__ void k_u_gw(const float* __restrict__ gw_part, int T, int ntile, int 
     }
 }
 
+// ---------------------------------------------------------------------------
+// the whole forward, and the whole backward, of a tile of shots on chip
+// ---------------------------------------------------------------------------
+// For codes with rows and columns of degree at most 8 whose messages of
+// kShots shots fit in an SM's shared memory, one block runs every iteration of
+// a tile of kShots shots there, so the messages never leave the SM: per
+// iteration a row pass (E -> D, or gD -> gE) and a column pass (D -> E, or gE ->
+// gD), each over the same words.  A thread handles one row or column for four
+// shots (16-byte accesses); edge e's kShots values start at word
+// kShots * tile_slot(e), which puts the accesses of consecutive rows of degree 8
+// in different banks.  The forward keeps what the adjoint needs of every
+// iteration, in place of the message checkpoints: per (row, shot) the two
+// smallest magnitudes, their edges and the signs (10 bytes), per (node, shot)
+// Lambda_j(t).  gE(t) is zero but on the two edges of a row that hold its
+// minima, whose magnitudes lie below L_MAX, so the adjoint of the clamp needs no
+// look at E(t).  Weight gradients are summed over a block's tiles in order in
+// the block's own partial, then over the blocks: deterministic.
+//
+// Bound: 4 shared-memory transfers per edge and shot (6912 wavefronts per
+// iteration of 8 shots on the phenomenological DEM, 3.3 us) and the issue slots
+// of both passes, against HBM traffic of 20 bytes per edge, pass and shot
+// before.
+constexpr int kShots = kTileShots;
+constexpr int kTileThreads = 512;
+constexpr int kMaxDeg = 8;
+
+struct TileArgs {
+    const int* row_ptr;
+    const int* row_col;
+    const int4* col_word;    // [N][CAP / 4]: words of the column's edges (kShots * tile_slot), -1 past its degree
+    const float* lam;
+    int M, N, E, T;
+    float L;
+    long long B;
+    int ntile;               // tiles of kShots shots
+    const float* w;          // [T][E]
+    unsigned char* s8;       // [ntile][M] the syndrome bits of the tile's shots
+    unsigned char* y8;       // [ntile][N] their errors
+    float* m1;               // [ntile][T][M][kShots]
+    float* m2;
+    uint16_t* pk;            // own signs of the row's edges (bits 0..7), edges of m1 and m2 (4 bits each, 15: none)
+    float* lamT;             // [ntile][T][N][kShots]
+    float* loss_part;        // [T][ntile]
+    float* gw_part;          // [blocks][T][E]
+    int blocks, threads;
+};
+
+__host__ __device__ inline size_t tile_smem(int M, int N, int E)
+{
+    const size_t e4 = ((size_t)E + 3) & ~size_t(3);
+    return e4 * kShots * sizeof(float) + (((size_t)M + (size_t)N + 15) & ~size_t(15)) + 2 * 16 * sizeof(float);
+}
+__device__ __forceinline__ float4* tile_at(float* x, int e, int half)
+{
+    return reinterpret_cast<float4*>(x + kShots * tile_slot(e) + 4 * half);
+}
+// the words of a column's edges
+template <int CAP>
+__device__ __forceinline__ void column_words(const TileArgs& a, int j, int (&e)[CAP])
+{
+#pragma unroll
+    for (int h = 0; h < CAP / 4; ++h) {
+        const int4 v = __ldg(a.col_word + (size_t)j * (CAP / 4) + h);
+        e[4 * h] = v.x; e[4 * h + 1] = v.y; e[4 * h + 2] = v.z; e[4 * h + 3] = v.w;
+    }
+}
+// signed minimum of two messages: the magnitude's minimum with the product's sign
+__device__ __forceinline__ float xmin(float a, float b)
+{
+    float r;
+    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+// bits << 1 with the sign of v below
+__device__ __forceinline__ uint32_t push_sign(uint32_t bits, float v)
+{
+    return __funnelshift_l(__float_as_uint(v), bits, 1);
+}
+// the row's weights or gradients as two 16-byte accesses where it has eight
+// edges at an aligned place
+__device__ __forceinline__ bool row_aligned(const float* p, int rb, int deg)
+{
+    return deg == kMaxDeg && ((reinterpret_cast<uintptr_t>(p + rb) & 15u) == 0);
+}
+__device__ __forceinline__ bool row_weights(const float* wt, int rb, int deg, float (&wv)[kMaxDeg])
+{
+    const bool wide = row_aligned(wt, rb, deg);
+    if (wide) {
+        const float4 w0 = __ldg(reinterpret_cast<const float4*>(wt + rb));
+        const float4 w1 = __ldg(reinterpret_cast<const float4*>(wt + rb) + 1);
+        wv[0] = w0.x; wv[1] = w0.y; wv[2] = w0.z; wv[3] = w0.w;
+        wv[4] = w1.x; wv[5] = w1.y; wv[6] = w1.z; wv[7] = w1.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < kMaxDeg; ++k) wv[k] = k < deg ? __ldg(wt + rb + k) : 0.f;
+    }
+    return wide;
+}
+// softplus(x) as above; below 2^-12 the two terms of log1p's series are within
+// e^2 / 3 of it, and most nodes are there
+__device__ __forceinline__ float softplus_tail(float x)
+{
+    const float e = expf(-fabsf(x));
+    const float l = e < 0x1p-12f ? fmaf(-0.5f * e, e, e) : log1pf(e);
+    return fmaxf(x, 0.f) + l;
+}
+
+template <int CAP>
+__global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const uint32_t* __restrict__ synd,
+                                                            const uint32_t* __restrict__ errs, int WM, int WN,
+                                                            float* __restrict__ llr)
+{
+    extern __shared__ __align__(16) float sm[];
+    float* const x = sm;
+    unsigned char* const sb = reinterpret_cast<unsigned char*>(sm + (((size_t)a.E + 3) & ~size_t(3)) * kShots);
+    unsigned char* const yb = sb + a.M;
+    float* const red = reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15)));   // [2][16]
+    const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
+        const long long b0 = (long long)tile * kShots;
+        // the tile's syndrome and error bits, one byte per row and node
+        for (int q = threadIdx.x; q < a.M + a.N; q += blockDim.x) {
+            const bool row = q < a.M;
+            const int i = row ? q : q - a.M, W = row ? WM : WN;
+            const uint32_t* src = row ? synd : errs;
+            uint32_t v = 0;
+#pragma unroll
+            for (int c = 0; c < kShots; ++c)
+                if (b0 + c < a.B) v |= ((__ldg(src + (size_t)(b0 + c) * W + (i >> 5)) >> (i & 31)) & 1u) << c;
+            sb[q] = (unsigned char)v;
+            if (row) a.s8[(size_t)tile * a.M + i] = (unsigned char)v;
+            else a.y8[(size_t)tile * a.N + i] = (unsigned char)v;
+        }
+        for (int q = threadIdx.x; q < 2 * a.E; q += blockDim.x) {          // E(0)
+            const float v = fminf(fmaxf(__ldg(a.lam + __ldg(a.row_col + (q >> 1))), -a.L), a.L);
+            *tile_at(x, q >> 1, q & 1) = make_float4(v, v, v, v);
+        }
+        __syncthreads();
+        for (int t = 1; t <= a.T; ++t) {
+            const float* wt = a.w + (size_t)(t - 1) * (size_t)a.E;
+            const size_t rec = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.M * kShots;
+            for (int q = threadIdx.x; q < 2 * a.M; q += blockDim.x) {
+                const int i = q >> 1, half = q & 1;
+                const int rb = __ldg(a.row_ptr + i), deg = __ldg(a.row_ptr + i + 1) - rb;
+                const uint32_t s4 = (uint32_t)sb[i] >> (4 * half);
+                float wv[kMaxDeg];
+                row_weights(wt, rb, deg, wv);
+                float4 v[kMaxDeg];
+#pragma unroll
+                for (int k = 0; k < kMaxDeg; ++k)
+                    v[k] = k < deg ? *tile_at(x, rb + k, half) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+                float r1[4], r2[4];
+                uint32_t rp[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    // each edge's signed minimum over the others (capped at
+                    // L_MAX, with the syndrome sign) from running minima from
+                    // both ends; the two smallest magnitudes are the least of
+                    // all and the largest of these
+                    float out[kMaxDeg];
+                    out[kMaxDeg - 1] = INFINITY;
+#pragma unroll
+                    for (int k = kMaxDeg - 1; k > 0; --k)
+                        out[k - 1] = k == kMaxDeg - 1 ? comp(v[k], c) : xmin(comp(v[k], c), out[k]);
+                    float pre = __uint_as_float(__float_as_uint(a.L) | (((s4 >> c) & 1u) << 31));
+#pragma unroll
+                    for (int k = 0; k < kMaxDeg; ++k) {
+                        out[k] = k == kMaxDeg - 1 ? pre : xmin(pre, out[k]);
+                        pre = xmin(pre, comp(v[k], c));
+                    }
+                    const float m1 = fabsf(pre);
+                    float m2 = m1;
+#pragma unroll
+                    for (int k = 0; k < kMaxDeg; ++k) m2 = fmaxf(m2, fabsf(out[k]));   // (past the degree: m1)
+                    // their edges (the lowest among equals, none at L_MAX) and
+                    // the own signs, bit by bit: m - |x| has its sign bit set
+                    // where |x| > m
+                    uint32_t above1 = ~0u, above2 = ~0u, neg = 0u;
+#pragma unroll
+                    for (int k = kMaxDeg - 1; k >= 0; --k) {
+                        const float y = comp(v[k], c);
+                        above1 = push_sign(above1, m1 - fabsf(y));
+                        above2 = push_sign(above2, m2 - fabsf(y));
+                        neg = push_sign(neg, y);
+                        setc(v[k], c, __fmul_rn(wv[k], out[k]));
+                    }
+                    const uint32_t at1 = m1 < a.L ? ~above1 : 0u;
+                    const uint32_t first = at1 & (0u - at1);
+                    const uint32_t at2 = m2 < a.L ? ~above2 & ~first : 0u;
+                    const uint32_t i1 = at1 ? (uint32_t)__ffs((int)at1) - 1u : 15u;
+                    const uint32_t i2 = at2 ? (uint32_t)__ffs((int)at2) - 1u : 15u;
+                    r1[c] = m1;
+                    r2[c] = m2;
+                    rp[c] = (neg & 0xFFu) | (i1 << 8) | (i2 << 12);
+                }
+#pragma unroll
+                for (int k = 0; k < kMaxDeg; ++k)
+                    if (k < deg) *tile_at(x, rb + k, half) = v[k];
+                const size_t at = rec + (size_t)i * kShots + 4 * half;
+                *reinterpret_cast<float4*>(a.m1 + at) = make_float4(r1[0], r1[1], r1[2], r1[3]);
+                *reinterpret_cast<float4*>(a.m2 + at) = make_float4(r2[0], r2[1], r2[2], r2[3]);
+                *reinterpret_cast<uint2*>(a.pk + at) = make_uint2(rp[0] | (rp[1] << 16), rp[2] | (rp[3] << 16));
+            }
+            __syncthreads();
+            float loss = 0.f;
+            const size_t nod = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.N * kShots;
+            for (int q = threadIdx.x; q < 2 * a.N; q += blockDim.x) {
+                const int j = q >> 1, half = q & 1;
+                int e[CAP];
+                column_words<CAP>(a, j, e);
+                const float lj = __ldg(a.lam + j);
+                float4 post = make_float4(lj, lj, lj, lj);
+                float4 v[CAP];
+#pragma unroll
+                for (int k = 0; k < CAP; ++k) {
+                    if (e[k] >= 0) {
+                        v[k] = *reinterpret_cast<const float4*>(x + e[k] + 4 * half);
+                        post.x = __fadd_rn(post.x, v[k].x);
+                        post.y = __fadd_rn(post.y, v[k].y);
+                        post.z = __fadd_rn(post.z, v[k].z);
+                        post.w = __fadd_rn(post.w, v[k].w);
+                    }
+                }
+                // (unclamped: the row pass caps the magnitudes at L_MAX)
+#pragma unroll
+                for (int k = 0; k < CAP; ++k) {
+                    if (e[k] >= 0)
+                        *reinterpret_cast<float4*>(x + e[k] + 4 * half) =
+                            make_float4(__fsub_rn(post.x, v[k].x), __fsub_rn(post.y, v[k].y),
+                                        __fsub_rn(post.z, v[k].z), __fsub_rn(post.w, v[k].w));
+                }
+                *reinterpret_cast<float4*>(a.lamT + nod + (size_t)j * kShots + 4 * half) = post;
+                const uint32_t y4 = (uint32_t)yb[j] >> (4 * half);
+                const long long b = b0 + 4 * half;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float p = comp(post, c);
+                    const float l = softplus_tail(((y4 >> c) & 1u) ? p : -p);
+                    loss += b + c < a.B ? l : 0.f;
+                    if (llr && b + c < a.B)
+                        llr[((size_t)(t - 1) * (size_t)a.B + (size_t)(b + c)) * (size_t)a.N + j] = p;
+                }
+            }
+            loss = warp_sum(loss);
+            if (lane == 0) red[16 * (t & 1) + wid] = loss;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                double l = 0.0;
+                for (int k = 0; k < nw; ++k) l += (double)red[16 * (t & 1) + k];
+                a.loss_part[(size_t)(t - 1) * a.ntile + tile] = (float)l;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <int CAP>
+__global__ void __launch_bounds__(kTileThreads, 1) k_u_backward(TileArgs a, const float* __restrict__ gout, double scale)
+{
+    extern __shared__ __align__(16) float sm[];
+    float* const x = sm;
+    unsigned char* const sb = reinterpret_cast<unsigned char*>(sm + (((size_t)a.E + 3) & ~size_t(3)) * kShots);
+    unsigned char* const yb = sb + a.M;
+    float* const part = a.gw_part + (size_t)blockIdx.x * (size_t)a.T * (size_t)a.E;
+    for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
+        const bool fresh = tile == (int)blockIdx.x;
+        const long long b0 = (long long)tile * kShots;
+        for (int q = threadIdx.x; q < a.M; q += blockDim.x) sb[q] = a.s8[(size_t)tile * a.M + q];
+        for (int q = threadIdx.x; q < a.N; q += blockDim.x) yb[q] = a.y8[(size_t)tile * a.N + q];
+        __syncthreads();
+        for (int t = a.T; t >= 1; --t) {
+            // the objective's derivative with respect to the term of iteration t:
+            // through the total ([0]) and through the term itself ([t])
+            const float gs = (float)(((double)__ldg(gout) + (double)__ldg(gout + t)) * scale);
+            const size_t nod = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.N * kShots;
+            for (int q = threadIdx.x; q < 2 * a.N; q += blockDim.x) {
+                const int j = q >> 1, half = q & 1;
+                int e[CAP];
+                column_words<CAP>(a, j, e);
+                const float4 post = __ldg(reinterpret_cast<const float4*>(a.lamT + nod + (size_t)j * kShots + 4 * half));
+                const uint32_t y4 = (uint32_t)yb[j] >> (4 * half);
+                const long long b = b0 + 4 * half;
+                float4 gl;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    // d BCE / d Lambda = sigmoid(Lambda) - 1 + e_j
+                    // (1 + e^-Lambda rounds to 1 above 16.64, where most nodes are)
+                    const float p = comp(post, c);
+                    const float sg = p > 16.7f ? 1.f : 1.f / (1.f + expf(-p));
+                    setc(gl, c, (b + c < a.B) ? gs * (sg - 1.f + (float)((y4 >> c) & 1u)) : 0.f);
+                }
+                float4 g[CAP];
+#pragma unroll
+                for (int k = 0; k < CAP; ++k) {
+                    g[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (t < a.T && e[k] >= 0) {
+                        g[k] = *reinterpret_cast<const float4*>(x + e[k] + 4 * half);
+                        gl.x += g[k].x; gl.y += g[k].y; gl.z += g[k].z; gl.w += g[k].w;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < CAP; ++k)
+                    if (e[k] >= 0)
+                        *reinterpret_cast<float4*>(x + e[k] + 4 * half) =
+                            make_float4(gl.x - g[k].x, gl.y - g[k].y, gl.z - g[k].z, gl.w - g[k].w);
+            }
+            __syncthreads();
+            const float* wt = a.w + (size_t)(t - 1) * (size_t)a.E;
+            float* gwt = part + (size_t)(t - 1) * (size_t)a.E;
+            const size_t rec = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.M * kShots;
+            for (int q = threadIdx.x; q < ((2 * a.M + 31) & ~31); q += blockDim.x) {
+                const bool in = q < 2 * a.M;
+                const int i = in ? q >> 1 : 0, half = q & 1;
+                const int rb = __ldg(a.row_ptr + i), deg = in ? __ldg(a.row_ptr + i + 1) - rb : 0;
+                const size_t at = rec + (size_t)i * kShots + 4 * half;
+                const float4 m1v = __ldg(reinterpret_cast<const float4*>(a.m1 + at));
+                const float4 m2v = __ldg(reinterpret_cast<const float4*>(a.m2 + at));
+                const uint2 pv = __ldg(reinterpret_cast<const uint2*>(a.pk + at));
+                const uint32_t s4 = (uint32_t)sb[i] >> (4 * half);
+                uint32_t neg[4], sig[4];
+                int i1[4], i2[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t p = (c < 2 ? pv.x : pv.y) >> (16 * (c & 1));
+                    neg[c] = p & 0xFFu;
+                    i1[c] = (int)((p >> 8) & 15u);
+                    i2[c] = (int)((p >> 12) & 15u);
+                    // bit k: the sign of the product over the other edges
+                    sig[c] = (((uint32_t)__popc(neg[c]) ^ (s4 >> c)) & 1u) ? ~neg[c] : neg[c];
+                }
+                float acc1[4] = {0.f, 0.f, 0.f, 0.f}, g1[4] = {0.f, 0.f, 0.f, 0.f}, gw[kMaxDeg], wv[kMaxDeg];
+                const bool wide = row_weights(wt, rb, deg, wv);
+#pragma unroll
+                for (int k = 0; k < kMaxDeg; ++k) {
+                    gw[k] = 0.f;
+                    if (k < deg) {
+                        const float4 g = *tile_at(x, rb + k, half);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const float gd = __uint_as_float(__float_as_uint(comp(g, c)) ^ (((sig[c] >> k) & 1u) << 31));
+                            gw[k] += gd * (k == i1[c] ? comp(m2v, c) : comp(m1v, c));
+                            const float gm = gd * wv[k];
+                            if (k == i1[c]) g1[c] = gm; else acc1[c] += gm;
+                        }
+                    }
+                    // the tile's other four shots are in the next lane
+                    gw[k] += __shfl_xor_sync(0xffffffffu, gw[k], 1);
+                }
+                if (wide && row_aligned(gwt, rb, deg)) {
+                    float4* o = reinterpret_cast<float4*>(gwt + rb) + half;
+                    float4 r = half ? make_float4(gw[4], gw[5], gw[6], gw[7]) : make_float4(gw[0], gw[1], gw[2], gw[3]);
+                    if (!fresh) {
+                        const float4 p = *o;
+                        r.x += p.x; r.y += p.y; r.z += p.z; r.w += p.w;
+                    }
+                    *o = r;
+                } else if (half == 0) {
+#pragma unroll
+                    for (int k = 0; k < kMaxDeg; ++k)
+                        if (k < deg) gwt[rb + k] = fresh ? gw[k] : gwt[rb + k] + gw[k];
+                }
+                if (t > 1) {
+#pragma unroll
+                    for (int k = 0; k < kMaxDeg; ++k) {
+                        if (k < deg) {
+                            float4 o;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                // d|E|/dE = sign(E), 0 at 0
+                                const float m = k == i1[c] ? comp(m1v, c) : comp(m2v, c);
+                                float r = k == i1[c] ? acc1[c] : g1[c];
+                                r = __uint_as_float(__float_as_uint(r) ^ (((neg[c] >> k) & 1u) << 31));
+                                setc(o, c, (k == i1[c] || (k == i2[c] && i1[c] != 15)) && m > 0.f ? r : 0.f);
+                            }
+                            *tile_at(x, rb + k, half) = o;
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// weight gradients of the tiled backward: the blocks' partial sums in order
+__global__ void k_u_gw_blocks(const float* __restrict__ part, long long n, int blocks, float* __restrict__ grad)
+{
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
+        double s = 0.0;
+        for (int k = 0; k < blocks; ++k) s += (double)part[(size_t)k * (size_t)n + (size_t)q];
+        grad[q] = (float)s;
+    }
+}
+
+// the tiled path's arrays in the caller's workspace; false where a degree, the
+// shared memory or the workspace (whose size the general passes set) does not
+// allow it
+bool tile_plan(const DevGraph& g, const DecCfg& cfg, int device, long long B, int T, const float* w, char* base,
+               size_t have, TileArgs* out)
+{
+    if (g.max_row_deg > kMaxDeg || g.tile_word == nullptr || g.max_row_deg < 1) return false;
+    const size_t smem = tile_smem(g.M, g.N, g.E);
+    int optin = 0, sms = 0;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || smem > (size_t)optin)
+        return false;
+    TileArgs a{};
+    a.row_ptr = g.row_ptr; a.row_col = g.row_col; a.col_word = g.tile_word; a.lam = g.lam;
+    a.M = g.M; a.N = g.N; a.E = g.E; a.T = T; a.L = cfg.L; a.B = B; a.w = w;
+    a.ntile = (int)((B + kShots - 1) / kShots);
+    // a thread per four shots of a row or of two columns, at most kTileThreads;
+    // as many blocks as fit at once, or fewer with the same number of tiles each
+    const int want = std::max(2 * g.M, g.N);
+    a.threads = std::min(kTileThreads, std::max(64, (want + 31) / 32 * 32));
+    const int fit = sms * std::max(1, std::min((int)((size_t)optin / smem), kTileThreads / a.threads));
+    const int rounds = (a.ntile + fit - 1) / fit;
+    a.blocks = (a.ntile + rounds - 1) / rounds;
+    const size_t nt = (size_t)a.ntile, TM = (size_t)T * (size_t)g.M * kShots, TN = (size_t)T * (size_t)g.N * kShots;
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* p = base + off;
+        off += a256(bytes);
+        return p;
+    };
+    a.s8 = (unsigned char*)take(nt * (size_t)g.M);
+    a.y8 = (unsigned char*)take(nt * (size_t)g.N);
+    a.m1 = (float*)take(sizeof(float) * nt * TM);
+    a.m2 = (float*)take(sizeof(float) * nt * TM);
+    a.pk = (uint16_t*)take(sizeof(uint16_t) * nt * TM);
+    a.lamT = (float*)take(sizeof(float) * nt * TN);
+    a.loss_part = (float*)take(sizeof(float) * nt * (size_t)T);
+    a.gw_part = (float*)take(sizeof(float) * (size_t)a.blocks * (size_t)T * (size_t)g.E);
+    if (off > have) return false;
+    *out = a;
+    return true;
+}
+
 // register cache for rows / columns of degree at most 4 or 8, none beyond
 int cap_of(int max_deg) { return max_deg <= 4 ? 4 : (max_deg <= 8 ? 8 : 0); }
 
@@ -565,6 +1003,21 @@ int bsd_unrolled_forward(const bsd_decoder* dec, const uint32_t* d_syndromes, co
     const size_t EB = (size_t)g->E * (size_t)a.Bp;
     LaunchHooks hks;
     const LaunchHooks* hk = decoder_hooks(dec, s, &hks) ? &hks : nullptr;
+    TileArgs ta;
+    if (tile_plan(*g, *cfg, device, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
+        const size_t smem = tile_smem(g->M, g->N, g->E);
+        auto kf = g->max_col_deg <= 4 ? k_u_forward<4> : k_u_forward<8>;
+        if (CUDA_FAILED(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+            return BSD_ERR_CUDA;
+        {
+            Timed tm(hk, kKindCheck);
+            kf<<<ta.blocks, ta.threads, smem, s>>>(ta, d_syndromes, d_errors, g->WM, g->WN, d_llr);
+        }
+        Timed tm(hk, kKindOther);
+        k_u_loss<<<T, 256, 0, s>>>(ta.loss_part, 1, ta.ntile, 1.0 / ((double)B * (double)g->N), d_loss);
+        k_u_loss_total<<<1, 32, 0, s>>>(T, d_loss);
+        return CUDA_FAILED(cudaGetLastError()) ? BSD_ERR_CUDA : BSD_OK;
+    }
     {
         Timed tm(hk, kKindOther);
         k_u_planes<<<1024, 256, 0, s>>>(d_syndromes, B, g->WM, g->M, a.Bp, u.sT);
@@ -611,6 +1064,20 @@ int bsd_unrolled_backward(const bsd_decoder* dec, int64_t B, int32_t T, int32_t 
     const dim3 gcol(a.ntile, grid_y(g->N)), grow(a.ntile, grid_y(g->M));
     LaunchHooks hks;
     const LaunchHooks* hk = decoder_hooks(dec, s, &hks) ? &hks : nullptr;
+    TileArgs ta;
+    if (tile_plan(*g, *cfg, device, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
+        const size_t smem = tile_smem(g->M, g->N, g->E);
+        auto kb = g->max_col_deg <= 4 ? k_u_backward<4> : k_u_backward<8>;
+        if (CUDA_FAILED(cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+            return BSD_ERR_CUDA;
+        {
+            Timed tm(hk, kKindBVar);
+            kb<<<ta.blocks, ta.threads, smem, s>>>(ta, d_grad_loss, scale);
+        }
+        Timed tm(hk, kKindOther);
+        k_u_gw_blocks<<<1024, 128, 0, s>>>(ta.gw_part, (long long)T * g->E, ta.blocks, d_grad_weights);
+        return CUDA_FAILED(cudaGetLastError()) ? BSD_ERR_CUDA : BSD_OK;
+    }
     int cur = 0;                               // gE(t) lives in u.gE[cur]
     const int C = (T + k - 1) / k;
     for (int c = C - 1; c >= 0; --c) {

@@ -95,6 +95,10 @@ inline int words_of(long long bits) { return (int)((bits + 31) / 32); }
 // this many slots
 constexpr long long kBatchMinEdges = 16384;
 constexpr int kBatchDefaultSlots = 2048;
+// by default the batch runs on at least this many shots: below, its passes over
+// the graph for the last few slots take longer than the per-candidate kernel
+// (4300 shots of the synthetic DEM, 75 of them failing: 9.5 against 2 ms)
+constexpr int kBatchMinQueue = 65536;
 // the second-iteration screen is built while the columns next to flipped
 // detectors are expected to be at most this share of all
 constexpr double kScreen2MaxShare = 0.125;
@@ -696,6 +700,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     }
 
     DecCfg& cfg = dec->cfg;
+    cfg.bs_min_queue = params->batch_slots == 0 ? kBatchMinQueue : 0;
     cfg.max_rounds = params->max_rounds;
     cfg.w = params->beam_width;
     cfg.initial_iters = params->initial_iters;
@@ -751,10 +756,13 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     long long S = (long long)(((double)budget - (double)A * win_b) / seed_b);
     if (S > (1ll << 22)) S = 1ll << 22;
     if (S < A) S = A;
-    // with the batched seed BP a chunk can hold far more shots than the seed
-    // store: only the shots it hands on need an entry, and they are decoded
-    // in windows of S
-    const long long S1 = bs_slots > 0 ? (1ll << 22) : 0;
+    // a chunk can hold more shots than the seed store where most seeds end the
+    // search: only the others need an entry, and those that find none are
+    // decoded again in windows of S.  With the batched seed BP 4M; else 4 S, as
+    // far as the two lists of a chunk's shots take no more than 1/2048 of the
+    // workspace (10^5 shots of the phenomenological DEM with w = 64 are one chunk
+    // instead of four, each with its own last failing shots)
+    long long S1 = bs_slots > 0 ? (1ll << 22) : NR == 1 ? std::min(4 * S, budget >> 14) : 0;
     for (;;) {
         const size_t wb = work_layout(g, cfg, S, A, nullptr, nullptr, bs_slots, S1);
         if (cudaMalloc(&dec->work_mem, wb) == cudaSuccess) { dec->work_bytes = wb; break; }
@@ -763,6 +771,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
         if (S == 1 && A == 1) { bsd_destroy(dec); return BSD_ERR_OOM; }
         S = S > 1 ? S / 2 : 1;
         A = A > 1 ? A / 2 : 1;
+        if (bs_slots == 0) S1 = std::min(S1, 4 * S);
     }
     Work& w = dec->w;
     work_layout(g, cfg, S, A, (char*)dec->work_mem, &w, bs_slots, S1);
@@ -878,11 +887,11 @@ static void prof_collect(bsd_decoder* d)
     d->ev_used = 0;
 }
 
-// shots per chunk: the seed store, or with the batched seed BP the larger
-// chunk whose handed-on shots it decodes in windows of the seed store
+// shots per chunk: the seed store, or the larger chunk whose handed-on shots
+// are decoded in windows of it
 static long long chunk_of(const bsd_decoder* dec)
 {
-    return (dec->ls.batch && dec->w.bs_slots > 0) ? dec->w.S1 : dec->w.S;
+    return ((dec->ls.batch && dec->w.bs_slots > 0) || dec->w.bs_slots == 0) ? dec->w.S1 : dec->w.S;
 }
 
 static int decode_impl(bsd_decoder* dec, const uint32_t* d_synd, long long base, long long n, const Outputs& o,

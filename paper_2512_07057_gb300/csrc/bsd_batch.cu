@@ -75,25 +75,29 @@ __device__ __forceinline__ BsRange bs_range(const Work& w, int items)
 }  // namespace
 
 // fill the slots with the first queued shots (every shot of the chunk when no
-// screen ran) and open the loop
-__global__ void k_bs_begin(Work w, int screened, cudaGraphConditionalHandle cond, int use_cond)
+// screen ran) and open the loop; a queue of fewer than min_queue shots goes to
+// the per-candidate kernel at once
+__global__ void k_bs_begin(Work w, int screened, int min_queue, cudaGraphConditionalHandle cond, int use_cond)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&w.stats[2], 1ull);
     const long long chunk_n = w.desc->chunk_n;
     const int nq = screened ? *((volatile int*)&w.ctr->n_queue) : (int)chunk_n;
     const int Bs = w.bs_slots;
+    const bool hand_on = nq < min_queue;
+    if (hand_on)
+        for (int k = threadIdx.x; k < nq; k += blockDim.x) w.fail[k] = screened ? w.queue[k] : k;
     for (int b = threadIdx.x; b < Bs; b += blockDim.x) {
-        w.bs_shot[b] = b < nq ? (screened ? w.queue[b] : b) : -1;
+        w.bs_shot[b] = b < nq && !hand_on ? (screened ? w.queue[b] : b) : -1;
         w.bs_t[b] = 0;
         w.bs_nl[b] = 0;
     }
     if (threadIdx.x == 0) {
-        const int n0 = nq < Bs ? nq : Bs;
+        const int n0 = hand_on ? 0 : nq < Bs ? nq : Bs;
         w.ctr->bs_claim = n0;
         w.ctr->bs_run = n0 > 0 ? 1 : 0;
         w.ctr->bs_active_next = 0;
         w.ctr->bs_done_blocks = 0;
-        w.ctr->n_fail = 0;
+        w.ctr->n_fail = hand_on ? nq : 0;
         if (use_cond) cudaGraphSetConditional(cond, n0 > 0 ? 1u : 0u);
     }
 }
@@ -463,8 +467,8 @@ int add_batch_nodes(cudaGraph_t graph, cudaGraphNode_t dep, cudaGraphNode_t* las
     if (CUDA_FAILED(cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault))) return -2;
     int use = 1;
     cudaGraphNode_t nb, nw;
-    void* bargs[] = {&w, &screened, &cond, &use};
-    int rc = add_node(graph, &nb, dep ? &dep : nullptr, (void*)k_bs_begin, 1, 256, bargs);
+    void* bargs[] = {&w, &screened, &cfg.bs_min_queue, &cond, &use};
+    int rc = add_node(graph, &nb, dep ? &dep : nullptr, (void*)k_bs_begin, 1, 1024, bargs);
     cudaGraphNodeParams cp{};
     if (!rc) {
         cp.type = cudaGraphNodeTypeConditional;
@@ -492,7 +496,7 @@ int launch_batch_direct(const DevGraph& g, const DecCfg& cfg, const Work& w, con
                         cudaStream_t s, const LaunchHooks* hk, int* host_word)
 {
     const cudaGraphConditionalHandle none{};
-    k_bs_begin<<<1, 256, 0, s>>>(w, screened, none, 0);
+    k_bs_begin<<<1, 1024, 0, s>>>(w, screened, cfg.bs_min_queue, none, 0);
     if (CUDA_FAILED(cudaGetLastError())) return -2;
     const int gc = grid_pass(w, g.M, kRowsPerThread), gv = grid_pass(w, g.N, kColsPerThread);
     const int gr = grid_retire(ls, w);

@@ -116,6 +116,8 @@ constexpr int kTileShots = 8;
 __host__ __device__ inline int tile_slot(int e) { return e ^ ((e >> 3) & 3); }
 
 struct DecCfg {
+    int bs_min_queue;      // the batched seed BP runs on at least this many shots, fewer go to the
+                           // per-candidate kernel
     int max_rounds, w, initial_iters, iters_per_round, num_results;
     float alpha, L;        // L: L_MAX as the storage format holds it
     double tie_guard;      // near-tie margin (0: no flags)
@@ -180,7 +182,7 @@ struct RunDesc {
     Outputs out;
     long long chunk_base;  // index of the chunk's first shot in the caller's batch
     long long chunk_n;     // shots in the chunk
-    int win_base;          // batched seed BP: first entry of the fail list in the current window
+    int win_base;          // first entry of the fail list in the current window
 };
 
 // per-chunk counters (reset by k_begin_chunk)
@@ -195,7 +197,7 @@ struct Counters {
     int bs_run;            // the batch has active slots: another iteration runs
     int bs_active_next;    // active slots after the current retirement (counted by its blocks)
     int bs_done_blocks;    // blocks of the current retirement that have finished
-    int n_fail;            // shots passed on to the per-candidate seed kernel
+    int n_fail;            // shots on the fail list
     // the beam over the n_active entries of the seed store
     unsigned b_head;       // tickets drawn from the ring of items
     unsigned b_tail;       // items put on it
@@ -225,9 +227,9 @@ constexpr long long kBeamEntries = 4096;
 constexpr int kErrBeam = 2;                   // Counters::err: the beam left a shot behind
 
 struct Work {
-    long long S;           // shots per chunk = seed-store entries
-    long long S1;          // with the batched seed BP: shots per chunk (>= S); the shots it hands on are
-                           // decoded from the seed on in windows of S
+    long long S;           // seed-store entries
+    long long S1;          // shots per chunk (>= S); those the batched seed BP hands on, or that find the
+                           // store full, are decoded from the seed on in windows of S
     long long A;           // window entries: shots whose beam runs at once
     int SB;                // words per slot bit record: sp[WM] mask[WN] vals[WN] ehat[WN]
     int* queue;            // [S1] chunk-local shots the screens passed on to the seed BP
@@ -240,7 +242,7 @@ struct Work {
     int* bs_t;             // [Bs] iterations the slot's shot has run
     int* bs_nl;            // [Bs] columns with e^_j(t) = 1 found in the current iteration
     int* bs_list;          // [kBsList][Bs] those columns
-    int* fail;             // [S1] shots the batch passes on to the per-candidate seed kernel
+    int* fail;             // [S1] shots for the windows: handed on by the batch, or the store was full
     // seed store [S]
     unsigned char* seedE;  // [S][Epad] messages in the storage format
     uint32_t* seedBits;    // [S][SB]

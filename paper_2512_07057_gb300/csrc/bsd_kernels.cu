@@ -102,7 +102,12 @@ struct WarpGroup {
     __device__ __forceinline__ int index() const { return threadIdx.x >> 5; }       // candidate slot of the block
     __device__ __forceinline__ int per_block() const { return blockDim.x >> 5; }
     __device__ __forceinline__ void sync() const { __syncwarp(); }
-    __device__ __forceinline__ bool any(bool p) const { return __any_sync(FULLMASK, p); }
+    __device__ __forceinline__ bool any(bool p) const
+    {
+        const bool r = __any_sync(FULLMASK, p);
+        __syncwarp();
+        return r;
+    }
     __device__ __forceinline__ int bcast(int v) const { return __shfl_sync(FULLMASK, v, 0); }
     __device__ __forceinline__ uint32_t xor_all(uint32_t v) const
     {
@@ -159,7 +164,7 @@ constexpr size_t kSelectBytes = 2 * kMaxBeam * (sizeof(double) + 2 * sizeof(int)
 __host__ __device__ inline size_t warp_smem_bytes(const DevGraph& g)
 {
     const size_t n = align16((size_t)g.e_bytes * (size_t)g.Epad) + det_region_bytes(g) +
-                     align16(sizeof(float) * (size_t)g.Npad) + align16(sizeof(uint32_t) * (size_t)(2 * g.WM + 3 * g.WN));
+                     align16(sizeof(float) * (size_t)g.Npad) + align16(sizeof(uint32_t) * (size_t)(2 * g.WM + 3 * g.WN + 1));
     return n > kSelectBytes ? n : kSelectBytes;   // the selection's scratch lies over the candidate's state
 }
 
@@ -173,6 +178,7 @@ struct WarpState {
     uint32_t* mask;    // [WN]
     uint32_t* vals;    // [WN]
     uint32_t* ehat;    // [WN]
+    uint32_t* ab;      // [1] a lower-index sibling has succeeded (early abort)
 };
 
 __device__ inline WarpState carve(char* base, const DevGraph& g)
@@ -189,6 +195,7 @@ __device__ inline WarpState carve(char* base, const DevGraph& g)
     s.mask = b + 2 * g.WM;
     s.vals = b + 2 * g.WM + g.WN;
     s.ehat = b + 2 * g.WM + 2 * g.WN;
+    s.ab = b + 2 * g.WM + 3 * g.WN;
     return s;
 }
 
@@ -1070,6 +1077,7 @@ struct JaggedEngine {
                     }
                 }
             }
+            if (ab.key != nullptr && grp.rank() == 0) st.ab[0] = ab.hit(ab_key) ? 1u : 0u;
             grp.sync();
             // ---- error-node pass (Eqs. 2-4) and syndrome parity; each warp owns
             // whole 32-column words of e^ (one column per lane)
@@ -1111,14 +1119,16 @@ struct JaggedEngine {
                 if (lane == 0) st.ehat[jb >> 5] = bal;
             }
             grp.sync();
-            // ---- stopping rule: H e^(t) = s'
+            // ---- stopping rule: H e^(t) = s' (the vote's barrier also keeps the
+            // next iteration's writes to par behind these reads); a child that
+            // succeeds in the iteration at whose end it would stop has succeeded
             uint32_t nz = 0;
             for (int q = grp.rank(); q < g.WM; q += grp.size()) nz |= st.par[q];
+            const bool gone = ab.key != nullptr && st.ab[0] != 0u;
             ok = !grp.any(nz != 0u);
             iters = t;
-            grp.sync();
             if (ok && stop) break;
-            if (ab.key != nullptr && grp.any(grp.rank() == 0 && ab.hit(ab_key))) { ok = 0; break; }
+            if (gone) { ok = 0; break; }
         }
         *success = ok;
         return iters;
@@ -1270,11 +1280,15 @@ __global__ void k_begin_chunk(Work w, const uint32_t* synd, Outputs out, long lo
 }
 
 // graph only, after the seed kernel: run the beam only if some shot of the
-// chunk needs it
-__global__ void k_beam_gate(Work w, cudaGraphConditionalHandle cond)
+// chunk needs it, and (windows) the loop over windows after it only if a shot
+// found the seed store full
+__global__ void k_beam_gate(Work w, cudaGraphConditionalHandle cond, cudaGraphConditionalHandle cwin, int windows)
 {
     count_launch(w);
-    if (threadIdx.x == 0) cudaGraphSetConditional(cond, w.ctr->n_active > 0 ? 1u : 0u);
+    if (threadIdx.x == 0) {
+        cudaGraphSetConditional(cond, w.ctr->n_active > 0 ? 1u : 0u);
+        if (windows) cudaGraphSetConditional(cwin, w.ctr->n_fail > 0 ? 1u : 0u);
+    }
 }
 
 // counters of a beam search over the n_active entries of the seed store: the
@@ -1283,8 +1297,9 @@ __global__ void k_beam_begin(Work w, int beam_width)
 {
     count_launch(w);
     if (threadIdx.x == 0) {
-        const int n = w.ctr->n_active;
+        const int n = (int)((long long)w.ctr->n_active < w.S ? (long long)w.ctr->n_active : w.S);
         const int cnt = (long long)n < w.A ? n : (int)w.A;
+        w.ctr->n_active = n;
         w.ctr->b_head = 0u;
         w.ctr->b_tail = 2u * (unsigned)cnt;
         w.ctr->b_left = n;
@@ -1717,6 +1732,7 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
             // the records of E0(1) over the other columns: the first two of the
             // row's four smallest; a row that has fewer (more than two of the
             // four are next to flipped detectors) is read whole
+#pragma unroll 4
             for (int i = lane; i < g.M; i += 32) {
                 const float4 a0 = __ldg(g.row4 + 2 * i), a1 = __ldg(g.row4 + 2 * i + 1);
                 const float x[4] = {a0.x, a0.z, a1.x, a1.z};
@@ -1866,12 +1882,16 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
     count_launch(w);
     eng.load_graph(g, st);
     unsigned long long seed_iters = 0;           // BP iterations (group rank 0)
-    // a warp claims its shots kBatch at a time (one atomic per batch on the
-    // chunk's counter, which a million one-iteration seeds would otherwise
-    // hit a million times); a block candidate one at a time
-    constexpr int kBatch = Eng::Grp::kBlock ? 1 : 4;
+    // a warp claims its shots four at a time (one atomic per batch on the
+    // chunk's counter, which a million one-iteration seeds would otherwise hit a
+    // million times), but one at a time once the shots left are few for the
+    // grid, and where each is many iterations: a block candidate's, and those a
+    // screen passed on (four failing seeds in one warp held up the end of the
+    // kernel: 10^5 shots of depolarizing noise on [[144,12,12]] 6.7 -> 4.4 ms)
+    const int total_warps = (int)(gridDim.x * grp.per_block());
     // the shots: every shot of the chunk (screened = 0), those the screen
-    // passed on (1), or those the batched seed BP passed on (2)
+    // passed on (1), or the current window of the fail list (2: those the
+    // batched seed BP passed on, or that found the seed store full)
     const int wb = screened == 2 ? *((volatile int*)&w.desc->win_base) : 0;
     const int* list = screened == 2 ? w.fail + wb : w.queue;
     int nq = screened ? *((volatile int*)&w.ctr->n_queue) : 0;
@@ -1883,10 +1903,11 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
     int kcur = 0, kend = 0;                      // claimed slots [kcur, kend), the same in the whole group
     for (;;) {
         if (kcur >= kend) {
+            const int batch = (Eng::Grp::kBlock || screened || dp->chunk_n - kend < 16ll * total_warps) ? 1 : 4;
             int base = 0;
-            if (grp.rank() == 0) base = atomicAdd(&w.ctr->claim_seed, kBatch);
+            if (grp.rank() == 0) base = atomicAdd(&w.ctr->claim_seed, batch);
             kcur = grp.bcast(base);
-            kend = kcur + kBatch;
+            kend = kcur + batch;
         }
         const int k = kcur++;
         // after a screen, the shots it passed on; else every shot of the chunk
@@ -1926,8 +1947,14 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
         long long S;
         eng.argmin_score(g, st, cfg.tie_guard, &np, &S, &tie);
         int a = 0;
-        if (grp.rank() == 0) a = atomicAdd(&w.ctr->n_active, 1);
+        if (grp.rank() == 0) {
+            a = atomicAdd(&w.ctr->n_active, 1);
+            // a full store (a chunk may be larger): the shot is decoded again in
+            // a window after this one's beam
+            if (a >= w.S) w.fail[atomicAdd(&w.ctr->n_fail, 1)] = b;
+        }
         a = grp.bcast(a);
+        if (a >= w.S) continue;
         // the seed path (Alg. 3): snapshot, s' = s, no fixed node, e^, next_pos
         eng.save_E(g, st, w.seedE + (size_t)a * snap_bytes(g));
         uint32_t* bits = w.seedBits + (size_t)a * (size_t)w.SB;
@@ -2565,10 +2592,12 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     g.det_bytes = gkind < 2 ? 0 : (int)align16(sizeof(float2) * (size_t)g.M);
     const size_t generic_bytes = warp_smem_bytes(g);
     // automatic choice: the small engine where it fits; otherwise a warp per
-    // candidate while eight or more candidates fit on an SM, a block of 8
-    // warps per candidate beyond
+    // candidate while eight or more candidates fit on an SM, a block of 16
+    // warps per candidate beyond (8 / 16 warps: 10^5 shots of the
+    // phenomenological DEM at p = 3e-3 3.42 / 2.88 ms, 5 x 10^4 in half
+    // precision 0.87 / 0.74, 3 x 10^5 of the synthetic DEM 11.2 / 10.7)
     int gw = group_warps;
-    if (gw == 0) gw = (skind >= 0 || generic_bytes * 8 <= (size_t)max_optin) ? 1 : 8;
+    if (gw == 0) gw = (skind >= 0 || generic_bytes * 8 <= (size_t)max_optin) ? 1 : 16;
     const bool weighted = cfg.weights != nullptr;
     int eng, wpb;
     if (gw >= 2) {
@@ -2713,10 +2742,16 @@ static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, c
         k_beam_end<<<1, 32, 0, s>>>(w);
         return CUDA_FAILED(cudaGetLastError()) ? -2 : 0;
     };
-    if (!(ls.batch && w.bs_slots > 0)) return seed_and_beam(ls.screen);
-    // batched seed BP over the chunk, then the shots it handed on in windows
-    // of at most S (the seed store)
-    if (launch_batch_direct(g, cfg, w, ls, ls.screen, s, hk, host_n_active)) return -2;
+    // the seed BP of the chunk: batched, or per candidate with the beam of the
+    // shots that fit the seed store; then the shots handed on, in windows of at
+    // most S (the store)
+    const bool batched = ls.batch && w.bs_slots > 0;
+    if (batched) {
+        if (launch_batch_direct(g, cfg, w, ls, ls.screen, s, hk, host_n_active)) return -2;
+    } else {
+        const int rc = seed_and_beam(ls.screen);
+        if (rc || w.S1 <= w.S || cfg.max_rounds == 0) return rc;
+    }
     if (CUDA_FAILED(cudaMemcpyAsync(host_n_active, &w.ctr->n_fail, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
         CUDA_FAILED(cudaStreamSynchronize(s)))
         return -2;
@@ -2762,14 +2797,14 @@ static int add_kernel(cudaGraph_t graph, cudaGraphNode_t* node, const cudaGraphN
 // left } after `dep` in `graph`
 template <class Eng>
 static int add_beam_nodes(cudaGraph_t graph, cudaGraphNode_t dep, cudaGraphNode_t* last, DevGraph& g, DecCfg& cfg,
-                          Work& w, const LaunchShape& ls)
+                          Work& w, const LaunchShape& ls, cudaGraphConditionalHandle cwin = 0, int windows = 0)
 {
     int rc = 0;
     cudaGraphConditionalHandle cbeam;
     cudaGraphNode_t gate, beam, begin, ring, entries, round, end;
     if (CUDA_FAILED(cudaGraphConditionalHandleCreate(&cbeam, graph, 0, cudaGraphCondAssignDefault))) rc = -2;
     if (!rc) {
-        void* gargs[] = {&w, &cbeam};
+        void* gargs[] = {&w, &cbeam, &cwin, &windows};
         rc = add_kernel(graph, &gate, &dep, (void*)k_beam_gate, 1, 32, 0, gargs);
     }
     cudaGraphNodeParams cp{};
@@ -2823,46 +2858,49 @@ static int build_graph_t(const DevGraph& g0, const DecCfg& cfg0, const Work& w0,
         rc = add_kernel(graph, &scr, &scr1, screen2_func(ls.dv_screen, g.prec), ls.grid_screen2, 32 * kScreenWarps,
                         ls.smem_screen2, cargs);
     }
+    // WHILE (shots handed on remain) { window start, the seed kernel on at most
+    // S of them, the beam, window end } after `dep`
+    auto add_windows = [&](cudaGraphNode_t dep, cudaGraphConditionalHandle cwin) {
+        cudaGraphNode_t wwin;
+        cudaGraphNodeParams cp{};
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = cwin;
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        if (CUDA_FAILED(cudaGraphAddNode(&wwin, graph, &dep, nullptr, 1, &cp))) { rc = -2; return; }
+        cudaGraph_t body = cp.conditional.phGraph_out[0];
+        cudaGraphNode_t wbeg, wseed, wend;
+        int keep = -1, from = 2;
+        void* bargs[] = {&w, &keep};
+        void* wargs[] = {&g, &cfg, &w, &from};
+        rc = add_kernel(body, &wbeg, nullptr, (void*)k_win_begin, 1, 32, 0, bargs);
+        if (!rc) rc = add_kernel(body, &wseed, &wbeg, (void*)k_seed<Eng>, ls.grid_seed, threads, ls.smem_bp, wargs);
+        cudaGraphNode_t tail = wseed;
+        if (!rc && cfg.max_rounds > 0) rc = add_beam_nodes<Eng>(body, wseed, &tail, g, cfg, w, ls);
+        void* eargs[] = {&w, &cwin};
+        if (!rc) rc = add_kernel(body, &wend, &tail, (void*)k_win_end, 1, 32, 0, eargs);
+    };
+    cudaGraphConditionalHandle cwin = 0;
+    const int windows = !batched && w.S1 > w.S && cfg.max_rounds > 0;
+    if (!rc && (batched || windows) &&
+        CUDA_FAILED(cudaGraphConditionalHandleCreate(&cwin, graph, 0, cudaGraphCondAssignDefault)))
+        rc = -2;
     if (!batched) {
-        // seed, then the beam
+        // seed, then the beam, then the shots that found the store full
         if (!rc)
             rc = add_kernel(graph, &seed, ls.screen ? &scr : nullptr, (void*)k_seed<Eng>, ls.grid_seed, threads,
                             ls.smem_bp, sargs);
-        if (!rc && cfg.max_rounds > 0) rc = add_beam_nodes<Eng>(graph, seed, &last, g, cfg, w, ls);
+        if (!rc && cfg.max_rounds > 0) rc = add_beam_nodes<Eng>(graph, seed, &last, g, cfg, w, ls, cwin, windows);
+        if (!rc && windows) add_windows(last, cwin);
     } else {
-        // the batched seed BP over the chunk, then WHILE (shots handed on
-        // remain) { window start, the seed kernel on at most S of them, the
-        // beam, window end }
-        cudaGraphNode_t bs, wgate, wwin;
-        cudaGraphConditionalHandle cwin;
+        // the batched seed BP over the chunk, then the shots it handed on
+        cudaGraphNode_t bs, wgate;
         if (!rc) rc = add_batch_nodes(graph, ls.screen ? scr : nullptr, &bs, g, cfg, w, ls, ls.screen);
-        if (!rc && CUDA_FAILED(cudaGraphConditionalHandleCreate(&cwin, graph, 0, cudaGraphCondAssignDefault)))
-            rc = -2;
         if (!rc) {
             void* gargs[] = {&w, &cwin};
             rc = add_kernel(graph, &wgate, &bs, (void*)k_win_gate, 1, 32, 0, gargs);
         }
-        cudaGraphNodeParams cp{};
-        if (!rc) {
-            cp.type = cudaGraphNodeTypeConditional;
-            cp.conditional.handle = cwin;
-            cp.conditional.type = cudaGraphCondTypeWhile;
-            cp.conditional.size = 1;
-            if (CUDA_FAILED(cudaGraphAddNode(&wwin, graph, &wgate, nullptr, 1, &cp))) rc = -2;
-        }
-        if (!rc) {
-            cudaGraph_t body = cp.conditional.phGraph_out[0];
-            cudaGraphNode_t wbeg, wend;
-            int keep = -1;
-            void* bargs[] = {&w, &keep};
-            rc = add_kernel(body, &wbeg, nullptr, (void*)k_win_begin, 1, 32, 0, bargs);
-            if (!rc)
-                rc = add_kernel(body, &seed, &wbeg, (void*)k_seed<Eng>, ls.grid_seed, threads, ls.smem_bp, sargs);
-            cudaGraphNode_t tail = seed;
-            if (!rc && cfg.max_rounds > 0) rc = add_beam_nodes<Eng>(body, seed, &tail, g, cfg, w, ls);
-            void* eargs[] = {&w, &cwin};
-            if (!rc) rc = add_kernel(body, &wend, &tail, (void*)k_win_end, 1, 32, 0, eargs);
-        }
+        if (!rc) add_windows(wgate, cwin);
     }
     cudaGraphExec_t gx = nullptr;
     if (!rc && CUDA_FAILED(cudaGraphInstantiate(&gx, graph, 0))) rc = -2;
@@ -2906,7 +2944,7 @@ size_t work_head_bytes()
 size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long A, char* base, Work* w,
                    int bs_slots, long long S1)
 {
-    if (bs_slots <= 0 || S1 < S) S1 = S;
+    if (S1 < S) S1 = S;
     const size_t W2 = 2 * (size_t)cfg.w;
     const size_t SB = (size_t)g.WM + 3 * (size_t)g.WN;
     const size_t NR = (size_t)cfg.num_results;
@@ -2960,11 +2998,11 @@ size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long 
         v.bs_t = (int*)take(sizeof(int) * Bs);
         v.bs_nl = (int*)take(sizeof(int) * Bs);
         v.bs_list = (int*)take(sizeof(int) * Bs * (size_t)kBsList);
-        v.fail = (int*)take(sizeof(int) * (size_t)S1);
     }
+    if (bs_slots > 0 || S1 > S) v.fail = (int*)take(sizeof(int) * (size_t)S1);
     // the first screen's queue for the second lies where the chunk's later
     // steps write (the hand-on list of the batch, or the seed store's shots)
-    v.queue1 = bs_slots > 0 ? v.fail : v.seed_shot;
+    v.queue1 = v.fail != nullptr || base == nullptr ? v.fail : v.seed_shot;
     if (w) *w = v;
     return off;
 }

@@ -499,6 +499,28 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
             std::memcpy(&colRD[((size_t)j * rdk + k) * 2 + 1], &r, 4);
         }
     }
+    // the first screen's edge table: the edge's column, and in bit 31 whether a
+    // flip of the edge's row alone gives e^_j(1) = 1 (Eqs. 3-4 in the screen's
+    // order on D0 with that message's sign flipped)
+    std::vector<uint32_t> scrC((size_t)(E > 0 ? E : 1), 0u);
+    const bool screens = all_pos && rdk > 0 && params->num_results == 1;
+    std::vector<int> byD(screens ? (size_t)E : 0);          // each column's edges in ascending order of D0 > 0
+    for (int j = 0; j < N && screens; ++j) {
+        int* const o = byD.data() + col_ptr[j];
+        const int deg = col_ptr[j + 1] - col_ptr[j];
+        for (int k = 0; k < deg; ++k) {
+            const int e = col_edge[col_ptr[j] + k];
+            int at = k;
+            for (; at > 0 && D0[o[at - 1]] > D0[e]; --at) o[at] = o[at - 1];
+            o[at] = e;
+        }
+        for (int k = 0; k < deg; ++k) {
+            float post = lam[j] - D0[o[k]];                 // the flipped message is the smallest
+            for (int k2 = 0; k2 < deg; ++k2)
+                if (k2 != k) post = post + D0[o[k2]];
+            scrC[o[k]] = (uint32_t)j | (post <= 0.f ? 0x80000000u : 0u);
+        }
+    }
     // the second-iteration screen's tables: E0(1), the messages after one
     // iteration with s = 0 (D0 of the column's other edges added to Lambda_j in
     // ascending order, clamped and rounded to the storage format), and each
@@ -509,7 +531,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     // p = 1e-3 to 3e-3) of the columns it pays; at 78% (depolarizing noise on
     // [[144,12,12]], p = 0.05) 3% of the shots converge at t = 2.
     std::vector<float> E1, row4;
-    if (all_pos && rdk > 0 && N < 65536 && params->num_results == 1) {
+    if (screens && N < 65536) {
         double next = 0.0;
         for (int i = 0; i < M; ++i) {
             double q = 1.0;
@@ -518,27 +540,29 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
         }
         if (next <= kScreen2MaxShare * N) {
             E1.assign((size_t)E, 0.f);
-            std::vector<int> ord;
             for (int j = 0; j < N; ++j) {
-                ord.assign(col_edge.begin() + col_ptr[j], col_edge.begin() + col_ptr[j + 1]);
-                std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return D0[a] < D0[b]; });
-                for (int e : ord) {
+                for (int k = col_ptr[j]; k < col_ptr[j + 1]; ++k) {
                     float acc = lam[j];
-                    for (int e2 : ord)
-                        if (e2 != e) acc = acc + D0[e2];
+                    for (int k2 = col_ptr[j]; k2 < col_ptr[j + 1]; ++k2)
+                        if (k2 != k) acc = acc + D0[byD[k2]];
                     const float v = store_round(std::fmin(std::fmax(acc, -L), L));
-                    E1[e] = v == 0.f ? 0.f : v;
+                    E1[byD[k]] = v == 0.f ? 0.f : v;
                 }
             }
             row4.assign((size_t)M * 8, 0.f);
             for (int i = 0; i < M; ++i) {
-                ord.resize(H_row_ptr[i + 1] - H_row_ptr[i]);
-                for (size_t k = 0; k < ord.size(); ++k) ord[k] = H_row_ptr[i] + (int)k;
-                std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return E1[a] < E1[b]; });
+                float x[4] = {L, L, L, L};
+                int c[4] = {-1, -1, -1, -1};
+                for (int e = H_row_ptr[i]; e < H_row_ptr[i + 1]; ++e) {
+                    // (a message at L_MAX is kept before the padding)
+                    int at = 4;
+                    while (at > 0 && (E1[e] < x[at - 1] || c[at - 1] < 0)) --at;
+                    for (int k = 3; k > at; --k) { x[k] = x[k - 1]; c[k] = c[k - 1]; }
+                    if (at < 4) { x[at] = E1[e]; c[at] = H_col_idx[e]; }
+                }
                 for (size_t k = 0; k < 4; ++k) {
-                    const int c = k < ord.size() ? H_col_idx[ord[k]] : -1;
-                    row4[(size_t)i * 8 + 2 * k] = k < ord.size() ? E1[ord[k]] : L;
-                    std::memcpy(&row4[(size_t)i * 8 + 2 * k + 1], &c, 4);
+                    row4[(size_t)i * 8 + 2 * k] = x[k];
+                    std::memcpy(&row4[(size_t)i * 8 + 2 * k + 1], &c[k], 4);
                 }
             }
         }
@@ -591,6 +615,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     gb += align256(sizeof(int) * colperm.size());
     gb += align256(sizeof(int2) * colseq.size());
     gb += align256(sizeof(float) * colRD.size());
+    gb += align256(sizeof(uint32_t) * scrC.size());
     gb += align256(sizeof(float) * E1.size()) + align256(sizeof(float) * row4.size());
     // the single-warp engine's rows of H as column sets (the stopping rule's parities)
     std::vector<uint32_t> shrow;
@@ -630,6 +655,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     unsigned char* d_lamEc = carve<unsigned char>(p, lamEc_st.size());
     int* d_colperm = colperm.empty() ? nullptr : carve<int>(p, colperm.size());
     int2* d_colseq = colseq.empty() ? nullptr : carve<int2>(p, colseq.size());
+    uint32_t* d_scrC = carve<uint32_t>(p, scrC.size());
     float* d_E1 = E1.empty() ? nullptr : carve<float>(p, E1.size());
     float* d_row4 = row4.empty() ? nullptr : carve<float>(p, row4.size());
     float* d_colRD = colRD.empty() ? nullptr : carve<float>(p, colRD.size());
@@ -662,6 +688,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
                !CUDA_FAILED(cudaMemcpy(d_colperm, colperm.data(), sizeof(int) * colperm.size(), cudaMemcpyHostToDevice))) &&
               (colseq.empty() ||
                !CUDA_FAILED(cudaMemcpy(d_colseq, colseq.data(), sizeof(int2) * colseq.size(), cudaMemcpyHostToDevice))) &&
+              !CUDA_FAILED(cudaMemcpy(d_scrC, scrC.data(), sizeof(uint32_t) * scrC.size(), cudaMemcpyHostToDevice)) &&
               (E1.empty() ||
                (!CUDA_FAILED(cudaMemcpy(d_E1, E1.data(), sizeof(float) * E1.size(), cudaMemcpyHostToDevice)) &&
                 !CUDA_FAILED(cudaMemcpy(d_row4, row4.data(), sizeof(float) * row4.size(), cudaMemcpyHostToDevice)))) &&
@@ -690,6 +717,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     g.colperm = d_colperm; g.colseq = d_colseq;
     g.colRD = reinterpret_cast<const float4*>(d_colRD); g.colRDk = rdk;
     for (int d = 0; d < kMaxColDeg + 2; ++d) { g.dstart[d] = dstart[d]; g.dbase[d] = dbase[d]; }
+    g.scrC = d_scrC;
     g.E1 = d_E1; g.row4 = reinterpret_cast<const float4*>(d_row4);
     g.scol = d_scol; g.sD0 = d_sD0; g.slamE = d_slamE; g.shrow = d_shrow;
     dec->generic_pos = jpos;

@@ -90,6 +90,7 @@ struct DevGraph {
     // the degree bounds 3, 6 and 16 (two pairs per float4)
     const float4* colRD;   // [Npad][colRDk / 2]
     int colRDk;
+    const uint32_t* scrC;  // [E] column of CSR edge e; bit 31: with its row the column's only flipped one, e^_j(1) = 1
     // second-iteration screen (null where it does not pay): per row the four
     // smallest E0(1) -- E(1) for s = 0, every Lambda_j > 0 -- with their
     // columns, ascending, padded with (L_MAX, -1); and E0(1) of every CSR edge

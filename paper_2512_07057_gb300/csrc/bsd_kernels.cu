@@ -1381,12 +1381,18 @@ __global__ void k_win_end(Work w, cudaGraphConditionalHandle cond)
 // t = 1 with this e^, and a converged seed with one result reads neither E(1)
 // nor sum_LLR.  The others go to the seed BP through the queue.  The state of
 // a warp is four bit vectors, so many shots are in flight per SM.
+//
+// Most columns next to a flipped detector are next to one only, and whether
+// that flip alone makes e^_j(1) = 1 does not depend on the shot: it is a bit of
+// the edge (DevGraph::scrC).  So Eqs. 2-4 are formed only for the columns met
+// a second time and those whose bit is set (of about 285 columns per shot of
+// the synthetic DEM some 10 are; 10^6 shots 5.4 -> 2.1 ms).
 constexpr int kScreenWarps = 8;
 constexpr int kMaxFlip = 128;
 
 __host__ __device__ inline size_t screen_warp_words(const DevGraph& g)
 {
-    return 2 * (size_t)g.WN + 2 * (size_t)g.WM + 2 * (size_t)kMaxFlip;
+    return 2 * (size_t)g.WN + 2 * (size_t)g.WM + 2 * (size_t)kMaxFlip + 64;
 }
 
 // (more: the shots that do not converge go to the second-iteration screen)
@@ -1401,6 +1407,7 @@ __global__ void k_screen(DevGraph g, DecCfg cfg, Work w, int more)
     uint32_t* par = sp + g.WM;
     int* fst = reinterpret_cast<int*>(par + g.WM);    // [kMaxFlip] flipped detectors, then their first edges
     int* foff = fst + kMaxFlip;                       // [kMaxFlip] their edges' offsets in the shot's list
+    int* cand = foff + kMaxFlip;                      // [64] columns to form
     count_launch(w);
     const RunDesc* dp = w.desc;
     const long long n = dp->chunk_n;
@@ -1465,23 +1472,14 @@ __global__ void k_screen(DevGraph g, DecCfg cfg, Work w, int more)
                     tot += __shfl_sync(FULLMASK, incl, 31);
                 }
                 __syncwarp();
-                // one (detector, edge) pair per lane: the column on the edge
-                for (int t = lane; t < tot; t += 32) {
-                    int lo = 0, hi = nflip - 1;                    // last detector with foff <= t
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (foff[mid] <= t) lo = mid; else hi = mid - 1;
-                    }
-                    const int e0 = fst[lo] + (t - foff[lo]);
-                    const int j = __ldg(g.row_col + e0);
-                    const uint32_t bit = 1u << (j & 31);
-                    if (atomicOr(&seen[j >> 5], bit) & bit) continue;   // another flipped detector has it
-                    // D_{i'->j}(1) on the column's edges: the check message of
-                    // E(0) on the edge (the same for every shot: E(0) > 0 on
-                    // every edge, so it is alpha times the row's minimum over the
-                    // other edges, positive) with the syndrome bit of its row as
-                    // the sign; two (message, row) pairs per 16-byte load, padding
-                    // (+inf, -1) past the column's degree
+                // D_{i'->j}(1) on the column's edges: the check message of
+                // E(0) on the edge (the same for every shot: E(0) > 0 on
+                // every edge, so it is alpha times the row's minimum over the
+                // other edges, positive) with the syndrome bit of its row as
+                // the sign; two (message, row) pairs per 16-byte load, padding
+                // (+inf, -1) past the column's degree.  (A column listed twice
+                // is formed twice with the same result.)
+                auto form = [&](int j) {
                     constexpr int KD = DV == 3 ? 4 : DV;
                     const float4* cr = g.colRD + (size_t)j * (KD / 2);
                     float v[KD];
@@ -1513,13 +1511,45 @@ __global__ void k_screen(DevGraph g, DecCfg cfg, Work w, int more)
                     for (int k = 0; k < KD; ++k)
                         if (k < deg) post = __fadd_rn(post, v[k]);
                     upd += (unsigned long long)deg;
-                    if (post <= 0.f) {                            // Eq. 4
-                        atomicOr(&eh[j >> 5], bit);
+                    const uint32_t bit = 1u << (j & 31);
+                    if (post <= 0.f && !(atomicOr(&eh[j >> 5], bit) & bit)) {   // Eq. 4
 #pragma unroll
                         for (int k = 0; k < KD; ++k)
                             if (rr[k] >= 0) atomicXor(&par[rr[k] >> 5], 1u << (rr[k] & 31));
                     }
+                };
+                // one (detector, edge) pair per lane: the column on the edge,
+                // listed when another flipped detector had it or its bit is set
+                int nc = 0;
+                for (int t0 = 0; t0 < tot; t0 += 32) {
+                    const int t = t0 + lane;
+                    bool add = false;
+                    int j = 0;
+                    if (t < tot) {
+                        int lo = 0, hi = nflip - 1;                // last detector with foff <= t
+                        while (lo < hi) {
+                            const int mid = (lo + hi + 1) >> 1;
+                            if (foff[mid] <= t) lo = mid; else hi = mid - 1;
+                        }
+                        const uint32_t c = __ldg(g.scrC + fst[lo] + (t - foff[lo]));
+                        j = (int)(c & 0x7fffffffu);
+                        const uint32_t bit = 1u << (j & 31);
+                        add = (atomicOr(&seen[j >> 5], bit) & bit) || (c >> 31);
+                    }
+                    const uint32_t bal = __ballot_sync(FULLMASK, add);
+                    if (add) cand[nc + __popc(bal & ((1u << lane) - 1u))] = j;
+                    nc += __popc(bal);
+                    __syncwarp();
+                    if (nc >= 32) {
+                        form(cand[lane]);
+                        const int rest = lane < nc - 32 ? cand[32 + lane] : 0;
+                        __syncwarp();
+                        cand[lane] = rest;
+                        nc -= 32;
+                        __syncwarp();
+                    }
                 }
+                if (lane < nc) form(cand[lane]);
                 __syncwarp();
                 nz = 0;
                 for (int q = lane; q < g.WM; q += 32) nz |= par[q];
@@ -1559,18 +1589,18 @@ __global__ void k_screen(DevGraph g, DecCfg cfg, Work w, int more)
 // those end here, after about 300 columns each way instead of two passes over
 // 35110 edges.
 constexpr int kScreen2Cols = 1024;       // columns next to flipped detectors, and
-constexpr int kScreen2Cand = 512;        // columns that may flip at t = 2, of one shot
+constexpr int kScreen2Cand = 512;        // columns to form at t = 2 (some of them more than once), of one shot
 
 __host__ __device__ inline size_t screen2_warp_words(const DevGraph& g)
 {
-    return (size_t)g.WN + 3 * (size_t)g.WM + 2 * (size_t)kMaxFlip + (kScreen2Cols + kScreen2Cand) / 2 +
+    return (size_t)g.WN + 3 * (size_t)g.WM + 3 * (size_t)kMaxFlip + (kScreen2Cols + kScreen2Cand) / 2 +
            2 * (size_t)g.M;
 }
 
-// the set rows of a bit set: each one's first edge (first) and its edges'
-// offset (off) in the list of all their edges; returns the rows, *tot = the
-// edges (nothing is listed when there are more than kMaxFlip)
-__device__ inline int list_rows(const DevGraph& g, const uint32_t* bits, int* first, int* off, int* tot)
+// the set rows of a bit set (rows): each one's first edge (first) and its
+// edges' offset (off) in the list of all their edges; returns their number,
+// *tot = the edges (nothing is listed when there are more than kMaxFlip)
+__device__ inline int list_rows(const DevGraph& g, const uint32_t* bits, int* rows, int* first, int* off, int* tot)
 {
     const int lane = threadIdx.x & 31;
     int n = 0;
@@ -1586,7 +1616,7 @@ __device__ inline int list_rows(const DevGraph& g, const uint32_t* bits, int* fi
         }
         int k = n + incl - c;
         if (k + c <= kMaxFlip) {
-            for (uint32_t w2 = word; w2 != 0u; w2 &= w2 - 1u) first[k++] = 32 * q + __ffs(w2) - 1;
+            for (uint32_t w2 = word; w2 != 0u; w2 &= w2 - 1u) rows[k++] = 32 * q + __ffs(w2) - 1;
         }
         n += __shfl_sync(FULLMASK, incl, 31);
     }
@@ -1597,7 +1627,7 @@ __device__ inline int list_rows(const DevGraph& g, const uint32_t* bits, int* fi
         const int k = k0 + lane;
         int rb = 0, d = 0;
         if (k < n) {
-            const int i = first[k];
+            const int i = rows[k];
             rb = __ldg(g.row_ptr + i);
             d = __ldg(g.row_ptr + i + 1) - rb;
         }
@@ -1617,13 +1647,17 @@ __device__ inline int list_rows(const DevGraph& g, const uint32_t* bits, int* fi
     return n;
 }
 
-// the columns on the listed rows' edges that `seen` does not hold yet, appended
-// to list[cap]; returns the list's length, above cap when it overflows
-__device__ inline int list_columns(const DevGraph& g, const int* first, const int* off, int n, int tot,
-                                   uint32_t* seen, uint16_t* list, int len, int cap)
+// the columns on the listed rows' edges, appended to list[cap]: those `seen` does
+// not hold yet, or with m2 (the rows' second smallest magnitudes at m2[2 i + 1])
+// those it holds and those whose Lambda_j one negative message of the row could
+// bring to 0; returns the list's length, above cap when it overflows
+template <bool kBound>
+__device__ inline int list_columns(const DevGraph& g, const int* rows, const int* first, const int* off, int n, int tot,
+                                   uint32_t* seen, uint16_t* list, int len, int cap, const uint32_t* m2, float alpha)
 {
     const int lane = threadIdx.x & 31;
-    for (int t0 = 0; t0 < tot && len <= cap; t0 += 32) {
+#pragma unroll 2
+    for (int t0 = 0; t0 < tot; t0 += 32) {
         const int t = t0 + lane;
         bool add = false;
         int j = 0;
@@ -1635,7 +1669,11 @@ __device__ inline int list_columns(const DevGraph& g, const int* first, const in
             }
             j = __ldg(g.row_col + first[lo] + (t - off[lo]));
             const uint32_t bit = 1u << (j & 31);
-            add = !(atomicOr(&seen[j >> 5], bit) & bit);
+            const bool had = atomicOr(&seen[j >> 5], bit) & bit;
+            if (kBound)
+                add = had || !(__fsub_rn(__ldg(g.lam + j), __fmul_rn(alpha, __uint_as_float(m2[2 * rows[lo] + 1]))) > 0.f);
+            else
+                add = !had;
         }
         const uint32_t bal = __ballot_sync(FULLMASK, add);
         const int at = len + __popc(bal & ((1u << lane) - 1u));
@@ -1647,18 +1685,29 @@ __device__ inline int list_columns(const DevGraph& g, const int* first, const in
 }
 
 // E_{j->i}(1) of column j in the storage format's values: v[k] on row rr[k],
-// k < the column's degree (returned)
+// k < the column's degree (returned); its table entry is loaded ahead
+template <int KD>
+struct ColumnIn {
+    float4 q[KD / 2];
+    float lam;
+};
+template <int KD>
+__device__ __forceinline__ void load_column(const DevGraph& g, int j, ColumnIn<KD>& in)
+{
+#pragma unroll
+    for (int h = 0; h < KD / 2; ++h) in.q[h] = __ldg(g.colRD + (size_t)j * (KD / 2) + h);
+    in.lam = __ldg(g.lam + j);
+}
 template <int KD, int P>
-__device__ __forceinline__ int column_E1(const DevGraph& g, const uint32_t* sp, int j, float L, float (&v)[KD],
+__device__ __forceinline__ int column_E1(const ColumnIn<KD>& in, const uint32_t* sp, float L, float (&v)[KD],
                                          int (&rr)[KD])
 {
     using S = Store<P>;
-    const float4* cr = g.colRD + (size_t)j * (KD / 2);
     float d[KD];
     int deg = 0;
 #pragma unroll
     for (int h = 0; h < KD / 2; ++h) {
-        const float4 q = __ldg(cr + h);
+        const float4 q = in.q[h];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int r = __float_as_int(u ? q.w : q.y);
@@ -1679,7 +1728,7 @@ __device__ __forceinline__ int column_E1(const DevGraph& g, const uint32_t* sp, 
             }
         }
     }
-    const float lj = __ldg(g.lam + j);
+    const float lj = in.lam;
 #pragma unroll
     for (int k = 0; k < KD; ++k) {                            // Eq. 2: leave d_i out
         float acc = lj;
@@ -1694,7 +1743,7 @@ __device__ __forceinline__ int column_E1(const DevGraph& g, const uint32_t* sp, 
 }
 
 template <int DV, int P>
-__global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCfg cfg, Work w)
+__global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCfg cfg, Work w, int min_queue)
 {
     extern __shared__ __align__(16) uint32_t ssm[];
     constexpr int KD = DV == 3 ? 4 : DV;
@@ -1705,7 +1754,8 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
     uint32_t* sp = bits + g.WN;
     uint32_t* pr = sp + g.WM;                                        // P_i
     uint32_t* par = pr + g.WM;                                       // s xor H e^(2)
-    int* first = reinterpret_cast<int*>(par + g.WM);
+    int* rows = reinterpret_cast<int*>(par + g.WM);
+    int* first = rows + kMaxFlip;
     int* off = first + kMaxFlip;
     uint16_t* cols = reinterpret_cast<uint16_t*>(off + kMaxFlip);
     uint16_t* cand = cols + kScreen2Cols;
@@ -1713,6 +1763,13 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
     const RunDesc* dp = w.desc;
     const int nq = *((volatile int*)&w.ctr->n_queue1);
     const int nw = gridDim.x * kScreenWarps;
+    // few shots: a warp here takes longer over one than the seed kernel's
+    // candidate group over two iterations, and the groups are free
+    if (nq < min_queue) {
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nq; k += gridDim.x * blockDim.x) w.queue[k] = w.queue1[k];
+        if (blockIdx.x == 0 && threadIdx.x == 0) w.ctr->n_queue = nq;
+        return;
+    }
     const float L = cfg.L;
     unsigned long long upd = 0;                                      // message updates formed (lane)
     unsigned long long ended = 0;
@@ -1725,13 +1782,15 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
         __syncwarp();
         bool conv = false;
         int tot;
-        const int nflip = list_rows(g, sp, first, off, &tot);
-        const int nc = nflip <= kMaxFlip ? list_columns(g, first, off, nflip, tot, bits, cols, 0, kScreen2Cols)
+        const int nflip = list_rows(g, sp, rows, first, off, &tot);
+        const int nc = nflip <= kMaxFlip ? list_columns<false>(g, rows, first, off, nflip, tot, bits, cols, 0,
+                                                               kScreen2Cols, nullptr, 0.f)
                                          : kScreen2Cols + 1;
         if (nc <= kScreen2Cols) {
-            // the records of E0(1) over the other columns: the first two of the
-            // row's four smallest; a row that has fewer (more than two of the
-            // four are next to flipped detectors) is read whole
+            // the records of E0(1) over the other columns: none on a flipped
+            // row, whose columns are all listed; else the first two of the row's
+            // four smallest, and a row that has fewer (more than two of the four
+            // are next to flipped detectors) is read whole
 #pragma unroll 4
             for (int i = lane; i < g.M; i += 32) {
                 const float4 a0 = __ldg(g.row4 + 2 * i), a1 = __ldg(g.row4 + 2 * i + 1);
@@ -1749,7 +1808,9 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
                         ++n;
                     }
                 }
-                if (n < 2) {
+                if ((sp[i >> 5] >> (i & 31)) & 1u) {
+                    m1 = m2 = L;
+                } else if (n < 2) {
                     m1 = m2 = L;
                     for (int e = __ldg(g.row_ptr + i); e < __ldg(g.row_ptr + i + 1); ++e) {
                         const int j = __ldg(g.row_col + e);
@@ -1767,22 +1828,28 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
             __syncwarp();
             // the messages of the columns next to flipped detectors; the larger
             // of a message and the minimum it meets goes on to the second one,
-            // which in the end is the least of all but the minimum
+            // which in the end is the least of all but the minimum (and one that
+            // is not below the second one now never changes either)
             int ncand = 0;
+            ColumnIn<KD> in, next;
+            int j = lane < nc ? cols[lane] : 0;
+            load_column<KD>(g, j, in);
             for (int t0 = 0; t0 < nc; t0 += 32) {
                 bool neg = false;
-                int j = 0;
+                const int jn = t0 + 32 + lane < nc ? cols[t0 + 32 + lane] : 0;
+                load_column<KD>(g, jn, next);
                 if (t0 + lane < nc) {
-                    j = cols[t0 + lane];
                     float v[KD];
                     int rr[KD];
-                    const int deg = column_E1<KD, P>(g, sp, j, L, v, rr);
+                    const int deg = column_E1<KD, P>(in, sp, L, v, rr);
 #pragma unroll
                     for (int k = 0; k < KD; ++k) {
                         if (k < deg) {
                             const uint32_t a = __float_as_uint(fabsf(v[k]));
-                            const uint32_t old = atomicMin(&rec[2 * rr[k]], a);
-                            atomicMin(&rec[2 * rr[k] + 1], old > a ? old : a);
+                            if (a < *((volatile uint32_t*)&rec[2 * rr[k] + 1])) {
+                                const uint32_t old = atomicMin(&rec[2 * rr[k]], a);
+                                atomicMin(&rec[2 * rr[k] + 1], old > a ? old : a);
+                            }
                             if (v[k] < 0.f) {
                                 neg = true;
                                 atomicXor(&pr[rr[k] >> 5], 1u << (rr[k] & 31));
@@ -1798,11 +1865,14 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
                     if (at < kScreen2Cand) cand[at] = (uint16_t)j;
                 }
                 ncand += __popc(bal);
+                in = next;
+                j = jn;
             }
             __syncwarp();
             if (ncand <= kScreen2Cand) {
-                const int nodd = list_rows(g, pr, first, off, &tot);
-                ncand = nodd <= kMaxFlip ? list_columns(g, first, off, nodd, tot, bits, cand, ncand, kScreen2Cand)
+                const int nodd = list_rows(g, pr, rows, first, off, &tot);
+                ncand = nodd <= kMaxFlip ? list_columns<true>(g, rows, first, off, nodd, tot, bits, cand, ncand,
+                                                              kScreen2Cand, rec, cfg.alpha)
                                          : kScreen2Cand + 1;
             }
             if (ncand <= kScreen2Cand) {
@@ -1812,7 +1882,9 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
                     const int j = cand[t];
                     float v[KD];
                     int rr[KD];
-                    const int deg = column_E1<KD, P>(g, sp, j, L, v, rr);
+                    ColumnIn<KD> in;
+                    load_column<KD>(g, j, in);
+                    const int deg = column_E1<KD, P>(in, sp, L, v, rr);
 #pragma unroll
                     for (int k = 0; k < KD; ++k) {            // Eq. 1
                         if (k < deg) {
@@ -1832,13 +1904,13 @@ __global__ void __launch_bounds__(32 * kScreenWarps) k_screen2(DevGraph g, DecCf
                             if (v[k] > v[k + 1]) { const float tv = v[k]; v[k] = v[k + 1]; v[k + 1] = tv; }
                         }
                     }
-                    float post = __ldg(g.lam + j);            // Eq. 3 in ascending order
+                    float post = in.lam;                      // Eq. 3 in ascending order
 #pragma unroll
                     for (int k = 0; k < KD; ++k)
                         if (k < deg) post = __fadd_rn(post, v[k]);
                     upd += (unsigned long long)deg;
-                    if (post <= 0.f) {                        // Eq. 4
-                        atomicOr(&bits[j >> 5], 1u << (j & 31));
+                    const uint32_t bit = 1u << (j & 31);
+                    if (post <= 0.f && !(atomicOr(&bits[j >> 5], bit) & bit)) {   // Eq. 4
 #pragma unroll
                         for (int k = 0; k < KD; ++k)
                             if (k < deg) atomicXor(&par[rr[k] >> 5], 1u << (rr[k] & 31));
@@ -2176,19 +2248,32 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
     } else {
         // results collection in visit order (dedupe by equality, App. B)
         unsigned long long sum = 0;
+        int nres = __ldcg(w.res_n + a);
         for (int c = 0; c < nch && !done; ++c) {
             const int fl = sc->flags[c];
             if (!(fl & 1)) continue;
             sum += (unsigned long long)sc->iters[c];
             if (!(fl & 2)) continue;
             const uint32_t* eb = w.slotBits + slot_index(w, cb, a, c, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
-            const int nres = __ldcg(w.res_n + a);
             bool dup = false;
-            for (int q = 0; q < nres && !dup; ++q) {
-                const uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + q) * g.WN;
-                bool eq = true;
-                for (int x = lane; x < g.WN; x += 32) eq = eq && (__ldcg(rb + x) == __ldcg(eb + x));
-                dup = __all_sync(FULLMASK, eq);
+            if (g.WN <= 32) {
+                // a stored result per lane (one memory round trip per success
+                // instead of one per stored result)
+                bool same = false;
+                for (int q = lane; q < nres; q += 32) {
+                    const uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + q) * g.WN;
+                    uint32_t diff = 0u;
+                    for (int x = 0; x < g.WN; ++x) diff |= __ldcg(rb + x) ^ __ldcg(eb + x);
+                    same = same || diff == 0u;
+                }
+                dup = __any_sync(FULLMASK, same);
+            } else {
+                for (int q = 0; q < nres && !dup; ++q) {
+                    const uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + q) * g.WN;
+                    bool eq = true;
+                    for (int x = lane; x < g.WN; x += 32) eq = eq && (__ldcg(rb + x) == __ldcg(eb + x));
+                    dup = __all_sync(FULLMASK, eq);
+                }
             }
             if (!dup) {
                 uint32_t* rb = w.res_bits + ((size_t)a * cfg.num_results + nres) * g.WN;
@@ -2201,7 +2286,7 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
                     w.res_n[a] = nres + 1;
                 }
                 __syncwarp();
-                if (nres + 1 >= cfg.num_results) {
+                if (++nres >= cfg.num_results) {
                     near |= near_upto(c);
                     finalize_results(g, cfg, w, d.out, a, gb, acc + sum, near ? ST_NEAR : 0u);
                     done = true;
@@ -2549,6 +2634,12 @@ static int occupancy(int threads, size_t smem_bp, int* bps)
     return 0;
 }
 
+// the second screen runs on at least this many shots: two for every candidate
+// group of the seed kernel
+static int screen2_min_queue(const LaunchShape& ls)
+{
+    return 2 * ls.grid_seed * (ls.group_warps >= 2 ? 1 : ls.warps_per_block);
+}
 static void* screen2_func(int dv, int prec)
 {
     if (dv == 0)
@@ -2711,12 +2802,13 @@ static int launch_chunk_t(const DevGraph& g, const DecCfg& cfg, const Work& w, c
         DevGraph gg = g;
         DecCfg cc = cfg;
         Work ww = w;
-        int more = ls.grid_screen2 > 0;
+        int more = ls.grid_screen2 > 0, min_queue = screen2_min_queue(ls);
         void* cargs[] = {&gg, &cc, &ww, &more};
+        void* margs[] = {&gg, &cc, &ww, &min_queue};
         if (CUDA_FAILED(cudaLaunchKernel(screen_func(ls), dim3((unsigned)ls.grid_screen), dim3(32 * kScreenWarps),
                                          cargs, ls.smem_screen, s)) ||
             (more && CUDA_FAILED(cudaLaunchKernel(screen2_func(ls.dv_screen, g.prec), dim3((unsigned)ls.grid_screen2),
-                                                  dim3(32 * kScreenWarps), cargs, ls.smem_screen2, s))))
+                                                  dim3(32 * kScreenWarps), margs, ls.smem_screen2, s))))
             return -2;
         if (hk) hk->after(hk->ctx, 11);
     }
@@ -2848,15 +2940,16 @@ static int build_graph_t(const DevGraph& g0, const DecCfg& cfg0, const Work& w0,
     const bool batched = ls.batch && w.bs_slots > 0;
     int screened = batched ? 2 : ls.screen;
     void* sargs[] = {&g, &cfg, &w, &screened};
-    int more = ls.grid_screen2 > 0;
+    int more = ls.grid_screen2 > 0, min_queue = screen2_min_queue(ls);
     void* cargs[] = {&g, &cfg, &w, &more};
+    void* margs[] = {&g, &cfg, &w, &min_queue};
     if (ls.screen)
         rc = add_kernel(graph, &scr, nullptr, screen_func(ls), ls.grid_screen, 32 * kScreenWarps, ls.smem_screen,
                         cargs);
     if (ls.screen && more && !rc) {
         cudaGraphNode_t scr1 = scr;
         rc = add_kernel(graph, &scr, &scr1, screen2_func(ls.dv_screen, g.prec), ls.grid_screen2, 32 * kScreenWarps,
-                        ls.smem_screen2, cargs);
+                        ls.smem_screen2, margs);
     }
     // WHILE (shots handed on remain) { window start, the seed kernel on at most
     // S of them, the beam, window end } after `dep`

@@ -331,9 +331,12 @@ bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int co
         per_sweep += d * (d - 1) / 2;
     }
     const int max_sweeps = (int)std::min<double>(kSweeps, 5e7 / per_sweep);
+    // (a given order starts close to what the search reaches: it ends at the
+    // first sweep that takes off less than a tenth)
     int best = ex, stale = 0;
-    for (int sw = 0; sw < max_sweeps && ex > 0 && stale < kPatience; ++sw) {
-        if (ex < best) { best = ex; stale = 0; } else if (sw > 0) { ++stale; }
+    for (int sw = 0; sw < max_sweeps && ex > 0 && stale < (start ? 1 : kPatience); ++sw) {
+        if (ex < (start && sw > 0 ? 0.9 * best : best)) { best = ex; stale = 0; } else if (sw > 0) { ++stale; }
+        if (start && stale) break;
         for (int i = M - 1; i > 0; --i) std::swap(order[i], order[rng.below((uint32_t)i + 1)]);
         for (int i : order) {
             for (int a = row_ptr[i]; a < row_ptr[i + 1]; ++a) {

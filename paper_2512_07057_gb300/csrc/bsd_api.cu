@@ -464,12 +464,12 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
         jD0.assign((size_t)(E > 0 ? E : 1), 0.f);
         for (long long e = 0; e < E; ++e) jD0[jpos[e]] = D0[e];
     }
-    // the columns' words in a tile of the unrolled decoder's on-chip path
+    // the places of the columns' edges in a tile of the unrolled decoder's on-chip path
     const int tcap = max_col <= 4 ? 4 : max_col <= 8 ? 8 : 0;
-    std::vector<int> tile_word((size_t)tcap * N, -1);
-    for (int j = 0; j < N && tcap > 0; ++j)
+    std::vector<uint16_t> tile_slots(E <= 65528 ? (size_t)tcap * N : 0, 0xffffu);
+    for (int j = 0; j < N && !tile_slots.empty(); ++j)
         for (int k = 0; k < col_ptr[j + 1] - col_ptr[j]; ++k)
-            tile_word[(size_t)tcap * j + k] = kTileShots * tile_slot(col_edge[col_ptr[j] + k]);
+            tile_slots[(size_t)tcap * j + k] = (uint16_t)tile_slot(col_edge[col_ptr[j] + k]);
     // E(0) of column j in the storage format (every edge of the column holds it)
     std::vector<unsigned char> lamEc_st((size_t)Npad * msg_bytes, 0);
     for (int j = 0; j < N; ++j) {
@@ -608,7 +608,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     gb += align256(sizeof(long long) * N);
     gb += align256(sizeof(float4) * M);
     gb += align256(sizeof(float) * Epad);
-    gb += align256(sizeof(int) * tile_word.size());
+    gb += align256(sizeof(uint16_t) * tile_slots.size());
     gb += align256(sizeof(int) * colW.size()) + align256(colG.size()) + align256(sizeof(int2) * rowQ.size()) +
           align256(sizeof(int) * jplanes.size()) + align256(sizeof(float) * jD0.size());
     gb += align256(lamEc_st.size());
@@ -646,7 +646,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     long long* d_lamq = carve<long long>(p, N);
     float4* d_rs0 = carve<float4>(p, M);
     float* d_D0 = carve<float>(p, Epad);
-    int* d_tile_word = tile_word.empty() ? nullptr : carve<int>(p, tile_word.size());
+    uint16_t* d_tile_slots = tile_slots.empty() ? nullptr : carve<uint16_t>(p, tile_slots.size());
     int* d_colW = colW.empty() ? nullptr : carve<int>(p, colW.size());
     uint8_t* d_colG = colG.empty() ? nullptr : carve<uint8_t>(p, colG.size());
     int2* d_rowQ = rowQ.empty() ? nullptr : carve<int2>(p, rowQ.size());
@@ -675,8 +675,8 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
               !CUDA_FAILED(cudaMemcpy(d_lamq, lamq.data(), sizeof(long long) * N, cudaMemcpyHostToDevice)) &&
               !CUDA_FAILED(cudaMemcpy(d_rs0, rs0.data(), sizeof(float4) * M, cudaMemcpyHostToDevice)) &&
               !CUDA_FAILED(cudaMemcpy(d_D0, D0.data(), sizeof(float) * Epad, cudaMemcpyHostToDevice)) &&
-              (tile_word.empty() ||
-               !CUDA_FAILED(cudaMemcpy(d_tile_word, tile_word.data(), sizeof(int) * tile_word.size(), cudaMemcpyHostToDevice))) &&
+              (tile_slots.empty() ||
+               !CUDA_FAILED(cudaMemcpy(d_tile_slots, tile_slots.data(), sizeof(uint16_t) * tile_slots.size(), cudaMemcpyHostToDevice))) &&
               (colW.empty() ||
                (!CUDA_FAILED(cudaMemcpy(d_colW, colW.data(), sizeof(int) * colW.size(), cudaMemcpyHostToDevice)) &&
                 !CUDA_FAILED(cudaMemcpy(d_colG, colG.data(), colG.size(), cudaMemcpyHostToDevice)) &&
@@ -710,7 +710,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     g.all_lam_pos = all_pos;
     g.row_ptr = d_row_ptr; g.row_col = d_row_col; g.col_ptr = d_col_ptr; g.col_edge = d_col_edge; g.col_row = d_col_row;
     g.lam = d_lam; g.lamE = d_lamE; g.hcol = d_hcol; g.acol = d_acol; g.lamq = d_lamq; g.rs0 = d_rs0; g.D0 = d_D0;
-    g.tile_word = reinterpret_cast<const int4*>(d_tile_word);
+    g.tile_slots = reinterpret_cast<const uint2*>(d_tile_slots);
     g.colW = d_colW; g.colK = colK; g.colG = d_colG; g.rowQ = d_rowQ; g.jplanes = d_jplanes; g.jD0 = d_jD0;
     for (int k = 0; k < kJaggedPlanes; ++k) g.jplane[k] = k < (int)jplanes.size() ? jplanes[k] : 0;
     g.lamEc = d_lamEc;

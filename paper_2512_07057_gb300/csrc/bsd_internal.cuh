@@ -76,8 +76,8 @@ struct DevGraph {
     const int* jplanes;    // [max_row_deg]
     int jplane[16];
     const float* jD0;      // [E] D0 at those words
-    const int4* tile_word; // [N][1 or 2] kTileShots * tile_slot of the column's edges, -1 past its degree
-                           // (one int4 for column degrees up to 4, two up to 8; null above)
+    const uint2* tile_slots;  // [N][1 or 2] tile_slot of the column's edges, 16 bits each, 0xffff past its
+                              // degree (one uint2 for column degrees up to 4, two up to 8; null above)
     const void* lamEc;     // [Npad] E(0) of column j (clamp(Lambda_j)) in the storage format
     // the columns ordered by degree (batched seed BP): colperm[q] is the
     // column at position q, the columns of degree d hold positions

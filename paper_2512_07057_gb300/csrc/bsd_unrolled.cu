@@ -476,7 +476,7 @@ constexpr int kMaxDeg = 8;
 struct TileArgs {
     const int* row_ptr;
     const int* row_col;
-    const int4* col_word;    // [N][CAP / 4]: words of the column's edges (kShots * tile_slot), -1 past its degree
+    const uint2* col_slot;   // [N][CAP / 4]: tile_slot of the column's edges, 16 bits each, 0xffff past its degree
     const float* lam;
     int M, N, E, T;
     float L;
@@ -497,21 +497,31 @@ struct TileArgs {
 __host__ __device__ inline size_t tile_smem(int M, int N, int E)
 {
     const size_t e4 = ((size_t)E + 3) & ~size_t(3);
-    return e4 * kShots * sizeof(float) + (((size_t)M + (size_t)N + 15) & ~size_t(15)) + 2 * 16 * sizeof(float);
+    return e4 * kShots * sizeof(float) + (((size_t)M + (size_t)N + 15) & ~size_t(15)) + 2 * 16 * sizeof(float) +
+           sizeof(uint16_t) * ((size_t)M + 1);
 }
 __device__ __forceinline__ float4* tile_at(float* x, int e, int half)
 {
     return reinterpret_cast<float4*>(x + kShots * tile_slot(e) + 4 * half);
 }
-// the words of a column's edges
+// the places of a column's edges, as they are stored and one by one
 template <int CAP>
-__device__ __forceinline__ void column_words(const TileArgs& a, int j, int (&e)[CAP])
-{
+struct ColumnSlots {
+    uint2 v[CAP / 4];
+    __device__ __forceinline__ void load(const TileArgs& a, int j)
+    {
 #pragma unroll
-    for (int h = 0; h < CAP / 4; ++h) {
-        const int4 v = __ldg(a.col_word + (size_t)j * (CAP / 4) + h);
-        e[4 * h] = v.x; e[4 * h + 1] = v.y; e[4 * h + 2] = v.z; e[4 * h + 3] = v.w;
+        for (int h = 0; h < CAP / 4; ++h) v[h] = __ldg(a.col_slot + (size_t)j * (CAP / 4) + h);
     }
+    __device__ __forceinline__ uint32_t at(int k) const
+    {
+        const uint32_t w = (k & 2) ? v[k / 4].y : v[k / 4].x;
+        return (k & 1) ? w >> 16 : w & 0xffffu;
+    }
+};
+__device__ __forceinline__ float4* slot_at(float* x, uint32_t slot, int half)
+{
+    return reinterpret_cast<float4*>(x + kShots * slot + 4 * half);
 }
 // signed minimum of two messages: the magnitude's minimum with the product's sign
 __device__ __forceinline__ float xmin(float a, float b)
@@ -564,6 +574,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const
     unsigned char* const sb = reinterpret_cast<unsigned char*>(sm + (((size_t)a.E + 3) & ~size_t(3)) * kShots);
     unsigned char* const yb = sb + a.M;
     float* const red = reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15)));   // [2][16]
+    uint16_t* const rp = reinterpret_cast<uint16_t*>(red + 32);                                           // row_ptr
+    for (int q = threadIdx.x; q <= a.M; q += blockDim.x) rp[q] = (uint16_t)__ldg(a.row_ptr + q);
     const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
         const long long b0 = (long long)tile * kShots;
@@ -588,12 +600,21 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const
         for (int t = 1; t <= a.T; ++t) {
             const float* wt = a.w + (size_t)(t - 1) * (size_t)a.E;
             const size_t rec = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.M * kShots;
+            // (each task's table entries are loaded while the one before runs)
+            float wn[kMaxDeg];
+            if ((int)threadIdx.x < 2 * a.M)
+                row_weights(wt, rp[threadIdx.x >> 1], rp[(threadIdx.x >> 1) + 1] - rp[threadIdx.x >> 1], wn);
             for (int q = threadIdx.x; q < 2 * a.M; q += blockDim.x) {
                 const int i = q >> 1, half = q & 1;
-                const int rb = __ldg(a.row_ptr + i), deg = __ldg(a.row_ptr + i + 1) - rb;
+                const int rb = rp[i], deg = rp[i + 1] - rb;
                 const uint32_t s4 = (uint32_t)sb[i] >> (4 * half);
                 float wv[kMaxDeg];
-                row_weights(wt, rb, deg, wv);
+#pragma unroll
+                for (int k = 0; k < kMaxDeg; ++k) wv[k] = wn[k];
+                if (q + (int)blockDim.x < 2 * a.M) {
+                    const int in = (q + (int)blockDim.x) >> 1;
+                    row_weights(wt, rp[in], rp[in + 1] - rp[in], wn);
+                }
                 float4 v[kMaxDeg];
 #pragma unroll
                 for (int k = 0; k < kMaxDeg; ++k)
@@ -653,17 +674,26 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const
             __syncthreads();
             float loss = 0.f;
             const size_t nod = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.N * kShots;
+            ColumnSlots<CAP> en;
+            float ln = 0.f;
+            if ((int)threadIdx.x < 2 * a.N) {
+                en.load(a, threadIdx.x >> 1);
+                ln = __ldg(a.lam + (threadIdx.x >> 1));
+            }
             for (int q = threadIdx.x; q < 2 * a.N; q += blockDim.x) {
                 const int j = q >> 1, half = q & 1;
-                int e[CAP];
-                column_words<CAP>(a, j, e);
-                const float lj = __ldg(a.lam + j);
+                const ColumnSlots<CAP> e = en;
+                const float lj = ln;
+                if (q + (int)blockDim.x < 2 * a.N) {
+                    en.load(a, (q + (int)blockDim.x) >> 1);
+                    ln = __ldg(a.lam + ((q + (int)blockDim.x) >> 1));
+                }
                 float4 post = make_float4(lj, lj, lj, lj);
                 float4 v[CAP];
 #pragma unroll
                 for (int k = 0; k < CAP; ++k) {
-                    if (e[k] >= 0) {
-                        v[k] = *reinterpret_cast<const float4*>(x + e[k] + 4 * half);
+                    if (e.at(k) != 0xffffu) {
+                        v[k] = *slot_at(x, e.at(k), half);
                         post.x = __fadd_rn(post.x, v[k].x);
                         post.y = __fadd_rn(post.y, v[k].y);
                         post.z = __fadd_rn(post.z, v[k].z);
@@ -673,8 +703,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const
                 // (unclamped: the row pass caps the magnitudes at L_MAX)
 #pragma unroll
                 for (int k = 0; k < CAP; ++k) {
-                    if (e[k] >= 0)
-                        *reinterpret_cast<float4*>(x + e[k] + 4 * half) =
+                    if (e.at(k) != 0xffffu)
+                        *slot_at(x, e.at(k), half) =
                             make_float4(__fsub_rn(post.x, v[k].x), __fsub_rn(post.y, v[k].y),
                                         __fsub_rn(post.z, v[k].z), __fsub_rn(post.w, v[k].w));
                 }
@@ -710,6 +740,9 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_backward(TileArgs a, cons
     float* const x = sm;
     unsigned char* const sb = reinterpret_cast<unsigned char*>(sm + (((size_t)a.E + 3) & ~size_t(3)) * kShots);
     unsigned char* const yb = sb + a.M;
+    uint16_t* const rp = reinterpret_cast<uint16_t*>(
+        reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15))) + 32);                // row_ptr
+    for (int q = threadIdx.x; q <= a.M; q += blockDim.x) rp[q] = (uint16_t)__ldg(a.row_ptr + q);
     float* const part = a.gw_part + (size_t)blockIdx.x * (size_t)a.T * (size_t)a.E;
     for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
         const bool fresh = tile == (int)blockIdx.x;
@@ -722,11 +755,22 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_backward(TileArgs a, cons
             // through the total ([0]) and through the term itself ([t])
             const float gs = (float)(((double)__ldg(gout) + (double)__ldg(gout + t)) * scale);
             const size_t nod = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.N * kShots;
+            // (each task's loads are issued while the one before runs; a task's
+            // Lambda lies at nod + 4 q)
+            ColumnSlots<CAP> en;
+            float4 pn = make_float4(0.f, 0.f, 0.f, 0.f);
+            if ((int)threadIdx.x < 2 * a.N) {
+                en.load(a, threadIdx.x >> 1);
+                pn = __ldg(reinterpret_cast<const float4*>(a.lamT + nod) + threadIdx.x);
+            }
             for (int q = threadIdx.x; q < 2 * a.N; q += blockDim.x) {
                 const int j = q >> 1, half = q & 1;
-                int e[CAP];
-                column_words<CAP>(a, j, e);
-                const float4 post = __ldg(reinterpret_cast<const float4*>(a.lamT + nod + (size_t)j * kShots + 4 * half));
+                const ColumnSlots<CAP> e = en;
+                const float4 post = pn;
+                if (q + (int)blockDim.x < 2 * a.N) {
+                    en.load(a, (q + (int)blockDim.x) >> 1);
+                    pn = __ldg(reinterpret_cast<const float4*>(a.lamT + nod) + q + blockDim.x);
+                }
                 const uint32_t y4 = (uint32_t)yb[j] >> (4 * half);
                 const long long b = b0 + 4 * half;
                 float4 gl;
@@ -742,29 +786,37 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_backward(TileArgs a, cons
 #pragma unroll
                 for (int k = 0; k < CAP; ++k) {
                     g[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (t < a.T && e[k] >= 0) {
-                        g[k] = *reinterpret_cast<const float4*>(x + e[k] + 4 * half);
+                    if (t < a.T && e.at(k) != 0xffffu) {
+                        g[k] = *slot_at(x, e.at(k), half);
                         gl.x += g[k].x; gl.y += g[k].y; gl.z += g[k].z; gl.w += g[k].w;
                     }
                 }
 #pragma unroll
                 for (int k = 0; k < CAP; ++k)
-                    if (e[k] >= 0)
-                        *reinterpret_cast<float4*>(x + e[k] + 4 * half) =
+                    if (e.at(k) != 0xffffu)
+                        *slot_at(x, e.at(k), half) =
                             make_float4(gl.x - g[k].x, gl.y - g[k].y, gl.z - g[k].z, gl.w - g[k].w);
             }
             __syncthreads();
             const float* wt = a.w + (size_t)(t - 1) * (size_t)a.E;
             float* gwt = part + (size_t)(t - 1) * (size_t)a.E;
             const size_t rec = ((size_t)tile * a.T + (size_t)(t - 1)) * (size_t)a.M * kShots;
+            // (a task's records lie at rec + 4 q)
+            float4 m1n, m2n;
+            uint2 pvn;
+            auto load_record = [&](int q) {
+                m1n = __ldg(reinterpret_cast<const float4*>(a.m1 + rec) + q);
+                m2n = __ldg(reinterpret_cast<const float4*>(a.m2 + rec) + q);
+                pvn = __ldg(reinterpret_cast<const uint2*>(a.pk + rec) + q);
+            };
+            load_record((int)threadIdx.x < 2 * a.M ? (int)threadIdx.x : 0);
             for (int q = threadIdx.x; q < ((2 * a.M + 31) & ~31); q += blockDim.x) {
                 const bool in = q < 2 * a.M;
                 const int i = in ? q >> 1 : 0, half = q & 1;
-                const int rb = __ldg(a.row_ptr + i), deg = in ? __ldg(a.row_ptr + i + 1) - rb : 0;
-                const size_t at = rec + (size_t)i * kShots + 4 * half;
-                const float4 m1v = __ldg(reinterpret_cast<const float4*>(a.m1 + at));
-                const float4 m2v = __ldg(reinterpret_cast<const float4*>(a.m2 + at));
-                const uint2 pv = __ldg(reinterpret_cast<const uint2*>(a.pk + at));
+                const int rb = rp[i], deg = in ? rp[i + 1] - rb : 0;
+                const float4 m1v = m1n, m2v = m2n;
+                const uint2 pv = pvn;
+                if (q + (int)blockDim.x < 2 * a.M) load_record(q + (int)blockDim.x);
                 const uint32_t s4 = (uint32_t)sb[i] >> (4 * half);
                 uint32_t neg[4], sig[4];
                 int i1[4], i2[4];
@@ -847,14 +899,14 @@ __global__ void k_u_gw_blocks(const float* __restrict__ part, long long n, int b
 bool tile_plan(const DevGraph& g, const DecCfg& cfg, int device, long long B, int T, const float* w, char* base,
                size_t have, TileArgs* out)
 {
-    if (g.max_row_deg > kMaxDeg || g.tile_word == nullptr || g.max_row_deg < 1) return false;
+    if (g.max_row_deg > kMaxDeg || g.tile_slots == nullptr || g.E > 65528 || g.max_row_deg < 1) return false;
     const size_t smem = tile_smem(g.M, g.N, g.E);
     int optin = 0, sms = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || smem > (size_t)optin)
         return false;
     TileArgs a{};
-    a.row_ptr = g.row_ptr; a.row_col = g.row_col; a.col_word = g.tile_word; a.lam = g.lam;
+    a.row_ptr = g.row_ptr; a.row_col = g.row_col; a.col_slot = g.tile_slots; a.lam = g.lam;
     a.M = g.M; a.N = g.N; a.E = g.E; a.T = T; a.L = cfg.L; a.B = B; a.w = w;
     a.ntile = (int)((B + kShots - 1) / kShots);
     // a thread per four shots of a row or of two columns, at most kTileThreads;

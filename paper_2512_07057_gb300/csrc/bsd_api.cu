@@ -57,9 +57,7 @@ struct bsd_decoder {
     long long rr_cap = 0;                    // capacity of the flagged list
     float* weights_mem = nullptr;            // [wT][Epad] weights of weighted min-sum (bsd_set_weights),
                                              // then the same at the single-warp engine's words
-    int small_excess = -1;                   // single-warp placement: bank loads above three left (-1: none)
-    int small_extent = 0;                    // words it spans
-    std::vector<int> small_addr;             // its word of every CSR edge
+    std::vector<int> small_addr;             // the single-warp placement's word of every CSR edge
     std::vector<int> generic_pos;            // the generic engines' word of every CSR edge (empty: CSR order)
     // the single-syndrome request loop (bsd_serve_*)
     ServeBox* serve_h = nullptr;             // mailbox, host-mapped (null when not serving)
@@ -312,8 +310,8 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     const int WM = words_of(M), WN = words_of(N), WK = words_of(K);
     // the single-warp engine's placement of the messages, for the codes it
     // can run (at most 5 words of columns, 3 of rows); Epad covers it
-    SmallLayout sl;
-    const bool has_sl = N <= 32 * kSmallMaxCpl && M <= 32 * kSmallMaxRpl && small_layout(M, N, H_row_ptr, H_col_idx, &sl);
+    SmallLocal sl;
+    const bool has_sl = N <= 32 * kSmallMaxCpl && M <= 32 * kSmallMaxRpl && small_local_layout(M, N, H_row_ptr, H_col_idx, &sl);
     int Epad = (int)((E + 7) / 8 * 8);
     if (has_sl) Epad = std::max(Epad, (sl.extent + 7) / 8 * 8);
     const int Npad = (N + 3) / 4 * 4;
@@ -410,8 +408,8 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
         sD0.assign(Epad, 0.f);
         slamE_st.assign((size_t)Epad * msg_bytes, 0);
         for (long long e = 0; e < E; ++e) {
-            sD0[sl.addr[e]] = D0[e];
-            std::memcpy(&slamE_st[(size_t)sl.addr[e] * msg_bytes], &lamE_st[(size_t)e * msg_bytes], msg_bytes);
+            sD0[sl.word[e]] = D0[e];
+            std::memcpy(&slamE_st[(size_t)sl.word[e] * msg_bytes], &lamE_st[(size_t)e * msg_bytes], msg_bytes);
         }
     }
     // the generic engines' column table: (edge, row) of the k-th edge of column
@@ -435,7 +433,7 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
         }
         for (int q = 0; q < M; ++q) rowQ.push_back(make_int2(ord[q], rdeg(ord[q])));
         GenericLayout gl;
-        const bool has_gl = generic_layout(M, N, H_row_ptr, H_col_idx, colK, &gl, start.data());
+        const bool has_gl = generic_layout(M, N, H_row_ptr, H_col_idx, colK, &gl, start.data(), true);
         jpos = has_gl ? gl.pos : start;
         // a group of 32 columns of one degree keeps its edges in the first slots
         colW.assign((size_t)colK * Npad, -1);
@@ -619,14 +617,25 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     gb += align256(sizeof(float) * E1.size()) + align256(sizeof(float) * row4.size());
     // the single-warp engine's rows of H as column sets (the stopping rule's parities)
     std::vector<uint32_t> shrow;
+    std::vector<int4> scol;
+    std::vector<int> sword;
     if (has_sl) {
         shrow.assign((size_t)kSmallRowWords * 32 * WM, 0u);
+        std::vector<int> pos(N, 0);
+        sword.assign((size_t)3 * N, 0);
+        for (int q = 0; q < 32 * WN; ++q) {
+            const int j = sl.col[q];
+            scol.push_back(make_int4(j, sl.slot[3 * (size_t)q], sl.slot[3 * (size_t)q + 1], sl.slot[3 * (size_t)q + 2]));
+            if (j < 0) continue;
+            pos[j] = q;
+            for (int k = 0; k < 3; ++k) sword[3 * (size_t)j + k] = sl.slot[3 * (size_t)q + k];
+        }
         for (int i = 0; i < M; ++i)
             for (int e = H_row_ptr[i]; e < H_row_ptr[i + 1]; ++e)
-                shrow[(size_t)kSmallRowWords * i + H_col_idx[e] / 32] |= 1u << (H_col_idx[e] % 32);
+                shrow[(size_t)kSmallRowWords * i + pos[H_col_idx[e]] / 32] |= 1u << (pos[H_col_idx[e]] % 32);
     }
     if (has_sl) {
-        gb += align256(sizeof(uint32_t) * sl.col.size());
+        gb += align256(sizeof(int4) * scol.size()) + align256(sizeof(int) * sword.size());
         gb += align256(sizeof(float) * sD0.size());
         gb += align256(slamE_st.size());
         gb += align256(sizeof(uint32_t) * shrow.size());
@@ -659,7 +668,8 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     float* d_E1 = E1.empty() ? nullptr : carve<float>(p, E1.size());
     float* d_row4 = row4.empty() ? nullptr : carve<float>(p, row4.size());
     float* d_colRD = colRD.empty() ? nullptr : carve<float>(p, colRD.size());
-    uint32_t* d_scol = has_sl ? carve<uint32_t>(p, sl.col.size()) : nullptr;
+    int4* d_scol = has_sl ? carve<int4>(p, scol.size()) : nullptr;
+    int* d_sword = has_sl ? carve<int>(p, sword.size()) : nullptr;
     float* d_sD0 = has_sl ? carve<float>(p, sD0.size()) : nullptr;
     unsigned char* d_slamE = has_sl ? carve<unsigned char>(p, slamE_st.size()) : nullptr;
     uint32_t* d_shrow = has_sl ? carve<uint32_t>(p, shrow.size()) : nullptr;
@@ -695,7 +705,8 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
               (colRD.empty() ||
                !CUDA_FAILED(cudaMemcpy(d_colRD, colRD.data(), sizeof(float) * colRD.size(), cudaMemcpyHostToDevice))) &&
               (!has_sl ||
-               (!CUDA_FAILED(cudaMemcpy(d_scol, sl.col.data(), sizeof(uint32_t) * sl.col.size(), cudaMemcpyHostToDevice)) &&
+               (!CUDA_FAILED(cudaMemcpy(d_scol, scol.data(), sizeof(int4) * scol.size(), cudaMemcpyHostToDevice)) &&
+                !CUDA_FAILED(cudaMemcpy(d_sword, sword.data(), sizeof(int) * sword.size(), cudaMemcpyHostToDevice)) &&
                 !CUDA_FAILED(cudaMemcpy(d_sD0, sD0.data(), sizeof(float) * sD0.size(), cudaMemcpyHostToDevice)) &&
                 !CUDA_FAILED(cudaMemcpy(d_slamE, slamE_st.data(), slamE_st.size(), cudaMemcpyHostToDevice)) &&
                 !CUDA_FAILED(cudaMemcpy(d_shrow, shrow.data(), sizeof(uint32_t) * shrow.size(), cudaMemcpyHostToDevice))));
@@ -719,12 +730,10 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
     for (int d = 0; d < kMaxColDeg + 2; ++d) { g.dstart[d] = dstart[d]; g.dbase[d] = dbase[d]; }
     g.scrC = d_scrC;
     g.E1 = d_E1; g.row4 = reinterpret_cast<const float4*>(d_row4);
-    g.scol = d_scol; g.sD0 = d_sD0; g.slamE = d_slamE; g.shrow = d_shrow;
+    g.scol = d_scol; g.sword = d_sword; g.sD0 = d_sD0; g.slamE = d_slamE; g.shrow = d_shrow;
     dec->generic_pos = jpos;
     if (has_sl) {
-        dec->small_excess = sl.excess;
-        dec->small_extent = sl.extent;
-        dec->small_addr = sl.addr;
+        dec->small_addr = sl.word;
     }
 
     DecCfg& cfg = dec->cfg;

@@ -98,16 +98,19 @@ struct DevGraph {
     const float* E1;       // [E]
     int dstart[kMaxColDeg + 2];
     int dbase[kMaxColDeg + 2];
-    // the single-warp engine's shared-memory placement of a candidate's
-    // messages (codes with every row of degree 6 and every column of degree
-    // 3; bsd_layout.cu): the pair h of row i at word h small_plane_stride(M)
-    // + 2 i, and scol[3 j + k] = (word << 16) | row for the k-th edge of
-    // column j; sD0 and slamE hold D0 and E(0) at those words (Epad covers
+    // the single-warp engine's placement of a candidate's messages (codes with
+    // every row of degree 6 and every column of degree 3; bsd_layout.cu): the
+    // pair h of row i at word h small_plane_stride(M) + 2 i.  A lane processes
+    // the columns scol[lane + 32 c].x; the words of their edges follow, and in
+    // all but the last group the first one is of the pair 0 of a row of the same
+    // lane, so that message stays in a register.  sword holds the words by
+    // natural column.  sD0 and slamE hold D0 and E(0) at those words (Epad covers
     // the placement)
-    const uint32_t* scol;  // [3 N], null when the code has no such placement
+    const int4* scol;      // [32 WN] (column or -1, three words), null when the code has no such placement
+    const int* sword;      // [3 N]
     const float* sD0;      // [Epad]
     const void* slamE;     // [Epad] in the storage format
-    const uint32_t* shrow; // [32 ceil(M / 32)][kSmallRowWords] with the placement: the columns of row i of H
+    const uint32_t* shrow; // [32 ceil(M / 32)][kSmallRowWords] with the placement: the positions of row i's columns
                            // as a bit set (the stopping rule's parities); zero past M
 };
 
@@ -127,7 +130,17 @@ struct DecCfg {
     int wT;                // iteration t of a BP call uses row min(t, wT) - 1
 };
 
-// the single-warp engine's placement of a code's messages (bsd_layout.cu):
+// the single-warp engine's placement: the column at each of the 32 CPL positions
+// (-1: none), the word of every CSR edge, the three words of each position's column
+// (all but the last group: the register-held one first), the words spanned; false
+// when the code is not of row degree 6 and column degree 3 with ceil(M / 32) =
+// RPL >= 2 and ceil(N / 32) = 2 RPL - 1
+struct SmallLocal {
+    std::vector<int> col, word, slot;
+    int extent, extra;                    // extra: wavefronts that bank conflicts add to the error pass
+};
+bool small_local_layout(int M, int N, const int* row_ptr, const int* col_idx, SmallLocal* out);
+// an earlier placement of the same words, exported for inspection:
 // plane bases A[0..2], the word of every CSR edge, the per-(column, k) table,
 // the words spanned and the bank loads above three the search left (0: both
 // passes conflict-free); false when the code is not of row degree 6 and
@@ -154,7 +167,7 @@ struct GenericLayout {
 constexpr int kGenericLayoutMaxEdges = 1 << 20;
 // (start: the words to permute within each row, null for the storage windows)
 bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, GenericLayout* out,
-                    const int* start = nullptr);
+                    const int* start = nullptr, bool quick = false);
 constexpr int kJaggedPlanes = 16;        // planes whose offsets travel with the kernel parameters
 // the placement's plane stride for codes of M rows (the engine holds
 // ceil(M / 32) rows per lane); every plane spans 2 M <= 64 ceil(M / 32) words

@@ -506,16 +506,18 @@ struct GenericEngine {
 };
 
 // SmallEngine: codes with every column of degree exactly 3, every row of
-// degree exactly RD = 6, N <= 32*CPL, M <= 32*RPL and fewer than 65536 edges
-// -- the bivariate bicycle codes.  A candidate's messages sit at the words of
-// the code's placement (bsd_layout.cu): the pair h of row i at h kPlane + 2 i,
-// so the detector pass moves 32 consecutive pairs per access, and the error
-// pass gathers and scatters through a per-(column, k) word table chosen to
-// put the 32 lanes in 32 distinct banks.  With single-precision storage D is
-// written over E (each word belongs to one row and to one (column, k), so
-// either pass reads its words before it writes them); 16-bit storage keeps D
-// in float beside E.  Each lane keeps its columns' shared-memory addresses,
-// Lambda_j, sum_LLR and its first row's columns in registers.
+// degree exactly RD = 6, N <= 32*CPL, M <= 32*RPL -- the bivariate bicycle
+// codes.  A candidate's messages sit at the words of the code's placement
+// (bsd_layout.cu): the pair h of row i at h kPlane + 2 i, so the detector pass
+// moves 32 consecutive pairs per access.  The columns are dealt to the lanes so
+// that each row of a full group of 32 rows has two columns in its own lane: the
+// messages on these edges (128 of 432 on [[144,12,12]]) stay in registers between
+// the passes.  The other words are spread over the banks of their column group.
+// With single-precision storage D is written over E (each word belongs to one
+// row and to one (column, k), so either pass reads its words before it writes
+// them); 16-bit storage keeps D in float beside E.  Each lane keeps its columns'
+// shared-memory addresses, Lambda_j, sum_LLR and its first row's columns in
+// registers.
 //
 // What bounds the iteration: 4 shared-memory transfers per edge (54
 // wavefronts at 100% for 432 edges), and the ALU pipe, which runs min, max,
@@ -592,29 +594,41 @@ struct SmallEngine {
     static constexpr bool kPriorStart = !W;  // unweighted runs from E(0) start from the table D0
     static constexpr bool kPriorSetsSums = false;
     static constexpr bool kInPlace = P == 0; // D over E
+    static constexpr int LC = 2 * (RPL - 1); // column groups with a register-held message
     WarpGroup grp;
     using S = Store<P>;
     static_assert(RD == 6, "the placement holds rows of degree 6");
+    static_assert(CPL == LC + 1, "every full row group has two column groups of its own, the last columns one");
     static constexpr int kPlane = small_plane_stride_rpl(RPL);   // words between a row's pairs
-    uint32_t ca[CPL][3];   // shared-memory address of the D message on the k-th edge of column lane + 32 c
-    uint32_t hq[CPL];      // the columns of row `lane` of H
+    uint32_t ca[CPL][3];   // shared-memory address of the D message on the k-th edge of the lane's column c
+    uint32_t hq[CPL];      // the columns of row `lane` of H, by position
     float sum[CPL];
-    uint32_t mb;           // bit c: column lane + 32 c is masked or beyond N
+    uint32_t mb;           // bit c: the lane's column c is masked or there is none
 
     static __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+    // the storage format's value of a message
+    static __device__ __forceinline__ float rnd(float x)
+    {
+        if constexpr (P == 0) return x;
+        typename S::T t;
+        S::st(&t, 0, x);
+        return S::ld(&t, 0);
+    }
+    static __device__ __forceinline__ int column(const DevGraph& g, int c)
+    {
+        return __ldg(&g.scol[(threadIdx.x & 31) + 32 * c].x);
+    }
     __device__ void load_graph(const DevGraph& g, const WarpState& st)
     {
         const int lane = threadIdx.x & 31;
         const uint32_t base = saddr(kInPlace ? st.E : (void*)st.D);
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
-            const int j = lane + 32 * c;
-            ca[c][0] = ca[c][1] = ca[c][2] = base;
+            const int4 q = __ldg(g.scol + lane + 32 * c);
             hq[c] = __ldg(g.shrow + (size_t)kSmallRowWords * lane + c);
-            if (j < g.N) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) ca[c][k] = base + 4u * (__ldg(g.scol + 3 * j + k) >> 16);
-            }
+            ca[c][0] = base + 4u * (uint32_t)q.y;
+            ca[c][1] = base + 4u * (uint32_t)q.z;
+            ca[c][2] = base + 4u * (uint32_t)q.w;
         }
     }
     __device__ void start_prior(const DevGraph& g, const WarpState& st) const
@@ -634,7 +648,7 @@ struct SmallEngine {
     {
         const int lane = threadIdx.x & 31;
         if (lane < 3)
-            Store<P>::st(reinterpret_cast<typename Store<P>::T*>(st.E), __ldg(g.scol + 3 * j + lane) >> 16, L);
+            Store<P>::st(reinterpret_cast<typename Store<P>::T*>(st.E), __ldg(g.sword + 3 * j + lane), L);
     }
     __device__ void clear_sums(const DevGraph&, const WarpState&)
     {
@@ -650,18 +664,22 @@ struct SmallEngine {
         typename S::T* const E = reinterpret_cast<typename S::T*>(st.E);
         const uint32_t dbase = saddr(kInPlace ? st.E : (void*)st.D);
         const uint32_t drow = dbase + 8u * lane;         // D of the lane's first row
-        // Lambda_j of the lane's columns; +inf for a masked column or one past
-        // N: its messages and posterior are then +inf, which the detector
-        // pass reads as L_MAX and positive (the sentinel of a masked node) and
-        // Eq. 4 as e^_j = 0, with no test in the loop
+        // Lambda_j of the lane's columns; +inf for a masked column or a position
+        // without one: its messages and posterior are then +inf, which the
+        // detector pass reads as L_MAX and positive (the sentinel of a masked
+        // node) and Eq. 4 as e^_j = 0, with no test in the loop
         float l[CPL];
+        // the messages of the edges between the lane's rows and its columns:
+        // E after the error-node pass, D after the detector pass
+        float own[LC];
         mb = 0u;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
-            const int j = lane + 32 * c;
-            const bool out = j >= g.N || ((st.mask[c] >> lane) & 1u);
+            const int j = column(g, c);
+            const bool out = j < 0 || ((st.mask[j >> 5] >> (j & 31)) & 1u);
             if (out) mb |= 1u << c;
             l[c] = out ? INFINITY : __ldg(g.lam + j);
+            if (c < LC) own[c] = S::ld(E, 2 * (lane + 32 * (c / 2)) + (c & 1));
         }
         // L_MAX with the sign (-1)^{s'_i} of the lane's rows (s' is fixed for the run)
         float sL[RPL];
@@ -672,7 +690,7 @@ struct SmallEngine {
         }
         int iters = 0;
         int ok = 0;
-        uint32_t bal[CPL];     // e^ words of the last iteration (the same in every lane)
+        uint32_t bal[CPL];     // e^ by position in the last iteration (the same in every lane)
 #pragma unroll
         for (int c = 0; c < CPL; ++c) bal[c] = 0u;
         for (int t = 1; t <= max_iters; ++t) {
@@ -691,11 +709,15 @@ struct SmallEngine {
                         const uint32_t sb = __float_as_uint(sL[r]) & 0x80000000u;
 #pragma unroll
                         for (int h = 0; h < 3; ++h) {
-                            const int wd = h * kPlane + 2 * i;
-                            const float2 v = __ldg(reinterpret_cast<const float2*>(g.sD0 + wd));
-                            sts2(drow + 4u * (h * kPlane + 64 * r),
-                                 make_float2(__uint_as_float(__float_as_uint(v.x) ^ sb),
-                                             __uint_as_float(__float_as_uint(v.y) ^ sb)));
+                            const float2 v = __ldg(reinterpret_cast<const float2*>(g.sD0 + h * kPlane + 2 * i));
+                            const float2 d = make_float2(__uint_as_float(__float_as_uint(v.x) ^ sb),
+                                                         __uint_as_float(__float_as_uint(v.y) ^ sb));
+                            if (h == 0 && r < RPL - 1) {
+                                own[2 * (r < RPL - 1 ? r : 0)] = d.x;
+                                own[2 * (r < RPL - 1 ? r : 0) + 1] = d.y;
+                            } else {
+                                sts2(drow + 4u * (h * kPlane + 64 * r), d);
+                            }
                         }
                     }
                 }
@@ -703,11 +725,16 @@ struct SmallEngine {
 #pragma unroll
                 for (int r = 0; r < RPL; ++r) {
                     const int i = lane + 32 * r;
-                    if (i < g.M) {
+                    const bool held = r < RPL - 1;       // the row's pair 0 is in registers (a full row group)
+                    const int o = held ? 2 * r : 0;
+                    if (held || i < g.M) {
                         float2 x[3];
 #pragma unroll
-                        for (int h = 0; h < 3; ++h)
-                            x[h] = kInPlace ? lds2(drow + 4u * (h * kPlane + 64 * r)) : S::ld2(E, h * kPlane + 2 * i);
+                        for (int h = 0; h < 3; ++h) {
+                            if (held && h == 0) x[h] = make_float2(own[o], own[o + 1]);
+                            else
+                                x[h] = kInPlace ? lds2(drow + 4u * (h * kPlane + 64 * r)) : S::ld2(E, h * kPlane + 2 * i);
+                        }
                         // D_{i->j} = alpha (-1)^{s_i} prod sign min over the other
                         // five messages (R3, R4): p[h] the signed minimum of pair
                         // h, q[h] that of the other two pairs capped at L_MAX with
@@ -723,8 +750,13 @@ struct SmallEngine {
                         for (int h = 0; h < 3; ++h) {
                             float2 w2 = alpha2;
                             if (W) w2 = __ldg(reinterpret_cast<const float2*>(wt + h * kPlane + 2 * i));
-                            sts2(drow + 4u * (h * kPlane + 64 * r),
-                                 mul2(w2, make_float2(xmin(x[h].y, q[h]), xmin(x[h].x, q[h]))));
+                            const float2 d = mul2(w2, make_float2(xmin(x[h].y, q[h]), xmin(x[h].x, q[h])));
+                            if (held && h == 0) {
+                                own[o] = d.x;
+                                own[o + 1] = d.y;
+                            } else {
+                                sts2(drow + 4u * (h * kPlane + 64 * r), d);
+                            }
                         }
                     }
                 }
@@ -733,14 +765,14 @@ struct SmallEngine {
             // ---- error-node pass (Eqs. 2-4), the next column's messages loaded
             // before this one's are stored
             float v[2][3];
+            auto load_column = [&](int c, float (&d)[3]) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) v[0][k] = lds(ca[0][k]);
+                for (int k = 0; k < 3; ++k) d[k] = (k == 0 && c < LC) ? own[c < LC ? c : 0] : lds(ca[c][k]);
+            };
+            load_column(0, v[0]);
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
-                if (c + 1 < CPL) {
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) v[(c + 1) & 1][k] = lds(ca[c + 1][k]);
-                }
+                if (c + 1 < CPL) load_column(c + 1, v[(c + 1) & 1]);
                 const float v0 = v[c & 1][0], v1 = v[c & 1][1], v2 = v[c & 1][2];
                 // Eq. 2: each message leaves its own detector out; the other two
                 // are added in ascending order.  Messages are stored unclamped:
@@ -755,17 +787,18 @@ struct SmallEngine {
                 const float2 e2p = add2(add2(ll, make_float2(lo01, fminf(lo01, v2))),
                                         make_float2(hi01, fmin3(hi01, hi02, hi12)));
                 const float post = __fadd_rn(e2p.y, fmaxf(hi01, v2));
-                const bool inr = c + 1 < CPL || lane + 32 * c < g.N;   // only the last word may pass N
+                const bool inr = c < LC || lane + 32 * c < g.N;   // only the last group may pass N
+                const float e[3] = {e01.x, e01.y, e2p.x};
+                if (c < LC) own[c < LC ? c : 0] = rnd(e[0]);
                 if (inr) {
-                    const float e[3] = {e01.x, e01.y, e2p.x};
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
+                    for (int k = c < LC ? 1 : 0; k < 3; ++k) {
                         if (kInPlace) sts(ca[c][k], e[k]);
                         else S::st(E, (ca[c][k] - dbase) >> 2, e[k]);
                     }
                 }
                 sum[c] = __fadd_rn(sum[c], post);           // unused for masked columns
-                if (kPostOut && t == max_iters && inr) post_out[lane + 32 * c] = post;
+                if (kPostOut && t == max_iters && inr) post_out[column(g, c)] = post;
                 bal[c] = __ballot_sync(FULLMASK, post <= 0.f);                       // Eq. 4
             }
             __syncwarp();
@@ -792,17 +825,27 @@ struct SmallEngine {
             if (ok && stop) break;
             if (ab.key != nullptr && __any_sync(FULLMASK, lane == 0 && ab.hit(ab_key))) { ok = 0; break; }
         }
-        // e^ of the last iteration run
+        // the register-held messages join the others, and e^ of the last
+        // iteration run goes back to natural order
 #pragma unroll
-        for (int c = 0; c < CPL; ++c)
-            if (lane == c && iters > 0) st.ehat[c] = bal[c];
+        for (int c = 0; c < LC; ++c) S::st(E, 2 * (lane + 32 * (c / 2)) + (c & 1), own[c]);
+        if (iters > 0) {
+            if (lane < CPL) st.ehat[lane] = 0u;
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                if ((bal[c] >> lane) & 1u) {
+                    const int j = column(g, c);
+                    atomicOr(&st.ehat[j >> 5], 1u << (j & 31));
+                }
+            }
+        }
         *success = ok;
         return iters;
     }
-    __device__ void argmin_score(const DevGraph&, const WarpState&, double guard, int* np, long long* S,
+    __device__ void argmin_score(const DevGraph& g, const WarpState&, double guard, int* np, long long* S,
                                  int* tie)
     {
-        const int lane = threadIdx.x & 31;
         float best = INFINITY, second = INFINITY;
         int bj = -1;
         unsigned long long s = 0;
@@ -810,17 +853,18 @@ struct SmallEngine {
         for (int c = 0; c < CPL; ++c) {
             if ((mb >> c) & 1u) continue;
             const float a = fabsf(sum[c]);
-            two_smallest(a, lane + 32 * c, &best, &second, &bj);
+            merge_argmin(best, second, bj, a, INFINITY, column(g, c));
             s += fixq(a);
         }
         reduce_argmin_score(grp, best, second, bj, s, guard, np, S, tie);
     }
     __device__ void write_sums(const DevGraph& g, const WarpState&, float* dst)
     {
-        const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int c = 0; c < CPL; ++c)
-            if (lane + 32 * c < g.N) dst[lane + 32 * c] = sum[c];
+        for (int c = 0; c < CPL; ++c) {
+            const int j = column(g, c);
+            if (j >= 0) dst[j] = sum[c];
+        }
     }
 };
 

@@ -65,6 +65,8 @@ constexpr int kRowDeg = 6;
 constexpr int kColDeg = 3;
 constexpr int kTries = 16;      // local-search restarts
 constexpr int kSweeps = 200;    // sweeps per restart
+constexpr int kLocalTries = 6;  // draws of the columns that rows own
+constexpr int kLocalSweeps = 60; // sweeps per draw
 
 struct Rng {                    // xorshift64*: a fixed, reproducible sequence
     uint64_t s;
@@ -297,7 +299,7 @@ void colour_group_n(const std::vector<int>& eu, const std::vector<int>& ev, int 
 }  // namespace
 
 bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, GenericLayout* out,
-                    const int* start)
+                    const int* start, bool quick)
 {
     if (M < 1 || N < 1 || colK < 1 || colK > kMaxColour) return false;
     const int E = row_ptr[M];
@@ -331,12 +333,12 @@ bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int co
         per_sweep += d * (d - 1) / 2;
     }
     const int max_sweeps = (int)std::min<double>(kSweeps, 5e7 / per_sweep);
-    // (a given order starts close to what the search reaches: it ends at the
-    // first sweep that takes off less than a tenth)
+    // (quick: the given order starts close to what the search reaches, and it
+    // ends at the first sweep that takes off less than a tenth)
     int best = ex, stale = 0;
-    for (int sw = 0; sw < max_sweeps && ex > 0 && stale < (start ? 1 : kPatience); ++sw) {
-        if (ex < (start && sw > 0 ? 0.9 * best : best)) { best = ex; stale = 0; } else if (sw > 0) { ++stale; }
-        if (start && stale) break;
+    for (int sw = 0; sw < max_sweeps && ex > 0 && stale < (quick ? 1 : kPatience); ++sw) {
+        if (ex < (quick && sw > 0 ? 0.9 * best : best)) { best = ex; stale = 0; } else if (sw > 0) { ++stale; }
+        if (quick && stale) break;
         for (int i = M - 1; i > 0; --i) std::swap(order[i], order[rng.below((uint32_t)i + 1)]);
         for (int i : order) {
             for (int a = row_ptr[i]; a < row_ptr[i + 1]; ++a) {
@@ -411,6 +413,203 @@ bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int co
         }
         for (size_t x = 0; x < ids.size(); ++x) out->kedge[(size_t)colour[x] * N + col_idx[ids[x]]] = ids[x];
     }
+    return true;
+}
+
+}  // namespace bsd
+
+namespace bsd {
+
+// the single-warp engine's placement: rows in natural order, columns in the
+// order of the lanes that process them.  Which two of its columns a row owns is
+// drawn anew until the other words meet almost no bank conflict or kLocalTries is
+// reached; the draw with the fewest is kept.
+bool small_local_layout(int M, int N, const int* row_ptr, const int* col_idx, SmallLocal* out)
+{
+    const int RPL = (M + 31) / 32, CPL = (N + 31) / 32, LC = 2 * (RPL - 1);
+    if (RPL < 2 || CPL != LC + 1 || N != 2 * M) return false;
+    const int E = row_ptr[M];
+    std::vector<std::vector<int>> cedges(N);
+    std::vector<int> erow(E);
+    for (int i = 0; i < M; ++i) {
+        if (row_ptr[i + 1] - row_ptr[i] != kRowDeg) return false;
+        for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+            erow[e] = i;
+            cedges[col_idx[e]].push_back(e);
+        }
+    }
+    for (int j = 0; j < N; ++j)
+        if (cedges[j].size() != kColDeg) return false;
+    const int full = 32 * (RPL - 1), P = small_plane_stride(M);
+    // (a start of the sequence whose first draw leaves 2 extra wavefronts of 24 on
+    // [[144,12,12]] and none on [[72,12,6]])
+    Rng rng{7142492453195352267ull};
+    int best = -1;
+    std::vector<int> order(N), seen(M), via(M), queue, start, rp(M + 1), ci, id, pos(N), own(N);
+    for (int j = 0; j < N; ++j) order[j] = j;
+    for (int t = 0; t < kLocalTries && (best < 0 || best > RPL - 1); ++t) {
+        // two columns of its own for every row (augmenting paths; every row has
+        // six columns and every column three rows, so the assignment exists)
+        for (int j = N - 1; j > 0 && t > 0; --j) std::swap(order[j], order[rng.below((uint32_t)j + 1)]);
+        std::fill(own.begin(), own.end(), -1);
+        std::fill(seen.begin(), seen.end(), -1);
+        std::vector<std::vector<int>> has(M);
+        for (int j0 : order) {
+            // breadth-first over rows; from a full row, on to the columns it holds
+            queue.clear();
+            auto visit = [&](int j) {
+                const int first = (int)rng.below(kColDeg);
+                for (int k = 0; k < kColDeg; ++k) {
+                    const int i = erow[cedges[j][(first + k) % kColDeg]];
+                    if (seen[i] != j0) { seen[i] = j0; via[i] = j; queue.push_back(i); }
+                }
+            };
+            visit(j0);
+            int end = -1;
+            for (size_t q = 0; q < queue.size() && end < 0; ++q) {
+                if (has[queue[q]].size() < 2) end = queue[q];
+                else
+                    for (int j : has[queue[q]]) visit(j);
+            }
+            if (end < 0) return false;
+            for (int i = end; i >= 0;) {
+                const int j = via[i], from = own[j];
+                if (from >= 0) has[from].erase(std::find(has[from].begin(), has[from].end(), j));
+                own[j] = i;
+                has[i].push_back(j);
+                i = from;
+            }
+        }
+        // a full row's own columns go to groups 2 r and 2 r + 1 (in either order),
+        // the others to the last; the other edges take words 2..5 of a full row,
+        // all six of the last ones.  Swaps of two words of a row, and of a row's
+        // two own columns, while the loads above each group's degree fall
+        auto group = [&](int j) {
+            const int i = own[j];
+            return i < full ? 2 * (i / 32) + (has[i][1] == j ? 1 : 0) : LC;
+        };
+        std::vector<std::vector<int>> word(M);               // edges by word of the row
+        std::vector<int> cnt((size_t)CPL * 32, 0), at(E, 0);
+        auto bank = [&](int i, int q) { return ((q >> 1) * P + 2 * i + (q & 1)) & 31; };
+        for (int i = 0; i < M; ++i) {
+            word[i].assign(kRowDeg, -1);
+            int q = i < full ? 2 : 0;
+            for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+                if (i < full && own[col_idx[e]] == i) continue;
+                word[i][q] = e;
+                at[e] = q;
+                cnt[(size_t)group(col_idx[e]) * 32 + bank(i, q)]++;
+                ++q;
+            }
+        }
+        auto cap = [&](int g) { return g < LC ? 2 : 3; };
+        auto over = [&](int g, int b) { return std::max(0, cnt[(size_t)g * 32 + b] - cap(g)); };
+        int ex = 0;
+        for (int g = 0; g < CPL; ++g)
+            for (int b = 0; b < 32; ++b) ex += over(g, b);
+        for (int sw = 0; sw < kLocalSweeps && ex > 0; ++sw) {
+            for (int n = 0; n < M && ex > 0; ++n) {
+                const int i = (int)rng.below((uint32_t)M);
+                for (int x = i < full ? 2 : 0; x < kRowDeg; ++x)
+                    for (int y = x + 1; y < kRowDeg; ++y) {
+                        const int gx = group(col_idx[word[i][x]]), gy = group(col_idx[word[i][y]]);
+                        if (gx == gy) continue;
+                        const int bx = bank(i, x), by = bank(i, y);
+                        const int before = over(gx, bx) + over(gy, by) + over(gx, by) + over(gy, bx);
+                        cnt[(size_t)gx * 32 + bx]--; cnt[(size_t)gy * 32 + by]--;
+                        cnt[(size_t)gx * 32 + by]++; cnt[(size_t)gy * 32 + bx]++;
+                        const int after = over(gx, bx) + over(gy, by) + over(gx, by) + over(gy, bx);
+                        if (after < before || (after == before && rng.below(4) == 0)) {
+                            std::swap(word[i][x], word[i][y]);
+                            at[word[i][x]] = x;
+                            at[word[i][y]] = y;
+                            ex += after - before;
+                        } else {
+                            cnt[(size_t)gx * 32 + bx]++; cnt[(size_t)gy * 32 + by]++;
+                            cnt[(size_t)gx * 32 + by]--; cnt[(size_t)gy * 32 + bx]--;
+                        }
+                    }
+                if (i >= full) continue;
+                const int g0 = 2 * (i / 32);
+                auto move = [&](int j, int from, int to) {
+                    int d = 0;
+                    for (int e : cedges[j]) {
+                        if (erow[e] == i) continue;
+                        const int b = bank(erow[e], at[e]);
+                        d -= over(from, b) + over(to, b);
+                        cnt[(size_t)from * 32 + b]--;
+                        cnt[(size_t)to * 32 + b]++;
+                        d += over(from, b) + over(to, b);
+                    }
+                    return d;
+                };
+                const int d = move(has[i][0], g0, g0 + 1) + move(has[i][1], g0 + 1, g0);
+                if (d < 0 || (d == 0 && rng.below(4) == 0)) {
+                    std::swap(has[i][0], has[i][1]);
+                    ex += d;
+                } else {
+                    move(has[i][0], g0 + 1, g0);
+                    move(has[i][1], g0, g0 + 1);
+                }
+            }
+        }
+        SmallLocal s;
+        s.col.assign((size_t)32 * CPL, -1);
+        int next = 32 * LC;
+        for (int i = 0; i < M; ++i)
+            for (int k = 0; k < 2; ++k) {
+                const int q = i < full ? 32 * (2 * (i / 32) + k) + i % 32 : next++;
+                s.col[q] = has[i][k];
+                pos[has[i][k]] = q;
+            }
+        ci.clear(); id.clear(); start.clear();
+        s.word.assign(E, 0);
+        rp[0] = 0;
+        for (int i = 0; i < M; ++i) {
+            for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+                const int j = col_idx[e];
+                if (i < full && own[j] == i) {
+                    s.word[e] = 2 * i + (has[i][1] == j ? 1 : 0);
+                    continue;
+                }
+                ci.push_back(pos[j]);
+                id.push_back(e);
+                start.push_back((at[e] >> 1) * P + 2 * i + (at[e] & 1));
+            }
+            rp[i + 1] = (int)ci.size();
+        }
+        GenericLayout gl;
+        if (!generic_layout(M, N, rp.data(), ci.data(), kColDeg, &gl, start.data(), true)) return false;
+        for (size_t x = 0; x < id.size(); ++x) s.word[id[x]] = gl.pos[x];
+        s.slot.assign((size_t)32 * CPL * kColDeg, 0);
+        for (int q = 0; q < N; ++q) {
+            int k = 0;
+            int* w = s.slot.data() + (size_t)kColDeg * q;
+            if (q < 32 * LC)
+                for (int e : cedges[s.col[q]])
+                    if (erow[e] == own[s.col[q]]) w[k++] = s.word[e];
+            for (int c = 0; c < kColDeg; ++c) {
+                const int x = gl.kedge[(size_t)c * N + q];
+                if (x >= 0 && k < kColDeg) w[k++] = s.word[id[x]];
+            }
+            if (k != kColDeg) return false;
+        }
+        // extra wavefronts of the error pass's accesses
+        int extra = 0;
+        for (int g = 0; g < CPL; ++g)
+            for (int k = g < LC ? 1 : 0; k < kColDeg; ++k) {
+                int load[32] = {0}, most = 0;
+                for (int q = 32 * g; q < std::min(N, 32 * g + 32); ++q)
+                    most = std::max(most, ++load[s.slot[(size_t)kColDeg * q + k] & 31]);
+                extra += most - 1;
+            }
+        if (best < 0 || extra < best) {
+            best = extra;
+            *out = s;
+        }
+    }
+    out->extent = 2 * P + 2 * M;
+    out->extra = best;
     return true;
 }
 

@@ -277,6 +277,7 @@ struct Work {
     int* near;             // [A] a near-tie met by this shot's search so far
     unsigned long long* first_ok;  // [A] (round stamp << 32) | ~c of the lowest-index successful child so far
     BeamEntry* ent;        // [A]
+    int2* kid;             // [A][2w] (parent's child index of the round before, the node to fix) of a round's children
     uint32_t* ring;        // items to run, Counters::b_mask + 1 slots in use
     Counters* ctr;
     RunDesc* desc;

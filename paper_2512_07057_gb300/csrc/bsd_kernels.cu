@@ -1244,29 +1244,25 @@ __device__ inline size_t slot_index(const Work& w, int bank, int a, int c, int W
     return ((size_t)bank * (size_t)w.A + (size_t)a) * (size_t)W2 + (size_t)c;
 }
 
-// the parent of the rank-k path of window entry a in round r: the seed-store
-// entry of its shot for r = 1, else the slot of the previous round that won
-// rank k
+// a parent in round r: the seed-store entry of the shot for r = 1, else child
+// `slot` of the round before
 struct SlotRef {
     const unsigned char* E;   // snapshot, Epad messages in the storage format
     const uint32_t* bits;
-    const SlotMeta* meta;
 };
 
-__device__ inline SlotRef parent_ref(const DevGraph& g, const DecCfg& cfg, const Work& w, int r, int seed,
-                                     int a, int k)
+__device__ inline SlotRef parent_ref(const DevGraph& g, const DecCfg& cfg, const Work& w, int r, int seed, int a,
+                                     int slot)
 {
     SlotRef s;
     if (r == 1) {
         const size_t e = (size_t)seed;
         s.E = w.seedE + e * snap_bytes(g);
         s.bits = w.seedBits + e * (size_t)w.SB;
-        s.meta = w.seedMeta + e;
     } else {
-        const size_t e = slot_index(w, (r - 1) & 1, a, __ldcg(w.set_idx + (size_t)a * cfg.w + k), 2 * cfg.w);
+        const size_t e = slot_index(w, (r - 1) & 1, a, slot, 2 * cfg.w);
         s.E = w.slotE + e * snap_bytes(g);
         s.bits = w.slotBits + e * (size_t)w.SB;
-        s.meta = w.slotMeta + e;
     }
     return s;
 }
@@ -1348,10 +1344,9 @@ __global__ void k_beam_begin(Work w, int beam_width)
         w.ctr->b_tail = 2u * (unsigned)cnt;
         w.ctr->b_left = n;
         w.ctr->b_next = cnt;
-        // the ring for these entries: at most 2w items of each are on it at
-        // once, and it has at least twice as many slots
+        // the ring for these entries: at most 2w items of each are on it at once
         uint32_t slots = 4;
-        while ((unsigned long long)slots < 4ull * (unsigned long long)cnt * (unsigned)beam_width) slots *= 2;
+        while ((unsigned long long)slots < 2ull * (unsigned long long)cnt * (unsigned)beam_width) slots *= 2;
         w.ctr->b_mask = slots - 1;
     }
 }
@@ -2109,10 +2104,16 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
 // slot still full when the ring has come round gives its item back to the
 // pusher, which pushes it again; a group that has waited kIdleNs leaves
 // and marks its ticket's slot, and the pusher that meets the mark pushes its
-// item again too.  No item is lost, no wait is unbounded, and the running
-// groups alone finish the work, so nothing rests on two groups being resident
-// at once.
+// item again too.  (Each group holds one ticket at most and there are no more
+// groups than slots, so a ticket's pusher has come and taken the mark back before
+// the slot's next ticket is drawn.)  No item is lost, no wait is unbounded, and
+// the running groups alone finish the work, so nothing rests on two groups being
+// resident at once.
 constexpr unsigned long long kIdleNs = 1000ull * 1000 * 1000;
+
+// orders this thread's memory operations, and those of the threads it has
+// synchronised with, before and after an atomic that passes them on
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p)
 {
@@ -2143,21 +2144,14 @@ __device__ inline void push_item(const Work& w, uint32_t item)
     }
 }
 
-// the next item, or kRingEmpty when every shot has ended (or none came for kIdleNs)
-__device__ inline uint32_t draw_item(const Work& w)
+// the item of a ticket, or kRingEmpty when every shot has ended (or none came for
+// kIdleNs)
+__device__ inline uint32_t draw_item(const Work& w, uint32_t ticket)
 {
-    uint32_t* slot = w.ring + (atomicAdd(&w.ctr->b_head, 1u) & w.ctr->b_mask);
+    uint32_t* slot = w.ring + (ticket & w.ctr->b_mask);
+    uint32_t it = atomicExch(slot, kRingEmpty);
     unsigned long long t0 = 0ull;
-    for (unsigned spins = 0;; ++spins) {
-        const uint32_t v = ld_relaxed(slot);
-        if (v != kRingEmpty && v != kRingLeft) {
-            const uint32_t it = atomicExch(slot, kRingEmpty);
-            if (it != kRingEmpty && it != kRingLeft) {
-                __threadfence();               // the item before what it names
-                return it;
-            }
-            continue;
-        }
+    for (unsigned spins = 0; it == kRingEmpty; ++spins) {
         if ((spins & 3u) == 0u && ld_relaxed(reinterpret_cast<const uint32_t*>(&w.ctr->b_left)) == 0u) return kRingEmpty;
         if (spins >= 4u) __nanosleep(200);
         if ((spins & 63u) == 0u) {
@@ -2165,7 +2159,10 @@ __device__ inline uint32_t draw_item(const Work& w)
             if (t0 == 0ull) t0 = t;
             else if (t - t0 > kIdleNs && atomicCAS(slot, kRingEmpty, kRingLeft) == kRingEmpty) return kRingEmpty;
         }
+        if (ld_relaxed(slot) != kRingEmpty) it = atomicExch(slot, kRingEmpty);
     }
+    fence_gpu();                               // the item before what it names
+    return it;
 }
 
 struct SelScratch {
@@ -2198,6 +2195,7 @@ __device__ inline void init_entry(const DevGraph& g, const DecCfg& cfg, const Wo
         w.res_n[a] = sm.success ? 1 : 0;
         w.near[a] = sm.flags & 1;      // the seed path branches on its argmin
         w.ent[a] = BeamEntry{e, 1, 2, stamp};
+        w.kid[(size_t)a * 2 * cfg.w] = w.kid[(size_t)a * 2 * cfg.w + 1] = make_int2(-1, sm.next_pos);
     }
     __syncwarp();
 }
@@ -2247,7 +2245,7 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
     const int nch = 2 * npar;
     // gather the children of this round in canonical order c = 2 * rank + val
     for (int c = lane; c < nch; c += 32) {
-        const int pnp = __ldcg(&parent_ref(g, cfg, w, r, ent.seed, a, c >> 1).meta->next_pos);
+        const int pnp = __ldcg(w.kid + (size_t)a * W2 + c).y;
         int fl = 0, it = 0;
         double scv = 0.0;
         if (pnp >= 0) {
@@ -2423,7 +2421,7 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
                 if (best != 0x7fffffff)
                     eb = w.slotBits + slot_index(w, cb, a, best, W2) * (size_t)w.SB + g.WM + 2 * g.WN;
                 else
-                    eb = parent_ref(g, cfg, w, r, ent.seed, a, 0).bits + g.WM + 2 * g.WN;
+                    eb = parent_ref(g, cfg, w, r, ent.seed, a, __ldcg(w.kid + (size_t)a * W2).x).bits + g.WM + 2 * g.WN;
                 finalize_shot<WarpGroup, false, true>(g, d.out, gb, eb, ST_FAILED | (near ? ST_NEAR : 0u), acc);
             }
             done = true;
@@ -2437,10 +2435,12 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
                 w.ent[a] = BeamEntry{ent.seed, r + 1, 2 * tot, ent.stamp + 1};
             }
             __syncwarp();
-            __threadfence();                   // the entry before its items
             for (int k = lane; k < keep; k += 32) {
                 const int c = __ldcg(w.set_idx + (size_t)a * cfg.w + k);
-                if (__ldcg(&w.slotMeta[slot_index(w, cb, a, c, W2)].next_pos) >= 0) {
+                const int np = __ldcg(&w.slotMeta[slot_index(w, cb, a, c, W2)].next_pos);
+                w.kid[(size_t)a * W2 + 2 * k] = w.kid[(size_t)a * W2 + 2 * k + 1] = make_int2(c, np);
+                if (np >= 0) {
+                    fence_gpu();               // the entry and the child before its items
                     push_item(w, ring_item(a, 2 * k));
                     push_item(w, ring_item(a, 2 * k + 1));
                 }
@@ -2455,12 +2455,14 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
         e = __shfl_sync(FULLMASK, e, 0);
         if (e < w.ctr->n_active) {
             init_entry(g, cfg, w, a, e, ent.stamp + 1);
-            __threadfence();
-            if (lane < 2) push_item(w, ring_item(a, lane));
+            if (lane < 2) {
+                fence_gpu();
+                push_item(w, ring_item(a, lane));
+            }
         }
         __syncwarp();
         if (lane == 0) {
-            __threadfence();
+            fence_gpu();
             atomicSub(&w.ctr->b_left, 1);
         }
     }
@@ -2477,21 +2479,23 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(Dev
     const auto& grp = eng.grp;
     char* const own = smem + (size_t)grp.index() * warp_smem_bytes(g);
     const WarpState st = carve(own, g);
-    // never more tickets waiting than half the ring
-    if ((uint32_t)(blockIdx.x * grp.per_block() + grp.index()) > w.ctr->b_mask / 2) return;
+    // no more tickets waiting than slots
+    if ((uint32_t)(blockIdx.x * grp.per_block() + grp.index()) > w.ctr->b_mask) return;
     const int W2 = 2 * cfg.w;
     unsigned long long ran = 0;                // BP iterations (group rank 0)
+    uint32_t ticket = 0;                       // the next item's (group rank 0)
+    if (grp.rank() == 0) ticket = atomicAdd(&w.ctr->b_head, 1u);
     for (;;) {
         uint32_t item = kRingEmpty;
-        if (grp.rank() == 0) item = draw_item(w);
+        if (grp.rank() == 0) item = draw_item(w, ticket);
         item = (uint32_t)grp.bcast((int)item);
         if (item == kRingEmpty) break;
         const int a = ring_entry(item), c = ring_child(item);
         const BeamEntry ent = load_entry(w.ent + a);
+        const int2 kid = __ldcg(w.kid + (size_t)a * W2 + c);
         const int r = ent.round;
-        const int k = c >> 1, v = c & 1;
-        const SlotRef par = parent_ref(g, cfg, w, r, ent.seed, a, k);
-        const int pos = __ldcg(&par.meta->next_pos);
+        const int v = c & 1, pos = kid.y;
+        const SlotRef par = parent_ref(g, cfg, w, r, ent.seed, a, kid.x);
         if (pos >= 0) {                        // (a path with no unmasked node has no children)
             const size_t cslot = slot_index(w, r & 1, a, c, W2);
             // s' of the child: flip the detectors of pos when it is fixed to 1
@@ -2567,15 +2571,19 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(Dev
                 }
             }
         }
-        // the slot before the count; the round's last child selects
-        __threadfence();
+        // the slot before the count; the round's last child selects (the next
+        // ticket is drawn on the way)
         grp.sync();
         int last = 0;
         if (grp.rank() == 0) {
+            ticket = atomicAdd(&w.ctr->b_head, 1u);
+            fence_gpu();
             last = atomicSub(&w.ent[a].pending, 1) == 1 ? 1 : 0;
-            __threadfence();
+            if (last) fence_gpu();
         }
-        if (grp.bcast(last)) {
+        last = grp.bcast(last);
+        grp.sync();
+        if (last) {
             if (grp.warp() == 0) select_entry(g, cfg, w, a, reinterpret_cast<SelScratch*>(own));
             grp.sync();
         }
@@ -3121,10 +3129,11 @@ size_t work_layout(const DevGraph& g, const DecCfg& cfg, long long S, long long 
     v.res_n = (int*)take(sizeof(int) * (size_t)A);
     v.first_ok = (unsigned long long*)take(sizeof(unsigned long long) * (size_t)A);
     v.near = (int*)take(sizeof(int) * (size_t)A);
-    // a power of two of at least 2 * A * 2w slots (k_beam_begin)
+    // a power of two of at least A * 2w slots (k_beam_begin)
     size_t slots = 4;
-    while (slots < 2 * (size_t)A * W2) slots *= 2;
+    while (slots < (size_t)A * W2) slots *= 2;
     v.ring = (uint32_t*)take(sizeof(uint32_t) * slots);
+    v.kid = (int2*)take(sizeof(int2) * (size_t)A * W2);
     // the batched seed BP's slots and the shots it passes on
     v.bs_slots = bs_slots;
     if (bs_slots > 0) {

@@ -13,8 +13,8 @@
 //   lamq[N]               Lambda_j on the 2^-16 fixed-point grid (weights)
 //   rs0[M]                the detector records of E(0) (a seed run's first check pass, up to the syndrome)
 //   D0[Epad]              the check messages of E(0) with the scale alpha, before the syndrome sign
-//   colW[colK][Npad]      word of the edge in slot k of column j at the jagged
-//                         engine's placement, -1 for an empty slot
+//   colW[colK][Npad]      word of the edge in slot k of the column at position p
+//                         at the jagged engine's placement, -1 for an empty slot
 //   lamEc[Npad]           clamp(Lambda_j) in the storage format (E(0) of every edge of column j)
 //
 // Workspace (one decoder):
@@ -69,9 +69,13 @@ struct DevGraph {
     // up to 6; bsd_layout.cu): the rows in order of falling degree, the k-th
     // edges of all rows that have one adjacent: the k-th edge of the row of rank
     // q at word jplane[k] + q (jplane[] holds the first kJaggedPlanes, jplanes all)
-    const int* colW;       // [colK][Npad] word of the edge in slot k of column j, -1: empty
+    const int* colW;       // [colK][Npad] word of the edge in slot k of the column at position p, -1: empty
+    const int* colJ;       // [N] column at position p, null: column p
+    const int* colN;       // [colK][Npad] the words by column
+    const int* colF;       // [colK][Npad] the rows of the column at position p, -1: past its degree
     int colK;              // 3 or 6 (the engine's degree bound), 0 when colW is absent
     const uint8_t* colG;   // [ceil(N / 32)] degree of the group's columns, + 8 when they differ
+    const uint8_t* rowG;   // [ceil(M / 32)] largest degree of 32 ranks' rows, + 32 when they differ; 64 above 16
     const int2* rowQ;      // [M] (row, degree) of rank q
     const int* jplanes;    // [max_row_deg]
     int jplane[16];

@@ -895,7 +895,8 @@ template <> struct SortNet<6> { static constexpr int n = 12; static constexpr un
 // their messages twice instead).  The error pass runs the exact network of the
 // columns' degree where the 32 columns of a group have the same one (degree 3
 // without a sort, as the single-warp engine), and one padded to the largest
-// degree where they differ.  Masked columns and the clamp are handled as in the
+// degree where they differ; a code most of whose groups would differ has its
+// columns dealt to the groups by degree (DevGraph::colJ).  Masked columns and the clamp are handled as in the
 // single-warp engine.
 //
 // Before (records of the two smallest magnitudes per row, one thread per CSR
@@ -913,6 +914,7 @@ struct JaggedEngine {
     static constexpr bool kPriorStart = !W;       // unweighted runs from E(0) start from the table D0
     static constexpr bool kPriorSetsSums = true;  // a run from E(0) needs no cleared sums
     using S = Store<P>;
+    static constexpr int kRegWords = G::kBlock ? 1 : 6;
     G grp;
 
     // the storage format's value of a message
@@ -932,7 +934,7 @@ struct JaggedEngine {
             const float v = S::ld(reinterpret_cast<const typename S::T*>(g.lamEc), j);
 #pragma unroll
             for (int k = 0; k < DV; ++k) {
-                const int e = __ldg(g.colW + (size_t)k * g.Npad + j);
+                const int e = __ldg(g.colN + (size_t)k * g.Npad + j);
                 if (e >= 0) E[e] = v;
             }
         }
@@ -972,7 +974,7 @@ struct JaggedEngine {
     __device__ void fix_node(const DevGraph& g, const WarpState& st, int j, float L) const
     {
         for (int k = grp.rank(); k < DV; k += grp.size()) {
-            const int e = __ldg(g.colW + (size_t)k * g.Npad + j);
+            const int e = __ldg(g.colN + (size_t)k * g.Npad + j);
             if (e >= 0) reinterpret_cast<float*>(st.E)[e] = L;
         }
     }
@@ -981,44 +983,52 @@ struct JaggedEngine {
         for (int j = grp.rank(); j < g.N; j += grp.size()) st.sumllr[j] = 0.f;
     }
 
-    // D over E on the row of rank q, of degree deg <= RD, whose words start at eb
-    template <int RD>
+    // D over E on the row of rank q, of degree RD (kSame) or deg <= RD
+    template <int RD, bool kSame>
     static __device__ __forceinline__ void row_pass(const DevGraph& g, uint32_t eb, int q, int deg, float sL, float alpha,
                                                     const float* wt)
     {
         float x[RD], after[RD];
+        uint32_t a[RD];
 #pragma unroll
-        for (int k = 0; k < RD; ++k) x[k] = k < deg ? lds(eb + 4u * (uint32_t)(g.jplane[k] + q)) : INFINITY;
+        for (int k = 0; k < RD; ++k) {
+            a[k] = eb + 4u * (uint32_t)(g.jplane[k] + q);
+            x[k] = kSame || k < deg ? lds(a[k]) : INFINITY;
+        }
         after[RD - 1] = INFINITY;                  // the messages after k
 #pragma unroll
         for (int k = RD - 1; k > 0; --k) after[k - 1] = k == RD - 1 ? x[k] : xmin(x[k], after[k]);
         float before = sL;                         // those before k, capped, with the syndrome sign
 #pragma unroll
-        for (int k = 0; k < RD; ++k) {
-            if (k < deg) {
-                const float m = k == RD - 1 ? before : xmin(before, after[k]);
-                sts(eb + 4u * (uint32_t)(g.jplane[k] + q), __fmul_rn(W ? __ldg(wt + g.jplane[k] + q) : alpha, m));
+        for (int k = 0; k < RD; k += 2) {
+            const int k1 = k + 1 < RD ? k + 1 : k;
+            const float m0 = k == RD - 1 ? before : xmin(before, after[k]);
+            before = xmin(before, x[k]);
+            const float m1 = k1 == RD - 1 ? before : xmin(before, after[k1]);
+            if (k1 + 1 < RD) before = xmin(before, x[k1]);
+            float2 w2 = make_float2(alpha, alpha);
+            if (W) {
+                if (kSame || k < deg) w2.x = __ldg(wt + g.jplane[k] + q);
+                if (kSame || k1 < deg) w2.y = __ldg(wt + g.jplane[k1] + q);
             }
-            if (k + 1 < RD) before = xmin(before, x[k]);
+            const float2 d = mul2(w2, make_float2(m0, m1));
+            if (kSame || k < deg) sts(a[k], d.x);
+            if (k1 > k && (kSame || k1 < deg)) sts(a[k1], d.y);
         }
     }
 
     // Eqs. 2-3 for a column of degree DD (kSame), or at most DD with holes in its
     // slots: the messages over the column's words, the posterior returned
     template <int DD, bool kSame>
-    static __device__ __forceinline__ float column(const DevGraph& g, uint32_t eb, int j, float l)
+    static __device__ __forceinline__ float column(uint32_t eb, const int (&word)[DV], float l)
     {
         if constexpr (DD == 0) {
             return l;
         } else {
             float v[DD];
             uint32_t a[DD];
-            const int* cw = g.colW + j;
 #pragma unroll
-            for (int k = 0; k < DD; ++k) {
-                const int e = __ldg(cw + (size_t)k * g.Npad);
-                a[k] = (kSame || e >= 0) ? eb + 4u * (uint32_t)e : 0xffffffffu;
-            }
+            for (int k = 0; k < DD; ++k) a[k] = (kSame || word[k] >= 0) ? eb + 4u * (uint32_t)word[k] : 0xffffffffu;
 #pragma unroll
             for (int k = 0; k < DD; ++k) v[k] = (kSame || a[k] != 0xffffffffu) ? lds(a[k]) : INFINITY;
             if constexpr (DD == 3 && kSame) {
@@ -1074,7 +1084,19 @@ struct JaggedEngine {
         for (int t = 1; t <= max_iters; ++t) {
             unsigned long long ab_key = 0ull;
             if (ab.key != nullptr && grp.rank() == 0) ab_key = *((volatile const unsigned long long*)ab.key);
-            for (int q = grp.rank(); q < g.WM; q += grp.size()) st.par[q] = st.sp[q];
+            // H e^(t): with a warp per candidate and few words of rows, the XOR of
+            // the set columns of H in the lanes' registers, else of their rows
+            // in shared memory
+            const bool inreg = !G::kBlock && g.WM <= kRegWords;
+            uint32_t hx[kRegWords];
+            if (inreg) {
+#pragma unroll
+                for (int q = 0; q < kRegWords; ++q) hx[q] = 0u;
+            } else {
+                for (int q = grp.rank(); q < g.WM; q += grp.size()) st.par[q] = st.sp[q];
+            }
+            if (g.colJ != nullptr)
+                for (int q = grp.rank(); q < g.WN; q += grp.size()) st.ehat[q] = 0u;
             // weighted min-sum: row min(t, wT) - 1 of the weights in place of alpha
             const float* wt = W ? cfg.weights + (size_t)((t < cfg.wT ? t : cfg.wT) - 1) * (size_t)g.Epad : nullptr;
             // ---- detector pass (Eq. 1); a run from E(0) takes its first check
@@ -1091,13 +1113,16 @@ struct JaggedEngine {
                     continue;
                 }
                 const float sL = __uint_as_float(__float_as_uint(cfg.L) | sb);
-                const int dmax = __ldg(&g.rowQ[q & ~31].y);       // the warp's largest degree
-                if (dmax <= 8) {
-                    row_pass<8>(g, eb, q, rd.y, sL, cfg.alpha, wt);
-                } else if (dmax <= 12) {
-                    row_pass<12>(g, eb, q, rd.y, sL, cfg.alpha, wt);
-                } else if (dmax <= 16) {
-                    row_pass<16>(g, eb, q, rd.y, sL, cfg.alpha, wt);
+                // the warp's largest degree, + 32 when its rows have another too
+                const int dmax = __ldg(g.rowG + (q >> 5));
+                if (dmax == 8) {
+                    row_pass<8, true>(g, eb, q, 8, sL, cfg.alpha, wt);
+                } else if (dmax == 12) {
+                    row_pass<12, true>(g, eb, q, 12, sL, cfg.alpha, wt);
+                } else if ((dmax & 31) <= 8 && dmax < 64) {
+                    row_pass<8, false>(g, eb, q, rd.y, sL, cfg.alpha, wt);
+                } else if ((dmax & 31) <= 16 && dmax < 64) {
+                    row_pass<16, false>(g, eb, q, rd.y, sL, cfg.alpha, wt);
                 } else {
                     // the two smallest magnitudes and the sign parity, then D:
                     // the minimum over the others is m2 on an edge holding the
@@ -1125,49 +1150,84 @@ struct JaggedEngine {
             grp.sync();
             // ---- error-node pass (Eqs. 2-4) and syndrome parity; each warp owns
             // whole 32-column words of e^ (one column per lane)
+            // (the next group's table entries are loaded while this one runs)
+            int nj = 0, nw[DV], ng = 0;
+            float nl = 0.f;
+            auto fetch = [&](int jb) {
+                if (jb >= g.N) return;
+                const int p = min(jb + lane, g.N - 1);
+                ng = __ldg(g.colG + (jb >> 5));
+                nj = g.colJ != nullptr ? __ldg(g.colJ + p) : p;
+#pragma unroll
+                for (int k = 0; k < DV; ++k) nw[k] = __ldg(g.colW + (size_t)k * g.Npad + p);
+                nl = __ldg(g.lam + nj);
+            };
+            fetch(32 * grp.warp());
             for (int jb = 32 * grp.warp(); jb < g.N; jb += 32 * grp.nwarps()) {
-                const int j = jb + lane;
+                const int gd = ng, j = nj, p = jb + lane;
+                int wd[DV];
+#pragma unroll
+                for (int k = 0; k < DV; ++k) wd[k] = nw[k];
+                const float lj = nl;
+                fetch(jb + 32 * grp.nwarps());
                 bool ebit = false;
-                const int gd = __ldg(g.colG + (jb >> 5));
-                if (j < g.N) {
-                    const float l = ((st.mask[jb >> 5] >> lane) & 1u) ? INFINITY : __ldg(g.lam + j);
+                if (p < g.N) {
+                    const float l = ((st.mask[j >> 5] >> (j & 31)) & 1u) ? INFINITY : lj;
+                    const float before = prior ? 0.f : st.sumllr[j];
                     float post;
                     switch (gd) {
-                        case 0: post = column<0, true>(g, eb, j, l); break;
-                        case 1: post = column<1, true>(g, eb, j, l); break;
-                        case 2: post = column<2, true>(g, eb, j, l); break;
-                        case 3: post = column<3, true>(g, eb, j, l); break;
-                        case 9: case 10: case 11: post = column<3, false>(g, eb, j, l); break;
+                        case 0: post = column<0, true>(eb, wd, l); break;
+                        case 1: post = column<1, true>(eb, wd, l); break;
+                        case 2: post = column<2, true>(eb, wd, l); break;
+                        case 3: post = column<3, true>(eb, wd, l); break;
+                        case 9: case 10: case 11: post = column<3, false>(eb, wd, l); break;
                         default:
                             if constexpr (DV == 6) {
-                                if (gd == 4) post = column<4, true>(g, eb, j, l);
-                                else if (gd == 5) post = column<5, true>(g, eb, j, l);
-                                else if (gd == 6) post = column<6, true>(g, eb, j, l);
-                                else post = column<6, false>(g, eb, j, l);
+                                if (gd == 4) post = column<4, true>(eb, wd, l);
+                                else if (gd == 5) post = column<5, true>(eb, wd, l);
+                                else if (gd == 6) post = column<6, true>(eb, wd, l);
+                                else post = column<6, false>(eb, wd, l);
                             } else {
                                 post = l;
                             }
                     }
                     // a run from E(0) starts its sums here (0 + post, as a sum from zero)
-                    st.sumllr[j] = __fadd_rn(prior ? 0.f : st.sumllr[j], post);
+                    st.sumllr[j] = __fadd_rn(before, post);
                     if (kPostOut && t == max_iters) post_out[j] = post;
                     ebit = post <= 0.f;                               // Eq. 4
                     if (ebit) {
-                        for (int k = __ldg(g.col_ptr + j); k < __ldg(g.col_ptr + j + 1); ++k) {
-                            const int r = __ldg(g.col_row + k);
-                            atomicXor(&st.par[r >> 5], 1u << (r & 31));
+                        if (g.colJ != nullptr) atomicOr(&st.ehat[j >> 5], 1u << (j & 31));
+                        if (inreg) {
+#pragma unroll
+                            for (int q = 0; q < kRegWords; ++q)
+                                if (q < g.WM) hx[q] ^= __ldg(g.hcol + (size_t)j * g.WM + q);
+                        } else {
+                            int rr[DV];
+#pragma unroll
+                            for (int k = 0; k < DV; ++k) rr[k] = __ldg(g.colF + (size_t)k * g.Npad + p);
+#pragma unroll
+                            for (int k = 0; k < DV; ++k)
+                                if (rr[k] >= 0) atomicXor(&st.par[rr[k] >> 5], 1u << (rr[k] & 31));
                         }
                     }
                 }
-                const uint32_t bal = __ballot_sync(FULLMASK, ebit);
-                if (lane == 0) st.ehat[jb >> 5] = bal;
+                if (g.colJ == nullptr) {
+                    const uint32_t bal = __ballot_sync(FULLMASK, ebit);
+                    if (lane == 0) st.ehat[jb >> 5] = bal;
+                }
             }
             grp.sync();
             // ---- stopping rule: H e^(t) = s' (the vote's barrier also keeps the
             // next iteration's writes to par behind these reads); a child that
             // succeeds in the iteration at whose end it would stop has succeeded
             uint32_t nz = 0;
-            for (int q = grp.rank(); q < g.WM; q += grp.size()) nz |= st.par[q];
+            if (inreg) {
+#pragma unroll
+                for (int q = 0; q < kRegWords; ++q)
+                    if (q < g.WM) nz |= __reduce_xor_sync(FULLMASK, hx[q]) ^ st.sp[q];
+            } else {
+                for (int q = grp.rank(); q < g.WM; q += grp.size()) nz |= st.par[q];
+            }
             const bool gone = ab.key != nullptr && st.ab[0] != 0u;
             ok = !grp.any(nz != 0u);
             iters = t;

@@ -470,7 +470,9 @@ __global__ void k_u_gw(const float* __restrict__ gw_part, int T, int ntile, int 
 // of both passes, against HBM traffic of 20 bytes per edge, pass and shot
 // before.
 constexpr int kShots = kTileShots;
-constexpr int kTileThreads = 512;
+// the forward's row pass holds a row's messages and weights (128 registers)
+constexpr int kFwdThreads = 512;
+constexpr int kBwdThreads = 768;
 constexpr int kMaxDeg = 8;
 
 struct TileArgs {
@@ -497,7 +499,7 @@ struct TileArgs {
 __host__ __device__ inline size_t tile_smem(int M, int N, int E)
 {
     const size_t e4 = ((size_t)E + 3) & ~size_t(3);
-    return e4 * kShots * sizeof(float) + (((size_t)M + (size_t)N + 15) & ~size_t(15)) + 2 * 16 * sizeof(float) +
+    return e4 * kShots * sizeof(float) + (((size_t)M + (size_t)N + 15) & ~size_t(15)) + 2 * 32 * sizeof(float) +
            sizeof(uint16_t) * ((size_t)M + 1);
 }
 __device__ __forceinline__ float4* tile_at(float* x, int e, int half)
@@ -565,7 +567,7 @@ __device__ __forceinline__ float softplus_tail(float x)
 }
 
 template <int CAP>
-__global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const uint32_t* __restrict__ synd,
+__global__ void __launch_bounds__(kFwdThreads, 1) k_u_forward(TileArgs a, const uint32_t* __restrict__ synd,
                                                             const uint32_t* __restrict__ errs, int WM, int WN,
                                                             float* __restrict__ llr)
 {
@@ -573,8 +575,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const
     float* const x = sm;
     unsigned char* const sb = reinterpret_cast<unsigned char*>(sm + (((size_t)a.E + 3) & ~size_t(3)) * kShots);
     unsigned char* const yb = sb + a.M;
-    float* const red = reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15)));   // [2][16]
-    uint16_t* const rp = reinterpret_cast<uint16_t*>(red + 32);                                           // row_ptr
+    float* const red = reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15)));   // [2][32]
+    uint16_t* const rp = reinterpret_cast<uint16_t*>(red + 64);                                           // row_ptr
     for (int q = threadIdx.x; q <= a.M; q += blockDim.x) rp[q] = (uint16_t)__ldg(a.row_ptr + q);
     const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
@@ -721,11 +723,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const
                 }
             }
             loss = warp_sum(loss);
-            if (lane == 0) red[16 * (t & 1) + wid] = loss;
+            if (lane == 0) red[32 * (t & 1) + wid] = loss;
             __syncthreads();
             if (threadIdx.x == 0) {
                 double l = 0.0;
-                for (int k = 0; k < nw; ++k) l += (double)red[16 * (t & 1) + k];
+                for (int k = 0; k < nw; ++k) l += (double)red[32 * (t & 1) + k];
                 a.loss_part[(size_t)(t - 1) * a.ntile + tile] = (float)l;
             }
         }
@@ -734,14 +736,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_u_forward(TileArgs a, const
 }
 
 template <int CAP>
-__global__ void __launch_bounds__(kTileThreads, 1) k_u_backward(TileArgs a, const float* __restrict__ gout, double scale)
+__global__ void __launch_bounds__(kBwdThreads, 1) k_u_backward(TileArgs a, const float* __restrict__ gout, double scale)
 {
     extern __shared__ __align__(16) float sm[];
     float* const x = sm;
     unsigned char* const sb = reinterpret_cast<unsigned char*>(sm + (((size_t)a.E + 3) & ~size_t(3)) * kShots);
     unsigned char* const yb = sb + a.M;
     uint16_t* const rp = reinterpret_cast<uint16_t*>(
-        reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15))) + 32);                // row_ptr
+        reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15))) + 64);                // row_ptr
     for (int q = threadIdx.x; q <= a.M; q += blockDim.x) rp[q] = (uint16_t)__ldg(a.row_ptr + q);
     float* const part = a.gw_part + (size_t)blockIdx.x * (size_t)a.T * (size_t)a.E;
     for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
@@ -909,11 +911,11 @@ bool tile_plan(const DevGraph& g, const DecCfg& cfg, int device, long long B, in
     a.row_ptr = g.row_ptr; a.row_col = g.row_col; a.col_slot = g.tile_slots; a.lam = g.lam;
     a.M = g.M; a.N = g.N; a.E = g.E; a.T = T; a.L = cfg.L; a.B = B; a.w = w;
     a.ntile = (int)((B + kShots - 1) / kShots);
-    // a thread per four shots of a row or of two columns, at most kTileThreads;
+    // a thread per four shots of a row or of two columns, at most kFwdThreads or kBwdThreads;
     // as many blocks as fit at once, or fewer with the same number of tiles each
     const int want = std::max(2 * g.M, g.N);
-    a.threads = std::min(kTileThreads, std::max(64, (want + 31) / 32 * 32));
-    const int fit = sms * std::max(1, std::min((int)((size_t)optin / smem), kTileThreads / a.threads));
+    a.threads = std::max(64, (want + 31) / 32 * 32);
+    const int fit = sms * std::max(1, std::min((int)((size_t)optin / smem), kFwdThreads / a.threads));
     const int rounds = (a.ntile + fit - 1) / fit;
     a.blocks = (a.ntile + rounds - 1) / rounds;
     const size_t nt = (size_t)a.ntile, TM = (size_t)T * (size_t)g.M * kShots, TN = (size_t)T * (size_t)g.N * kShots;
@@ -1063,7 +1065,7 @@ int bsd_unrolled_forward(const bsd_decoder* dec, const uint32_t* d_syndromes, co
             return BSD_ERR_CUDA;
         {
             Timed tm(hk, kKindCheck);
-            kf<<<ta.blocks, ta.threads, smem, s>>>(ta, d_syndromes, d_errors, g->WM, g->WN, d_llr);
+            kf<<<ta.blocks, std::min(ta.threads, kFwdThreads), smem, s>>>(ta, d_syndromes, d_errors, g->WM, g->WN, d_llr);
         }
         Timed tm(hk, kKindOther);
         k_u_loss<<<T, 256, 0, s>>>(ta.loss_part, 1, ta.ntile, 1.0 / ((double)B * (double)g->N), d_loss);
@@ -1124,7 +1126,7 @@ int bsd_unrolled_backward(const bsd_decoder* dec, int64_t B, int32_t T, int32_t 
             return BSD_ERR_CUDA;
         {
             Timed tm(hk, kKindBVar);
-            kb<<<ta.blocks, ta.threads, smem, s>>>(ta, d_grad_loss, scale);
+            kb<<<ta.blocks, std::min(ta.threads, kBwdThreads), smem, s>>>(ta, d_grad_loss, scale);
         }
         Timed tm(hk, kKindOther);
         k_u_gw_blocks<<<1024, 128, 0, s>>>(ta.gw_part, (long long)T * g->E, ta.blocks, d_grad_weights);

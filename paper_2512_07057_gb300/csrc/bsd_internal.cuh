@@ -379,6 +379,9 @@ struct ServeBox {
 };
 int launch_serve(const DevGraph& g, const DecCfg& cfg, const LaunchShape& ls, ServeBox* box, uint32_t last,
                  unsigned long long idle_ns, void* stream);
+// plain BP on tiles of shots (bsd_unrolled.cu); 1 where it does not apply
+int launch_llr_tiles(const DevGraph& g, const DecCfg& cfg, const LaunchShape& ls, const uint32_t* synd, long long B,
+                     int T, float* llr, float* sum_llr, void* stream);
 int launch_bp_llr(const DevGraph& g, const DecCfg& cfg, const LaunchShape& ls, const uint32_t* synd,
                   long long B, int T, float* llr, float* sum_llr, void* stream);
 // single-precision re-runs of near-tie shots

@@ -3334,7 +3334,12 @@ int launch_bp_llr(const DevGraph& g, const DecCfg& cfg, const LaunchShape& ls, c
                   int T, float* llr, float* sum_llr, void* stream)
 {
     cudaStream_t s = (cudaStream_t)stream;
-    long long blocks = (B + ls.warps_per_block - 1) / ls.warps_per_block;
+    if (g.scol == nullptr) {                                 // (the single-warp engine's codes run there)
+        const int rc = launch_llr_tiles(g, cfg, ls, synd, B, T, llr, sum_llr, stream);
+        if (rc <= 0) return rc;
+    }
+    const int per_block = ls.group_warps > 1 ? 1 : ls.warps_per_block;     // candidates
+    long long blocks = (B + per_block - 1) / per_block;
     if (blocks > ls.grid_round) blocks = ls.grid_round;
     if (blocks < 1) blocks = 1;
     switch (ls.dv) {

@@ -938,6 +938,147 @@ bool tile_plan(const DevGraph& g, const DecCfg& cfg, int device, long long B, in
     return true;
 }
 
+// plain BP (Eqs. 1-3 with the scale alpha, the sums in ascending order) for T
+// iterations on the same tiles: Lambda_j(T), and the sum of Lambda_j(t) held by the
+// thread of (column, half tile) over the iterations.  For column degrees up to 3,
+// whose ordered sums need no sort.  Bound by shared memory (each message read and
+// written twice per iteration).  8192 shots of the phenomenological DEM, T = 20:
+// 2.47 ms as candidates of 16 warps, 1.08 here; the sums in memory 1.36 (3.5 GB
+// through L2), 640 threads and 9 sums 1.13, 768 and 7 1.21 (both spill).
+constexpr int kLlrThreads = 512, kLlrHeld = 11;
+
+__global__ void __launch_bounds__(kLlrThreads, 1) k_llr_tiles(TileArgs a, float alpha, const uint32_t* __restrict__ synd,
+                                                              int WM, float* __restrict__ llr,
+                                                              float* __restrict__ sum_llr)
+{
+    extern __shared__ __align__(16) float sm[];
+    float* const x = sm;
+    unsigned char* const sb = reinterpret_cast<unsigned char*>(sm + (((size_t)a.E + 3) & ~size_t(3)) * kShots);
+    uint16_t* const rp = reinterpret_cast<uint16_t*>(
+        reinterpret_cast<float*>(sb + (((size_t)a.M + (size_t)a.N + 15) & ~size_t(15))) + 64);                // row_ptr
+    for (int q = threadIdx.x; q <= a.M; q += blockDim.x) rp[q] = (uint16_t)__ldg(a.row_ptr + q);
+    for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
+        const long long b0 = (long long)tile * kShots;
+        for (int i = threadIdx.x; i < a.M; i += blockDim.x) {
+            uint32_t v = 0;
+#pragma unroll
+            for (int c = 0; c < kShots; ++c)
+                if (b0 + c < a.B) v |= ((__ldg(synd + (size_t)(b0 + c) * WM + (i >> 5)) >> (i & 31)) & 1u) << c;
+            sb[i] = (unsigned char)v;
+        }
+        for (int q = threadIdx.x; q < 2 * a.E; q += blockDim.x) {          // E(0)
+            const float v = fminf(fmaxf(__ldg(a.lam + __ldg(a.row_col + (q >> 1))), -a.L), a.L);
+            *tile_at(x, q >> 1, q & 1) = make_float4(v, v, v, v);
+        }
+        __syncthreads();
+        float4 sum[kLlrHeld];
+#pragma unroll
+        for (int r = 0; r < kLlrHeld; ++r) sum[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int t = 1; t <= a.T; ++t) {
+            for (int q = threadIdx.x; q < 2 * a.M; q += blockDim.x) {
+                const int i = q >> 1, half = q & 1;
+                const int rb = rp[i], deg = rp[i + 1] - rb;
+                const uint32_t s4 = (uint32_t)sb[i] >> (4 * half);
+                float4 v[kMaxDeg];
+#pragma unroll
+                for (int k = 0; k < kMaxDeg; ++k)
+                    v[k] = k < deg ? *tile_at(x, rb + k, half) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    // signed minima over the others from running ones from both
+                    // ends, capped at L_MAX with the syndrome sign
+                    float out[kMaxDeg];
+                    out[kMaxDeg - 1] = INFINITY;
+#pragma unroll
+                    for (int k = kMaxDeg - 1; k > 0; --k)
+                        out[k - 1] = k == kMaxDeg - 1 ? comp(v[k], c) : xmin(comp(v[k], c), out[k]);
+                    float pre = __uint_as_float(__float_as_uint(a.L) | (((s4 >> c) & 1u) << 31));
+#pragma unroll
+                    for (int k = 0; k < kMaxDeg; ++k) {
+                        const float m = k == kMaxDeg - 1 ? pre : xmin(pre, out[k]);
+                        if (k + 1 < kMaxDeg) pre = xmin(pre, comp(v[k], c));
+                        setc(v[k], c, __fmul_rn(alpha, m));
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kMaxDeg; ++k)
+                    if (k < deg) *tile_at(x, rb + k, half) = v[k];
+            }
+            __syncthreads();
+            ColumnSlots<4> en;
+            float ln = 0.f;
+            if ((int)threadIdx.x < 2 * a.N) {
+                en.load(a, threadIdx.x >> 1);
+                ln = __ldg(a.lam + (threadIdx.x >> 1));
+            }
+#pragma unroll
+            for (int r = 0; r < kLlrHeld; ++r) {
+                const int q = threadIdx.x + r * blockDim.x;
+                if (q >= 2 * a.N) break;
+                const int j = q >> 1, half = q & 1;
+                const ColumnSlots<4> e = en;
+                const float lj = ln;
+                if (q + (int)blockDim.x < 2 * a.N) {
+                    en.load(a, (q + (int)blockDim.x) >> 1);
+                    ln = __ldg(a.lam + ((q + (int)blockDim.x) >> 1));
+                }
+                const long long b = b0 + 4 * half;
+                float4 v[3];
+                int deg = 0;
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    if (e.at(k) != 0xffffu) {
+                        v[k] = *slot_at(x, e.at(k), half);
+                        deg = k + 1;
+                    }
+                float4 post = make_float4(lj, lj, lj, lj);
+                if (deg == 3) {
+                    float4 o[3];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float v0 = comp(v[0], c), v1 = comp(v[1], c), v2 = comp(v[2], c);
+                        const float lo12 = fminf(v1, v2), hi12 = fmaxf(v1, v2);
+                        const float lo02 = fminf(v0, v2), hi02 = fmaxf(v0, v2);
+                        const float lo01 = fminf(v0, v1), hi01 = fmaxf(v0, v1);
+                        setc(o[0], c, __fadd_rn(__fadd_rn(lj, lo12), hi12));
+                        setc(o[1], c, __fadd_rn(__fadd_rn(lj, lo02), hi02));
+                        setc(o[2], c, __fadd_rn(__fadd_rn(lj, lo01), hi01));
+                        // smallest, median (the least of the pair maxima), largest
+                        const float mid = fminf(hi01, fminf(hi02, hi12));
+                        setc(post, c, __fadd_rn(__fadd_rn(__fadd_rn(lj, fminf(lo01, v2)), mid), fmaxf(hi01, v2)));
+                    }
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) *slot_at(x, e.at(k), half) = o[k];
+                } else if (deg == 2) {
+                    float4 o[2];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float v0 = comp(v[0], c), v1 = comp(v[1], c);
+                        setc(o[0], c, __fadd_rn(lj, v1));
+                        setc(o[1], c, __fadd_rn(lj, v0));
+                        setc(post, c, __fadd_rn(__fadd_rn(lj, fminf(v0, v1)), fmaxf(v0, v1)));
+                    }
+                    *slot_at(x, e.at(0), half) = o[0];
+                    *slot_at(x, e.at(1), half) = o[1];
+                } else if (deg == 1) {
+                    *slot_at(x, e.at(0), half) = post;
+                    post = make_float4(__fadd_rn(lj, v[0].x), __fadd_rn(lj, v[0].y), __fadd_rn(lj, v[0].z),
+                                       __fadd_rn(lj, v[0].w));
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    setc(sum[r], c, __fadd_rn(comp(sum[r], c), comp(post, c)));
+                    if (t != a.T || b + c >= a.B) continue;
+                    const size_t at = (size_t)(b + c) * (size_t)a.N + j;
+                    llr[at] = comp(post, c);
+                    if (sum_llr) sum_llr[at] = comp(sum[r], c);
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // register cache for rows / columns of degree at most 4 or 8, none beyond
 int cap_of(int max_deg) { return max_deg <= 4 ? 4 : (max_deg <= 8 ? 8 : 0); }
 
@@ -1019,6 +1160,35 @@ void launch_var(const UArgs& a, const DevGraph& g, const float* D, float* Eout, 
 }
 
 }  // namespace
+
+// plain BP on tiles of shots where it applies: single precision, no weights, rows
+// of at most 8 and columns of at most 3 edges, the tile in shared memory; 1 where
+// not.  A wave of tiles takes the time of one tile: against candidates of one warp
+// each (864 columns, T = 20) 82 us for any batch up to 8 per SM where they take
+// 290-350; a candidate of 16 warps (2592 columns) is done sooner while each SM has
+// at most two, 66-98 us against 150, and later from three on, 187.
+int launch_llr_tiles(const DevGraph& g, const DecCfg& cfg, const LaunchShape& ls, const uint32_t* synd, long long B, int T, float* llr,
+                     float* sum_llr, void* stream)
+{
+    int device = 0, optin = 0, sms = 0;
+    const size_t smem = tile_smem(g.M, g.N, g.E);
+    if (g.prec != 0 || cfg.weights != nullptr || g.max_row_deg > kMaxDeg || g.max_row_deg < 1 || g.max_col_deg > 3 ||
+        g.tile_slots == nullptr || cudaGetDevice(&device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || smem > (size_t)optin ||
+        (ls.group_warps > 1 && B < 3ll * sms))
+        return 1;
+    TileArgs a{};
+    a.row_ptr = g.row_ptr; a.row_col = g.row_col; a.col_slot = g.tile_slots; a.lam = g.lam;
+    a.M = g.M; a.N = g.N; a.E = g.E; a.T = T; a.L = cfg.L; a.B = B;
+    a.ntile = (int)((B + kShots - 1) / kShots);
+    if (CUDA_FAILED(cudaFuncSetAttribute(k_llr_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return -2;
+    const int threads = std::min(kLlrThreads, std::max(64, (std::max(2 * g.M, g.N) + 31) / 32 * 32));
+    const int fit = sms * std::max(1, std::min((int)((size_t)optin / smem), kLlrThreads / threads));
+    if (2ll * g.N > (long long)kLlrHeld * threads) return 1;
+    k_llr_tiles<<<std::min(a.ntile, fit), threads, smem, (cudaStream_t)stream>>>(a, cfg.alpha, synd, g.WM, llr, sum_llr);
+    return CUDA_FAILED(cudaGetLastError()) ? -2 : 0;
+}
 }  // namespace bsd
 
 using namespace bsd;

@@ -107,9 +107,11 @@ typedef struct {
                                   with the scale alpha and num_results = 1: the seed BP of many
                                   shots runs at once over this many slots, messages streamed
                                   through device memory with the shots contiguous; 0 the library
-                                  default (codes of at least 16384 edges: 2048 slots; smaller
-                                  codes: none), -1 never, else 256..65536 (rounded
-                                  down to a multiple of 256); at most a quarter of the workspace;
+                                  default (codes of at least 16384 edges: 2048 slots, run when at
+                                  least 65536 shots of a chunk wait for a seed BP; smaller
+                                  codes: none), -1 never, else 256..65536 (rounded down to a
+                                  multiple of 256; any number of shots); at most a quarter of
+                                  the workspace;
                                   results do not depend on it */
 } bsd_params;
 
@@ -247,7 +249,8 @@ int bsd_bp_llr(bsd_decoder *dec, const uint32_t *d_syndromes, int64_t B, int32_t
 int bsd_sync_error(bsd_decoder *dec);
 
 /* Sizes and launch shape: any pointer may be NULL.  chunk_shots is the
- * number of shots decoded per internal pass (bounded by the workspace). */
+ * size of the seed store, the shots with a failing seed BP that are decoded per
+ * internal pass (bounded by the workspace). */
 int bsd_get_info(const bsd_decoder *dec, int32_t *M, int32_t *N, int32_t *K, int32_t *n_edges,
                  int64_t *chunk_shots, int64_t *workspace_bytes);
 
@@ -257,16 +260,17 @@ int bsd_get_info(const bsd_decoder *dec, int32_t *M, int32_t *N, int32_t *K, int
  * launch shape uses them.  Any pointer may be NULL. */
 int bsd_get_batch(const bsd_decoder *dec, int32_t *slots, int32_t *active);
 
-/* Where the single-warp engine keeps a candidate's messages in shared memory
+/* A conflict-free placement of a candidate's messages in shared memory
  * (a layout choice of this library; the paper's Eqs. 1-3 do not depend on
  * it).  For codes with every row of degree 6 and every column of degree 3
  * (the bivariate bicycle codes) the pair h of row i is at word plane[h] + 2 i
  * with plane[h] = h (64 ceil(M / 32) + 12), and the error-node pass reads the
  * k-th edge of column j at col_word[3 j + k].
  * The rows' edge orders and the columns' k orders are searched so that both
- * passes touch 32 distinct banks per access; bsd_create builds the same
- * placement for codes of at most 160 columns and 96 rows.  Host only; nothing
- * is allocated on a device.
+ * passes touch 32 distinct banks per access.  The engine of codes of at most
+ * 160 columns and 96 rows uses the same words; its own placement also deals the
+ * columns to the lanes, so that a warp can keep a third of the messages in
+ * registers.  Host only; nothing is allocated on a device.
  *   M, N, H_row_ptr, H_col_idx  host, H in CSR as for bsd_create
  *   plane      host int32[3]: out, the plane bases
  *   edge_word  host int32[E]: out, the word of CSR edge e (E = H_row_ptr[M])
@@ -284,7 +288,9 @@ int bsd_small_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32
  * edges permuted inside the row's storage window, each column's edges in the
  * k slots of the padded column table (colK = 3 for a largest column degree of
  * 3 or less, else 6), chosen so that the 32 lanes of an error-pass access
- * meet distinct banks where possible.  bsd_create builds the same placement.
+ * meet distinct banks where possible.  bsd_create runs the same search over the
+ * storage of its engine for these codes, where the rows stand by falling degree
+ * with their k-th edges side by side.
  * Host only; nothing is allocated on a device.
  *   M, N, H_row_ptr, H_col_idx  host, H in CSR as for bsd_create
  *   edge_word  host int32[E]: out, the element of CSR edge e
@@ -308,14 +314,17 @@ int bsd_profile_enable(bsd_decoder *dec, int enable);
  * read: the summed event-timed duration in milliseconds and the launch count
  * of each kernel kind (index 0: seed BP, 1: the beam -- expand, masked BP and
  * selection of every round, 2: the beam's set-up), the full BP iterations executed on the
- * device (index 0: seed candidates, 1: round candidates, counting children
+ * device (index 0: seed candidates, two for each run that the second screen below
+ * ends, 1: round candidates, counting children
  * evaluated after a shot's first success, 2: the part of index 0 run by the
  * batched seed BP of bsd_params.batch_slots), the number of kernels of this
  * library that ran for this decoder (counted on the device, with or without
  * timing enabled), and the message updates done by first-iteration screens
  * of seed runs (with every Lambda_j > 0, the scale alpha and one result, a
  * seed run first forms e^(1) from the columns next to flipped detectors
- * only, since no other column can flip at t = 1; a run that converges there
+ * only, since no other column can flip at t = 1, and for sparse syndromes a
+ * second screen forms e^(2) from those that can flip at t = 2; a run that
+ * converges there
  * ends after that partial iteration, which is counted here and not as a full
  * iteration).  While timing is enabled the kernels are launched one by one so
  * that events can bracket them; otherwise each chunk runs as one CUDA graph.
@@ -325,10 +334,11 @@ int bsd_profile_read(bsd_decoder *dec, double ms[3], int64_t launches[3], uint64
 
 /* Kernel kinds timed while timing is enabled: 0..2 as above, then the
  * unrolled decoder's passes (bsd_unrolled_forward / _backward): 3 check pass,
- * 4 error-node pass, 5 error-node adjoint, 6 check adjoint, 7 its other
+ * 4 error-node pass, 5 error-node adjoint, 6 check adjoint (on tiles of shots, where
+ * the code allows it, 3 is the whole forward and 5 the whole backward), 7 its other
  * kernels (bit planes, initial messages, loss and gradient reductions), then
  * the batched seed BP: 8 its check pass, 9 its error-node pass, 10 its
- * stopping test and refill, and 11 the first-iteration screen of seed runs. */
+ * stopping test and refill, and 11 the screens of seed runs. */
 #define BSD_PROFILE_KINDS 12
 
 /* Synchronise the stream of the last timed launch, then return and reset the

@@ -2,10 +2,10 @@
 //
 // One warp owns one BP candidate (the seed path of a shot, or one child of a
 // beam round) and keeps its whole state in shared memory: the edge messages
-// E_{j->i}, a compact 8-byte per-detector record (min1, min2 with the sign
-// parity in both sign bits) standing in for the detector-to-error messages
-// D_{i->j} (the single-warp engine keeps D per edge instead), sum_LLR, and
-// the bit vectors s', mask, vals, e^ and the running syndrome parity.
+// E_{j->i}, over which the single-warp and jagged engines write the
+// detector-to-error messages D_{i->j} and back (the generic engine keeps a
+// compact 8-byte per-detector record, min1 and min2 with the sign parity in both
+// sign bits, in D's place), sum_LLR, and the bit vectors s', mask, vals, e^ and the running syndrome parity.
 //
 // Kernels (all persistent: warps claim work with one atomic per item and
 // exit when the item counter runs out, so uneven iteration counts balance):

@@ -1,9 +1,9 @@
 // bsd_layout.cu -- where the BP engines keep each edge's messages in shared
 // memory (host code, run once when a decoder is created).
 //
-// Generic engines (column degree bound 3 or 6; generic_layout): a row's
-// edges occupy the row's window [row_ptr[i], row_ptr[i + 1]) in any order
-// (the detector pass reduces the window with order-independent operations),
+// Jagged engine (column degree bound 3 or 6; generic_layout): a row's
+// edges occupy the row's places (given by the caller) in any order (the detector
+// pass reduces them with order-independent operations),
 // and a column's edges may take any k slots of the padded column table (the
 // error pass sorts its inputs).  A local search over swaps within rows
 // spreads each group of 32 columns over the banks (at most the group's
@@ -12,7 +12,9 @@
 // search leaves a bank above that, each edge takes the free slot whose bank
 // is least loaded.  Columns may keep holes in their slots.
 //
-// Single-warp engine (small_layout):
+// Single-warp engine: small_local_layout (described there) deals the columns to the
+// lanes; small_layout, an earlier placement of the same words with the columns in
+// their own order, is exported for inspection and described here:
 //
 // The single-warp engine (codes with every row of degree 6 and every column of
 // degree 3) runs two passes per BP iteration over a candidate's messages in

@@ -6,6 +6,10 @@
 //     loss = sum_{t=1..T} mean_{b,j} BCE(sigmoid(-Lambda_j(t)), e_j)
 // with respect to the weights.
 //
+// Codes with rows and columns of at most 8 edges whose messages fit in shared
+// memory for 8 shots run on chip, one block per tile of shots (described at
+// kShots below).  The other codes run the passes described here.
+//
 // Layout: every per-edge array is [E][Bp] and every per-node array [N][Bp]
 // (shots contiguous; Bp = B rounded up to the 512-shot tile of a block), so a
 // warp's 32 threads x 4 shots move 512 contiguous bytes of one edge.  The
@@ -470,7 +474,9 @@ __global__ void k_u_gw(const float* __restrict__ gw_part, int T, int ntile, int 
 // of both passes, against HBM traffic of 20 bytes per edge, pass and shot
 // before.
 constexpr int kShots = kTileShots;
-// the forward's row pass holds a row's messages and weights (128 registers)
+// the forward's row pass holds a row's messages and weights (128 registers; 640
+// threads spill: 1.24 against 1.21 ms at B = 4096, T = 20 on the phenomenological
+// DEM); the backward fits in 80 (512 threads 1.64 ms, 640 1.49, 768 1.47, 1024 1.57)
 constexpr int kFwdThreads = 512;
 constexpr int kBwdThreads = 768;
 constexpr int kMaxDeg = 8;

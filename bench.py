@@ -471,6 +471,10 @@ def alu_roofline(prof, E: int, dev: int, traffic_case: str, shots: int = 0, msg_
     dom_kind, name, updates = max(cands, key=lambda c: kinds_ms[c[0]])
     launches = max(1, int(kinds_ln[dom_kind]))
     ms_launch = float(kinds_ms[dom_kind]) / launches
+    if name == "k_seed" and kinds_ln[11] > 0:
+        # the runs that the second screen ends are counted with the seed iterations (two each): one stage
+        name, updates = "k_screen+k_seed", updates + screen
+        ms_launch += float(kinds_ms[11]) / launches
     upd_launch = updates / launches
     ops_tops = OPS_PER_UPDATE * upd_launch / (ms_launch * 1e-3) / 1e12
     share = float(kinds_ms[dom_kind] / max(kinds_ms[[0, 1, 2, 8, 9, 10, 11]].sum(), 1e-9))
@@ -493,8 +497,9 @@ def alu_roofline(prof, E: int, dev: int, traffic_case: str, shots: int = 0, msg_
         roofline = {"bound": "alu", "achieved": ops_tops, "peak": alu_peak_tops, "unit": "Tops/s",
                     "frac": ops_tops / alu_peak_tops, "traffic": None,
                     "peak_source": f"{sms} SMs x {LANES_PER_SM} lanes x {sm_mhz_max:.0f} MHz (sm_max_mhz {pk_kind})",
-                    "msg_updates_counted": "full BP iterations x E (k_seed, k_round) or the edges the "
-                                           "first-iteration screens formed (k_screen)", **common}
+                    "msg_updates_counted": "full BP iterations x E (k_seed, k_round; two for a seed run that "
+                                           "the second screen ends) and the edges the first screen formed",
+                    **common}
     # DRAM bytes per unit of work from an ncu capture of a smaller case
     # (profiles/), scaled to this run's average launch; null once the kernel
     # sources differ from the ones that were captured
@@ -959,19 +964,28 @@ def run_unrolled(args, rank: int, world: int, local_rank: int):
         ms_total = float(t.item())
     E, N, M = prob.n_edges, prob.N, prob.M
     Bp = (Bn + 511) // 512 * 512
-    names = {3: "k_u_check", 4: "k_u_var", 5: "k_u_bvar", 6: "k_u_bcheck"}
+    # on tiles of shots the whole forward and the whole backward are one kernel each
+    tiled = int(prof["launches"][4]) == 0
+    names = {3: "k_u_forward", 5: "k_u_backward"} if tiled else \
+            {3: "k_u_check", 4: "k_u_var", 5: "k_u_bvar", 6: "k_u_bcheck"}
     per_kind = {names[kd]: {"ms_per_step": float(prof["ms"][kd]) / args.steps,
                             "launches_per_step": float(prof["launches"][kd]) / args.steps} for kd in names}
     dom = max(names, key=lambda kd: prof["ms"][kd])
     launch_ms = float(prof["ms"][dom]) / max(1, int(prof["launches"][dom]))
-    alg = unrolled_bytes_per_launch(dom, E, N, M, Bp, T)
     pk, pk_kind = peaks()
-    hbm = float(pk.get("hbm_gbs", 6800.0))
+    if tiled:
+        # both kernels read and write every message twice per iteration in shared memory (128 bytes per clock and SM)
+        alg = 16.0 * E * Bn * T
+        sms = torch.cuda.get_device_properties(dev).multi_processor_count
+        peak, bound, source = sms * 128 * 2.07, "shared memory", f"{sms} SMs x 128 B x 2070 MHz"
+    else:
+        alg = unrolled_bytes_per_launch(dom, E, N, M, Bp, T)
+        peak, bound, source = float(pk.get("hbm_gbs", 6800.0)), "hbm", f"hbm_gbs ({pk_kind})"
     achieved = alg / (launch_ms * 1e-3) / 1e9
-    roofline = {"kernel": names[dom], "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
-                "frac": achieved / hbm, "traffic": None, "algorithmic_bytes_per_launch": alg, "launch_ms": launch_ms,
+    roofline = {"kernel": names[dom], "bound": bound, "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak, "traffic": None, "algorithmic_bytes_per_launch": alg, "launch_ms": launch_ms,
                 "kernel_share": float(prof["ms"][dom] / max(prof["ms"][3:7].sum(), 1e-9)),
-                "peak_source": f"hbm_gbs ({pk_kind})",
+                "peak_source": source,
                 "measured_in": "second timed region: same steps, each pass launched between CUDA events"}
     tr_rec = _traffic_record(names[dom], E)
     if tr_rec is not None and tr_rec[1] == "launch":
@@ -980,8 +994,8 @@ def run_unrolled(args, rank: int, world: int, local_rank: int):
                                      "the launches of one training step of this workload"
     steps_s = ms_total * 1e-3
     value = world * Bn * args.steps / steps_s
-    # edge updates: forward T iterations, the recomputed T, the adjoint T (check + error pass each)
-    upd = 3.0 * T * E * Bn
+    # edge updates: forward T iterations, the recomputed T (passes only), the adjoint T (check + error pass each)
+    upd = (2.0 if tiled else 3.0) * T * E * Bn
     line = {
         "metric": METRIC, "value": value, "unit": "training syndromes/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_total / args.steps, "higher_is_better": True, "scaling": "weak",
@@ -992,13 +1006,11 @@ def run_unrolled(args, rank: int, world: int, local_rank: int):
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "edge_updates_per_s": world * upd * args.steps / steps_s,
         "kernels": per_kind, "roofline": roofline, "clocks": clocks,
-        # per step: forward 2 bit-plane + 1 initial-message + T check + T error + 1 loss kernels; backward
-        # T recomputed check + T recomputed error + T error-adjoint + T check-adjoint + 1 gradient kernels
-        "gpu_launches": (6 * T + 5) * args.steps,
-        "timed_launches_per_step": {"check": float(prof["launches"][3]) / args.steps,
-                                    "error": float(prof["launches"][4]) / args.steps,
-                                    "error_adjoint": float(prof["launches"][5]) / args.steps,
-                                    "check_adjoint": float(prof["launches"][6]) / args.steps},
+        # per step, on tiles: forward, two loss reductions, backward, gradient reduction; on passes: forward
+        # 2 bit-plane + 1 initial-message + T check + T error + 1 loss kernels; backward T recomputed check +
+        # T recomputed error + T error-adjoint + T check-adjoint + 1 gradient kernels
+        "gpu_launches": (5 if tiled else 6 * T + 5) * args.steps,
+        "timed_launches_per_step": {names[kd]: float(prof["launches"][kd]) / args.steps for kd in names},
     }
     if rank == 0 and not args.no_e2e:
         line["e2e"] = _unrolled_e2e(tr, w, opt, prob, Bn, args, dev)

@@ -232,13 +232,6 @@ struct __align__(16) BeamEntry {
     int stamp;             // of the round, never 0, grows over the shots of the entry
 };
 
-// an item of the ring: child c (< 2w <= 128) of window entry a, never one of
-// the two marks
-constexpr uint32_t kRingEmpty = 0u;
-constexpr uint32_t kRingLeft = 0xffffffffu;   // the group that held this slot's ticket has left
-__host__ __device__ inline uint32_t ring_item(int a, int c) { return (((uint32_t)a << 7) | (uint32_t)c) + 1u; }
-__host__ __device__ inline int ring_entry(uint32_t it) { return (int)((it - 1u) >> 7); }
-__host__ __device__ inline int ring_child(uint32_t it) { return (int)((it - 1u) & 127u); }
 // window entries in use at once: enough that the items of their shots (two in
 // the first round, up to 2w later) keep every candidate group busy
 constexpr long long kBeamEntries = 4096;

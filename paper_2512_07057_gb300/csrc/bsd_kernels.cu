@@ -43,6 +43,7 @@
 
 #include "bsd_device.cuh"
 #include "bsd_internal.cuh"
+#include "bsd_ring.cuh"
 
 namespace bsd {
 
@@ -108,7 +109,13 @@ struct WarpGroup {
         __syncwarp();
         return r;
     }
-    __device__ __forceinline__ int bcast(int v) const { return __shfl_sync(FULLMASK, v, 0); }
+    // (a shuffle passes the value, the barrier what lane 0 has seen before it)
+    __device__ __forceinline__ int bcast(int v) const
+    {
+        const int r = __shfl_sync(FULLMASK, v, 0);
+        __syncwarp();
+        return r;
+    }
     __device__ __forceinline__ uint32_t xor_all(uint32_t v) const
     {
 #pragma unroll
@@ -2159,18 +2166,10 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_seed(DevG
 // GPU idle: 10^6 [[144,12,12]] shots at p = 0.05 took 280 launches of 21.3 ms
 // in all.)
 //
-// The ring: a group draws a ticket (b_head) and waits for the item that will
-// be put at it (b_tail).  An item is exchanged in and out of its slot, so a
-// slot still full when the ring has come round gives its item back to the
-// pusher, which pushes it again; a group that has waited kIdleNs leaves
-// and marks its ticket's slot, and the pusher that meets the mark pushes its
-// item again too.  (Each group holds one ticket at most and there are no more
-// groups than slots, so a ticket's pusher has come and taken the mark back before
-// the slot's next ticket is drawn.)  No item is lost, no wait is unbounded, and
-// the running groups alone finish the work, so nothing rests on two groups being
-// resident at once.
-constexpr unsigned long long kIdleNs = 1000ull * 1000 * 1000;
-
+// The ring (bsd_ring.cuh): a group draws a ticket and waits for the item that will
+// be put at its slot; it draws the next one when its child, and the selection after
+// it, are done.  The running groups alone finish the work: a group that has waited a
+// second without an item leaves.
 // orders this thread's memory operations, and those of the threads it has
 // synchronised with, before and after an atomic that passes them on
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
@@ -2188,40 +2187,24 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+struct GpuRing {
+    static __device__ __forceinline__ uint32_t add(uint32_t* p, uint32_t v) { return atomicAdd(p, v); }
+    static __device__ __forceinline__ uint32_t cas(uint32_t* p, uint32_t want, uint32_t v) { return atomicCAS(p, want, v); }
+    static __device__ __forceinline__ uint32_t and_(uint32_t* p, uint32_t v) { return atomicAnd(p, v); }
+    static __device__ __forceinline__ uint32_t load(const uint32_t* p) { return ld_relaxed(p); }
+    static __device__ __forceinline__ void pause() { __nanosleep(200); }
+    static __device__ __forceinline__ unsigned long long now() { return global_ns(); }
+};
+
 __device__ inline void push_item(const Work& w, uint32_t item)
 {
-    for (;;) {
-        uint32_t* slot = w.ring + (atomicAdd(&w.ctr->b_tail, 1u) & w.ctr->b_mask);
-        const uint32_t old = atomicExch(slot, item);
-        if (old == kRingEmpty) return;
-        if (old == kRingLeft) {
-            // this ticket's group has left: take the item back unless the
-            // ring's next lap has drawn it already
-            if (atomicCAS(slot, item, kRingEmpty) != item) return;
-        } else {
-            item = old;                        // an item of the lap before, not drawn yet
-        }
-    }
+    ring_push<GpuRing>(w.ring, &w.ctr->b_tail, w.ctr->b_mask, item);
 }
 
-// the item of a ticket, or kRingEmpty when every shot has ended (or none came for
-// kIdleNs)
 __device__ inline uint32_t draw_item(const Work& w, uint32_t ticket)
 {
-    uint32_t* slot = w.ring + (ticket & w.ctr->b_mask);
-    uint32_t it = atomicExch(slot, kRingEmpty);
-    unsigned long long t0 = 0ull;
-    for (unsigned spins = 0; it == kRingEmpty; ++spins) {
-        if ((spins & 3u) == 0u && ld_relaxed(reinterpret_cast<const uint32_t*>(&w.ctr->b_left)) == 0u) return kRingEmpty;
-        if (spins >= 4u) __nanosleep(200);
-        if ((spins & 63u) == 0u) {
-            const unsigned long long t = global_ns();
-            if (t0 == 0ull) t0 = t;
-            else if (t - t0 > kIdleNs && atomicCAS(slot, kRingEmpty, kRingLeft) == kRingEmpty) return kRingEmpty;
-        }
-        if (ld_relaxed(slot) != kRingEmpty) it = atomicExch(slot, kRingEmpty);
-    }
-    fence_gpu();                               // the item before what it names
+    const uint32_t it = ring_draw<GpuRing>(w.ring, w.ctr->b_mask, reinterpret_cast<const uint32_t*>(&w.ctr->b_left), ticket);
+    if (it != kRingEmpty) fence_gpu();         // the item before what it names
     return it;
 }
 
@@ -2543,11 +2526,9 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(Dev
     if ((uint32_t)(blockIdx.x * grp.per_block() + grp.index()) > w.ctr->b_mask) return;
     const int W2 = 2 * cfg.w;
     unsigned long long ran = 0;                // BP iterations (group rank 0)
-    uint32_t ticket = 0;                       // the next item's (group rank 0)
-    if (grp.rank() == 0) ticket = atomicAdd(&w.ctr->b_head, 1u);
     for (;;) {
         uint32_t item = kRingEmpty;
-        if (grp.rank() == 0) item = draw_item(w, ticket);
+        if (grp.rank() == 0) item = draw_item(w, atomicAdd(&w.ctr->b_head, 1u));
         item = (uint32_t)grp.bcast((int)item);
         if (item == kRingEmpty) break;
         const int a = ring_entry(item), c = ring_child(item);
@@ -2631,12 +2612,10 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_round(Dev
                 }
             }
         }
-        // the slot before the count; the round's last child selects (the next
-        // ticket is drawn on the way)
+        // the slot before the count; the round's last child selects
         grp.sync();
         int last = 0;
         if (grp.rank() == 0) {
-            ticket = atomicAdd(&w.ctr->b_head, 1u);
             fence_gpu();
             last = atomicSub(&w.ent[a].pending, 1) == 1 ? 1 : 0;
             if (last) fence_gpu();

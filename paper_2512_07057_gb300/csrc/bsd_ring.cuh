@@ -1,0 +1,98 @@
+// bsd_ring.cuh -- the ring of beam items: how candidate groups pass children on.
+//
+// Written over a policy Ops (atomics, a relaxed load, a pause, a clock), so that
+// the host can run the same code in any interleaving; the kernels use GpuRing
+// (bsd_kernels.cu).
+//
+// A group draws a ticket (one add to the head) and waits at the ticket's slot; a
+// pusher takes the next ticket of the tail and puts its item there.  An item is
+// whatever comes first at a slot: tickets of several laps may wait at one slot
+// while a pusher is between its two steps, and items are interchangeable.  What
+// must hold is the count: every ticket drawn is matched by one push, or cancelled
+// by one mark.
+//   * A group that has waited kIdleNs leaves: it puts the mark kRingLeft into its
+//     empty slot.  The pusher that meets the mark takes it away and pushes its
+//     item at another ticket.  A group of a later lap that meets the mark leaves it
+//     (atomicAnd takes an item and keeps a mark).
+//   * A pusher never puts an item over another one: it waits for the slot's group.
+//     That group only has to take the item, since no group holds a ticket while it
+//     selects or pushes (an item undrawn has a group: at most as many items are
+//     undrawn as the ring has slots, so the ticket one lap before the pusher's has
+//     been drawn).  A group that held a ticket while it pushed would make the
+//     pusher wait for it; one that put its item over the other and pushed that
+//     again would leave one group at the slot waiting for ever.
+// No item is lost and no wait is unbounded.
+#pragma once
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define BSD_RING_FN __host__ __device__ __forceinline__
+#define BSD_RING_DEV __device__ __forceinline__
+#else
+#define BSD_RING_FN inline
+#define BSD_RING_DEV inline
+#endif
+
+namespace bsd {
+
+// an item of the ring: child c (< 2w <= 128) of window entry a (< 2^20), never
+// one of the two marks
+constexpr uint32_t kRingEmpty = 0u;
+constexpr uint32_t kRingLeft = 0x80000000u;   // the group that held this slot's ticket has left
+BSD_RING_FN uint32_t ring_item(int a, int c) { return (((uint32_t)a << 7) | (uint32_t)c) + 1u; }
+BSD_RING_FN int ring_entry(uint32_t it) { return (int)((it - 1u) >> 7); }
+BSD_RING_FN int ring_child(uint32_t it) { return (int)((it - 1u) & 127u); }
+BSD_RING_FN bool ring_has_item(uint32_t v) { return (v & ~kRingLeft) != 0u; }
+
+constexpr unsigned long long kIdleNs = 1000ull * 1000 * 1000;
+constexpr unsigned long long kStuckNs = 16ull * kIdleNs;   // past any wait that can come about
+
+template <class Ops>
+BSD_RING_DEV void ring_push(uint32_t* ring, uint32_t* tail, uint32_t mask, uint32_t item)
+{
+    for (;;) {
+        uint32_t* const slot = ring + (Ops::add(tail, 1u) & mask);
+        uint32_t want = kRingEmpty;
+        unsigned long long t0 = 0ull;
+        for (;;) {
+            const uint32_t old = Ops::cas(slot, want, want == kRingLeft ? kRingEmpty : item);
+            if (old == want) {
+                if (want == kRingEmpty) return;
+                if (want != kRingLeft) item = want;            // (past kStuckNs: pushed in its place)
+                break;
+            }
+            want = old == kRingLeft ? kRingLeft : kRingEmpty;
+            if (ring_has_item(old)) {                          // its group is about to take it
+                Ops::pause();
+                const unsigned long long t = Ops::now();
+                if (t0 == 0ull) t0 = t;
+                else if (t - t0 > kStuckNs) want = old;
+            }
+        }
+    }
+}
+
+// the item of a ticket, or kRingEmpty when every shot has ended (*left = 0) or
+// none came for kIdleNs
+template <class Ops>
+BSD_RING_DEV uint32_t ring_draw(uint32_t* ring, uint32_t mask, const uint32_t* left, uint32_t ticket)
+{
+    uint32_t* const slot = ring + (ticket & mask);
+    uint32_t it = Ops::and_(slot, kRingLeft);
+    unsigned long long t0 = 0ull;
+    for (unsigned spins = 0; !ring_has_item(it); ++spins) {
+        if ((spins & 3u) == 0u && Ops::load(left) == 0u) return kRingEmpty;
+        if (spins >= 4u) Ops::pause();
+        if ((spins & 63u) == 0u) {
+            const unsigned long long t = Ops::now();
+            if (t0 == 0ull) t0 = t;
+            else if (t - t0 > kIdleNs && (Ops::cas(slot, kRingEmpty, kRingLeft) == kRingEmpty || t - t0 > kStuckNs))
+                return kRingEmpty;
+        }
+        it = Ops::load(slot);
+        if (ring_has_item(it)) it = Ops::and_(slot, kRingLeft);
+    }
+    return it;
+}
+
+}  // namespace bsd

@@ -53,6 +53,7 @@ struct DevGraph {
     int all_lam_pos;       // every Lambda_j > 0 (all p_j < 1/2)
     int det_bytes;         // per-warp detector-side shared memory (set with the engine)
     int e_bytes;           // bytes of a message in shared memory (set with the engine)
+    int sms, max_smem;     // the device's SMs and largest dynamic shared memory of a block (likewise)
     const int* row_ptr;
     const int* row_col;    // [E] column of CSR edge e
     const int* col_ptr;

@@ -2768,6 +2768,8 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     if (CUDA_FAILED(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device)) ||
         CUDA_FAILED(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)))
         return -2;
+    g.sms = sms;
+    g.max_smem = max_optin;
     // per-candidate state: the jagged engine keeps float messages, D over E;
     // the generic one the stored format and a record per detector
     g.e_bytes = gkind < 2 ? (int)sizeof(float) : g.msg_bytes;
@@ -3290,7 +3292,8 @@ static int launch_serve_t(const DevGraph& g, const DecCfg& cfg, const LaunchShap
 {
     const bool block = ls.group_warps >= 2;
     const size_t smem = block ? ls.smem_bp : warp_smem_bytes(g);
-    if (CUDA_FAILED(cudaFuncSetAttribute(k_serve<Eng>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+    // (the device maximum: see configure_kernels)
+    if (CUDA_FAILED(cudaFuncSetAttribute(k_serve<Eng>, cudaFuncAttributeMaxDynamicSharedMemorySize, g.max_smem)))
         return -2;
     k_serve<Eng><<<1, 32 * (block ? ls.group_warps : 1), smem, s>>>(g, cfg, box, last, idle_ns);
     return CUDA_FAILED(cudaGetLastError()) ? -2 : 0;

@@ -901,18 +901,24 @@ __global__ void k_u_gw_blocks(const float* __restrict__ part, long long n, int b
     }
 }
 
+// the limit belongs to the kernel, not to a decoder: always the device maximum, so
+// that a thread with a smaller code does not lower it between another's call and
+// its launch
+template <class F>
+bool allow_smem(const DevGraph& g, F* kernel)
+{
+    return !CUDA_FAILED(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g.max_smem));
+}
+
 // the tiled path's arrays in the caller's workspace; false where a degree, the
 // shared memory or the workspace (whose size the general passes set) does not
 // allow it
-bool tile_plan(const DevGraph& g, const DecCfg& cfg, int device, long long B, int T, const float* w, char* base,
+bool tile_plan(const DevGraph& g, const DecCfg& cfg, long long B, int T, const float* w, char* base,
                size_t have, TileArgs* out)
 {
     if (g.max_row_deg > kMaxDeg || g.tile_slots == nullptr || g.E > 65528 || g.max_row_deg < 1) return false;
     const size_t smem = tile_smem(g.M, g.N, g.E);
-    int optin = 0, sms = 0;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || smem > (size_t)optin)
-        return false;
+    if (smem > (size_t)g.max_smem) return false;
     TileArgs a{};
     a.row_ptr = g.row_ptr; a.row_col = g.row_col; a.col_slot = g.tile_slots; a.lam = g.lam;
     a.M = g.M; a.N = g.N; a.E = g.E; a.T = T; a.L = cfg.L; a.B = B; a.w = w;
@@ -921,7 +927,7 @@ bool tile_plan(const DevGraph& g, const DecCfg& cfg, int device, long long B, in
     // as many blocks as fit at once, or fewer with the same number of tiles each
     const int want = std::max(2 * g.M, g.N);
     a.threads = std::max(64, (want + 31) / 32 * 32);
-    const int fit = sms * std::max(1, std::min((int)((size_t)optin / smem), kFwdThreads / a.threads));
+    const int fit = g.sms * std::max(1, std::min((int)((size_t)g.max_smem / smem), kFwdThreads / a.threads));
     const int rounds = (a.ntile + fit - 1) / fit;
     a.blocks = (a.ntile + rounds - 1) / rounds;
     const size_t nt = (size_t)a.ntile, TM = (size_t)T * (size_t)g.M * kShots, TN = (size_t)T * (size_t)g.N * kShots;
@@ -1176,22 +1182,18 @@ void launch_var(const UArgs& a, const DevGraph& g, const float* D, float* Eout, 
 int launch_llr_tiles(const DevGraph& g, const DecCfg& cfg, const LaunchShape& ls, const uint32_t* synd, long long B, int T, float* llr,
                      float* sum_llr, void* stream)
 {
-    int device = 0, optin = 0, sms = 0;
     const size_t smem = tile_smem(g.M, g.N, g.E);
     if (g.prec != 0 || cfg.weights != nullptr || g.max_row_deg > kMaxDeg || g.max_row_deg < 1 || g.max_col_deg > 3 ||
-        g.tile_slots == nullptr || cudaGetDevice(&device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || smem > (size_t)optin ||
-        (ls.group_warps > 1 && B < 3ll * sms))
+        g.tile_slots == nullptr || smem > (size_t)g.max_smem || (ls.group_warps > 1 && B < 3ll * g.sms))
         return 1;
     TileArgs a{};
     a.row_ptr = g.row_ptr; a.row_col = g.row_col; a.col_slot = g.tile_slots; a.lam = g.lam;
     a.M = g.M; a.N = g.N; a.E = g.E; a.T = T; a.L = cfg.L; a.B = B;
     a.ntile = (int)((B + kShots - 1) / kShots);
-    if (CUDA_FAILED(cudaFuncSetAttribute(k_llr_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return -2;
     const int threads = std::min(kLlrThreads, std::max(64, (std::max(2 * g.M, g.N) + 31) / 32 * 32));
-    const int fit = sms * std::max(1, std::min((int)((size_t)optin / smem), kLlrThreads / threads));
+    const int fit = g.sms * std::max(1, std::min((int)((size_t)g.max_smem / smem), kLlrThreads / threads));
     if (2ll * g.N > (long long)kLlrHeld * threads) return 1;
+    if (!allow_smem(g, k_llr_tiles)) return -2;
     k_llr_tiles<<<std::min(a.ntile, fit), threads, smem, (cudaStream_t)stream>>>(a, cfg.alpha, synd, g.WM, llr, sum_llr);
     return CUDA_FAILED(cudaGetLastError()) ? -2 : 0;
 }
@@ -1234,11 +1236,10 @@ int bsd_unrolled_forward(const bsd_decoder* dec, const uint32_t* d_syndromes, co
     LaunchHooks hks;
     const LaunchHooks* hk = decoder_hooks(dec, s, &hks) ? &hks : nullptr;
     TileArgs ta;
-    if (tile_plan(*g, *cfg, device, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
+    if (tile_plan(*g, *cfg, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
         const size_t smem = tile_smem(g->M, g->N, g->E);
         auto kf = g->max_col_deg <= 4 ? k_u_forward<4> : k_u_forward<8>;
-        if (CUDA_FAILED(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-            return BSD_ERR_CUDA;
+        if (!allow_smem(*g, kf)) return BSD_ERR_CUDA;
         {
             Timed tm(hk, kKindCheck);
             kf<<<ta.blocks, std::min(ta.threads, kFwdThreads), smem, s>>>(ta, d_syndromes, d_errors, g->WM, g->WN, d_llr);
@@ -1295,11 +1296,10 @@ int bsd_unrolled_backward(const bsd_decoder* dec, int64_t B, int32_t T, int32_t 
     LaunchHooks hks;
     const LaunchHooks* hk = decoder_hooks(dec, s, &hks) ? &hks : nullptr;
     TileArgs ta;
-    if (tile_plan(*g, *cfg, device, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
+    if (tile_plan(*g, *cfg, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
         const size_t smem = tile_smem(g->M, g->N, g->E);
         auto kb = g->max_col_deg <= 4 ? k_u_backward<4> : k_u_backward<8>;
-        if (CUDA_FAILED(cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-            return BSD_ERR_CUDA;
+        if (!allow_smem(*g, kb)) return BSD_ERR_CUDA;
         {
             Timed tm(hk, kKindBVar);
             kb<<<ta.blocks, std::min(ta.threads, kBwdThreads), smem, s>>>(ta, d_grad_loss, scale);

@@ -462,8 +462,9 @@ __device__ inline void argmin_and_score(const G& grp, const DevGraph& g, const W
 // BP engines: how one warp runs the iterations of one candidate
 // ----------------------------------------------------------------------------
 // GenericEngine: any code whose column degree is at most DV (used for degrees
-// above 6); graph tables are read from global memory (L1-resident) and sum_LLR
-// lives in shared memory.
+// above 6, and for 16-bit messages that do not fit on chip as the floats of the
+// jagged engine); graph tables are read from global memory (L1-resident) and
+// sum_LLR lives in shared memory.
 template <int DV, int P, bool W = false, class G = WarpGroup>
 struct GenericEngine {
     using Grp = G;
@@ -2666,7 +2667,7 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_bp_llr(De
 // engine id = 3 * kind + storage precision, or 15 + kind for weighted min-sum;
 // kinds: 0, 1 jagged with column degree bound 3 / 6, 2 generic (16), 3: small (CPL 3,
 // RPL 2, row degree 6), 4: small (CPL 5, RPL 3, row degree 6); precision 0
-// float, 1 binary16, 2 bfloat16
+// float, 1 binary16, 2 bfloat16; then the blocks of warps and the wide engines below
 #define BSD_KIND_ALIASES(P, SFX)                          \
     using Generic3##SFX = JaggedEngine<3, P>;             \
     using Generic6##SFX = JaggedEngine<6, P>;             \
@@ -2694,6 +2695,17 @@ BSD_BLOCK_ALIASES(3, JaggedEngine)
 BSD_BLOCK_ALIASES(6, JaggedEngine)
 BSD_BLOCK_ALIASES(16, GenericEngine)
 constexpr int kBlockEngine = 20;
+// the generic engine with 16-bit messages on chip, for codes of column degree up to 6
+// whose messages do not fit there as floats: id 32 + 4 * kind + 2 (a block) +
+// (0 binary16, 1 bfloat16)
+#define BSD_WIDE_ALIASES(DV)                                             \
+    using Wide##DV##_f16 = GenericEngine<DV, 1>;                         \
+    using Wide##DV##_bf16 = GenericEngine<DV, 2>;                        \
+    using WideBlock##DV##_f16 = GenericEngine<DV, 1, false, BlockGroup>; \
+    using WideBlock##DV##_bf16 = GenericEngine<DV, 2, false, BlockGroup>;
+BSD_WIDE_ALIASES(3)
+BSD_WIDE_ALIASES(6)
+constexpr int kWideEngine = 32;
 #define BSD_ENGINES(X)                                                                          \
     X(0, Generic3_f32) X(1, Generic3_f16) X(2, Generic3_bf16)                                   \
     X(3, Generic6_f32) X(4, Generic6_f16) X(5, Generic6_bf16)                                   \
@@ -2703,7 +2715,9 @@ constexpr int kBlockEngine = 20;
     X(15, Generic3_w) X(16, Generic6_w) X(17, Generic16_w) X(18, Small326_w) X(19, Small536_w)  \
     X(20, Block3_f32) X(21, Block3_f16) X(22, Block3_bf16) X(23, Block3_w)                      \
     X(24, Block6_f32) X(25, Block6_f16) X(26, Block6_bf16) X(27, Block6_w)                      \
-    X(28, Block16_f32) X(29, Block16_f16) X(30, Block16_bf16) X(31, Block16_w)
+    X(28, Block16_f32) X(29, Block16_f16) X(30, Block16_bf16) X(31, Block16_w)                  \
+    X(32, Wide3_f16) X(33, Wide3_bf16) X(34, WideBlock3_f16) X(35, WideBlock3_bf16)             \
+    X(36, Wide6_f16) X(37, Wide6_bf16) X(38, WideBlock6_f16) X(39, WideBlock6_bf16)
 
 template <class Eng>
 static int set_attrs(size_t smem_bp)
@@ -2774,22 +2788,30 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     // the generic one the stored format and a record per detector
     g.e_bytes = gkind < 2 ? (int)sizeof(float) : g.msg_bytes;
     g.det_bytes = gkind < 2 ? 0 : (int)align16(sizeof(float2) * (size_t)g.M);
-    const size_t generic_bytes = warp_smem_bytes(g);
     // automatic choice: the small engine where it fits; otherwise a warp per
     // candidate while eight or more candidates fit on an SM, a block of 16
     // warps per candidate beyond (8 / 16 warps: 10^5 shots of the
     // phenomenological DEM at p = 3e-3 3.42 / 2.88 ms, 5 x 10^4 in half
     // precision 0.87 / 0.74, 3 x 10^5 of the synthetic DEM 11.2 / 10.7)
     int gw = group_warps;
-    if (gw == 0) gw = (skind >= 0 || generic_bytes * 8 <= (size_t)max_optin) ? 1 : 16;
+    if (gw == 0) gw = (skind >= 0 || warp_smem_bytes(g) * 8 <= (size_t)max_optin) ? 1 : 16;
+    // 16-bit messages that do not fit as floats stay in 16 bits on chip (the
+    // generic engine's state: 2 E + 8 M + 4 N bytes against 4 E + 4 N): from about
+    // 45000 edges; 2 x 10^4 shots of a 1200 x 20000 code of 60000 edges 1.9 ms
+    const bool wide = gkind < 2 && skind < 0 && g.prec != 0 &&
+                      warp_smem_bytes(g) + (gw >= 2 ? 16 * sizeof(ArgRec) : 0) > (size_t)max_optin;
+    if (wide) {
+        g.e_bytes = g.msg_bytes;
+        g.det_bytes = (int)align16(sizeof(float2) * (size_t)g.M);
+    }
     const bool weighted = cfg.weights != nullptr;
     int eng, wpb;
     if (gw >= 2) {
-        eng = kBlockEngine + 4 * gkind + (weighted ? 3 : g.prec);
+        eng = wide ? kWideEngine + 4 * gkind + 2 + (g.prec - 1) : kBlockEngine + 4 * gkind + (weighted ? 3 : g.prec);
         wpb = gw;
     } else {
         const int kind = skind >= 0 ? skind : gkind;
-        eng = weighted ? kWeightedEngine + kind : 3 * kind + g.prec;
+        eng = weighted ? kWeightedEngine + kind : wide ? kWideEngine + 4 * gkind + (g.prec - 1) : 3 * kind + g.prec;
         // the small engine keeps D per edge in float (over E with single-precision
         // messages, else beside it)
         if (kind >= 3) {

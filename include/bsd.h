@@ -375,14 +375,21 @@ int bsd_set_weights(bsd_decoder *dec, const float *h_weights, int32_t T);
  * weights are not used.
  *
  * Workspace: device memory of bsd_unrolled_workspace() bytes, 256-byte
- * aligned, owned by the caller.  The forward stores E at the checkpoints
- * t = 0, k, 2k, ... (k = ckpt_every, 1 <= k <= T) and the bit planes of the
- * batch there; the backward recomputes each segment of k iterations from its
- * checkpoint.  A backward needs the forward of the same (B, T, k, weights,
- * workspace) before it, with the workspace untouched in between.
+ * aligned, owned by the caller.  A backward needs the forward of the same (B, T,
+ * k, weights, workspace) before it, with the workspace untouched in between
+ * (k = ckpt_every, 1 <= k <= T; no result depends on it).
  *
- * Memory: about (ceil(T/k) + k + 4) * E * Bp + k * N * Bp floats, Bp = B
- * rounded up to a multiple of 512. */
+ * Codes whose rows and columns have at most 8 edges and whose messages of 8
+ * shots fit in an SM's shared memory (about 7100 edges) run on chip in tiles of 8
+ * shots, whatever k is: the forward keeps T * (10 M + 4 N) bytes per shot for the
+ * backward, and each block T * E floats of weight gradients.  Above 8 GB they do
+ * so only where this is no more than the other codes' form would take with its
+ * best k.
+ *
+ * The other codes: the forward stores E at the checkpoints t = 0, k, 2k, ... and
+ * the bit planes of the batch; the backward recomputes each segment of k
+ * iterations from its checkpoint.  About (ceil(T/k) + k + 4) * E * Bp + k * N * Bp
+ * floats, Bp = B rounded up to a multiple of 512. */
 int bsd_unrolled_workspace(const bsd_decoder *dec, int64_t B, int32_t T, int32_t ckpt_every, int64_t *bytes);
 
 /*   d_syndromes  device, B x ceil(M/32) words (bitpacked like bsd_decode)

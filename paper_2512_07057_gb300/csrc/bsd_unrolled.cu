@@ -910,11 +910,16 @@ bool allow_smem(const DevGraph& g, F* kernel)
     return !CUDA_FAILED(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g.max_smem));
 }
 
-// the tiled path's arrays in the caller's workspace; false where a degree, the
-// shared memory or the workspace (whose size the general passes set) does not
-// allow it
-bool tile_plan(const DevGraph& g, const DecCfg& cfg, long long B, int T, const float* w, char* base,
-               size_t have, TileArgs* out)
+// The tiled path's arrays in the caller's workspace (base may be null: their size
+// only).  It runs wherever the code allows it, whatever ckpt_every is: the interval
+// changes no bit of the results.  It keeps 10 bytes per (row, shot) and 4 per (node,
+// shot) of every iteration, on the phenomenological DEM 0.96 of what the passes need
+// with their best interval at T = 20 and 1.27 at T = 30; so that no training that fit
+// the device stops fitting, a workspace above kTileBytes is taken only where the
+// passes' smallest is no smaller.
+constexpr size_t kTileBytes = size_t(8) << 30;
+bool tile_plan(const DevGraph& g, const DecCfg& cfg, long long B, int T, const float* w, char* base, TileArgs* out,
+               size_t* bytes)
 {
     if (g.max_row_deg > kMaxDeg || g.tile_slots == nullptr || g.E > 65528 || g.max_row_deg < 1) return false;
     const size_t smem = tile_smem(g.M, g.N, g.E);
@@ -932,9 +937,9 @@ bool tile_plan(const DevGraph& g, const DecCfg& cfg, long long B, int T, const f
     a.blocks = (a.ntile + rounds - 1) / rounds;
     const size_t nt = (size_t)a.ntile, TM = (size_t)T * (size_t)g.M * kShots, TN = (size_t)T * (size_t)g.N * kShots;
     size_t off = 0;
-    auto take = [&](size_t bytes) {
-        char* p = base + off;
-        off += a256(bytes);
+    auto take = [&](size_t n) {
+        char* p = base ? base + off : nullptr;
+        off += a256(n);
         return p;
     };
     a.s8 = (unsigned char*)take(nt * (size_t)g.M);
@@ -945,9 +950,23 @@ bool tile_plan(const DevGraph& g, const DecCfg& cfg, long long B, int T, const f
     a.lamT = (float*)take(sizeof(float) * nt * TN);
     a.loss_part = (float*)take(sizeof(float) * nt * (size_t)T);
     a.gw_part = (float*)take(sizeof(float) * (size_t)a.blocks * (size_t)T * (size_t)g.E);
-    if (off > have) return false;
-    *out = a;
+    if (off > kTileBytes) {
+        // (the passes' size falls, then rises with the interval, turning below sqrt(T) + 1)
+        size_t least = SIZE_MAX;
+        for (long long k = 1; k <= T && (k - 1) * (k - 1) <= T; ++k)
+            least = std::min(least, layout(g, B, T, (int)k, nullptr).bytes);
+        if (off > least) return false;
+    }
+    if (out) *out = a;
+    *bytes = off;
     return true;
+}
+
+// bytes of the caller's workspace, on the path that runs
+size_t work_bytes_of(const DevGraph& g, const DecCfg& cfg, long long B, int T, int k)
+{
+    size_t bytes = 0;
+    return tile_plan(g, cfg, B, T, nullptr, nullptr, nullptr, &bytes) ? bytes : layout(g, B, T, k, nullptr).bytes;
 }
 
 // plain BP (Eqs. 1-3 with the scale alpha, the sums in ascending order) for T
@@ -1211,7 +1230,7 @@ int bsd_unrolled_workspace(const bsd_decoder* dec, int64_t B, int32_t T, int32_t
     if (!bytes) return BSD_ERR_INVALID_ARG;
     const int rc = check_args(dec, B, T, ckpt_every, &g, &cfg, &device);
     if (rc) return rc;
-    *bytes = (int64_t)layout(*g, B, T, ckpt_every, nullptr).bytes;
+    *bytes = (int64_t)work_bytes_of(*g, *cfg, B, T, ckpt_every);
     return BSD_OK;
 }
 
@@ -1225,18 +1244,16 @@ int bsd_unrolled_forward(const bsd_decoder* dec, const uint32_t* d_syndromes, co
     int rc = check_args(dec, B, T, ckpt_every, &g, &cfg, &device);
     if (rc) return rc;
     if (!d_syndromes || !d_errors || !d_weights || !d_loss || !d_work) return BSD_ERR_INVALID_ARG;
-    const ULayout u = layout(*g, B, T, ckpt_every, (char*)d_work);
-    if (work_bytes < (int64_t)u.bytes || ((uintptr_t)d_work & 255u)) return BSD_ERR_INVALID_ARG;
+    if (work_bytes < (int64_t)work_bytes_of(*g, *cfg, B, T, ckpt_every) || ((uintptr_t)d_work & 255u))
+        return BSD_ERR_INVALID_ARG;
     DeviceScope ds(device);
     if (!ds.ok) return BSD_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const UArgs a = make_args(*g, *cfg, B, T, d_weights, u);
-    const int k = ckpt_every;
-    const size_t EB = (size_t)g->E * (size_t)a.Bp;
     LaunchHooks hks;
     const LaunchHooks* hk = decoder_hooks(dec, s, &hks) ? &hks : nullptr;
     TileArgs ta;
-    if (tile_plan(*g, *cfg, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
+    size_t tile_bytes;
+    if (tile_plan(*g, *cfg, B, T, d_weights, (char*)d_work, &ta, &tile_bytes)) {
         const size_t smem = tile_smem(g->M, g->N, g->E);
         auto kf = g->max_col_deg <= 4 ? k_u_forward<4> : k_u_forward<8>;
         if (!allow_smem(*g, kf)) return BSD_ERR_CUDA;
@@ -1249,6 +1266,10 @@ int bsd_unrolled_forward(const bsd_decoder* dec, const uint32_t* d_syndromes, co
         k_u_loss_total<<<1, 32, 0, s>>>(T, d_loss);
         return CUDA_FAILED(cudaGetLastError()) ? BSD_ERR_CUDA : BSD_OK;
     }
+    const ULayout u = layout(*g, B, T, ckpt_every, (char*)d_work);
+    const UArgs a = make_args(*g, *cfg, B, T, d_weights, u);
+    const int k = ckpt_every;
+    const size_t EB = (size_t)g->E * (size_t)a.Bp;
     {
         Timed tm(hk, kKindOther);
         k_u_planes<<<1024, 256, 0, s>>>(d_syndromes, B, g->WM, g->M, a.Bp, u.sT);
@@ -1282,21 +1303,17 @@ int bsd_unrolled_backward(const bsd_decoder* dec, int64_t B, int32_t T, int32_t 
     int rc = check_args(dec, B, T, ckpt_every, &g, &cfg, &device);
     if (rc) return rc;
     if (!d_weights || !d_grad_loss || !d_grad_weights || !d_work) return BSD_ERR_INVALID_ARG;
-    const ULayout u = layout(*g, B, T, ckpt_every, (char*)d_work);
-    if (work_bytes < (int64_t)u.bytes || ((uintptr_t)d_work & 255u)) return BSD_ERR_INVALID_ARG;
+    if (work_bytes < (int64_t)work_bytes_of(*g, *cfg, B, T, ckpt_every) || ((uintptr_t)d_work & 255u))
+        return BSD_ERR_INVALID_ARG;
     DeviceScope ds(device);
     if (!ds.ok) return BSD_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const UArgs a = make_args(*g, *cfg, B, T, d_weights, u);
-    const int k = ckpt_every;
-    const size_t EB = (size_t)g->E * (size_t)a.Bp, NB = (size_t)g->N * (size_t)a.Bp;
     const double scale = 1.0 / ((double)B * (double)g->N);
-    const int cap_c = cap_of(g->max_col_deg);
-    const dim3 gcol(a.ntile, grid_y(g->N)), grow(a.ntile, grid_y(g->M));
     LaunchHooks hks;
     const LaunchHooks* hk = decoder_hooks(dec, s, &hks) ? &hks : nullptr;
     TileArgs ta;
-    if (tile_plan(*g, *cfg, B, T, d_weights, (char*)d_work, u.bytes, &ta)) {
+    size_t tile_bytes;
+    if (tile_plan(*g, *cfg, B, T, d_weights, (char*)d_work, &ta, &tile_bytes)) {
         const size_t smem = tile_smem(g->M, g->N, g->E);
         auto kb = g->max_col_deg <= 4 ? k_u_backward<4> : k_u_backward<8>;
         if (!allow_smem(*g, kb)) return BSD_ERR_CUDA;
@@ -1308,6 +1325,12 @@ int bsd_unrolled_backward(const bsd_decoder* dec, int64_t B, int32_t T, int32_t 
         k_u_gw_blocks<<<1024, 128, 0, s>>>(ta.gw_part, (long long)T * g->E, ta.blocks, d_grad_weights);
         return CUDA_FAILED(cudaGetLastError()) ? BSD_ERR_CUDA : BSD_OK;
     }
+    const ULayout u = layout(*g, B, T, ckpt_every, (char*)d_work);
+    const UArgs a = make_args(*g, *cfg, B, T, d_weights, u);
+    const int k = ckpt_every;
+    const size_t EB = (size_t)g->E * (size_t)a.Bp, NB = (size_t)g->N * (size_t)a.Bp;
+    const int cap_c = cap_of(g->max_col_deg);
+    const dim3 gcol(a.ntile, grid_y(g->N)), grow(a.ntile, grid_y(g->M));
     int cur = 0;                               // gE(t) lives in u.gE[cur]
     const int C = (T + k - 1) / k;
     for (int c = C - 1; c >= 0; --c) {

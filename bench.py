@@ -1006,10 +1006,10 @@ def run_unrolled(args, rank: int, world: int, local_rank: int):
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "edge_updates_per_s": world * upd * args.steps / steps_s,
         "kernels": per_kind, "roofline": roofline, "clocks": clocks,
-        # per step, on tiles: forward, two loss reductions, backward, gradient reduction; on passes: forward
+        # per step, on tiles: weight scan, forward, two loss reductions, backward, gradient reduction; on passes: forward
         # 2 bit-plane + 1 initial-message + T check + T error + 1 loss kernels; backward T recomputed check +
         # T recomputed error + T error-adjoint + T check-adjoint + 1 gradient kernels
-        "gpu_launches": (5 if tiled else 6 * T + 5) * args.steps,
+        "gpu_launches": (6 if tiled else 6 * T + 5) * args.steps,
         "timed_launches_per_step": {names[kd]: float(prof["launches"][kd]) / args.steps for kd in names},
     }
     if rank == 0 and not args.no_e2e:

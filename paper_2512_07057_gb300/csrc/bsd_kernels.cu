@@ -2197,9 +2197,9 @@ struct GpuRing {
     static __device__ __forceinline__ unsigned long long now() { return global_ns(); }
 };
 
-__device__ inline void push_item(const Work& w, uint32_t item)
+__device__ inline void push_pair(const Work& w, uint32_t item)
 {
-    ring_push<GpuRing>(w.ring, &w.ctr->b_tail, w.ctr->b_mask, item);
+    ring_push_pair<GpuRing>(w.ring, &w.ctr->b_tail, w.ctr->b_mask, item);
 }
 
 __device__ inline uint32_t draw_item(const Work& w, uint32_t ticket)
@@ -2485,8 +2485,7 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
                 w.kid[(size_t)a * W2 + 2 * k] = w.kid[(size_t)a * W2 + 2 * k + 1] = make_int2(c, np);
                 if (np >= 0) {
                     fence_gpu();               // the entry and the child before its items
-                    push_item(w, ring_item(a, 2 * k));
-                    push_item(w, ring_item(a, 2 * k + 1));
+                    push_pair(w, ring_item(a, 2 * k));
                 }
             }
         }
@@ -2499,9 +2498,9 @@ __device__ __noinline__ void select_entry(const DevGraph& g, const DecCfg& cfg, 
         e = __shfl_sync(FULLMASK, e, 0);
         if (e < w.ctr->n_active) {
             init_entry(g, cfg, w, a, e, ent.stamp + 1);
-            if (lane < 2) {
+            if (lane == 0) {
                 fence_gpu();
-                push_item(w, ring_item(a, lane));
+                push_pair(w, ring_item(a, 0));
             }
         }
         __syncwarp();

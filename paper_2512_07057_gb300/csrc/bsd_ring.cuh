@@ -47,29 +47,41 @@ BSD_RING_FN bool ring_has_item(uint32_t v) { return (v & ~kRingLeft) != 0u; }
 constexpr unsigned long long kIdleNs = 1000ull * 1000 * 1000;
 constexpr unsigned long long kStuckNs = 16ull * kIdleNs;   // past any wait that can come about
 
+// an item whose ticket's slot holds `old`, not kRingEmpty
 template <class Ops>
-BSD_RING_DEV void ring_push(uint32_t* ring, uint32_t* tail, uint32_t mask, uint32_t item)
+BSD_RING_DEV void ring_settle(uint32_t* ring, uint32_t* tail, uint32_t mask, uint32_t* slot, uint32_t item, uint32_t old)
 {
+    unsigned long long t0 = 0ull;
     for (;;) {
-        uint32_t* const slot = ring + (Ops::add(tail, 1u) & mask);
-        uint32_t want = kRingEmpty;
-        unsigned long long t0 = 0ull;
-        for (;;) {
-            const uint32_t old = Ops::cas(slot, want, want == kRingLeft ? kRingEmpty : item);
-            if (old == want) {
-                if (want == kRingEmpty) return;
-                if (want != kRingLeft) item = want;            // (past kStuckNs: pushed in its place)
-                break;
-            }
-            want = old == kRingLeft ? kRingLeft : kRingEmpty;
-            if (ring_has_item(old)) {                          // its group is about to take it
-                Ops::pause();
-                const unsigned long long t = Ops::now();
-                if (t0 == 0ull) t0 = t;
-                else if (t - t0 > kStuckNs) want = old;
-            }
+        uint32_t want = old == kRingLeft ? kRingLeft : kRingEmpty;
+        if (ring_has_item(old)) {                              // its group is about to take it
+            Ops::pause();
+            const unsigned long long t = Ops::now();
+            if (t0 == 0ull) t0 = t;
+            else if (t - t0 > kStuckNs) want = old;
         }
+        old = Ops::cas(slot, want, want == kRingLeft ? kRingEmpty : item);
+        if (old != want) continue;
+        if (want == kRingEmpty) return;
+        if (want != kRingLeft) item = want;                    // (past kStuckNs: pushed in its place)
+        slot = ring + (Ops::add(tail, 1u) & mask);
+        t0 = 0ull;
+        old = Ops::cas(slot, kRingEmpty, item);
+        if (old == kRingEmpty) return;
     }
+}
+
+// push item and item + 1, the two children of a path: two tickets in one step, both
+// slots tried before either is waited for
+template <class Ops>
+BSD_RING_DEV void ring_push_pair(uint32_t* ring, uint32_t* tail, uint32_t mask, uint32_t item)
+{
+    const uint32_t t = Ops::add(tail, 2u);
+    uint32_t* const s0 = ring + (t & mask);
+    uint32_t* const s1 = ring + ((t + 1u) & mask);
+    const uint32_t o0 = Ops::cas(s0, kRingEmpty, item), o1 = Ops::cas(s1, kRingEmpty, item + 1u);
+    if (o0 != kRingEmpty) ring_settle<Ops>(ring, tail, mask, s0, item, o0);
+    if (o1 != kRingEmpty) ring_settle<Ops>(ring, tail, mask, s1, item + 1u, o1);
 }
 
 // the item of a ticket, or kRingEmpty when every shot has ended (*left = 0) or

@@ -70,7 +70,7 @@ struct HostRing {
 void run_lane()
 {
     Fiber& f = *S->cur;
-    for (uint32_t it : f.push) bsd::ring_push<HostRing>(S->ring.data(), &S->tail, S->mask, it);
+    for (uint32_t it : f.push) bsd::ring_push_pair<HostRing>(S->ring.data(), &S->tail, S->mask, it);
     f.push.clear();
     f.done = true;
     yield();
@@ -115,7 +115,8 @@ void run_group()
         std::vector<uint32_t> items;
         auto put = [&](int n) {
             s.pending[a] = n;
-            for (int k = 0; k < n; ++k) { s.out[a][k] = 1; items.push_back(bsd::ring_item(a, k)); }
+            for (int k = 0; k < n; ++k) s.out[a][k] = 1;
+            for (int k = 0; k < n; k += 2) items.push_back(bsd::ring_item(a, k));        // (a path's two children)
         };
         if (s.round[a] < s.rounds && s.rng.below(8) != 0) {
             ++s.round[a];

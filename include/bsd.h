@@ -267,10 +267,9 @@ int bsd_get_batch(const bsd_decoder *dec, int32_t *slots, int32_t *active);
  * with plane[h] = h (64 ceil(M / 32) + 12), and the error-node pass reads the
  * k-th edge of column j at col_word[3 j + k].
  * The rows' edge orders and the columns' k orders are searched so that both
- * passes touch 32 distinct banks per access.  The engine of codes of at most
- * 160 columns and 96 rows uses the same words; its own placement also deals the
- * columns to the lanes, so that a warp can keep a third of the messages in
- * registers.  Host only; nothing is allocated on a device.
+ * passes touch 32 distinct banks per access with the columns in their own order.
+ * No engine keeps its messages by it: that of these codes deals the columns to the
+ * lanes (bsd_lane_layout).  Host only; nothing is allocated on a device.
  *   M, N, H_row_ptr, H_col_idx  host, H in CSR as for bsd_create
  *   plane      host int32[3]: out, the plane bases
  *   edge_word  host int32[E]: out, the word of CSR edge e (E = H_row_ptr[M])
@@ -282,6 +281,27 @@ int bsd_get_batch(const bsd_decoder *dec, int32_t *slots, int32_t *active);
  * (another degree structure). */
 int bsd_small_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32_t *H_col_idx, int32_t *plane,
                      int32_t *edge_word, int32_t *col_word, int32_t *extent, int32_t *excess);
+
+/* Where the single-warp engine keeps a candidate's messages (a layout choice of
+ * this library, for codes with every row of degree 6 and every column of degree 3
+ * and 33 to 48 or 65 to 80 rows): the placement that bsd_create builds.  The rows' pairs lie as in bsd_small_layout.
+ * Each row of a group of 32 owns two of its columns, which its lane processes and
+ * whose edges with it are the row's pair 0, held in registers; the other columns
+ * follow in the last group.  Host only; nothing is allocated on a device.
+ *   M, N, H_row_ptr, H_col_idx  host, H in CSR as for bsd_create
+ *   edge_word  host int32[E]: out, the word of CSR edge e
+ *   lane_col   host int32[32 ceil(N / 32)]: out, the column at lane l of group g
+ *              at [32 g + l], -1 for none
+ *   lane_word  host int32[3 * 32 ceil(N / 32)]: out, the words of that column's
+ *              edges in the order of the error pass's accesses (in all groups but
+ *              the last the register-held one first)
+ *   extent     host int32: out, the words spanned
+ *   extra      host int32: out, the wavefronts that bank conflicts add to one
+ *              round of the error pass's accesses
+ * Errors: BSD_ERR_INVALID_ARG (null pointer, bad CSR), BSD_ERR_UNSUPPORTED
+ * (another degree structure or size). */
+int bsd_lane_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32_t *H_col_idx, int32_t *edge_word,
+                    int32_t *lane_col, int32_t *lane_word, int32_t *extent, int32_t *extra);
 
 /* Where the generic engines keep a candidate's messages (a layout choice of
  * this library, for codes with every column of degree at most 6): each row's

@@ -31,7 +31,7 @@ BSD_STATUS_FAILED = 4
 
 # every symbol include/bsd.h declares
 EXPORTS = ("bsd_params_default", "bsd_params_preset", "bsd_create", "bsd_decode", "bsd_decode_host",
-           "bsd_bp_llr", "bsd_sync_error", "bsd_get_info", "bsd_get_batch", "bsd_small_layout", "bsd_generic_layout", "bsd_serve_start", "bsd_serve_decode",
+           "bsd_bp_llr", "bsd_sync_error", "bsd_get_info", "bsd_get_batch", "bsd_small_layout", "bsd_lane_layout", "bsd_generic_layout", "bsd_serve_start", "bsd_serve_decode",
            "bsd_serve_stop", "bsd_profile_enable", "bsd_profile_read",
            "bsd_decode_noalloc", "bsd_set_weights", "bsd_unrolled_workspace", "bsd_unrolled_forward",
            "bsd_unrolled_backward", "bsd_profile_read_kinds", "bsd_autotune", "bsd_get_shape", "bsd_dem_parse",
@@ -90,6 +90,7 @@ def load(path: str | None = None) -> C.CDLL:
     lib.bsd_get_info.argtypes = [P] + [C.POINTER(C.c_int32)] * 4 + [C.POINTER(C.c_int64)] * 2
     lib.bsd_get_batch.argtypes = [P, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
     lib.bsd_small_layout.argtypes = [C.c_int32, C.c_int32, P, P, P, P, P, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
+    lib.bsd_lane_layout.argtypes = [C.c_int32, C.c_int32, P, P, P, P, P, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
     lib.bsd_generic_layout.argtypes = [C.c_int32, C.c_int32, P, P, P, P, C.POINTER(C.c_int32),
                                        C.POINTER(C.c_int32)]
     lib.bsd_decode_noalloc.argtypes = [P, P, C.c_int64, P, P, P, P, P]
@@ -208,8 +209,8 @@ def bsd_get_batch(dec) -> dict:
 
 
 def bsd_small_layout(M: int, N: int, row_ptr, col_idx) -> dict:
-    """The single-warp engine's shared-memory placement of H's messages (host
-    only): plane bases, the word of every CSR edge, the word of the k-th edge
+    """A conflict-free placement of H's messages in shared memory with the columns
+    in their own order (host only; no engine's): plane bases, the word of every CSR edge, the word of the k-th edge
     of every column ([N][3]), the words spanned and the bank loads above three
     left in the error-node pass."""
     import numpy as np
@@ -222,6 +223,24 @@ def bsd_small_layout(M: int, N: int, row_ptr, col_idx) -> dict:
     check(load().bsd_small_layout(int(M), int(N), rp.ctypes.data, ci.ctypes.data, plane.ctypes.data, ew.ctypes.data,
                                   cw.ctypes.data, C.byref(ext), C.byref(exc)), "bsd_small_layout")
     return dict(plane=plane, edge_word=ew, col_word=cw.reshape(int(N), 3), extent=ext.value, excess=exc.value)
+
+
+def bsd_lane_layout(M: int, N: int, row_ptr, col_idx) -> dict:
+    """The single-warp engine's shared-memory placement of H's messages (host
+    only): the word of every CSR edge, the column at every lane of every group
+    ([groups, 32], -1 none), its edges' words ([groups, 32, 3]), the words spanned
+    and the wavefronts that bank conflicts add to the error pass."""
+    import numpy as np
+    rp = np.ascontiguousarray(row_ptr, dtype=np.int32)
+    ci = np.ascontiguousarray(col_idx, dtype=np.int32)
+    groups = (int(N) + 31) // 32
+    ew = np.zeros(int(rp[-1]), np.int32)
+    lc = np.zeros((groups, 32), np.int32)
+    lw = np.zeros((groups, 32, 3), np.int32)
+    ext, extra = C.c_int32(), C.c_int32()
+    check(load().bsd_lane_layout(int(M), int(N), rp.ctypes.data, ci.ctypes.data, ew.ctypes.data, lc.ctypes.data,
+                                 lw.ctypes.data, C.byref(ext), C.byref(extra)), "bsd_lane_layout")
+    return dict(edge_word=ew, lane_col=lc, lane_word=lw, extent=ext.value, extra=extra.value)
 
 
 def bsd_generic_layout(M: int, N: int, row_ptr, col_idx) -> dict:

@@ -55,6 +55,7 @@
 #include "bsd_internal.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <vector>
 
@@ -67,8 +68,7 @@ constexpr int kRowDeg = 6;
 constexpr int kColDeg = 3;
 constexpr int kTries = 16;      // local-search restarts
 constexpr int kSweeps = 200;    // sweeps per restart
-constexpr int kLocalTries = 6;  // draws of the columns that rows own
-constexpr int kLocalSweeps = 60; // sweeps per draw
+constexpr int kLocalMoves = 20000; // moves of the single-warp engine's placement
 
 struct Rng {                    // xorshift64*: a fixed, reproducible sequence
     uint64_t s;
@@ -80,6 +80,7 @@ struct Rng {                    // xorshift64*: a fixed, reproducible sequence
         return (uint32_t)((s * 2685821657736338717ull) >> 32);
     }
     uint32_t below(uint32_t n) { return next() % n; }
+    uint32_t pick(uint32_t n) { return (uint32_t)(((uint64_t)next() * n) >> 32); }
 };
 
 int mod32(int x) { return ((x % 32) + 32) % 32; }
@@ -425,196 +426,305 @@ bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int co
 
 namespace bsd {
 
-// the single-warp engine's placement: rows in natural order, columns in the
-// order of the lanes that process them.  Which two of its columns a row owns is
-// drawn anew until the other words meet almost no bank conflict or kLocalTries is
-// reached; the draw with the fewest is kept.
+// The single-warp engine's placement: rows in natural order, columns in the order
+// of the lanes that process them.
+//
+// Each full row (of a group of 32 rows) owns two of its columns; they are dealt to
+// its lane in the groups 2 r and 2 r + 1, and their messages on that row stay in a
+// register.  The other columns form the last group.  The row's other four edges take
+// its words 2..5 (all six in the last rows).  An access of the error pass is free of
+// conflicts when each bank holds at most two words of a full group's columns (three
+// of the last one's): exactly two, as 64 words meet 32 banks, so a placement by
+// chance leaves some 20 words over.
+//
+// Annealing over the words within a row, the two sides of a row's own columns, and
+// the columns that rows own (one of the last group taken in, or one of another row,
+// which takes one of the last group instead); the cost is the sum of squared loads.
+// Four moves of five start at a word of an overloaded bank.  kLocalMoves bound it,
+// about 2 ms; many codes end earlier.  Extra wavefronts, beside the error pass's 11 (7
+// for up to 96 columns), on average and at most: 1.7 and 2 over 20 numberings of the
+// rows and columns of [[144,12,12]], 0.4 and 2 of [[72,12,6]], 1.7 and 4 over 20 random
+// (3, 6)-regular codes of 40 to 78 rows.  With the owned columns drawn at random and
+// only words and sides moved it was 6.3, 2.8 and 5.5, in three times the time.
 bool small_local_layout(int M, int N, const int* row_ptr, const int* col_idx, SmallLocal* out)
 {
     const int RPL = (M + 31) / 32, CPL = (N + 31) / 32, LC = 2 * (RPL - 1);
-    if (RPL < 2 || CPL != LC + 1 || N != 2 * M) return false;
+    if (RPL < 2 || CPL != LC + 1 || N != 2 * M || CPL > kSmallMaxCpl) return false;
     const int E = row_ptr[M];
-    std::vector<std::vector<int>> cedges(N);
-    std::vector<int> erow(E);
+    std::vector<int> cedge((size_t)kColDeg * N), deg(N, 0), erow(E);
     for (int i = 0; i < M; ++i) {
         if (row_ptr[i + 1] - row_ptr[i] != kRowDeg) return false;
         for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+            const int j = col_idx[e];
+            if (deg[j] == kColDeg) return false;
             erow[e] = i;
-            cedges[col_idx[e]].push_back(e);
+            cedge[(size_t)kColDeg * j + deg[j]++] = e;
         }
     }
-    for (int j = 0; j < N; ++j)
-        if (cedges[j].size() != kColDeg) return false;
     const int full = 32 * (RPL - 1), P = small_plane_stride(M);
-    // (a start of the sequence whose first draw leaves 2 extra wavefronts of 24 on
-    // [[144,12,12]] and none on [[72,12,6]])
-    Rng rng{7142492453195352267ull};
-    int best = -1;
-    std::vector<int> order(N), seen(M), via(M), queue, start, rp(M + 1), ci, id, pos(N), own(N);
-    for (int j = 0; j < N; ++j) order[j] = j;
-    for (int t = 0; t < kLocalTries && (best < 0 || best > RPL - 1); ++t) {
-        // two columns of its own for every row (augmenting paths; every row has
-        // six columns and every column three rows, so the assignment exists)
-        for (int j = N - 1; j > 0 && t > 0; --j) std::swap(order[j], order[rng.below((uint32_t)j + 1)]);
-        std::fill(own.begin(), own.end(), -1);
-        std::fill(seen.begin(), seen.end(), -1);
-        std::vector<std::vector<int>> has(M);
-        for (int j0 : order) {
-            // breadth-first over rows; from a full row, on to the columns it holds
-            queue.clear();
-            auto visit = [&](int j) {
-                const int first = (int)rng.below(kColDeg);
-                for (int k = 0; k < kColDeg; ++k) {
-                    const int i = erow[cedges[j][(first + k) % kColDeg]];
-                    if (seen[i] != j0) { seen[i] = j0; via[i] = j; queue.push_back(i); }
-                }
-            };
-            visit(j0);
-            int end = -1;
-            for (size_t q = 0; q < queue.size() && end < 0; ++q) {
-                if (has[queue[q]].size() < 2) end = queue[q];
-                else
-                    for (int j : has[queue[q]]) visit(j);
-            }
-            if (end < 0) return false;
-            for (int i = end; i >= 0;) {
-                const int j = via[i], from = own[j];
-                if (from >= 0) has[from].erase(std::find(has[from].begin(), has[from].end(), j));
-                own[j] = i;
-                has[i].push_back(j);
-                i = from;
-            }
-        }
-        // a full row's own columns go to groups 2 r and 2 r + 1 (in either order),
-        // the others to the last; the other edges take words 2..5 of a full row,
-        // all six of the last ones.  Swaps of two words of a row, and of a row's
-        // two own columns, while the loads above each group's degree fall
-        auto group = [&](int j) {
-            const int i = own[j];
-            return i < full ? 2 * (i / 32) + (has[i][1] == j ? 1 : 0) : LC;
-        };
-        std::vector<std::vector<int>> word(M);               // edges by word of the row
-        std::vector<int> cnt((size_t)CPL * 32, 0), at(E, 0);
-        auto bank = [&](int i, int q) { return ((q >> 1) * P + 2 * i + (q & 1)) & 31; };
-        for (int i = 0; i < M; ++i) {
-            word[i].assign(kRowDeg, -1);
-            int q = i < full ? 2 : 0;
-            for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
-                if (i < full && own[col_idx[e]] == i) continue;
-                word[i][q] = e;
-                at[e] = q;
-                cnt[(size_t)group(col_idx[e]) * 32 + bank(i, q)]++;
-                ++q;
-            }
-        }
-        auto cap = [&](int g) { return g < LC ? 2 : 3; };
-        auto over = [&](int g, int b) { return std::max(0, cnt[(size_t)g * 32 + b] - cap(g)); };
-        int ex = 0;
-        for (int g = 0; g < CPL; ++g)
-            for (int b = 0; b < 32; ++b) ex += over(g, b);
-        for (int sw = 0; sw < kLocalSweeps && ex > 0; ++sw) {
-            for (int n = 0; n < M && ex > 0; ++n) {
-                const int i = (int)rng.below((uint32_t)M);
-                for (int x = i < full ? 2 : 0; x < kRowDeg; ++x)
-                    for (int y = x + 1; y < kRowDeg; ++y) {
-                        const int gx = group(col_idx[word[i][x]]), gy = group(col_idx[word[i][y]]);
-                        if (gx == gy) continue;
-                        const int bx = bank(i, x), by = bank(i, y);
-                        const int before = over(gx, bx) + over(gy, by) + over(gx, by) + over(gy, bx);
-                        cnt[(size_t)gx * 32 + bx]--; cnt[(size_t)gy * 32 + by]--;
-                        cnt[(size_t)gx * 32 + by]++; cnt[(size_t)gy * 32 + bx]++;
-                        const int after = over(gx, bx) + over(gy, by) + over(gx, by) + over(gy, bx);
-                        if (after < before || (after == before && rng.below(4) == 0)) {
-                            std::swap(word[i][x], word[i][y]);
-                            at[word[i][x]] = x;
-                            at[word[i][y]] = y;
-                            ex += after - before;
-                        } else {
-                            cnt[(size_t)gx * 32 + bx]++; cnt[(size_t)gy * 32 + by]++;
-                            cnt[(size_t)gx * 32 + by]--; cnt[(size_t)gy * 32 + bx]--;
-                        }
-                    }
-                if (i >= full) continue;
-                const int g0 = 2 * (i / 32);
-                auto move = [&](int j, int from, int to) {
-                    int d = 0;
-                    for (int e : cedges[j]) {
-                        if (erow[e] == i) continue;
-                        const int b = bank(erow[e], at[e]);
-                        d -= over(from, b) + over(to, b);
-                        cnt[(size_t)from * 32 + b]--;
-                        cnt[(size_t)to * 32 + b]++;
-                        d += over(from, b) + over(to, b);
-                    }
-                    return d;
-                };
-                const int d = move(has[i][0], g0, g0 + 1) + move(has[i][1], g0 + 1, g0);
-                if (d < 0 || (d == 0 && rng.below(4) == 0)) {
-                    std::swap(has[i][0], has[i][1]);
-                    ex += d;
-                } else {
-                    move(has[i][0], g0 + 1, g0);
-                    move(has[i][1], g0, g0 + 1);
-                }
-            }
-        }
-        SmallLocal s;
-        s.col.assign((size_t)32 * CPL, -1);
-        int next = 32 * LC;
-        for (int i = 0; i < M; ++i)
-            for (int k = 0; k < 2; ++k) {
-                const int q = i < full ? 32 * (2 * (i / 32) + k) + i % 32 : next++;
-                s.col[q] = has[i][k];
-                pos[has[i][k]] = q;
-            }
-        ci.clear(); id.clear(); start.clear();
-        s.word.assign(E, 0);
-        rp[0] = 0;
-        for (int i = 0; i < M; ++i) {
-            for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+    Rng rng{1};
+    for (int k = 0; k < 8; ++k) rng.next();                    // (its first draws are small)
+    // two columns of its own for every full row (augmenting paths; a row has six
+    // columns and a column three rows, so the assignment exists)
+    std::vector<int> own(N, -1), seen(N, -1), via(N, -1), queue, rp(M + 1), ci, id, start, pos(N);
+    std::vector<int> has(2 * (size_t)full, -1);
+    for (int n = 0; n < 2 * full; ++n) {
+        // breadth-first over columns from row n / 2, through the rows that own them
+        queue.clear();
+        int end = -1;
+        std::vector<int> from(full, -1);                       // the column a row would give up
+        std::vector<char> met(full, 0);
+        met[n / 2] = 1;
+        std::vector<int> rows(1, n / 2);
+        for (size_t q = 0; q < rows.size() && end < 0; ++q) {
+            for (int e = row_ptr[rows[q]]; e < row_ptr[rows[q] + 1] && end < 0; ++e) {
                 const int j = col_idx[e];
-                if (i < full && own[j] == i) {
-                    s.word[e] = 2 * i + (has[i][1] == j ? 1 : 0);
-                    continue;
-                }
-                ci.push_back(pos[j]);
-                id.push_back(e);
-                start.push_back((at[e] >> 1) * P + 2 * i + (at[e] & 1));
+                if (seen[j] == n || own[j] == rows[q]) continue;
+                seen[j] = n;
+                via[j] = rows[q];
+                if (own[j] < 0) end = j;
+                else if (!met[own[j]]) { met[own[j]] = 1; from[own[j]] = j; rows.push_back(own[j]); }
             }
-            rp[i + 1] = (int)ci.size();
         }
-        GenericLayout gl;
-        if (!generic_layout(M, N, rp.data(), ci.data(), kColDeg, &gl, start.data(), true)) return false;
-        for (size_t x = 0; x < id.size(); ++x) s.word[id[x]] = gl.pos[x];
-        s.slot.assign((size_t)32 * CPL * kColDeg, 0);
-        for (int q = 0; q < N; ++q) {
-            int k = 0;
-            int* w = s.slot.data() + (size_t)kColDeg * q;
-            if (q < 32 * LC)
-                for (int e : cedges[s.col[q]])
-                    if (erow[e] == own[s.col[q]]) w[k++] = s.word[e];
-            for (int c = 0; c < kColDeg; ++c) {
-                const int x = gl.kedge[(size_t)c * N + q];
-                if (x >= 0 && k < kColDeg) w[k++] = s.word[id[x]];
-            }
-            if (k != kColDeg) return false;
-        }
-        // extra wavefronts of the error pass's accesses
-        int extra = 0;
-        for (int g = 0; g < CPL; ++g)
-            for (int k = g < LC ? 1 : 0; k < kColDeg; ++k) {
-                int load[32] = {0}, most = 0;
-                for (int q = 32 * g; q < std::min(N, 32 * g + 32); ++q)
-                    most = std::max(most, ++load[s.slot[(size_t)kColDeg * q + k] & 31]);
-                extra += most - 1;
-            }
-        if (best < 0 || extra < best) {
-            best = extra;
-            *out = s;
+        if (end < 0) return false;
+        for (int j = end;;) {
+            const int i = via[j], given = i == n / 2 ? -1 : from[i];
+            own[j] = i;
+            int* const h = &has[2 * (size_t)i];
+            if (given < 0) { h[n % 2] = j; break; }
+            h[h[0] == given ? 0 : 1] = j;
+            j = given;
         }
     }
-    out->extent = 2 * P + 2 * M;
-    out->extra = best;
+    std::vector<int> grp(N, LC);
+    for (int n = 0; n < 2 * full; ++n) grp[has[n]] = 2 * (n / 2 / 32) + n % 2;
+    // the words: word[6 i + q] the edge at word q of row i, at[e] its q, bk[e] its bank (-1: in a register)
+    std::vector<int> word((size_t)kRowDeg * M, -1), at(E, -1), bk(E, -1);
+    std::vector<std::vector<int>> words_of(32);                // word indices by bank
+    auto bank = [&](int i, int q) { return ((q >> 1) * P + 2 * i + (q & 1)) & 31; };
+    int cnt[kSmallMaxCpl * 32] = {0}, over[kSmallMaxCpl * 32], overpos[kSmallMaxCpl * 32], nover = 0;
+    int d = 0;                                                 // cost of the current move
+    auto cap = [&](int cell) { return cell < 32 * LC ? 2 : 3; };
+    auto shift = [&](int g, int b, int by) {
+        const int cell = 32 * g + b, c = cnt[cell];
+        cnt[cell] = c + by;
+        d += g < LC ? 2 * by * c + 1 : 4 * (std::max(0, c + by - 3) - std::max(0, c - 3));
+        if (by > 0 && c == cap(cell)) { overpos[cell] = nover; over[nover++] = cell; }
+        if (by < 0 && c == cap(cell) + 1) {
+            over[overpos[cell]] = over[--nover];
+            overpos[over[nover]] = overpos[cell];
+        }
+    };
+    for (int i = 0; i < M; ++i) {
+        int q = i < full ? 2 : 0;
+        for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+            if (own[col_idx[e]] == i) continue;
+            word[(size_t)kRowDeg * i + q] = e;
+            at[e] = q;
+            bk[e] = bank(i, q);
+            words_of[bk[e]].push_back(kRowDeg * i + q);
+            shift(grp[col_idx[e]], bk[e], 1);
+            ++q;
+        }
+    }
+    auto count = [&](int j, int by) {                          // column j's words in the loads
+        for (int k = 0; k < kColDeg; ++k) {
+            const int e = cedge[(size_t)kColDeg * j + k];
+            if (bk[e] >= 0) shift(grp[j], bk[e], by);
+        }
+    };
+    auto edge_in = [&](int j, int i) {
+        const int* e = &cedge[(size_t)kColDeg * j];
+        return erow[e[0]] == i ? e[0] : erow[e[1]] == i ? e[1] : e[2];
+    };
+    uint32_t odds[32] = {0};                                   // of taking a move that costs d
+    auto pass = [&] { return d <= 0 || (d < 32 && rng.next() < odds[d]); };
+    // edge e takes the word x of its row's edge f, which goes into a register
+    auto put = [&](int e, int f) {
+        at[e] = at[f];
+        bk[e] = bk[f];
+        bk[f] = -1;
+        word[(size_t)kRowDeg * erow[e] + at[e]] = e;
+    };
+    for (int n = 0; n < kLocalMoves && nover > 0; ++n) {
+        if (n % 512 == 0) {
+            const double T = 0.7 * std::pow(0.35, (double)n / kLocalMoves);
+            for (int k = 0; k < 32; ++k) odds[k] = (uint32_t)(4294967295.0 * std::exp(-k / T));
+        }
+        // a word of an overloaded bank, or one in five times any word
+        int e = -1;
+        if (rng.pick(5) != 0) {
+            const int cell = over[rng.pick((uint32_t)nover)];
+            const std::vector<int>& w = words_of[cell & 31];
+            uint32_t q = rng.pick((uint32_t)w.size());
+            while (grp[col_idx[word[w[q]]]] != cell >> 5) q = q + 1 < w.size() ? q + 1 : 0;
+            e = word[w[q]];
+        } else {
+            do e = (int)rng.pick((uint32_t)E); while (bk[e] < 0);
+        }
+        const int i = erow[e], j = col_idx[e], lo = i < full ? 2 : 0;
+        const uint32_t kind = rng.pick(10);
+        d = 0;
+        if (kind < 6 || (i >= full && own[j] < 0)) {
+            int y = lo + (int)rng.pick((uint32_t)(kRowDeg - lo - 1));
+            if (y >= at[e]) ++y;
+            const int f = word[(size_t)kRowDeg * i + y], ge = grp[j], gf = grp[col_idx[f]], be = bk[e], bf = bk[f];
+            if (ge == gf) continue;
+            shift(ge, be, -1); shift(ge, bf, 1); shift(gf, bf, -1); shift(gf, be, 1);
+            if (pass()) {
+                std::swap(word[(size_t)kRowDeg * i + at[e]], word[(size_t)kRowDeg * i + y]);
+                std::swap(at[e], at[f]);
+                std::swap(bk[e], bk[f]);
+            } else {
+                shift(gf, be, -1); shift(gf, bf, 1); shift(ge, bf, -1); shift(ge, be, 1);
+            }
+        } else if (own[j] >= 0 && (kind == 6 || i >= full)) {
+            int* const h = &has[2 * (size_t)own[j]];           // the two sides
+            auto swap_sides = [&] {
+                count(h[0], -1); count(h[1], -1);
+                std::swap(grp[h[0]], grp[h[1]]);
+                count(h[0], 1); count(h[1], 1);
+            };
+            swap_sides();
+            if (pass()) std::swap(h[0], h[1]); else swap_sides();
+        } else {
+            // row i owns j in place of its column g; the row i2 that owned j takes
+            // a column l of the last group, or g
+            const int side = (int)rng.pick(2), g = has[2 * (size_t)i + side], i2 = own[j], eg = edge_in(g, i);
+            int l = -1, el = -1, ej = -1, side2 = 0;
+            if (i2 >= 0) {
+                int cand[kRowDeg], nc = 0;
+                for (int q = 2; q < kRowDeg; ++q) {
+                    const int f = word[(size_t)kRowDeg * i2 + q];
+                    if (own[col_idx[f]] < 0 || col_idx[f] == g) cand[nc++] = f;
+                }
+                if (nc == 0) continue;
+                el = cand[rng.pick((uint32_t)nc)];
+                l = col_idx[el];
+                ej = edge_in(j, i2);
+                side2 = has[2 * (size_t)i2] == j ? 0 : 1;
+            }
+            const int gg = grp[g], gj = grp[j];
+            auto count_all = [&](int by) {
+                count(g, by); count(j, by);
+                if (l >= 0 && l != g) count(l, by);
+            };
+            count_all(-1);
+            put(eg, e);
+            own[g] = -1; grp[g] = LC;
+            own[j] = i; grp[j] = gg; has[2 * (size_t)i + side] = j;
+            if (l >= 0) { put(ej, el); own[l] = i2; grp[l] = gj; has[2 * (size_t)i2 + side2] = l; }
+            count_all(1);
+            if (pass()) continue;
+            count_all(-1);
+            if (l >= 0) { put(el, ej); own[l] = -1; grp[l] = LC; has[2 * (size_t)i2 + side2] = j; }
+            put(e, eg);
+            own[j] = i2; grp[j] = gj;
+            own[g] = i; grp[g] = gg; has[2 * (size_t)i + side] = g;
+            count_all(1);
+        }
+    }
+    SmallLocal s;
+    s.col.assign((size_t)32 * CPL, -1);
+    int next = 32 * LC;
+    for (int j = 0; j < N; ++j) {
+        const int i = own[j];
+        pos[j] = i < 0 ? next++ : 32 * grp[j] + i % 32;
+        s.col[pos[j]] = j;
+    }
+    s.word.assign(E, 0);
+    rp[0] = 0;
+    for (int i = 0; i < M; ++i) {
+        for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+            const int j = col_idx[e];
+            if (own[j] == i) {
+                s.word[e] = 2 * i + (grp[j] & 1);
+                continue;
+            }
+            ci.push_back(pos[j]);
+            id.push_back(e);
+            start.push_back((at[e] >> 1) * P + 2 * i + (at[e] & 1));
+        }
+        rp[i + 1] = (int)ci.size();
+    }
+    GenericLayout gl;
+    if (!generic_layout(M, N, rp.data(), ci.data(), kColDeg, &gl, start.data(), true)) return false;
+    for (size_t x = 0; x < id.size(); ++x) s.word[id[x]] = gl.pos[x];
+    // the columns' slots: the register-held word first; the two others of a full
+    // group's columns so that each bank's words fall to the two accesses in equal
+    // parts or one more to the one (colours in turn along trails through columns
+    // and banks, from banks of an odd load first)
+    s.slot.assign((size_t)32 * CPL * kColDeg, 0);
+    for (int g = 0; g < LC; ++g) {
+        int two[32][2], left[32] = {0}, who[32][2 * kRowDeg];
+        bool used[32] = {false};
+        for (int u = 0; u < 32; ++u) {
+            const int j = s.col[32 * g + u];
+            int k = 0;
+            for (int c = 0; c < kColDeg; ++c) {
+                const int e = cedge[(size_t)kColDeg * j + c];
+                if (own[j] == erow[e]) s.slot[(size_t)kColDeg * (32 * g + u)] = s.word[e];
+                else two[u][k++] = s.word[e];
+            }
+            for (k = 0; k < 2; ++k) {
+                const int b = two[u][k] & 31;
+                who[b][left[b]++] = u;
+            }
+        }
+        int load[32];
+        std::copy(left, left + 32, load);
+        for (int n = 0; n < 96; ++n) {                         // odd loads above two, the other odd ones, the rest
+            const int b0 = n & 31;
+            if (n < 64 ? !(load[b0] & 1) || (n < 32 && load[b0] < 3) : false) continue;
+            for (;;) {
+                int b = b0, steps = 0;
+                for (;; ++steps) {
+                    while (left[b] > 0 && used[who[b][left[b] - 1]]) --left[b];
+                    if (left[b] == 0) break;
+                    const int u = who[b][--left[b]];
+                    used[u] = true;
+                    const int first = (two[u][0] & 31) == b ? 0 : 1;
+                    int* const w = &s.slot[(size_t)kColDeg * (32 * g + u)];
+                    w[1] = two[u][first];
+                    w[2] = two[u][1 - first];
+                    b = two[u][1 - first] & 31;
+                }
+                if (steps == 0 || n < 64) break;
+            }
+        }
+    }
+    for (int q = 32 * LC; q < N; ++q) {
+        int k = 0;
+        for (int c = 0; c < kColDeg; ++c) {
+            const int x = gl.kedge[(size_t)c * N + q];
+            if (x >= 0 && k < kColDeg) s.slot[(size_t)kColDeg * q + k++] = s.word[id[x]];
+        }
+        if (k != kColDeg) return false;
+    }
+    s.extent = 2 * P + 2 * M;
+    s.extra = 0;                                               // wavefronts that conflicts add to the error pass
+    for (int g = 0; g < CPL; ++g)
+        for (int k = g < LC ? 1 : 0; k < kColDeg; ++k) {
+            int load[32] = {0}, most = 0;
+            for (int q = 32 * g; q < std::min(N, 32 * g + 32); ++q)
+                most = std::max(most, ++load[s.slot[(size_t)kColDeg * q + k] & 31]);
+            s.extra += most - 1;
+        }
+    *out = s;
+    return true;
+}
+
+// H as the exports take it: rows of ascending columns in range
+static bool csr_valid(int M, int N, const int32_t* row_ptr, const int32_t* col_idx)
+{
+    if (row_ptr[0] != 0) return false;
+    for (int i = 0; i < M; ++i) {
+        if (row_ptr[i + 1] < row_ptr[i]) return false;
+        for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+            if (col_idx[e] < 0 || col_idx[e] >= N) return false;
+            if (e > row_ptr[i] && col_idx[e] <= col_idx[e - 1]) return false;
+        }
+    }
     return true;
 }
 
@@ -626,14 +736,7 @@ extern "C" int bsd_small_layout(int32_t M, int32_t N, const int32_t* H_row_ptr, 
 {
     if (M < 1 || N < 1 || !H_row_ptr || !H_col_idx || !plane || !edge_word || !col_word || !extent || !excess)
         return BSD_ERR_INVALID_ARG;
-    if (H_row_ptr[0] != 0) return BSD_ERR_INVALID_ARG;
-    for (int i = 0; i < M; ++i) {
-        if (H_row_ptr[i + 1] < H_row_ptr[i]) return BSD_ERR_INVALID_ARG;
-        for (int e = H_row_ptr[i]; e < H_row_ptr[i + 1]; ++e) {
-            if (H_col_idx[e] < 0 || H_col_idx[e] >= N) return BSD_ERR_INVALID_ARG;
-            if (e > H_row_ptr[i] && H_col_idx[e] <= H_col_idx[e - 1]) return BSD_ERR_INVALID_ARG;
-        }
-    }
+    if (!bsd::csr_valid(M, N, H_row_ptr, H_col_idx)) return BSD_ERR_INVALID_ARG;
     bsd::SmallLayout sl;
     if (!bsd::small_layout(M, N, H_row_ptr, H_col_idx, &sl)) return BSD_ERR_UNSUPPORTED;
     for (int h = 0; h < 3; ++h) plane[h] = sl.A[h];
@@ -644,19 +747,31 @@ extern "C" int bsd_small_layout(int32_t M, int32_t N, const int32_t* H_row_ptr, 
     return BSD_OK;
 }
 
+extern "C" int bsd_lane_layout(int32_t M, int32_t N, const int32_t* H_row_ptr, const int32_t* H_col_idx,
+                               int32_t* edge_word, int32_t* lane_col, int32_t* lane_word, int32_t* extent,
+                               int32_t* extra)
+{
+    if (M < 1 || N < 1 || !H_row_ptr || !H_col_idx || !edge_word || !lane_col || !lane_word || !extent || !extra)
+        return BSD_ERR_INVALID_ARG;
+    if (!bsd::csr_valid(M, N, H_row_ptr, H_col_idx)) return BSD_ERR_INVALID_ARG;
+    bsd::SmallLocal sl;
+    if (N > 32 * bsd::kSmallMaxCpl || M > 32 * bsd::kSmallMaxRpl ||
+        !bsd::small_local_layout(M, N, H_row_ptr, H_col_idx, &sl))
+        return BSD_ERR_UNSUPPORTED;
+    std::copy(sl.word.begin(), sl.word.end(), edge_word);
+    std::copy(sl.col.begin(), sl.col.end(), lane_col);
+    std::copy(sl.slot.begin(), sl.slot.end(), lane_word);
+    *extent = sl.extent;
+    *extra = sl.extra;
+    return BSD_OK;
+}
+
 extern "C" int bsd_generic_layout(int32_t M, int32_t N, const int32_t* H_row_ptr, const int32_t* H_col_idx,
                                   int32_t* edge_word, int32_t* slot_edge, int32_t* colK, int32_t* excess)
 {
     if (M < 1 || N < 1 || !H_row_ptr || !H_col_idx || !edge_word || !slot_edge || !colK || !excess)
         return BSD_ERR_INVALID_ARG;
-    if (H_row_ptr[0] != 0) return BSD_ERR_INVALID_ARG;
-    for (int i = 0; i < M; ++i) {
-        if (H_row_ptr[i + 1] < H_row_ptr[i]) return BSD_ERR_INVALID_ARG;
-        for (int e = H_row_ptr[i]; e < H_row_ptr[i + 1]; ++e) {
-            if (H_col_idx[e] < 0 || H_col_idx[e] >= N) return BSD_ERR_INVALID_ARG;
-            if (e > H_row_ptr[i] && H_col_idx[e] <= H_col_idx[e - 1]) return BSD_ERR_INVALID_ARG;
-        }
-    }
+    if (!bsd::csr_valid(M, N, H_row_ptr, H_col_idx)) return BSD_ERR_INVALID_ARG;
     const int E = H_row_ptr[M];
     std::vector<int> cdeg(N, 0);
     for (int e = 0; e < E; ++e) cdeg[H_col_idx[e]]++;

@@ -1,0 +1,68 @@
+"""The single-warp engine's shared-memory placement (host logic, no GPU), the one
+bsd_create builds: every edge has its own word among its row's, each full row's pair
+0 holds the edges of two columns of its own lane, every column reads its three
+words, and few bank conflicts are left whatever the numbering of rows and columns."""
+import numpy as np
+import pytest
+
+from paper_2512_07057_gb300 import binding as B
+from paper_2512_07057_gb300 import workloads as W
+
+
+def _renumbered(prob, seed):
+    rng = np.random.default_rng(seed)
+    H = prob.H_dense()[rng.permutation(prob.M)][:, rng.permutation(prob.N)]
+    return W.problem_from_dense(H, np.zeros((1, prob.N), np.uint8), np.full(prob.N, 0.05))
+
+
+def _check(prob):
+    M, N, rp, ci = prob.M, prob.N, prob.H_row_ptr, prob.H_col_idx
+    lay = B.bsd_lane_layout(M, N, rp, ci)
+    ew, col, lw = lay["edge_word"], lay["lane_col"].reshape(-1), lay["lane_word"].reshape(-1, 3)
+    P, full = 64 * ((M + 31) // 32) + 12, 32 * ((M - 1) // 32)
+    groups = (N + 31) // 32
+    assert lay["extent"] == 2 * P + 2 * M
+    for i in range(M):                                       # a row's six words
+        assert sorted(ew[rp[i]:rp[i + 1]].tolist()) == sorted(h * P + 2 * i + u for h in range(3) for u in range(2))
+    assert sorted(c for c in col.tolist() if c >= 0) == list(range(N)) and (col[:N] >= 0).all()
+    words = [[] for _ in range(N)]
+    for e, j in enumerate(ci):
+        words[j].append(int(ew[e]))
+    for q in range(N):                                       # a column's three words
+        assert sorted(lw[q].tolist()) == sorted(words[col[q]])
+    for i in range(full):                                    # the register-held pair, in the row's own lane
+        for u in range(2):
+            assert lw[32 * (2 * (i // 32) + u) + i % 32, 0] == 2 * i + u
+    extra = 0
+    for g in range(groups):
+        for k in range(1 if g < groups - 1 else 0, 3):
+            extra += np.bincount(lw[32 * g:min(N, 32 * g + 32), k] % 32).max() - 1
+    assert lay["extra"] == extra
+    return extra
+
+
+@pytest.mark.parametrize("M", [33, 40, 48, 65, 72, 80])
+@pytest.mark.parametrize("seed", [1, 2])
+def test_placement_of_random_regular_codes(M, seed):
+    _check(W.random_regular_36(M, 0.05, seed))
+
+
+def test_no_numbering_of_a_code_is_placed_much_worse():
+    """Extra wavefronts beside the 11 (7) of the error pass: a search that fits one
+    numbering leaves 6 on [[144,12,12]] and 4 on [[72,12,6]] under others."""
+    for prob, most in ((W.bb144_code_capacity(0.05), 3), (W.bb72_code_capacity(0.05), 2)):
+        extra = [_check(prob)] + [_check(_renumbered(prob, s)) for s in range(10)]
+        assert max(extra) <= most and np.mean(extra) <= most - 1, extra
+
+
+def test_other_structures_are_unsupported():
+    for prob in (W.random_ldpc(40, 80, 4, 0.05, seed=1), W.random_regular_36(64, 0.05, 1), W.random_regular_36(32, 0.05, 1)):
+        with pytest.raises(B.BsdError) as ei:
+            B.bsd_lane_layout(prob.M, prob.N, prob.H_row_ptr, prob.H_col_idx)
+        assert ei.value.code == B.BSD_ERR_UNSUPPORTED
+    prob = W.bb72_code_capacity(0.05)
+    ci = prob.H_col_idx.copy()
+    ci[1] = ci[0]
+    with pytest.raises(B.BsdError) as ei:
+        B.bsd_lane_layout(prob.M, prob.N, prob.H_row_ptr, ci)
+    assert ei.value.code == B.BSD_ERR_INVALID_ARG

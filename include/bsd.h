@@ -303,14 +303,13 @@ int bsd_small_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32
 int bsd_lane_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32_t *H_col_idx, int32_t *edge_word,
                     int32_t *lane_col, int32_t *lane_word, int32_t *extent, int32_t *extra);
 
-/* Where the generic engines keep a candidate's messages (a layout choice of
+/* A placement of a candidate's messages in CSR storage (a layout choice of
  * this library, for codes with every column of degree at most 6): each row's
  * edges permuted inside the row's storage window, each column's edges in the
  * k slots of the padded column table (colK = 3 for a largest column degree of
  * 3 or less, else 6), chosen so that the 32 lanes of an error-pass access
- * meet distinct banks where possible.  bsd_create runs the same search over the
- * storage of its engine for these codes, where the rows stand by falling degree
- * with their k-th edges side by side.
+ * meet distinct banks where possible.  No engine keeps its messages by it: that of
+ * these codes is bsd_jagged_layout, whose search ends sooner.
  * Host only; nothing is allocated on a device.
  *   M, N, H_row_ptr, H_col_idx  host, H in CSR as for bsd_create
  *   edge_word  host int32[E]: out, the element of CSR edge e
@@ -323,6 +322,25 @@ int bsd_lane_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32_
  * (a column of degree above 6, or more than 2^20 edges). */
 int bsd_generic_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32_t *H_col_idx,
                        int32_t *edge_word, int32_t *slot_edge, int32_t *colK, int32_t *excess);
+
+/* Where the jagged engine keeps a candidate's messages (codes with every column of
+ * degree at most 6): the placement that bsd_create builds.  The rows stand by
+ * falling degree; the k-th words of all rows that have one lie side by side, so
+ * that the row of rank q has the words (rows with more than k edges, summed over
+ * the k before) + q.  Its edges are permuted among them, and the columns stand in
+ * their own order or by degree, so that the error pass's accesses, the k-th slots of
+ * 32 columns, meet few bank conflicts.  Host only; nothing is allocated on a device.
+ *   M, N, H_row_ptr, H_col_idx  host, H in CSR as for bsd_create
+ *   rank_row   host int32[M]: out, the row of rank q
+ *   edge_word  host int32[E]: out, the word of CSR edge e
+ *   column     host int32[N]: out, the column at position p
+ *   slot_edge  host int32[6 N]: out, the CSR edge in slot k of the column at
+ *              position p at [k * N + p], -1 for an empty slot (colK * N used)
+ *   colK       host int32: out, 3 or 6
+ * Errors: BSD_ERR_INVALID_ARG (null pointer, bad CSR), BSD_ERR_UNSUPPORTED
+ * (a column of degree above 6). */
+int bsd_jagged_layout(int32_t M, int32_t N, const int32_t *H_row_ptr, const int32_t *H_col_idx, int32_t *rank_row,
+                      int32_t *edge_word, int32_t *column, int32_t *slot_edge, int32_t *colK);
 
 /* Opt-in timing of this library's kernels (not part of the method): while
  * enabled, every kernel launch made by bsd_decode / bsd_decode_host is

@@ -31,7 +31,8 @@ BSD_STATUS_FAILED = 4
 
 # every symbol include/bsd.h declares
 EXPORTS = ("bsd_params_default", "bsd_params_preset", "bsd_create", "bsd_decode", "bsd_decode_host",
-           "bsd_bp_llr", "bsd_sync_error", "bsd_get_info", "bsd_get_batch", "bsd_small_layout", "bsd_lane_layout", "bsd_generic_layout", "bsd_serve_start", "bsd_serve_decode",
+           "bsd_bp_llr", "bsd_sync_error", "bsd_get_info", "bsd_get_batch", "bsd_small_layout", "bsd_lane_layout", "bsd_generic_layout", "bsd_jagged_layout",
+           "bsd_serve_start", "bsd_serve_decode",
            "bsd_serve_stop", "bsd_profile_enable", "bsd_profile_read",
            "bsd_decode_noalloc", "bsd_set_weights", "bsd_unrolled_workspace", "bsd_unrolled_forward",
            "bsd_unrolled_backward", "bsd_profile_read_kinds", "bsd_autotune", "bsd_get_shape", "bsd_dem_parse",
@@ -93,6 +94,7 @@ def load(path: str | None = None) -> C.CDLL:
     lib.bsd_lane_layout.argtypes = [C.c_int32, C.c_int32, P, P, P, P, P, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
     lib.bsd_generic_layout.argtypes = [C.c_int32, C.c_int32, P, P, P, P, C.POINTER(C.c_int32),
                                        C.POINTER(C.c_int32)]
+    lib.bsd_jagged_layout.argtypes = [C.c_int32, C.c_int32, P, P, P, P, P, P, C.POINTER(C.c_int32)]
     lib.bsd_decode_noalloc.argtypes = [P, P, C.c_int64, P, P, P, P, P]
     lib.bsd_profile_enable.argtypes = [P, C.c_int]
     lib.bsd_set_weights.argtypes = [P, P, C.c_int32]
@@ -244,7 +246,7 @@ def bsd_lane_layout(M: int, N: int, row_ptr, col_idx) -> dict:
 
 
 def bsd_generic_layout(M: int, N: int, row_ptr, col_idx) -> dict:
-    """The generic engines' placement of H's messages (host only): the
+    """A placement of H's messages in CSR storage (host only; no engine's): the
     element of every CSR edge, the CSR edge in every (k, column) slot
     ([colK][N], -1 empty), colK and the bank loads above the groups' largest
     degrees left by the search."""
@@ -258,6 +260,22 @@ def bsd_generic_layout(M: int, N: int, row_ptr, col_idx) -> dict:
                                     C.byref(ck), C.byref(exc)), "bsd_generic_layout")
     return dict(edge_word=ew, slot_edge=se[:ck.value * int(N)].reshape(ck.value, int(N)), colK=ck.value,
                 excess=exc.value)
+
+
+def bsd_jagged_layout(M: int, N: int, row_ptr, col_idx) -> dict:
+    """The jagged engine's placement of H's messages (host only): the row of every
+    rank, the word of every CSR edge, the column at every position, the CSR edge in
+    every (slot, position) ([colK][N], -1 empty) and colK."""
+    import numpy as np
+    rp = np.ascontiguousarray(row_ptr, dtype=np.int32)
+    ci = np.ascontiguousarray(col_idx, dtype=np.int32)
+    rows, ew = np.zeros(int(M), np.int32), np.zeros(int(rp[-1]), np.int32)
+    col, se = np.zeros(int(N), np.int32), np.zeros(6 * int(N), np.int32)
+    ck = C.c_int32()
+    check(load().bsd_jagged_layout(int(M), int(N), rp.ctypes.data, ci.ctypes.data, rows.ctypes.data, ew.ctypes.data,
+                                   col.ctypes.data, se.ctypes.data, C.byref(ck)), "bsd_jagged_layout")
+    return dict(rank_row=rows, edge_word=ew, column=col, slot_edge=se[:ck.value * int(N)].reshape(ck.value, int(N)),
+                colK=ck.value)
 
 
 def bsd_set_weights(dec, h_weights, T: int) -> None:

@@ -412,84 +412,42 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
             std::memcpy(&slamE_st[(size_t)sl.word[e] * msg_bytes], &lamE_st[(size_t)e * msg_bytes], msg_bytes);
         }
     }
-    // the generic engines' column table: (edge, row) of the k-th edge of column
-    // j at [k][j], (-1, -1) past the column's degree, for degree bounds 3 and 6
+    // the jagged engine's tables (column degree bounds 3 and 6): rows by falling
+    // degree, the planes of their k-th edges, the words of every column's edges
     const int colK = max_col <= 3 ? 3 : max_col <= 6 ? 6 : 0;
-    // the jagged engine's tables: rows by falling degree, the planes of their
-    // k-th edges, the words of every column's edges
     std::vector<int2> rowQ;
     std::vector<int> jplanes, colW, colN, colJ, colF, jpos;
     std::vector<uint8_t> colG, rowG;
     std::vector<float> jD0;
     if (colK > 0) {
-        std::vector<int> ord(M), start((size_t)E);
-        for (int i = 0; i < M; ++i) ord[i] = i;
-        auto rdeg = [&](int i) { return H_row_ptr[i + 1] - H_row_ptr[i]; };
-        std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return rdeg(x) > rdeg(y); });
-        jplanes.assign(max_row > 0 ? max_row : 1, 0);
-        for (int k = 0, at = 0; k < max_row; ++k) {
-            jplanes[k] = at;
-            for (int q = 0; q < M && rdeg(ord[q]) > k; ++q) start[(size_t)H_row_ptr[ord[q]] + k] = at++;
-        }
-        for (int q = 0; q < M; ++q) rowQ.push_back(make_int2(ord[q], rdeg(ord[q])));
+        JaggedLayout jl;
+        jagged_layout(M, N, H_row_ptr, H_col_idx, colK, &jl);
+        for (int q = 0; q < M; ++q)
+            rowQ.push_back(make_int2(jl.row[q], H_row_ptr[jl.row[q] + 1] - H_row_ptr[jl.row[q]]));
         for (int q = 0; q < M; q += 32) {
             const int hi = rowQ[q].y, lo = rowQ[std::min(M, q + 32) - 1].y;
             rowG.push_back((uint8_t)(hi > 16 ? 64 : hi + (lo < hi ? 32 : 0)));
         }
-        // the columns' positions: natural, or by degree where more than a quarter
-        // of the groups would hold several (columns of degree 2 to 6 at random,
-        // 35110 edges: the seed BP of 4300 shots 4.2 -> 3.5 ms together with the tables loaded ahead)
-        std::vector<int> order(N);
-        for (int j = 0; j < N; ++j) order[j] = j;
-        auto cdeg = [&](int j) { return col_ptr[j + 1] - col_ptr[j]; };
-        int several = 0;
-        for (int q = 0; q < WN; ++q) {
-            bool same = true;
-            for (int j = 32 * q; j < std::min(N, 32 * q + 32); ++j) same = same && cdeg(j) == cdeg(32 * q);
-            several += same ? 0 : 1;
-        }
-        if (4 * several > WN) {
-            std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cdeg(x) < cdeg(y); });
-            colJ = order;
-        }
-        // the edges with their column's position, for the search's column groups
-        std::vector<int> at(N), ci((size_t)(E > 0 ? E : 1));
-        for (int q = 0; q < N; ++q) at[order[q]] = q;
-        for (long long e = 0; e < E; ++e) ci[e] = at[H_col_idx[e]];
-        GenericLayout gl;
-        const bool has_gl = generic_layout(M, N, H_row_ptr, ci.data(), colK, &gl, start.data(), true);
-        jpos = has_gl ? gl.pos : start;
-        // a group of 32 columns of one degree keeps its edges in the first slots
+        jplanes = jl.plane;
+        jpos = jl.word;
+        if (jl.dealt) colJ = jl.order;
         colW.assign((size_t)colK * Npad, -1);
         colN.assign((size_t)colK * Npad, -1);
         colF.assign((size_t)colK * Npad, -1);
-        for (int p = 0; p < N; ++p)
-            for (int k = 0; k < cdeg(order[p]); ++k) colF[(size_t)k * Npad + p] = col_row[col_ptr[order[p]] + k];
         colG.assign((size_t)WN, 0);
         for (int q = 0; q < WN; ++q) {
             int lo = colK, hi = 0;
             for (int p = 32 * q; p < std::min(N, 32 * q + 32); ++p) {
-                lo = std::min(lo, cdeg(order[p]));
-                hi = std::max(hi, cdeg(order[p]));
+                const int j = jl.order[p], deg = col_ptr[j + 1] - col_ptr[j];
+                lo = std::min(lo, deg);
+                hi = std::max(hi, deg);
+                for (int k = 0; k < deg; ++k) colF[(size_t)k * Npad + p] = col_row[col_ptr[j] + k];
+                for (int k = 0; k < colK; ++k) {
+                    const int e = jl.slot[(size_t)k * N + p];
+                    if (e >= 0) colW[(size_t)k * Npad + p] = colN[(size_t)k * Npad + j] = jpos[e];
+                }
             }
             colG[q] = (uint8_t)(lo == hi ? hi : hi + 8);
-            for (int p = 32 * q; p < std::min(N, 32 * q + 32); ++p) {
-                const int j = order[p];
-                int slot[kMaxColDeg], rest[kMaxColDeg], nrest = 0;
-                for (int k = 0; k < colK; ++k) slot[k] = -1;
-                for (int k = 0; k < colK; ++k) {
-                    const int e = has_gl ? gl.kedge[(size_t)k * N + p] : (k < cdeg(j) ? col_edge[col_ptr[j] + k] : -1);
-                    if (e < 0) continue;
-                    if (k < hi) slot[k] = e; else rest[nrest++] = e;
-                }
-                for (int k = 0; k < hi && nrest > 0; ++k)
-                    if (slot[k] < 0) slot[k] = rest[--nrest];
-                for (int k = 0; k < hi; ++k)
-                    if (slot[k] >= 0) {
-                        colW[(size_t)k * Npad + p] = jpos[slot[k]];
-                        colN[(size_t)k * Npad + j] = jpos[slot[k]];
-                    }
-            }
         }
         jD0.assign((size_t)(E > 0 ? E : 1), 0.f);
         for (long long e = 0; e < E; ++e) jD0[jpos[e]] = D0[e];

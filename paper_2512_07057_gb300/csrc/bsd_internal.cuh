@@ -173,6 +173,17 @@ constexpr int kGenericLayoutMaxEdges = 1 << 20;
 // (start: the words to permute within each row, null for the storage windows)
 bool generic_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, GenericLayout* out,
                     const int* start = nullptr, bool quick = false);
+// the jagged engine's placement (column degree bound colK = 3 or 6): row[q] the row of
+// rank q, by falling degree; plane[k] the word of the k-th edge of rank 0; word[e] the
+// word of CSR edge e, plane[k] + q for some k of its row; order[p] the column at position
+// p, dealt = not its own order; slot[k N + p] the CSR edge in slot k of that column, -1:
+// empty (a group of 32 columns of one degree fills its first slots, any other those below
+// its largest degree)
+struct JaggedLayout {
+    std::vector<int> row, plane, word, order, slot;
+    bool dealt;
+};
+void jagged_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, JaggedLayout* out);
 constexpr int kJaggedPlanes = 16;        // planes whose offsets travel with the kernel parameters
 // the placement's plane stride for codes of M rows (the engine holds
 // ceil(M / 32) rows per lane); every plane spans 2 M <= 64 ceil(M / 32) words

@@ -714,6 +714,64 @@ bool small_local_layout(int M, int N, const int* row_ptr, const int* col_idx, Sm
     return true;
 }
 
+void jagged_layout(int M, int N, const int* row_ptr, const int* col_idx, int colK, JaggedLayout* out)
+{
+    const int E = row_ptr[M], WN = (N + 31) / 32;
+    JaggedLayout l;
+    auto rdeg = [&](int i) { return row_ptr[i + 1] - row_ptr[i]; };
+    for (int i = 0; i < M; ++i) l.row.push_back(i);
+    std::stable_sort(l.row.begin(), l.row.end(), [&](int x, int y) { return rdeg(x) > rdeg(y); });
+    std::vector<int> start((size_t)std::max(E, 1), 0);
+    l.plane.assign(std::max(1, rdeg(l.row[0])), 0);
+    for (int k = 0, at = 0; k < rdeg(l.row[0]); ++k) {
+        l.plane[k] = at;
+        for (int q = 0; q < M && rdeg(l.row[q]) > k; ++q) start[(size_t)row_ptr[l.row[q]] + k] = at++;
+    }
+    // the columns' positions: natural, or by degree where more than a quarter
+    // of the groups would hold several (columns of degree 2 to 6 at random,
+    // 35110 edges: the seed BP of 4300 shots 4.2 -> 3.5 ms together with the tables loaded ahead)
+    std::vector<int> cdeg(N, 0);
+    for (int e = 0; e < E; ++e) cdeg[col_idx[e]]++;
+    for (int j = 0; j < N; ++j) l.order.push_back(j);
+    int several = 0;
+    for (int q = 0; q < WN; ++q) {
+        bool same = true;
+        for (int j = 32 * q; j < std::min(N, 32 * q + 32); ++j) same = same && cdeg[j] == cdeg[32 * q];
+        several += same ? 0 : 1;
+    }
+    l.dealt = 4 * several > WN;
+    if (l.dealt) std::stable_sort(l.order.begin(), l.order.end(), [&](int x, int y) { return cdeg[x] < cdeg[y]; });
+    // the search over the rows' words, with the edges' columns by position
+    std::vector<int> at(N), ci((size_t)std::max(E, 1));
+    for (int p = 0; p < N; ++p) at[l.order[p]] = p;
+    for (int e = 0; e < E; ++e) ci[e] = at[col_idx[e]];
+    GenericLayout gl;
+    if (generic_layout(M, N, row_ptr, ci.data(), colK, &gl, start.data(), true)) {
+        l.word = gl.pos;
+        l.slot = gl.kedge;
+    } else {                                   // too many edges to search: as they come
+        l.word = start;
+        l.slot.assign((size_t)colK * N, -1);
+        std::vector<int> fill(N, 0);
+        for (int e = 0; e < E; ++e) l.slot[(size_t)fill[ci[e]]++ * N + ci[e]] = e;
+    }
+    for (int q = 0; q < WN; ++q) {
+        int hi = 0;
+        for (int p = 32 * q; p < std::min(N, 32 * q + 32); ++p) hi = std::max(hi, cdeg[l.order[p]]);
+        for (int p = 32 * q; p < std::min(N, 32 * q + 32); ++p) {
+            int free = 0;
+            for (int k = hi; k < colK; ++k) {
+                int& from = l.slot[(size_t)k * N + p];
+                if (from < 0) continue;
+                while (l.slot[(size_t)free * N + p] >= 0) ++free;
+                l.slot[(size_t)free * N + p] = from;
+                from = -1;
+            }
+        }
+    }
+    *out = l;
+}
+
 // H as the exports take it: rows of ascending columns in range
 static bool csr_valid(int M, int N, const int32_t* row_ptr, const int32_t* col_idx)
 {
@@ -784,5 +842,26 @@ extern "C" int bsd_generic_layout(int32_t M, int32_t N, const int32_t* H_row_ptr
     for (size_t q = 0; q < gl.kedge.size(); ++q) slot_edge[q] = gl.kedge[q];
     *colK = K;
     *excess = gl.excess;
+    return BSD_OK;
+}
+
+extern "C" int bsd_jagged_layout(int32_t M, int32_t N, const int32_t* H_row_ptr, const int32_t* H_col_idx,
+                                 int32_t* rank_row, int32_t* edge_word, int32_t* column, int32_t* slot_edge,
+                                 int32_t* colK)
+{
+    if (M < 1 || N < 1 || !H_row_ptr || !H_col_idx || !rank_row || !edge_word || !column || !slot_edge || !colK)
+        return BSD_ERR_INVALID_ARG;
+    if (!bsd::csr_valid(M, N, H_row_ptr, H_col_idx)) return BSD_ERR_INVALID_ARG;
+    std::vector<int> cdeg(N, 0);
+    for (int e = 0; e < H_row_ptr[M]; ++e) cdeg[H_col_idx[e]]++;
+    const int max_col = *std::max_element(cdeg.begin(), cdeg.end());
+    if (max_col > 6) return BSD_ERR_UNSUPPORTED;
+    *colK = max_col <= 3 ? 3 : 6;
+    bsd::JaggedLayout l;
+    bsd::jagged_layout(M, N, H_row_ptr, H_col_idx, *colK, &l);
+    std::copy(l.row.begin(), l.row.end(), rank_row);
+    std::copy(l.word.begin(), l.word.begin() + H_row_ptr[M], edge_word);
+    std::copy(l.order.begin(), l.order.end(), column);
+    std::copy(l.slot.begin(), l.slot.end(), slot_edge);
     return BSD_OK;
 }

@@ -106,6 +106,7 @@ def parse():
                     help="target CPU time of each side-by-side workload's oracle baseline")
     ap.add_argument("--train-steps", type=int, default=300, help="unrolled_training: steps before the LER judgement")
     ap.add_argument("--judge-shots", type=int, default=1_000_000, help="unrolled_training: held-out shots")
+    ap.add_argument("--details", default=None, help="file for the whole record (the result line is a short form)")
     a = ap.parse_args()
     if a.workload == "phenom_precision":
         if a.ps == "0.01,0.03,0.05":
@@ -182,6 +183,61 @@ class ClockSampler:
             return {"sm_mhz": None, "sm_max_mhz": None, "reasons": ["no samples"]}
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": max(smax), "reasons": sorted(reasons),
                 "samples": len(sm), "power_w_max": max(power) if power else None}
+
+
+# A result line is one JSON line of at most this many characters: what reads a run's
+# output may keep no more than its end.  --details FILE writes the whole record.
+LINE_LIMIT = 2600
+# what a result line always holds
+CONTRACT = ("impl", "unavailable", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+            "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks",
+            "roofline", "cpu_baseline", "msg_updates_per_s", "ler", "side_by_side")
+# explanations and tables that only the whole record holds
+DETAIL = {"timed", "sample_shots", "launch_shapes", "measured_in", "msg_updates_counted", "peak_source",
+          "traffic_source", "source", "dram_measured", "alu_view", "samples", "single_core", "record"}
+DETAILS_FILE = None
+
+
+def _pruned(x):
+    if isinstance(x, dict):
+        return {k: _pruned(v) for k, v in x.items() if k not in DETAIL}
+    if isinstance(x, list):
+        return [_pruned(v) for v in x]
+    return float(f"{x:.7g}") if isinstance(x, float) else x
+
+
+def _values(x, name=""):
+    """Every "value" of nested records, by its place."""
+    out = {}
+    for k, v in x.items():
+        if k == "value" and name:
+            out[name] = float(f"{v:.5g}")
+        elif isinstance(v, dict) and k not in ("cpu_baseline", "roofline", "e2e"):
+            out.update(_values(v, name if k in ("forms", "per_width") else f"{name}.{k}" if name else k))
+    return out
+
+
+def shorten(line: dict) -> dict:
+    """The line within LINE_LIMIT: details left out, the side-by-side runs as their
+    values, per-p records as their logical error rates, then whatever the contract
+    does not name, largest first."""
+    out = _pruned(line)
+    if "side_by_side" in line:
+        out["side_by_side"] = _values(line["side_by_side"])
+    if "per_p" in line:
+        out["ler"] = {p: v["ler"] for p, v in out.pop("per_p").items() if "ler" in v}
+    for key in sorted((k for k in out if k not in CONTRACT), key=lambda k: -len(json.dumps(out[k]))):
+        if len(json.dumps(out)) <= LINE_LIMIT:
+            break
+        out.pop(key)
+    return out
+
+
+def emit(line: dict) -> None:
+    if DETAILS_FILE:
+        with open(DETAILS_FILE, "w") as f:
+            json.dump(line, f)
+    print(json.dumps(line if len(json.dumps(line)) <= LINE_LIMIT else shorten(line)), flush=True)
 
 
 def make_phen_workload(rank: int, shots: int, ps=PHEN_PS):
@@ -311,7 +367,7 @@ def run_reference_unrolled(args):
             "cpu_baseline": {"value": value, "unit": "training syndromes/s", "cores": nth, "kind": "oracle",
                              "sample": sample},
             "e2e": {"value": value, "unit": "training syndromes/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def run_reference_synthetic(args):
@@ -341,7 +397,7 @@ def run_reference_synthetic(args):
             "config": {"workload": SYN_WORKLOAD, "shots_per_width_per_step": n, "l2": "n/a (host)"},
             "cpu_baseline": {"value": value, "unit": "syndromes/s", "cores": nth, "kind": "oracle", "sample": sample},
             "e2e": {"value": value, "unit": "syndromes/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def run_reference_latency(args):
@@ -375,7 +431,7 @@ def run_reference_latency(args):
                              "kind": "oracle", "sample": f"{n} single-syndrome decodes per case, one thread"},
             "e2e": {"value": 1e6 / mean_us, "unit": "syndromes/s (one at a time)", "h2d_bytes_per_step": 0,
                     "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def run_reference(args, rank: int):
@@ -426,7 +482,7 @@ def run_reference(args, rank: int):
             "config": {"workload": wl_name, "shots_per_p_per_step": n, "l2": "n/a (host)"},
             "cpu_baseline": {"value": value, "unit": "syndromes/s", "cores": nth, "kind": "oracle", "sample": sample},
             "e2e": {"value": value, "unit": "syndromes/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 KIND_NAMES = {0: "k_seed", 1: "k_round", 2: "beam set-up", 8: "k_bs_check", 9: "k_bs_var", 10: "k_bs_retire",
@@ -477,7 +533,8 @@ def alu_roofline(prof, E: int, dev: int, traffic_case: str, shots: int = 0, msg_
         ms_launch += float(kinds_ms[11]) / launches
     upd_launch = updates / launches
     ops_tops = OPS_PER_UPDATE * upd_launch / (ms_launch * 1e-3) / 1e12
-    share = float(kinds_ms[dom_kind] / max(kinds_ms[[0, 1, 2, 8, 9, 10, 11]].sum(), 1e-9))
+    stage = kinds_ms[dom_kind] + (kinds_ms[11] if name == "k_screen+k_seed" else 0.0)
+    share = float(stage / max(kinds_ms[[0, 1, 2, 8, 9, 10, 11]].sum(), 1e-9))
     common = {"kernel": name, "msg_updates_per_launch": upd_launch, "launch_ms": ms_launch, "kernel_share": share,
               "ops_per_msg_update": OPS_PER_UPDATE,
               "measured_in": "second timed region: same steps, each kernel launched alone between CUDA events "
@@ -694,7 +751,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
     if world == 1 and not args.no_side_by_side:
         line["side_by_side"] = side_by_side(args, dev)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
 
 
 def side_by_side(args, dev) -> dict:
@@ -872,7 +929,7 @@ def run_precision(args, rank: int, world: int, local_rank: int):
         line["cpu_baseline"] = res["cpu_baseline"]
         line["fp64_agreement"] = res["fp64_agreement"]
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
 
 
 def unrolled_bytes_per_launch(kind: int, E: int, N: int, M: int, Bp: int, T: int) -> float:
@@ -977,7 +1034,8 @@ def run_unrolled(args, rank: int, world: int, local_rank: int):
         # both kernels read and write every message twice per iteration in shared memory (128 bytes per clock and SM)
         alg = 16.0 * E * Bn * T
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
-        peak, bound, source = sms * 128 * 2.07, "shared memory", f"{sms} SMs x 128 B x 2070 MHz"
+        mhz = float(pk.get("sm_max_mhz", 2070.0))
+        peak, bound, source = sms * 128 * mhz * 1e-3, "shared memory", f"{sms} SMs x 128 B x {mhz:.0f} MHz ({pk_kind})"
     else:
         alg = unrolled_bytes_per_launch(dom, E, N, M, Bp, T)
         peak, bound, source = float(pk.get("hbm_gbs", 6800.0)), "hbm", f"hbm_gbs ({pk_kind})"
@@ -1020,7 +1078,7 @@ def run_unrolled(args, rank: int, world: int, local_rank: int):
         line["cpu_baseline"] = _unrolled_cpu_baseline(prob, T, args.cpu_seconds)
     tr.close()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
 
 
 def _unrolled_e2e(tr, w, opt, prob, Bn, args, dev):
@@ -1279,7 +1337,7 @@ def run_synthetic(args, rank: int, world: int, local_rank: int):
     if "cpu_baseline" in res:
         line["cpu_baseline"] = res["cpu_baseline"]
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
 
 
 def run_xyz(args, rank: int, world: int, local_rank: int):
@@ -1377,7 +1435,7 @@ def run_xyz(args, rank: int, world: int, local_rank: int):
     if rank == 0 and not args.no_e2e:
         line["e2e"] = e2e_host(decs, work, args, dev)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
     for d in decs:
         d.close()
 
@@ -1488,7 +1546,7 @@ def run_latency(args, rank: int, world: int, local_rank: int):
             "context": "the paper reports 99.9 percentile decoding times per syndrome on one CPU core for its "
                        "circuit-level [[144,12,12]] workload (Tables II-III); that workload is not available here"}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
 
 
 def run_num_results(args, rank: int, world: int, local_rank: int):
@@ -1578,7 +1636,7 @@ def run_num_results(args, rank: int, world: int, local_rank: int):
                                 "sample": f"first {n} shots of each p batch, beam64_32res_640iters, double-precision "
                                           f"oracle, {dt:.1f} s"}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
 
 
 def e2e_host(decs, work, args, dev):
@@ -1678,9 +1736,10 @@ def _source_hash(files=None) -> str:
 
 
 def main():
-    global NO_AUTOTUNE
+    global NO_AUTOTUNE, DETAILS_FILE
     args = parse()
     NO_AUTOTUNE = args.no_autotune
+    DETAILS_FILE = args.details
     world = int(os.environ.get("WORLD_SIZE", "1"))
     rank = int(os.environ.get("RANK", "0"))
     local_rank = int(os.environ.get("LOCAL_RANK", "0"))

@@ -306,7 +306,7 @@ def bsd_profile_enable(dec, enable: bool) -> None:
 
 
 def bsd_profile_read(dec) -> dict:
-    """Kernel times (ms) and launches per kind (seed, round, select), executed full iterations,
+    """Kernel times (ms) and launches per kind (seed, the beam, its set-up), executed full iterations,
     kernel launches, message updates of first-iteration screens."""
     import numpy as np
     ms = np.zeros(3, np.float64)
@@ -320,9 +320,9 @@ def bsd_profile_read(dec) -> dict:
 
 
 def bsd_profile_read_kinds(dec) -> dict:
-    """Event-timed ms and launches of every kernel kind (0 seed, 1 round, 2 select,
+    """Event-timed ms and launches of every kernel kind (0 seed, 1 the beam, 2 its set-up,
     3..6 unrolled check / error / error adjoint / check adjoint, 7 other unrolled,
-    8..10 batched seed check / error / retirement, 11 first-iteration screen)."""
+    8..10 batched seed check / error / retirement, 11 the screens)."""
     import numpy as np
     ms = np.zeros(BSD_PROFILE_KINDS, np.float64)
     ln = np.zeros(BSD_PROFILE_KINDS, np.int64)

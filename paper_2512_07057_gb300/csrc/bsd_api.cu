@@ -3,8 +3,8 @@
 // bsd_create validates (H, A, p) and the Alg. 3 parameters, builds the
 // device graph tables (CSR, per-column edge lists, column bitsets of H and A,
 // prior LLRs) and sizes the beam workspace; bsd_decode splits a batch into
-// chunks that fit the workspace and launches, per chunk, the seed kernel and
-// two kernels per beam round, all on the caller's stream.
+// chunks that fit the workspace and launches, per chunk, one graph on the caller's
+// stream: the screens, the seed BP and the beam in one persistent kernel.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -95,10 +95,19 @@ constexpr long long kBatchMinEdges = 16384;
 constexpr int kBatchDefaultSlots = 2048;
 // by default the batch runs on at least this many shots: below, its passes over
 // the graph for the last few slots take longer than the per-candidate kernel
-// (4300 shots of the synthetic DEM, 75 of them failing: 9.5 against 2 ms)
+// (4300 shots of the synthetic DEM, 75 of them failing: 9.5 against 2 ms).  The
+// same code with its priors times 4, seed BP only, per candidate / batched: 20400
+// shots waiting 6.2 / 10.4 ms, 40700 11.5 / 16.1, 67800 19.6 / 24.5, 203000 57.6 / 64.2;
+// in half precision 58.1 / 63.2.  So the batch has not been found faster on either
+// side since a candidate runs on 16 warps; the line keeps it off where it loses most.
 constexpr int kBatchMinQueue = 65536;
 // the second-iteration screen is built while the columns next to flipped
-// detectors are expected to be at most this share of all
+// detectors are expected to be at most this share of all.  5 x 10^4 shots, seed BP
+// only, with it / without: phenomenological DEM at a share of 0.06 0.68 / 0.96 ms, 0.12
+// 2.11 / 2.16, 0.16 3.31 / 2.86, 0.20 4.59 / 3.65; synthetic DEM (priors times 1 to 6)
+// 0.03 0.96 / 2.51, 0.10 5.24 / 9.25, 0.13 9.80 / 12.53, 0.19 16.87 / 16.96.  Depolarizing
+// noise, few of whose shots end at t = 2, does without it: 0.03 0.405 / 0.399, 0.08 0.78 /
+// 0.69, 0.15 1.24 / 1.10.
 constexpr double kScreen2MaxShare = 0.125;
 
 const char* kPresetNames[] = {"beam8_230iters", "beam32_340iters", "beam64_640iters", "beam64_32res_640iters"};
@@ -766,11 +775,10 @@ int bsd_create(int32_t M, int32_t N, int32_t K, const int32_t* H_row_ptr, const 
                          12.0 + cfg.w + 8.0 + NR * (4.0 * WN + 12.0) + 4.0 + 2.0 * W2 * sizeof(int2);
     long long budget = params->workspace_bytes > 0 ? params->workspace_bytes : (4ll << 30);
     // the batched seed BP's slots: the requested count, or by default for
-    // codes of at least kBatchMinEdges edges kBatchDefaultSlots (measured on
-    // GB300: on the 35k-edge synthetic DEM the batch decodes 1.8x faster than
-    // one candidate per block of warps in single precision, on the 6912-edge
-    // phenomenological DEM 1.6x slower, where the per-iteration launches
-    // dominate); at most a quarter of the workspace
+    // codes of at least kBatchMinEdges edges kBatchDefaultSlots (on the 6912-edge
+    // phenomenological DEM the per-iteration launches dominate: 1.6x slower than
+    // per candidate; for larger codes see kBatchMinQueue); at most a quarter of
+    // the workspace
     int bs_slots = 0;
     const bool bs_default = params->batch_slots == 0 && E >= kBatchMinEdges;
     if (dec->ls.batch && (params->batch_slots > 0 || bs_default)) {

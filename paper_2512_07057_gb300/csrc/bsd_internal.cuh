@@ -334,7 +334,7 @@ struct LaunchShape {
 // optional callbacks around every kernel launch; kinds 0 seed, 1 the beam,
 // 2 its set-up, 3..6 the unrolled decoder's check / error / error adjoint / check
 // adjoint passes, 7 its other kernels, 8..10 the batched seed BP's check pass,
-// error-node pass and retirement, 11 the first-iteration screen
+// error-node pass and retirement, 11 the screens
 constexpr int kProfKinds = BSD_PROFILE_KINDS;
 struct LaunchHooks {
     void (*before)(void* ctx, int kind);

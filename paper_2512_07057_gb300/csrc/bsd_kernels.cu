@@ -7,8 +7,9 @@
 // compact 8-byte per-detector record, min1 and min2 with the sign parity in both
 // sign bits, in D's place), sum_LLR, and the bit vectors s', mask, vals, e^ and the running syndrome parity.
 //
-// Kernels (all persistent: warps claim work with one atomic per item and
-// exit when the item counter runs out, so uneven iteration counts balance):
+// Kernels (all persistent: candidate groups claim shots with one atomic and leave
+// when the counter runs out, or draw children from the beam's ring and leave when
+// every shot has ended, so uneven iteration counts balance):
 //   k_screen<DV>  (generic engines, every Lambda_j > 0, one result) a warp per
 //                 shot forms e^(1) from the columns next to flipped detectors;
 //                 finalises the shots that converge there, queues the rest
@@ -31,9 +32,10 @@
 // contraction); scores and weights are summed exactly on a 2^-16 grid.
 //
 // Masked nodes: the messages of a masked error node are set to +L_MAX when it
-// is masked.  A +L_MAX input never lowers a minimum below that of the other
-// inputs and never flips a sign, so the check pass needs no mask test; the
-// error-node pass skips masked nodes, whose messages therefore stay +L_MAX.
+// is masked.  A +L_MAX input (or a larger one, which the check pass caps) never
+// lowers a minimum below that of the other inputs and never flips a sign, so the
+// check pass needs no mask test.  The generic engine's error-node pass skips masked
+// nodes; the others take Lambda_j = +inf for them, which makes their messages +inf.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -162,9 +164,9 @@ struct BlockGroup {
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 // per-warp shared-memory footprint of one BP candidate
-// detector-side region: M records of 16 bytes (GenericEngine), or one D
-// message per edge and at least M records (SmallEngine); g.det_bytes is set
-// with the engine choice
+// detector-side region: M records of 8 bytes (GenericEngine), one D per word
+// (SmallEngine with 16-bit messages), nothing where D lies over E; g.det_bytes is
+// set with the engine choice
 __host__ __device__ inline size_t det_region_bytes(const DevGraph& g) { return (size_t)g.det_bytes; }
 
 constexpr size_t kSelectBytes = 2 * kMaxBeam * (sizeof(double) + 2 * sizeof(int));
@@ -527,20 +529,20 @@ struct GenericEngine {
 // shared-memory addresses, Lambda_j, sum_LLR and its first row's columns in
 // registers.
 //
-// What bounds the iteration: 4 shared-memory transfers per edge (54
-// wavefronts at 100% for 432 edges), and the ALU pipe, which runs min, max,
-// compare, select and logic at 64 lanes per clock (an add or multiply runs on
-// the other pipe at 128).  So the detector pass takes each edge's minimum over
-// the other five directly, with the sign product in the same instruction
-// (min.xorsign.abs: the sign of the result is the xor of the operands'), 15
-// such operations per row of six instead of 13 min/max, 6 compares, 6 selects
-// and 12 logic operations; the cap at L_MAX carries the syndrome sign.  The
+// What bounds the iteration: 4 shared-memory transfers per edge that is not held
+// in a register (44 wavefronts on [[144,12,12]], 54 if all 432 edges were in
+// memory), and the ALU pipe, which runs min, max, compare, select and logic at 64
+// lanes per clock (an add or multiply runs on the other pipe at 128).  So the
+// detector pass takes each edge's minimum over the other five directly, with the
+// sign product in the same instruction (min.xorsign.abs: the sign of the result is
+// the xor of the operands'), 15 such operations per row of six instead of 13
+// min/max, 6 compares, 6 selects and 12 logic operations; the cap at L_MAX carries
+// the syndrome sign.  The
 // stopping rule tests the parity of e^ on rows 0..31 from registers and goes on
 // to the others only if these agree with s' (before: XOR of the set columns of
-// H in every column pass and three warp reductions).  k_round on 10^6
-// [[144,12,12]] shots at p = 0.05: 25.9 -> 17.4 ms; with 32 results on 3001
-// shots: 21.3 -> 13.7 ms, 94 cycles per SM and candidate iteration against
-// the 54 of its shared-memory transfers.
+// H in every column pass and three warp reductions).  The beam of 10^6
+// [[144,12,12]] shots at p = 0.05: 25.9 -> 17.4 ms, 15.1 with the ring and the
+// register-held messages: issue, ALU and shared memory at about 60% each.
 //
 // Every value it produces is the one GenericEngine produces (same operations,
 // same order; the placement only permutes where a row's edges and a column's
@@ -2668,8 +2670,8 @@ __global__ void __launch_bounds__(Eng::kMaxThreads, Eng::kMinBlocks) k_bp_llr(De
 // RPL 2, row degree 6), 4: small (CPL 5, RPL 3, row degree 6); precision 0
 // float, 1 binary16, 2 bfloat16; then the blocks of warps and the wide engines below
 #define BSD_KIND_ALIASES(P, SFX)                          \
-    using Generic3##SFX = JaggedEngine<3, P>;             \
-    using Generic6##SFX = JaggedEngine<6, P>;             \
+    using Jagged3##SFX = JaggedEngine<3, P>;              \
+    using Jagged6##SFX = JaggedEngine<6, P>;              \
     using Generic16##SFX = GenericEngine<16, P>;          \
     using Small326##SFX = SmallEngine<3, 2, 6, P>;        \
     using Small536##SFX = SmallEngine<5, 3, 6, P>;
@@ -2677,13 +2679,13 @@ BSD_KIND_ALIASES(0, _f32)
 BSD_KIND_ALIASES(1, _f16)
 BSD_KIND_ALIASES(2, _bf16)
 // weighted min-sum (per-edge, per-iteration weights), single-precision messages: id 15 + kind
-using Generic3_w = JaggedEngine<3, 0, true>;
-using Generic6_w = JaggedEngine<6, 0, true>;
+using Jagged3_w = JaggedEngine<3, 0, true>;
+using Jagged6_w = JaggedEngine<6, 0, true>;
 using Generic16_w = GenericEngine<16, 0, true>;
 using Small326_w = SmallEngine<3, 2, 6, 0, true>;
 using Small536_w = SmallEngine<5, 3, 6, 0, true>;
 constexpr int kWeightedEngine = 15;
-// a block of warps per candidate (generic engines only): id 20 + 4 * kind + (0 float, 1 binary16,
+// a block of warps per candidate (jagged and generic engines): id 20 + 4 * kind + (0 float, 1 binary16,
 // 2 bfloat16, 3 weighted float)
 #define BSD_BLOCK_ALIASES(DV, ENGINE)                                    \
     using Block##DV##_f32 = ENGINE<DV, 0, false, BlockGroup>;            \
@@ -2706,12 +2708,12 @@ BSD_WIDE_ALIASES(3)
 BSD_WIDE_ALIASES(6)
 constexpr int kWideEngine = 32;
 #define BSD_ENGINES(X)                                                                          \
-    X(0, Generic3_f32) X(1, Generic3_f16) X(2, Generic3_bf16)                                   \
-    X(3, Generic6_f32) X(4, Generic6_f16) X(5, Generic6_bf16)                                   \
+    X(0, Jagged3_f32) X(1, Jagged3_f16) X(2, Jagged3_bf16)                                      \
+    X(3, Jagged6_f32) X(4, Jagged6_f16) X(5, Jagged6_bf16)                                      \
     X(6, Generic16_f32) X(7, Generic16_f16) X(8, Generic16_bf16)                                \
     X(9, Small326_f32) X(10, Small326_f16) X(11, Small326_bf16)                                 \
     X(12, Small536_f32) X(13, Small536_f16) X(14, Small536_bf16)                                \
-    X(15, Generic3_w) X(16, Generic6_w) X(17, Generic16_w) X(18, Small326_w) X(19, Small536_w)  \
+    X(15, Jagged3_w) X(16, Jagged6_w) X(17, Generic16_w) X(18, Small326_w) X(19, Small536_w)    \
     X(20, Block3_f32) X(21, Block3_f16) X(22, Block3_bf16) X(23, Block3_w)                      \
     X(24, Block6_f32) X(25, Block6_f16) X(26, Block6_bf16) X(27, Block6_w)                      \
     X(28, Block16_f32) X(29, Block16_f16) X(30, Block16_bf16) X(31, Block16_w)                  \

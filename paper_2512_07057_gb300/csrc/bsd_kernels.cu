@@ -2793,7 +2793,10 @@ int configure_kernels(DevGraph& g, const DecCfg& cfg, int device, int group_warp
     // candidate while eight or more candidates fit on an SM, a block of 16
     // warps per candidate beyond (8 / 16 warps: 10^5 shots of the
     // phenomenological DEM at p = 3e-3 3.42 / 2.88 ms, 5 x 10^4 in half
-    // precision 0.87 / 0.74, 3 x 10^5 of the synthetic DEM 11.2 / 10.7)
+    // precision 0.87 / 0.74, 3 x 10^5 of the synthetic DEM 11.2 / 10.7).  The rule
+    // does not know the batch: of depolarizing noise on [[144,12,12]] at p = 0.03, 1 /
+    // 8 / 16 warps, 10^5 shots take 7.6 / 9.8 / 14.3 ms, 3000 1.22 / 0.58 / 0.66, 300
+    // 0.81 / 0.31 / 0.28 (bsd_autotune and group_warps choose otherwise)
     int gw = group_warps;
     if (gw == 0) gw = (skind >= 0 || warp_smem_bytes(g) * 8 <= (size_t)max_optin) ? 1 : 16;
     // 16-bit messages that do not fit as floats stay in 16 bits on chip (the

@@ -68,7 +68,7 @@ constexpr int kRowDeg = 6;
 constexpr int kColDeg = 3;
 constexpr int kTries = 16;      // local-search restarts
 constexpr int kSweeps = 200;    // sweeps per restart
-constexpr int kLocalMoves = 20000; // moves of the single-warp engine's placement
+constexpr int kLocalMoves = 10000; // moves of the single-warp engine's placement
 
 struct Rng {                    // xorshift64*: a fixed, reproducible sequence
     uint64_t s;
